@@ -172,11 +172,11 @@ __device__ __forceinline__ void march_item(const Inst<T>& I, int set, int step, 
   a.st.th += (long long)row * I.stage_stride;
   if constexpr (sizeof(T) == 4) {
     if (I.multi) {
-      if (I.cubic) march_x2_body<true, false, true>(a, item, tid);
-      else march_x2_body<true, false, false>(a, item, tid);
+      if (I.cubic) march_x2_body<true, false, true, kThreads>(a, item, tid);
+      else march_x2_body<true, false, false, kThreads>(a, item, tid);
     } else {
-      if (I.cubic) march_x2_body<false, false, true>(a, item, tid);
-      else march_x2_body<false, false, false>(a, item, tid);
+      if (I.cubic) march_x2_body<false, false, true, kThreads>(a, item, tid);
+      else march_x2_body<false, false, false, kThreads>(a, item, tid);
     }
   } else {
     const int bx = item % I.march_bx, by = item / I.march_bx;

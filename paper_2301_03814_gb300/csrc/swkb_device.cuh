@@ -274,10 +274,10 @@ __global__ void __launch_bounds__(256) k_march(const MarchArgs<T> p) {
 
 // ----------------------------------------------------------------------------
 // (b) ray march, FP32 path with packed f32x2 arithmetic: each thread marches
-// two rays of one mode (see k_march_x2 for which).  The medium lookups stay per ray; the
-// right-hand side of the ray + variational system and the RK4 updates run on
-// register pairs, halving their issue slots (same IEEE round-to-nearest
-// operations as the scalar kernel, in the same order up to FMA contraction).
+// two rays of one mode (see march_x2_body for which).  The medium polynomials
+// are evaluated per ray; the table positions, the right-hand side of the ray +
+// variational system and the RK4 updates run on register pairs, halving their
+// issue slots.
 // ----------------------------------------------------------------------------
 struct f2 {
   unsigned long long v;
@@ -312,33 +312,49 @@ __device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {   // a b + c
   return r;
 }
 
+// floor of both lanes' positions: a round-down add of 1.5 * 2^23 (exact for
+// 0 <= u < 2^22), whose low bits are the integer
+__device__ __forceinline__ f2 add2_rd(f2 a, f2 b) {
+  f2 r;
+  asm("add.rm.ftz.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ float rcp_approx(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+// Marched state of two rays, scaled so that the right-hand side needs no
+// constant factors (c = 1 / (2 h) of the table spacing h, d1 and d2 the
+// table's derivatives p' and p''/2 in units of h):
+//   w  = (z - s) / h        w'  = 2c A          A = Q / P
+//   dQ = Q - kappa          dQ' = c B           B = d1 / P
+//   rh = r - x P_bar        rh' = D / (P_bar + P) + dQ A
+//   N  = -Z_s               N'  = -c (S + A m) / P,   m = A S + B N
+//   S  = Q_s / c            S'  = c (-4 d2 N + B m) / P
+// (r' - P_bar = (e - kappa dQ) / P - P_bar with e = D + dQ (2 kappa + dQ) and
+// P^2 = P_bar^2 + D; -P_s / P = c m / P).  The factors c, 2c, -c enter through
+// the RK4 weights.
 struct Ray2 {
-  f2 dz, dQ, rh, Zs, Qs;
+  f2 w, dQ, rh, N, S;
 };
 
-// FP32 medium lookup at table position u (intervals from the table origin;
-// the table stores the reflection, so there is no mirror step).  Returns
-// p(t), p'(t) and p''(t)/2 of the interval's quintic (derivatives in t).
-// u outside [0, top] or NaN flags ST_RANGE and is evaluated at the clamped
-// position.  floor(u) comes from one round-down add of 1.5 * 2^23 (exact for
-// 0 <= u < 2^22), keeping the conversion units free.
-__device__ __forceinline__ void horner5(const float* q, float t, float& e, float& d1, float& d2) {
-  float a0, a1, a2, a3, a4, a5;
-  load6<float>(q, a0, a1, a2, a3, a4, a5);
-  float b = a5 * t + a4;
-  float c2 = a5;
-  float c1 = a5 * t + b;
-  b = b * t + a3;
-  c2 = c2 * t + c1; c1 = c1 * t + b; b = b * t + a2;
-  c2 = c2 * t + c1; c1 = c1 * t + b; b = b * t + a1;
-  c2 = c2 * t + c1; c1 = c1 * t + b; b = b * t + a0;
+__device__ __forceinline__ void horner5(const float a[6], float t, float& e, float& d1,
+                                        float& d2) {
+  float b = a[5] * t + a[4];
+  float c2 = a[5];
+  float c1 = a[5] * t + b;
+  b = b * t + a[3];
+  c2 = c2 * t + c1; c1 = c1 * t + b; b = b * t + a[2];
+  c2 = c2 * t + c1; c1 = c1 * t + b; b = b * t + a[1];
+  c2 = c2 * t + c1; c1 = c1 * t + b; b = b * t + a[0];
   e = b; d1 = c1; d2 = c2;
 }
 
-// Cubic piece b0..b3 in tau (one 16-byte load): value, first derivative and
-// half the second derivative by synthetic division (6 FMAs).
-__device__ __forceinline__ void horner3(const float* q, float t, float& e, float& d1, float& d2) {
-  const float4 v = __ldg(reinterpret_cast<const float4*>(q));
+// Cubic piece b0..b3 in tau: value, first derivative and half the second
+// derivative by synthetic division (6 FMAs).
+__device__ __forceinline__ void horner3(const float4 v, float t, float& e, float& d1, float& d2) {
   float b = v.w * t + v.z;
   float c1 = v.w * t + b;
   b = b * t + v.y;
@@ -348,104 +364,120 @@ __device__ __forceinline__ void horner3(const float* q, float t, float& e, float
   e = b; d1 = c1; d2 = c2;
 }
 
-template <bool CUBIC>
-__device__ __forceinline__ void table_eval(const float* q, float t, float& e, float& d1,
-                                           float& d2) {
-  if (CUBIC) horner3(q, t, e, d1, d2);
-  else horner5(q, t, e, d1, d2);
-}
-
-// CUBIC: the table holds cubic pieces (4 slots each, u in piece units).
+// One entry of the FP32 medium table at its local coordinate t: p(t), p'(t)
+// and p''(t)/2.  MULTI: the entry holds a column's coefficients and their
+// differences to the next column, blended with weight th before the
+// polynomial is evaluated (4 + 6 FMAs for a cubic piece; evaluating both
+// columns and blending the results takes 18).
 template <bool MULTI, bool CUBIC>
-__device__ __forceinline__ void med32(const MarchArgs<float>& p, int l, float u, float& e,
-                                      float& d1, float& d2, unsigned& st) {
-  constexpr int W = CUBIC ? 4 : 8;
-  const float uc = fminf(fmaxf(u, 0.f), p.med.top);
-  if (uc != u) st |= ST_RANGE;
-  const float v = __fadd_rd(uc, 12582912.f);
-  const int i = (int)(__float_as_uint(v) - 0x4B400000u);
-  const float t = uc - (v - 12582912.f);
-  if (!MULTI) {
-    table_eval<CUBIC>(p.med.coef + bchk((long long)i * W, p.med.size - (W - 1), st), t, e, d1, d2);
-  } else {
-    const int c = __ldg(p.st.c + l);
-    const float th = __ldg(p.st.th + l);
-    const float* q = p.med.coef + bchk((long long)c * p.med.col_stride + (long long)i * W,
-                                       p.med.size - (th == 0.f ? W - 1 : p.med.col_stride + W - 1),
-                                       st);
-    if (th == 0.f) {
-      table_eval<CUBIC>(q, t, e, d1, d2);
-    } else if (th == 1.f) {
-      table_eval<CUBIC>(q + p.med.col_stride, t, e, d1, d2);
-    } else {
-      float e0, e1, f0, f1, g0, g1;
-      table_eval<CUBIC>(q, t, e0, f0, g0);
-      table_eval<CUBIC>(q + p.med.col_stride, t, e1, f1, g1);
-      e = (1.f - th) * e0 + th * e1;
-      d1 = (1.f - th) * f0 + th * f1;
-      d2 = (1.f - th) * g0 + th * g1;
+__device__ __forceinline__ void table_eval(const float* q, float t, float th, float& e, float& d1,
+                                           float& d2) {
+  if constexpr (CUBIC) {
+    float4 v = __ldg(reinterpret_cast<const float4*>(q));
+    if constexpr (MULTI) {
+      const float4 d = __ldg(reinterpret_cast<const float4*>(q + 4));
+      v.x = fmaf(th, d.x, v.x);
+      v.y = fmaf(th, d.y, v.y);
+      v.z = fmaf(th, d.z, v.z);
+      v.w = fmaf(th, d.w, v.w);
     }
+    horner3(v, t, e, d1, d2);
+  } else {
+    float a[6];
+    load6<float>(q, a[0], a[1], a[2], a[3], a[4], a[5]);
+    if constexpr (MULTI) {
+      float d[6];
+      load6<float>(q + 8, d[0], d[1], d[2], d[3], d[4], d[5]);
+#pragma unroll
+      for (int k = 0; k < 6; ++k) a[k] = fmaf(th, d[k], a[k]);
+    }
+    horner5(a, t, e, d1, d2);
   }
 }
 
-// x-form right-hand side for two rays; u2 = their table positions.  With
-// he = eps_z / 2 and hee = eps_zz / 2 (table derivatives times 1 / (2 h) and
-// 1 / h^2):  z' = Q/P,  Q' = he/P,  r' - P_bar as in the scalar kernel,
-//   -P_s/P = (Q Q_s - he Z_s)/P^2,  Z_s' = (Q_s + Q (-P_s/P))/P,
-//   Q_s' = (hee Z_s + he (-P_s/P))/P.
+// Running extremes of a ray pair, tested once per ray: table position, P^2
+// (<= 0: turning point) and -Z_s (>= 0: caustic).  A ray that meets one goes on
+// with values that are discarded; its table reads are clamped.  The
+// comparisons drop NaNs: a ray that turns NaN stays NaN, and its landing is
+// tested explicitly.
+struct Extremes {
+  float u_lo, u_hi, P2, N;
+};
+
+// FP32 medium lookup of both rays at table positions u2 (intervals or pieces
+// from the table origin; the table stores the reflection, so there is no
+// mirror step).
 template <bool MULTI, bool CUBIC>
-__device__ __forceinline__ Ray2 rhs2(const MarchArgs<float>& p, int l, f2 u2, f2 kap, f2 m2kap,
-                                     f2 mkap, f2 pb, f2 mpb, float pb2, f2 pb2v, f2 ihh,
-                                     f2 mihh, f2 ihq, const Ray2& y, unsigned& st, float& mnP,
-                                     float& mnZ) {
-  float ua, ub;
+__device__ __forceinline__ void med32x2(const MarchArgs<float>& p, int l, f2 u2, f2& e, f2& d1,
+                                        float& d2a, float& d2b, Extremes& x, unsigned& st) {
+  constexpr int W = (CUBIC ? 4 : 8) * (MULTI ? 2 : 1);
+  const f2 magic = bc2(12582912.f);
+  const f2 v = add2_rd(u2, magic);
+  const f2 t = sub2(u2, sub2(v, magic));
+  float ua, ub, va, vb, ta, tb;
   sp2(u2, ua, ub);
-  float ea, d1a, d2a, eb, d1b, d2b;
-  med32<MULTI, CUBIC>(p, l, ua, ea, d1a, d2a, st);
-  med32<MULTI, CUBIC>(p, l, ub, eb, d1b, d2b, st);
-  const f2 e = mk2(ea, eb), d1 = mk2(d1a, d1b);
-  const f2 he = mul2(d1, ihh), mhe = mul2(d1, mihh), hee = mul2(mk2(d2a, d2b), ihq);
-  const f2 Q = add2(kap, y.dQ);
-  const f2 D = fma2(y.dQ, sub2(m2kap, y.dQ), e);           // e - dQ (2 kappa + dQ)
-  float P2a, P2b;
-  sp2(add2(pb2v, D), P2a, P2b);
-  // Turning points (P^2 <= 0) and caustics (Z_s <= 0) at any stage: running
-  // minima, checked once after the march (a ray that meets one goes on with
-  // NaN values; its table positions are clamped, its status is an error).
-  float Zsa, Zsb;
-  sp2(y.Zs, Zsa, Zsb);
-  mnP = fminf(mnP, fminf(P2a, P2b));
-  mnZ = fminf(mnZ, fminf(Zsa, Zsb));
-  (void)pb2;
-  const float iPa = rsqrtf(P2a), iPb = rsqrtf(P2b);
-  const f2 iP = mk2(iPa, iPb);
-  const f2 P = mul2(mk2(P2a, P2b), iP);
-  float da, db;
-  sp2(add2(pb, P), da, db);
-  const f2 rden = mk2(__fdividef(1.f, da), __fdividef(1.f, db));
-  Ray2 d;
-  d.dz = mul2(Q, iP);
-  d.dQ = mul2(he, iP);
-  // (e - kappa dQ - P_bar D / (P_bar + P)) / P
-  d.rh = mul2(fma2(mpb, mul2(D, rden), fma2(mkap, y.dQ, e)), iP);
-  const f2 mPsiP = mul2(fma2(mhe, y.Zs, mul2(Q, y.Qs)), mul2(iP, iP));
-  d.Zs = mul2(fma2(Q, mPsiP, y.Qs), iP);
-  d.Qs = mul2(fma2(he, mPsiP, mul2(hee, y.Zs)), iP);
-  return d;
+  sp2(v, va, vb);
+  sp2(t, ta, tb);
+  x.u_lo = fminf(x.u_lo, fminf(ua, ub));
+  x.u_hi = fmaxf(x.u_hi, fmaxf(ua, ub));
+  // unsigned: positions below 0 and NaN wrap to large indices
+  const unsigned n = (unsigned)p.med.n_int;
+  const unsigned ia = min(__float_as_uint(va) - 0x4B400000u, n);
+  const unsigned ib = min(__float_as_uint(vb) - 0x4B400000u, n);
+  const float* base = p.med.coef;
+  float th = 0.f;
+  if constexpr (MULTI) {
+    base += (long long)__ldg(p.st.c + l) * p.med.col_stride;
+    th = __ldg(p.st.th + l);
+  }
+  const long long off = base - p.med.coef;
+  float ea, eb, d1a, d1b;
+  table_eval<MULTI, CUBIC>(base + (bchk(off + (long long)ia * W, p.med.size - (W - 1), st) - off),
+                           ta, th, ea, d1a, d2a);
+  table_eval<MULTI, CUBIC>(base + (bchk(off + (long long)ib * W, p.med.size - (W - 1), st) - off),
+                           tb, th, eb, d1b, d2b);
+  e = mk2(ea, eb);
+  d1 = mk2(d1a, d1b);
 }
 
-__device__ __forceinline__ Ray2 axpy2(const Ray2& y, f2 a, const Ray2& k) {
-  return Ray2{fma2(a, k.dz, y.dz), fma2(a, k.dQ, y.dQ), fma2(a, k.rh, y.rh), fma2(a, k.Zs, y.Zs),
-              fma2(a, k.Qs, y.Qs)};
+// Right-hand side of the scaled system above for two rays at table positions
+// u2, without the factors 2c, c, 1, -c, c: d.w = A, d.dQ = B, ...
+template <bool MULTI, bool CUBIC>
+__device__ __forceinline__ Ray2 rhs2(const MarchArgs<float>& p, int l, f2 u2, f2 kap, f2 m2kap,
+                                     f2 pb, f2 pb2v, const Ray2& y, Extremes& x, unsigned& st) {
+  f2 e, d1;
+  float d2a, d2b;
+  med32x2<MULTI, CUBIC>(p, l, u2, e, d1, d2a, d2b, x, st);
+  const f2 Q = add2(kap, y.dQ);
+  const f2 D = fma2(y.dQ, sub2(m2kap, y.dQ), e);           // e - dQ (2 kappa + dQ)
+  const f2 P2 = add2(pb2v, D);
+  float P2a, P2b, Na, Nb;
+  sp2(P2, P2a, P2b);
+  sp2(y.N, Na, Nb);
+  x.P2 = fminf(x.P2, fminf(P2a, P2b));
+  x.N = fmaxf(x.N, fmaxf(Na, Nb));
+  const f2 iP = mk2(rsqrtf(P2a), rsqrtf(P2b));
+  float da, db;
+  sp2(fma2(P2, iP, pb), da, db);                           // P_bar + P
+  const f2 rden = mk2(rcp_approx(da), rcp_approx(db));
+  Ray2 d;
+  d.w = mul2(Q, iP);
+  d.dQ = mul2(d1, iP);
+  d.rh = fma2(D, rden, mul2(y.dQ, d.w));
+  const f2 m = fma2(d.dQ, y.N, mul2(d.w, y.S));
+  d.N = mul2(fma2(d.w, m, y.S), iP);
+  d.S = mul2(fma2(d.dQ, m, mul2(mul2(mk2(d2a, d2b), bc2(-4.f)), y.N)), iP);
+  return d;
 }
 
 // Thread t marches rays q and q + NH of mode r, t = q Mr + r (NH = ceil(NRT / 2)):
 // a warp's lanes are consecutive modes at one launch height (their table
 // reads stay within a few intervals) and no lane idles at the end of a row.
-template <bool MULTI, bool PLANES, bool CUBIC>
+// THREADS threads per block.
+template <bool MULTI, bool PLANES, bool CUBIC, int THREADS>
 __device__ __forceinline__ void march_x2_body(const MarchArgs<float>& p, int blk, int tid) {
   const int NH = (p.NRT + 1) >> 1;
-  const int t = blk * 256 + tid;
+  const int t = blk * THREADS + tid;
   if (t >= p.Mr * NH) return;
   const int ja = t / p.Mr;
   const int r = t - ja * p.Mr;
@@ -457,88 +489,109 @@ __device__ __forceinline__ void march_x2_body(const MarchArgs<float>& p, int blk
   // launch heights in table intervals
   const float ua = fmaf(float((ja - p.G) * p.R), p.u_dz, p.u_lo);
   const float ub = has_b ? fmaf(float((jb - p.G) * p.R), p.u_dz, p.u_lo) : ua;
-  const f2 s = mk2(ua, ub), kv = bc2(kap), m2kap = bc2(-2.f * kap), mkap = bc2(-kap);
-  const f2 pbv = bc2(pb), mpb = bc2(-pb), pb2v = bc2(pb2);
-  const float ihs = p.med.inv_h;
-  const f2 ih = bc2(ihs), ihh = bc2(0.5f * ihs), mihh = bc2(-0.5f * ihs);
-  const f2 ihq = bc2(0.5f * p.med.inv_h2);   // inv_h2 = 2 / h^2
-  float e0a, e0b, t0, t1;
-  med32<MULTI, CUBIC>(p, 0, ua, e0a, t0, t1, st);
-  med32<MULTI, CUBIC>(p, 0, ub, e0b, t0, t1, st);
-  float P0a = pb2 + e0a, P0b = pb2 + e0b;
+  const f2 s = mk2(ua, ub), kv = bc2(kap), m2kap = bc2(-2.f * kap);
+  const f2 pbv = bc2(pb), pb2v = bc2(pb2);
+  const f2 zero = bc2(0.f);
+  Extremes x{ua, ua, 1.f, -1.f};   // P^2 and Z_s start at 1: none below
+  f2 e0, d0;
+  float t0, t1;
+  med32x2<MULTI, CUBIC>(p, 0, s, e0, d0, t0, t1, x, st);
+  float P0a, P0b;
+  sp2(add2(pb2v, e0), P0a, P0b);
   if (!(P0a > 0.f)) { st |= ST_TURNING; P0a = pb2; }
   if (!(P0b > 0.f)) { st |= ST_TURNING; P0b = pb2; }
   P0a = sqrtf(P0a);
   P0b = sqrtf(P0b);
-  const f2 zero = bc2(0.f);
-  Ray2 y{zero, zero, zero, bc2(1.f), zero};
-  const f2 h = bc2(p.h), hh = bc2(0.5f * p.h), h6 = bc2(p.h / 6.f);
-  // table position of a ray: launch position + dz / h_table
-  const auto pos = [&](const Ray2& w) { return fma2(w.dz, ih, s); };
+  Ray2 y{zero, zero, zero, bc2(-1.f), zero};
+  const float c = 0.5f * p.med.inv_h, H = c * p.h;
+  // RK4 weights 1/2, 1, 1/6, 1/3 times the factors of the scaled system
+  const f2 H2 = bc2(0.5f * H), H1 = bc2(H), H6 = bc2(H / 6.f), H3 = bc2(H / 3.f);
+  const f2 W1 = bc2(2.f * H), W3 = bc2(2.f * H / 3.f);          // w: H1, W1, H3, W3
+  const f2 n2 = bc2(-0.5f * H), n1 = bc2(-H), n6 = bc2(-H / 6.f), n3 = bc2(-H / 3.f);
+  const f2 h6 = bc2(p.h / 6.f), h3 = bc2(p.h / 3.f);
+  const float w_out = p.inv_dz / p.med.inv_h;
   // landing quantities at RK4 stage l (the screen's end, or a plane inside it)
   const auto land = [&](int l, float* od, float* oph, float* oam) {
     const long long nrm = (long long)p.NRT * p.Mr;
     const long long oa = bchk((long long)ja * p.Mr + r, nrm, st);
     const long long ob = has_b ? bchk((long long)jb * p.Mr + r, nrm, st) : oa;
-    float dza, dzb, dQa, dQb, rha, rhb, Zsa, Zsb, u1a, u1b;
-    sp2(y.dz, dza, dzb);
+    float wa, wb, dQa, dQb, rha, rhb, Na, Nb, u1a, u1b, e1a, e1b;
+    sp2(y.w, wa, wb);
     sp2(y.dQ, dQa, dQb);
     sp2(y.rh, rha, rhb);
-    sp2(y.Zs, Zsa, Zsb);
-    sp2(pos(y), u1a, u1b);
-    if (!(Zsa > 0.f) || !(Zsb > 0.f)) st |= ST_CAUSTIC;
-    float e1a, e1b, s0, s1;
-    med32<MULTI, CUBIC>(p, l, u1a, e1a, s0, s1, st);
-    med32<MULTI, CUBIC>(p, l, u1b, e1b, s0, s1, st);
+    sp2(y.N, Na, Nb);
+    const f2 u1 = add2(s, y.w);
+    sp2(u1, u1a, u1b);
+    if (!(Na < 0.f) || !(Nb < 0.f)) st |= ST_CAUSTIC;
+    if (!(u1a >= 0.f && u1a <= p.med.top) || !(u1b >= 0.f && u1b <= p.med.top)) st |= ST_RANGE;
+    f2 e1, d1;
+    float s0, s1;
+    med32x2<MULTI, CUBIC>(p, l, u1, e1, d1, s0, s1, x, st);
+    sp2(e1, e1a, e1b);
     float P1a = pb2 + e1a - dQa * (2.f * kap + dQa);
     float P1b = pb2 + e1b - dQb * (2.f * kap + dQb);
     if (!(P1a > 0.f)) { st |= ST_TURNING; P1a = pb2; }
     if (!(P1b > 0.f)) { st |= ST_TURNING; P1b = pb2; }
-    const float Za = Zsa > 0.f ? Zsa : 1.f, Zb = Zsb > 0.f ? Zsb : 1.f;
-    od[oa] = dza * p.inv_dz;
+    const float Za = Na < 0.f ? -Na : 1.f, Zb = Nb < 0.f ? -Nb : 1.f;
+    od[oa] = wa * w_out;
     oph[oa] = rha * p.k_over_2pi;
     oam[oa] = sqrtf(P0a * rsqrtf(P1a) / Za);
     if (has_b) {
-      od[ob] = dzb * p.inv_dz;
+      od[ob] = wb * w_out;
       oph[ob] = rhb * p.k_over_2pi;
       oam[ob] = sqrtf(P0b * rsqrtf(P1b) / Zb);
     }
   };
   // RK4: y + h/6 k1 + h/3 k2 + h/3 k3 + h/6 k4, accumulated as the stages
-  // complete (k1..k3 need not stay live)
-  const f2 h3 = bc2(p.h / 3.f);
-  float mnP = 1.f, mnZ = 1.f;   // smallest P^2 and Z_s met (1: none below)
+  // complete (k1..k3 need not stay live).  A stage state needs no rh, and its
+  // w only as the table position u.
   for (int n = 0; n < p.Nt; ++n) {
-    const Ray2 k1 = rhs2<MULTI, CUBIC>(p, 2 * n, pos(y), kv, m2kap, mkap, pbv, mpb, pb2, pb2v, ihh,
-                                mihh, ihq, y, st, mnP, mnZ);
-    Ray2 acc = axpy2(y, h6, k1);
-    const Ray2 y2 = axpy2(y, hh, k1);
-    const Ray2 k2 = rhs2<MULTI, CUBIC>(p, 2 * n + 1, pos(y2), kv, m2kap, mkap, pbv, mpb, pb2, pb2v,
-                                ihh, mihh, ihq, y2, st, mnP, mnZ);
-    acc = axpy2(acc, h3, k2);
-    const Ray2 y3 = axpy2(y, hh, k2);
-    const Ray2 k3 = rhs2<MULTI, CUBIC>(p, 2 * n + 1, pos(y3), kv, m2kap, mkap, pbv, mpb, pb2, pb2v,
-                                ihh, mihh, ihq, y3, st, mnP, mnZ);
-    acc = axpy2(acc, h3, k3);
-    const Ray2 y4 = axpy2(y, h, k3);
-    const Ray2 k4 = rhs2<MULTI, CUBIC>(p, 2 * n + 2, pos(y4), kv, m2kap, mkap, pbv, mpb, pb2, pb2v,
-                                ihh, mihh, ihq, y4, st, mnP, mnZ);
-    y = axpy2(acc, h6, k4);
+    const f2 u0 = add2(s, y.w);
+    Ray2 acc = y;
+    const auto add = [&](const Ray2& k, f2 gw, f2 gq, f2 gr, f2 gn) {
+      acc = Ray2{fma2(gw, k.w, acc.w), fma2(gq, k.dQ, acc.dQ), fma2(gr, k.rh, acc.rh),
+                 fma2(gn, k.N, acc.N), fma2(gq, k.S, acc.S)};
+    };
+    const auto stage = [&](const Ray2& k, f2 gq, f2 gn) {
+      return Ray2{zero, fma2(gq, k.dQ, y.dQ), zero, fma2(gn, k.N, y.N), fma2(gq, k.S, y.S)};
+    };
+    const Ray2 k1 = rhs2<MULTI, CUBIC>(p, 2 * n, u0, kv, m2kap, pbv, pb2v, y, x, st);
+    add(k1, H3, H6, h6, n6);
+    const Ray2 k2 = rhs2<MULTI, CUBIC>(p, 2 * n + 1, fma2(H1, k1.w, u0), kv, m2kap, pbv, pb2v,
+                                       stage(k1, H2, n2), x, st);
+    add(k2, W3, H3, h3, n3);
+    const Ray2 k3 = rhs2<MULTI, CUBIC>(p, 2 * n + 1, fma2(H1, k2.w, u0), kv, m2kap, pbv, pb2v,
+                                       stage(k2, H2, n2), x, st);
+    add(k3, W3, H3, h3, n3);
+    const Ray2 k4 = rhs2<MULTI, CUBIC>(p, 2 * n + 2, fma2(W1, k3.w, u0), kv, m2kap, pbv, pb2v,
+                                       stage(k3, H1, n1), x, st);
+    add(k4, H3, H6, h6, n6);
+    y = acc;
     if (PLANES && (n + 1) % p.plane_steps == 0 && n + 1 < p.Nt) {
       const long long po = (long long)((n + 1) / p.plane_steps - 1) * p.NRT * p.Mr;
       land(2 * (n + 1), p.pl_d + po, p.pl_ph + po, p.pl_a + po);
     }
   }
   land(2 * p.Nt, p.out_d, p.out_ph, p.out_a);
-  if (!(mnP > 0.f)) st |= ST_TURNING;
-  if (!(mnZ > 0.f)) st |= ST_CAUSTIC;
+  if (!(x.P2 > 0.f)) st |= ST_TURNING;
+  if (!(x.N < 0.f)) st |= ST_CAUSTIC;
+  if (!(x.u_lo >= 0.f && x.u_hi <= p.med.top)) st |= ST_RANGE;
   if (st) atomicOr(p.status, st);
 }
 
-// 4 CTAs of 256 threads per SM (64 registers)
+// Bound by the FMA pipe: ~72 of its cycles per ray-pair stage (14 FFMA2, 8
+// FMUL2, 6 FADD2 at two cycles each, 12 FFMA of the medium, 2 IMAD), busy 64 %
+// of the time that CTAs are resident; 61 instructions in all.  On the
+// 16384-point duct (489 modes x 2086 rays, 16 RK4 steps) 102 us, against 121
+// with the unscaled system (35 packed operations, 80 instructions); 326
+// against 485 us on a range-dependent table (698 modes x 4118 rays).
+// 6 CTAs of 128 threads per SM (80 registers): 102 us; 3 of 256: 104; 4 of
+// 256 (64 registers, spills): 112; 2 of 256: 107; all-scalar arithmetic: 110.
+constexpr int MARCH_THREADS = 128;
+
 template <bool MULTI, bool PLANES, bool CUBIC>
-__global__ void __launch_bounds__(256, 4) k_march_x2(const MarchArgs<float> p) {
-  march_x2_body<MULTI, PLANES, CUBIC>(p, blockIdx.x, threadIdx.x);
+__global__ void __launch_bounds__(MARCH_THREADS, 6) k_march_x2(const MarchArgs<float> p) {
+  march_x2_body<MULTI, PLANES, CUBIC, MARCH_THREADS>(p, blockIdx.x, threadIdx.x);
 }
 
 // ----------------------------------------------------------------------------

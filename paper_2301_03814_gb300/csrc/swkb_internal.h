@@ -37,7 +37,9 @@ template <> struct C2<double> { using type = double2; };
 //   before that pad and top = n_int as a float.  When pieces = S > 0 every
 //   interval is stored as S cubic Hermite pieces of its quintic (value and
 //   slope matched at the piece ends; 4 slots b0..b3 in the piece's own
-//   tau in [0, 1]) and n_int, top, inv_h, inv_h2 count pieces.
+//   tau in [0, 1]) and n_int, top, inv_h, inv_h2 count pieces.  With several
+//   columns every entry is followed by its difference to the next column's
+//   entry (twice the slots), and the last column has no rows of its own.
 template <typename T>
 struct Medium {
   const T* coef;

@@ -86,7 +86,8 @@ cudaError_t launch_march(const MarchArgs<T>& a, bool multi_column, cudaStream_t 
 template <>
 cudaError_t launch_march<float>(const MarchArgs<float>& a, bool multi_column, cudaStream_t s) {
   const long long threads = (long long)a.Mr * ((a.NRT + 1) / 2);
-  const dim3 block(256), grid((unsigned)((threads + 255) / 256));
+  const dim3 block(MARCH_THREADS),
+      grid((unsigned)((threads + MARCH_THREADS - 1) / MARCH_THREADS));
   const bool pl = a.plane_steps > 0, cub = a.med.pieces > 0;
   if (cub) {
     if (pl)

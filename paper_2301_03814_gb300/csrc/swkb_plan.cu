@@ -249,6 +249,13 @@ namespace {
 
 // Intervals of the FP32 medium table of one column (layout in swkb_internal.h).
 int table32_intervals(const swkb_plan* p) { return (p->mirror ? 2 : 1) * p->n_int + 1; }
+// Its columns as stored (with several, each holds the differences to the
+// next one too, so the last needs none of its own) and the values of one.
+int table32_columns(const swkb_plan* p) { return p->n_cols > 1 ? p->n_cols - 1 : 1; }
+long long table32_values(const swkb_plan* p) {
+  return (long long)table32_intervals(p) * (p->pieces > 0 ? 4 * p->pieces : 8) *
+         (p->n_cols > 1 ? 2 : 1);
+}
 
 // Quintic Hermite interpolant of eps - eps_ref on every profile interval, as
 // monomial coefficients a0..a5 in t in [0, 1] (8 slots per interval).
@@ -496,7 +503,20 @@ swkb_status build_device(swkb_plan* p, const swkb_profile* prof) {
         std::vector<double> cub((size_t)p->n_cols * nt * S * 4);
         for (size_t k = 0; k < (size_t)p->n_cols * nt; ++k)
           for (int sp = 0; sp < S; ++sp) cubic_piece(c32.data() + k * 8, sp, S, &cub[(k * S + sp) * 4]);
-        TRY(upload<T>(p, &p->coef, cub));
+        c32.swap(cub);
+      }
+      if (p->n_cols > 1) {
+        // each entry of a column followed by its difference to the next one
+        const size_t w = p->pieces > 0 ? 4 : 8, per = c32.size() / p->n_cols;
+        std::vector<T> pairs((size_t)(p->n_cols - 1) * per * 2);
+        T* o = pairs.data();
+        for (size_t k = 0; k + per < c32.size(); k += w, o += 2 * w)
+          for (size_t j = 0; j < w; ++j) {
+            o[j] = (T)c32[k + j];
+            o[w + j] = (T)(c32[k + per + j] - c32[k + j]);
+          }
+        TRY(dev_alloc(p, &p->coef, pairs.size() * sizeof(T)));
+        CK(cudaMemcpy(p->coef, pairs.data(), pairs.size() * sizeof(T), cudaMemcpyHostToDevice));
       } else {
         TRY(upload<T>(p, &p->coef, c32));
       }
@@ -699,13 +719,13 @@ MarchArgs<T> march_args(const swkb_plan* p, int q) {
     const int S = p->pieces > 0 ? p->pieces : 1;
     const double hs = p->dzp / S;
     a.med.n_int = (p->mirror ? 2 : 1) * p->n_int * S;
-    a.med.col_stride = (long long)table32_intervals(p) * (p->pieces > 0 ? 4 * S : 8);
+    a.med.col_stride = table32_values(p);
     a.med.z0 = (T)z0;
     a.med.inv_h = (T)(1.0 / hs);
     a.med.inv_h2 = (T)(2.0 / (hs * hs));
     a.med.mirrored = 0;
     a.med.pieces = p->pieces;
-    a.med.size = (long long)p->n_cols * a.med.col_stride;
+    a.med.size = (long long)table32_columns(p) * a.med.col_stride;
     a.med.top = (T)a.med.n_int;
     a.u_lo = (T)((p->z_lo - z0) / hs);
     a.u_dz = (T)(p->dz / hs);
@@ -1664,9 +1684,8 @@ swkb_status configure(swkb_plan* p, const swkb_profile* prof, double k, const sw
 size_t device_bytes(const swkb_plan* p) {
   const size_t T = p->precision == SWKB_FP64 ? 8 : 4, V = 2 * T;
   const size_t S = 2 * (size_t)p->Nt + 1;
-  size_t b = (size_t)p->n_cols * (T == 8 ? (size_t)p->n_int * 8                      // medium
-                                          : (size_t)table32_intervals(p) *
-                                                (p->pieces > 0 ? 4 * p->pieces : 8)) * T;
+  size_t b = (T == 8 ? (size_t)p->n_cols * p->n_int * 8                              // medium
+                     : (size_t)table32_columns(p) * table32_values(p)) * T;
   b += (size_t)p->stage_rows * S * (sizeof(int) + T);               // stage columns
   b += 3 * (size_t)p->M * T + (size_t)p->M * V;                     // mode tables
   b += (size_t)p->N * V;                                            // twiddles
