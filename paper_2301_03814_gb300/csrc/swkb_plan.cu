@@ -302,12 +302,24 @@ void cubic_piece(const double* a, int s, int S, double* b) {
   b[3] = 2.0 * (f0 - f1) + d0 + d1;
 }
 
+// The smallest curvature deviation an FP32 march can tell: over one screen a
+// deviation d of eps_zz moves Z_s by at most d dx^2 / (4 P^2), P^2 >= eps_ref -
+// kappa_max^2; at 2^-26 P^2 / dx^2 that is an eighth of the rounding of Z_s.
+double curvature_floor(const swkb_plan* p) {
+  const double kmax = 2.0 * M_PI * p->n_max / (p->k * p->L);
+  return ldexp(std::max(p->eps_ref - kmax * kmax, 0.0), -26) / (p->dx * p->dx);
+}
+
 // FP32 plans evaluate each interval's quintic through S cubic Hermite pieces
 // (6 FMAs per lookup instead of 12).  S is the smallest of 1, 2, 4, 8, 16 for
 // which, at the quarter points of every piece, value, slope and curvature of
 // the pieces stay within 1e-7, 1e-6 and 1e-4 of the table's largest |e|, |e_z|
-// and |e_zz| (e = eps - eps_ref): far below what the FP32 march resolves.
-// 0 when none does (the quintic itself is evaluated).
+// and |e_zz| (e = eps - eps_ref): far below what the FP32 march resolves.  The
+// curvature's bound is not taken below curvature_floor: media broad against
+// the table spacing (or linear) have an e_zz of the order of the table's own
+// rounding, which no number of pieces reproduces (open lens of 131072 points,
+// spacing 1/16, width 7282: one piece instead of the quintic, 425 against 495
+// us per march).  0 when none does (the quintic itself is evaluated).
 int choose_pieces(const swkb_plan* p, const std::vector<double>& coef) {
   const double h = p->dzp;
   const size_t n = (size_t)p->n_cols * p->n_int;
@@ -322,7 +334,7 @@ int choose_pieces(const swkb_plan* p, const std::vector<double>& coef) {
       E2 = std::max(E2, fabs(d2) / (h * h));
     }
   }
-  const double tol[3] = {1e-7 * E0, 1e-6 * E1, 1e-4 * E2};
+  const double tol[3] = {1e-7 * E0, 1e-6 * E1, std::max(1e-4 * E2, curvature_floor(p))};
   // largest deviations of S pieces from the quintic (value, slope, curvature);
   // with stop set, returns as soon as one exceeds its bound
   auto worst = [&](int S, double dev[3], bool stop) {
@@ -365,7 +377,7 @@ int choose_pieces(const swkb_plan* p, const std::vector<double>& coef) {
 }
 
 // choose_pieces depends only on the table (and eps_ref, the ground
-// reflection): remembered by a 64-bit FNV-1a hash of those, so that the
+// reflection, the curvature floor): remembered by a 64-bit FNV-1a hash of those, so that the
 // budget estimate and the creation of the same request's plan scan it once.
 uint64_t table_hash(const swkb_plan* p, const swkb_profile* prof) {
   uint64_t h = 1469598103934665603ull;
@@ -377,7 +389,7 @@ uint64_t table_hash(const swkb_plan* p, const swkb_profile* prof) {
   mix(prof->eps, nt * sizeof(double));
   mix(prof->eps_z, nt * sizeof(double));
   mix(prof->eps_zz, nt * sizeof(double));
-  const double sc[2] = {p->eps_ref, p->dzp};
+  const double sc[3] = {p->eps_ref, p->dzp, curvature_floor(p)};
   const int ic[3] = {p->n_cols, p->n_p, p->mirror};
   mix(sc, sizeof(sc));
   mix(ic, sizeof(ic));
