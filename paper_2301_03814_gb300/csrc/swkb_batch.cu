@@ -86,7 +86,7 @@ struct Inst {
   double* out;                     // n_z complex128 output
   typename C2<T>::type* u;         // the plan's period field
   int n_z, N, mirror, q0, stage_rows, stage_stride, multi, cubic;
-  int march_bx, march_blocks, bracket_bx, fft1_blocks, fft2_blocks, resum_blocks, resum_pw;
+  int march_blocks, bracket_bx, fft1_blocks, fft2_blocks, resum_blocks, resum_pw;
   int reduce_n, out_off;
 };
 
@@ -179,9 +179,8 @@ __device__ __forceinline__ void march_item(const Inst<T>& I, int set, int step, 
       else march_x2_body<false, false, false, kThreads>(a, item, tid);
     }
   } else {
-    const int bx = item % I.march_bx, by = item / I.march_bx;
-    if (I.multi) march_body<T, true, false>(a, bx, by, tid & 31, tid >> 5);
-    else march_body<T, false, false>(a, bx, by, tid & 31, tid >> 5);
+    if (I.multi) march64_body<true, false, kThreads>(a, item, tid);
+    else march64_body<false, false, kThreads>(a, item, tid);
   }
 }
 
@@ -457,7 +456,7 @@ swkb_status build(swkb_batch* b, const swkb_request* reqs, const swkb_batch_opti
     I.n_z = pp.n_z; I.N = pp.N; I.mirror = pp.mirror; I.q0 = reqs[i].q0;
     I.stage_rows = pp.stage_rows; I.stage_stride = pp.stage_stride;
     I.multi = pp.n_cols > 1; I.cubic = pp.pieces > 0;
-    I.march_bx = pp.march_bx; I.march_blocks = pp.march_blocks; I.bracket_bx = pp.bracket_bx;
+    I.march_blocks = pp.march_blocks; I.bracket_bx = pp.bracket_bx;
     I.fft1_blocks = pp.fft1_blocks; I.fft2_blocks = pp.fft2_blocks;
     I.resum_blocks = pp.resum_blocks; I.resum_pw = pp.resum_pw;
     I.reduce_n = pp.reduce_n; I.out_off = pp.out_off;

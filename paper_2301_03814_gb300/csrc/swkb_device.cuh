@@ -88,13 +88,6 @@ __device__ __forceinline__ float minus_rint(float t) {
 }
 __device__ __forceinline__ double minus_rint(double t) { return t - rint(t); }
 
-// 1/sqrt: FP32 via the special-function unit (2 ulp), FP64 correctly-rounded
-// to 1 ulp.  Small-quotient division: FP32 fast (2 ulp), FP64 IEEE.
-__device__ __forceinline__ float rsqrt_t(float x) { return rsqrtf(x); }
-__device__ __forceinline__ double rsqrt_t(double x) { return rsqrt(x); }
-__device__ __forceinline__ float fdiv_t(float a, float b) { return __fdividef(a, b); }
-__device__ __forceinline__ double fdiv_t(double a, double b) { return a / b; }
-
 template <typename T>
 __device__ __forceinline__ void load6(const T* p, T& a0, T& a1, T& a2, T& a3, T& a4, T& a5);
 
@@ -116,160 +109,208 @@ __device__ __forceinline__ void load6<double>(const double* p, double& a0, doubl
 }
 
 // ----------------------------------------------------------------------------
-// medium: quintic in z per interval, linear in x between two columns
-// ----------------------------------------------------------------------------
-template <typename T>
-__device__ __forceinline__ void col_eval(const Medium<T>& m, int c, T zz, T& e, T& ez, T& ezz,
-                                         unsigned& st) {
-  const T u = (zz - m.z0) * m.inv_h;
-  // outside [0, n_int] (or NaN): flag; the interval index is clamped in
-  // integers (a flagged ray's values are discarded, its reads stay in bounds)
-  if (!(u >= T(0) && u <= T(m.n_int))) st |= ST_RANGE;
-  const int i = min(max((int)floor(u), 0), m.n_int - 1);
-  const T t = u - T(i);
-  T a0, a1, a2, a3, a4, a5;
-  load6<T>(m.coef + bchk((long long)c * m.col_stride + (long long)i * 8, m.size - 7, st), a0, a1,
-           a2, a3, a4, a5);
-  // Horner with derivatives (synthetic division): p, p', p''/2 at t
-  T b = a5 * t + a4;                                     // coefficient 4
-  T d2 = a5;                                             // coefficient 3
-  T d1 = a5 * t + b;
-  b = b * t + a3;
-  d2 = d2 * t + d1; d1 = d1 * t + b; b = b * t + a2;     // coefficient 2
-  d2 = d2 * t + d1; d1 = d1 * t + b; b = b * t + a1;     // coefficient 1
-  d2 = d2 * t + d1; d1 = d1 * t + b; b = b * t + a0;     // coefficient 0
-  e = b;
-  ez = d1 * m.inv_h;
-  ezz = d2 * m.inv_h2;   // inv_h2 = 2 / h^2
-}
-
-// eps - eps_ref, eps_z, eps_zz at RK4 stage l and height z.  MULTI: the
-// profile has several range columns (else column 0 everywhere).
-template <typename T, bool MULTI>
-__device__ __forceinline__ void medium_eval(const MarchArgs<T>& p, int l, T z, T& e, T& ez,
-                                            T& ezz, unsigned& st) {
-  T zz = z, sg = T(1);
-  if (p.med.mirrored) {
-    const T d = z - p.med.z_mirror;
-    sg = d < T(0) ? T(-1) : T(1);
-    zz = p.med.z_mirror + fabs(d);
-  }
-  if (!MULTI) {
-    col_eval(p.med, 0, zz, e, ez, ezz, st);
-  } else {
-    const int c = __ldg(p.st.c + l);
-    const T th = __ldg(p.st.th + l);
-    if (th == T(0)) {
-      col_eval(p.med, c, zz, e, ez, ezz, st);
-    } else if (th == T(1)) {
-      col_eval(p.med, c + 1, zz, e, ez, ezz, st);
-    } else {
-      T e0, ez0, ezz0, e1, ez1, ezz1;
-      col_eval(p.med, c, zz, e0, ez0, ezz0, st);
-      col_eval(p.med, c + 1, zz, e1, ez1, ezz1, st);
-      e = (T(1) - th) * e0 + th * e1;
-      ez = (T(1) - th) * ez0 + th * ez1;
-      ezz = (T(1) - th) * ezz0 + th * ezz1;
-    }
-  }
-  ez *= sg;
-}
-
-// ----------------------------------------------------------------------------
 // (b) ray march
 // ----------------------------------------------------------------------------
-template <typename T>
-struct Ray {
-  T dz, dQ, rh, Zs, Qs;
-};
-
-// x-form right-hand side (Eqs. charsys / charsys_s divided by x_t = 2P):
+// Both precisions march the same system, scaled so that the right-hand side
+// needs no constant factors (h the medium table's spacing, c = 1 / (2 h),
+// e = eps - eps_ref, d1 and d2 the table's p' and p''/2 in units of h):
+//   w  = (z - s) / h        w'  = 2c A          A = Q / P
+//   dQ = Q - kappa          dQ' = c B           B = d1 / P
+//   rh = r - x P_bar        rh' = D / (P_bar + P) + dQ A
+//   N  = -Z_s               N'  = -c (S + A m) / P,   m = A S + B N
+//   S  = Q_s / c            S'  = c (-4 d2 N + B m) / P
+// This is the x-form of Eqs. charsys / charsys_s divided by x_t = 2P
 //   z' = Q/P, Q' = eps_z/(2P), r' = (eps - kappa Q)/P,
 //   P_s = (eps_z Z_s - 2 Q Q_s)/(2P), Z_s' = (Q_s - Q P_s/P)/P,
 //   Q_s' = (eps_zz Z_s - eps_z P_s/P)/(2P)
-// in deviation form: with e = eps - eps_ref and D = e - dQ (2 kappa + dQ),
-// P^2 = P_bar^2 + D and r' - P_bar = (e - kappa dQ - P_bar D/(P_bar + P))/P.
-template <typename T, bool MULTI>
-__device__ __forceinline__ Ray<T> rhs(const MarchArgs<T>& p, int l, T s, T kap, T pb, T pb2,
-                                      const Ray<T>& y, unsigned& st) {
-  T e, ez, ezz;
-  medium_eval<T, MULTI>(p, l, s + y.dz, e, ez, ezz, st);
-  const T Q = kap + y.dQ;
-  const T D = e - y.dQ * (T(2) * kap + y.dQ);
-  T P2 = pb2 + D;
-  if (!(P2 > T(0))) { st |= ST_TURNING; P2 = pb2; }
-  if (!(y.Zs > T(0))) st |= ST_CAUSTIC;
-  const T iP = rsqrt_t(P2);
-  const T P = P2 * iP;
-  Ray<T> d;
-  d.dz = Q * iP;
-  d.dQ = T(0.5) * ez * iP;
-  d.rh = (e - kap * y.dQ - pb * fdiv_t(D, pb + P)) * iP;
-  const T PsiP = (ez * y.Zs - T(2) * Q * y.Qs) * (T(0.5) * iP * iP);   // P_s / P
-  d.Zs = (y.Qs - Q * PsiP) * iP;
-  d.Qs = T(0.5) * (ezz * y.Zs - ez * PsiP) * iP;
+// with D = e - dQ (2 kappa + dQ) = P^2 - P_bar^2, P - P_bar = D / (P_bar + P)
+// and -P_s / P = c m / P.  The factors c, 2c, -c enter through the RK4 weights.
+
+// 1/sqrt(x) and 1/x in FP64: the special-function unit's estimate (relative
+// error ~2^-20) corrected by one step of third order (Householder's
+// iterations: y (1 + e/2 + 3 e^2/8) with e = 1 - x y^2, and y (1 + e + e^2)
+// with e = 1 - x y), whose own error, ~2^-58, is below the rounding.  5 and 3
+// FP64 operations, for normal positive x.
+__device__ __forceinline__ double rsqrt64(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-(x * y), y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+__device__ __forceinline__ double rcp64(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+
+// FP64 medium lookup at table position u (intervals from the table origin;
+// grounded domains: from the ground, the table even about it): p(t), p'(t) and
+// p''(t)/2 of the interval's quintic.  The interval comes from the low bits of
+// a round-down add of 1.5 * 2^52, so that only three additions of the lookup
+// are FP64 work; positions outside the table (or its very top) take the slow
+// branch.  MULTI: the entry holds a column's coefficients and their
+// differences to the next column, blended with weight th (6 FMAs; a second
+// polynomial and its blend would take 18).
+template <bool MULTI>
+__device__ __forceinline__ void med64(const MarchArgs<double>& p, int l, double u, double& e,
+                                      double& d1, double& d2, unsigned& st) {
+  constexpr int W = MULTI ? 16 : 8;
+  const double magic = 6755399441055744.0;
+  const double z = p.med.mirrored ? fabs(u) : u;
+  const double v = __dadd_rd(z, magic);
+  int i = __double2loint(v);
+  double t = z - (v - magic);
+  if (__double2hiint(v) != 0x43380000 || (unsigned)i >= (unsigned)p.med.n_int) {
+    if (!(z >= 0.0 && z <= p.med.top)) st |= ST_RANGE;
+    i = z > 0.0 ? p.med.n_int - 1 : 0;
+    t = z > 0.0 ? 1.0 : 0.0;
+  }
+  const double* q = p.med.coef;
+  long long o = (long long)i * W;
+  double th = 0.0;
+  if constexpr (MULTI) {
+    o += (long long)__ldg(p.st.c + l) * p.med.col_stride;
+    th = __ldg(p.st.th + l);
+  }
+  q += bchk(o, p.med.size - (W - 1), st);
+  double a[6];
+  load6<double>(q, a[0], a[1], a[2], a[3], a[4], a[5]);
+  if constexpr (MULTI) {
+    double d[6];
+    load6<double>(q + 8, d[0], d[1], d[2], d[3], d[4], d[5]);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) a[k] = fma(th, d[k], a[k]);
+  }
+  // Horner with derivatives (synthetic division)
+  double b = a[5] * t + a[4];                             // coefficient 4
+  d2 = a[5];                                              // coefficient 3
+  d1 = a[5] * t + b;
+  b = b * t + a[3];
+  d2 = d2 * t + d1; d1 = d1 * t + b; b = b * t + a[2];    // coefficient 2
+  d2 = d2 * t + d1; d1 = d1 * t + b; b = b * t + a[1];    // coefficient 1
+  d2 = d2 * t + d1; d1 = d1 * t + b; b = b * t + a[0];    // coefficient 0
+  e = b;
+  // below the ground the slope changes sign (the sign bit of u)
+  if (p.med.mirrored)
+    d1 = __hiloint2double(__double2hiint(d1) ^ (__double2hiint(u) & (int)0x80000000),
+                          __double2loint(d1));
+}
+
+struct Ray {
+  double w, dQ, rh, N, S;
+};
+
+// Right-hand side without the factors 2c, c, 1, -c, c.  Turning points (P^2 <=
+// 0) and caustics (N >= 0) are running extremes of the high words (as integers,
+// off the FP64 pipe), tested once per ray.
+template <bool MULTI>
+__device__ __forceinline__ Ray rhs64(const MarchArgs<double>& p, int l, double u, double kap,
+                                     double pb, double pb2, const Ray& y, int& P2_lo, int& N_hi,
+                                     unsigned& st) {
+  double e, d1, d2;
+  med64<MULTI>(p, l, u, e, d1, d2, st);
+  const double Q = kap + y.dQ;
+  const double D = fma(-y.dQ, Q + kap, e);                // e - dQ (2 kappa + dQ)
+  const double P2 = pb2 + D;
+  P2_lo = min(P2_lo, __double2hiint(P2));
+  N_hi = max(N_hi, __double2hiint(y.N));
+  const double iP = rsqrt64(P2);
+  const double rden = rcp64(fma(P2, iP, pb));             // 1 / (P_bar + P)
+  Ray d;
+  d.w = Q * iP;
+  d.dQ = d1 * iP;
+  d.rh = fma(D, rden, y.dQ * d.w);
+  const double m = fma(d.dQ, y.N, d.w * y.S);
+  d.N = fma(d.w, m, y.S) * iP;
+  d.S = fma(d.dQ, m, (-4.0 * d2) * y.N) * iP;
   return d;
 }
 
-template <typename T>
-__device__ __forceinline__ Ray<T> axpy(const Ray<T>& y, T a, const Ray<T>& k) {
-  return Ray<T>{y.dz + a * k.dz, y.dQ + a * k.dQ, y.rh + a * k.rh, y.Zs + a * k.Zs,
-                y.Qs + a * k.Qs};
-}
-
-// Block (32, 8): lanes are 32 consecutive modes at one launch height, so a
-// warp's table reads stay within a few z-intervals; warps are 8 rays.
-template <typename T, bool MULTI, bool PLANES>
-__device__ __forceinline__ void march_body(const MarchArgs<T>& p, int bx, int by, int tx, int ty) {
-  const int r = bx * 32 + tx;       // marched mode (output column)
-  const int j = by * 8 + ty;
-  if (r >= p.Mr || j >= p.NRT) return;
+// Thread t marches ray j of mode r, t = j Mr + r: a warp's lanes are
+// consecutive modes at one launch height, so their table reads stay within a
+// few intervals.  THREADS threads per block.
+template <bool MULTI, bool PLANES, int THREADS>
+__device__ __forceinline__ void march64_body(const MarchArgs<double>& p, int blk, int tid) {
+  const long long t = (long long)blk * THREADS + tid;
+  if (t >= (long long)p.Mr * p.NRT) return;
+  const int j = (int)(t / p.Mr);
+  const int r = (int)(t - (long long)j * p.Mr);
   unsigned st = 0;
   const int i = r + p.mode_off;
-  const T kap = p.kappa[i], pb = p.pbar[i], pb2 = p.pbar2[i];
-  const T s = p.z_lo + T((j - p.G) * p.R) * p.dz;
-  T e, ez, ezz;
-  medium_eval<T, MULTI>(p, 0, s, e, ez, ezz, st);
-  T P0sq = pb2 + e;
-  if (!(P0sq > T(0))) { st |= ST_TURNING; P0sq = pb2; }
-  const T P0 = sqrt(P0sq);
-  Ray<T> y{T(0), T(0), T(0), T(1), T(0)};
-  const T h = p.h, hh = T(0.5) * p.h, h6 = p.h / T(6);
+  const double kap = p.kappa[i], pb = p.pbar[i], pb2 = p.pbar2[i];
+  const double s = fma((double)((j - p.G) * p.R), p.u_dz, p.u_lo);   // launch height in intervals
+  double e0, d0, d00;
+  med64<MULTI>(p, 0, s, e0, d0, d00, st);
+  double P0sq = pb2 + e0;
+  if (!(P0sq > 0.0)) { st |= ST_TURNING; P0sq = pb2; }
+  const double P0 = sqrt(P0sq);
+  Ray y{0.0, 0.0, 0.0, -1.0, 0.0};
+  const double H = 0.5 * p.med.inv_h * p.h;
+  const double H2 = 0.5 * H, H6 = H / 6.0, H3 = H / 3.0, W1 = 2.0 * H, W3 = 2.0 * H3;
+  const double h6 = p.h / 6.0, h3 = p.h / 3.0;
+  int P2_lo = 0x7fefffff, N_hi = (int)0x80000000;
   // landing quantities at RK4 stage l (the screen's end, or a plane inside it)
-  auto land = [&](int l, T* od, T* oph, T* oa) {
+  auto land = [&](int l, double* od, double* oph, double* oa) {
     const long long o = bchk((long long)j * p.Mr + r, (long long)p.NRT * p.Mr, st);
-    if (!(y.Zs > T(0))) st |= ST_CAUSTIC;
-    T e1, ez1, ezz1;
-    medium_eval<T, MULTI>(p, l, s + y.dz, e1, ez1, ezz1, st);
-    T P1sq = pb2 + e1 - y.dQ * (T(2) * kap + y.dQ);
-    if (!(P1sq > T(0))) { st |= ST_TURNING; P1sq = pb2; }
-    const T Zs = y.Zs > T(0) ? y.Zs : T(1);
-    od[o] = y.dz * p.inv_dz;
+    if (!(y.N < 0.0)) st |= ST_CAUSTIC;
+    double e1, f1, g1;
+    med64<MULTI>(p, l, s + y.w, e1, f1, g1, st);
+    double P1sq = pb2 + e1 - y.dQ * (2.0 * kap + y.dQ);
+    if (!(P1sq > 0.0)) { st |= ST_TURNING; P1sq = pb2; }
+    const double Zs = y.N < 0.0 ? -y.N : 1.0;
+    od[o] = y.w * (p.inv_dz / p.med.inv_h);
     oph[o] = y.rh * p.k_over_2pi;
-    oa[o] = sqrt(P0 * rsqrt_t(P1sq) / Zs);
+    oa[o] = sqrt(P0 * rsqrt(P1sq) / Zs);
   };
+  // RK4 accumulated as the stages complete; a stage state needs no rh, and its
+  // w only as the table position
   for (int n = 0; n < p.Nt; ++n) {
-    const Ray<T> k1 = rhs<T, MULTI>(p, 2 * n, s, kap, pb, pb2, y, st);
-    const Ray<T> k2 = rhs<T, MULTI>(p, 2 * n + 1, s, kap, pb, pb2, axpy(y, hh, k1), st);
-    const Ray<T> k3 = rhs<T, MULTI>(p, 2 * n + 1, s, kap, pb, pb2, axpy(y, hh, k2), st);
-    const Ray<T> k4 = rhs<T, MULTI>(p, 2 * n + 2, s, kap, pb, pb2, axpy(y, h, k3), st);
-    y.dz += h6 * (k1.dz + T(2) * k2.dz + T(2) * k3.dz + k4.dz);
-    y.dQ += h6 * (k1.dQ + T(2) * k2.dQ + T(2) * k3.dQ + k4.dQ);
-    y.rh += h6 * (k1.rh + T(2) * k2.rh + T(2) * k3.rh + k4.rh);
-    y.Zs += h6 * (k1.Zs + T(2) * k2.Zs + T(2) * k3.Zs + k4.Zs);
-    y.Qs += h6 * (k1.Qs + T(2) * k2.Qs + T(2) * k3.Qs + k4.Qs);
+    const double u0 = s + y.w;
+    Ray acc = y;
+    auto add = [&](const Ray& k, double gw, double gq, double gr) {
+      acc = Ray{fma(gw, k.w, acc.w), fma(gq, k.dQ, acc.dQ), fma(gr, k.rh, acc.rh),
+                fma(-gq, k.N, acc.N), fma(gq, k.S, acc.S)};
+    };
+    auto stage = [&](const Ray& k, double gq) {
+      return Ray{0.0, fma(gq, k.dQ, y.dQ), 0.0, fma(-gq, k.N, y.N), fma(gq, k.S, y.S)};
+    };
+    const Ray k1 = rhs64<MULTI>(p, 2 * n, u0, kap, pb, pb2, y, P2_lo, N_hi, st);
+    add(k1, H3, H6, h6);
+    const Ray k2 = rhs64<MULTI>(p, 2 * n + 1, fma(H, k1.w, u0), kap, pb, pb2, stage(k1, H2),
+                                P2_lo, N_hi, st);
+    add(k2, W3, H3, h3);
+    const Ray k3 = rhs64<MULTI>(p, 2 * n + 1, fma(H, k2.w, u0), kap, pb, pb2, stage(k2, H2),
+                                P2_lo, N_hi, st);
+    add(k3, W3, H3, h3);
+    const Ray k4 = rhs64<MULTI>(p, 2 * n + 2, fma(W1, k3.w, u0), kap, pb, pb2, stage(k3, H),
+                                P2_lo, N_hi, st);
+    add(k4, H3, H6, h6);
+    y = acc;
     if (PLANES && (n + 1) % p.plane_steps == 0 && n + 1 < p.Nt) {
       const long long po = (long long)((n + 1) / p.plane_steps - 1) * p.NRT * p.Mr;
       land(2 * (n + 1), p.pl_d + po, p.pl_ph + po, p.pl_a + po);
     }
   }
   land(2 * p.Nt, p.out_d, p.out_ph, p.out_a);
+  if (P2_lo <= 0) st |= ST_TURNING;
+  if (N_hi >= 0) st |= ST_CAUSTIC;
   if (st) atomicOr(p.status, st);
 }
 
-template <typename T, bool MULTI, bool PLANES>
-__global__ void __launch_bounds__(256) k_march(const MarchArgs<T> p) {
-  march_body<T, MULTI, PLANES>(p, blockIdx.x, blockIdx.y, threadIdx.x, threadIdx.y);
+// Bound by the FP64 pipe (2 operations per SM and clock, ~87 % busy): ~49 FP64
+// operations per stage (12 of them the quintic, 8 the two special functions).
+// On the 16384-point duct (489 modes x 2086 rays, 16 RK4 steps) 6.4 ms, against
+// 9.1 ms with the unscaled system, library rsqrt and division, and FP64
+// comparisons and conversions in the lookup (~66).  CTAs of 64 threads spread
+// small plans evenly: 65 modes x 704 rays on 152 SMs take 0.18 ms, against
+// 0.50 ms in CTAs of 256 (179 of them: two on some SMs, one on the others) that
+// evaluated both columns of a lookup.
+constexpr int MARCH64_THREADS = 64;
+
+template <bool MULTI, bool PLANES>
+__global__ void __launch_bounds__(MARCH64_THREADS) k_march(const MarchArgs<double> p) {
+  march64_body<MULTI, PLANES, MARCH64_THREADS>(p, blockIdx.x, threadIdx.x);
 }
 
 // ----------------------------------------------------------------------------
@@ -325,17 +366,7 @@ __device__ __forceinline__ float rcp_approx(float x) {
   return r;
 }
 
-// Marched state of two rays, scaled so that the right-hand side needs no
-// constant factors (c = 1 / (2 h) of the table spacing h, d1 and d2 the
-// table's derivatives p' and p''/2 in units of h):
-//   w  = (z - s) / h        w'  = 2c A          A = Q / P
-//   dQ = Q - kappa          dQ' = c B           B = d1 / P
-//   rh = r - x P_bar        rh' = D / (P_bar + P) + dQ A
-//   N  = -Z_s               N'  = -c (S + A m) / P,   m = A S + B N
-//   S  = Q_s / c            S'  = c (-4 d2 N + B m) / P
-// (r' - P_bar = (e - kappa dQ) / P - P_bar with e = D + dQ (2 kappa + dQ) and
-// P^2 = P_bar^2 + D; -P_s / P = c m / P).  The factors c, 2c, -c enter through
-// the RK4 weights.
+// Marched state of two rays (scaled as above).
 struct Ray2 {
   f2 w, dQ, rh, N, S;
 };

@@ -27,9 +27,9 @@ template <> struct C2<double> { using type = double2; };
 
 // Quintic medium table: per column, per z interval i, the monomial
 // coefficients a0..a5 of eps(z0 + (i + t) h) - eps_ref in t in [0, 1]
-// (8 slots per interval, the last two unused).
-//   FP64 plans: the profile's n_int intervals from z0 = z_a; grounded domains
-//   reflect z about z_mirror before the lookup.
+// (8 slots per interval, the last two unused).  Positions are in intervals.
+//   FP64 plans: the profile's n_int intervals from z0; grounded domains look
+//   up the magnitude of the position (the ground is at z0).
 //   FP32 plans: the reflection is stored instead (grounded domains: the
 //   mirror images of the n_int intervals below z_a, then the n_int intervals
 //   above), followed by one interval continuing the last one, so that a
@@ -37,17 +37,16 @@ template <> struct C2<double> { using type = double2; };
 //   before that pad and top = n_int as a float.  When pieces = S > 0 every
 //   interval is stored as S cubic Hermite pieces of its quintic (value and
 //   slope matched at the piece ends; 4 slots b0..b3 in the piece's own
-//   tau in [0, 1]) and n_int, top, inv_h, inv_h2 count pieces.  With several
-//   columns every entry is followed by its difference to the next column's
-//   entry (twice the slots), and the last column has no rows of its own.
+//   tau in [0, 1]) and n_int, top, inv_h count pieces.
+// With several columns every entry is followed by its difference to the next
+// column's entry (twice the slots), and the last column has no rows of its own.
 template <typename T>
 struct Medium {
   const T* coef;
   int n_int;
   long long col_stride;
-  T z0, inv_h, inv_h2;
+  T inv_h;
   int mirrored;
-  T z_mirror;
   T top;
   int pieces;   // FP32: > 0 when each entry is a cubic piece (4 slots), in piece units
   long long size;   // values in coef (all columns), for bounds-checked builds
@@ -71,8 +70,8 @@ struct MarchArgs {
   int Mr;           // marched modes (row length of the outputs)
   int mode_off;     // marched mode r is mode index r + mode_off (n = r + mode_off - n_max)
   int NRT, G, R, Nt;
-  T z_lo, dz, inv_dz, h, k_over_2pi;
-  T u_lo, u_dz;     // FP32 table position of grid point 0 and per grid point
+  T inv_dz, h, k_over_2pi;
+  T u_lo, u_dz;     // table position of grid point 0 and per grid point
   T* out_d;         // [NRT][Mr] landing offset from the launch grid point, grid units
   T* out_ph;        // [NRT][Mr] residual phase k (r - x P_bar) / (2 pi), turns
   T* out_a;         // [NRT][Mr] amplitude factor sqrt(P0 / (P1 Z_s))
@@ -219,8 +218,7 @@ template <typename T>
 struct PlanParts {
   int N, n_z, M, Mr, NRT, Nt, n_max, mirror, sym, N1, n_cols, pieces;
   int stage_rows, stage_stride;      // RK4 stage rows (screens q >= rows - 1 share the last)
-  int march_bx, march_blocks;        // FP64: ceil(Mr / 32) x ceil(NRT / 8) blocks of (32, 8);
-                                     // FP32: ceil(Mr ceil(NRT / 2) / 256) blocks of 256
+  int march_blocks;                  // blocks of 256: a thread per ray (FP64) or ray pair (FP32)
   int bracket_bx;                    // bracket blocks of 256 threads along the modes
   int resum_blocks, resum_pw;        // resummation blocks (tiles x mode groups), points per lane
   size_t resum_smem;                 // shared memory of one resummation block

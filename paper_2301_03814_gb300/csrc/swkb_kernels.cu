@@ -72,15 +72,16 @@ cudaError_t launch_fft(const FftArgs<T>& a, cudaStream_t s) {
   return launch_k(k_fft2<T>, dim3(modes), dim3(FFT2_THREADS), 0, s, a);
 }
 
-template <typename T>
-cudaError_t launch_march(const MarchArgs<T>& a, bool multi_column, cudaStream_t s) {
-  dim3 block(32, 8);
-  dim3 grid((a.Mr + 31) / 32, (a.NRT + 7) / 8);
+template <>
+cudaError_t launch_march<double>(const MarchArgs<double>& a, bool multi_column, cudaStream_t s) {
+  const long long threads = (long long)a.Mr * a.NRT;
+  const dim3 block(MARCH64_THREADS),
+      grid((unsigned)((threads + MARCH64_THREADS - 1) / MARCH64_THREADS));
   if (a.plane_steps > 0)
-    return multi_column ? launch_k(k_march<T, true, true>, grid, block, 0, s, a)
-                        : launch_k(k_march<T, false, true>, grid, block, 0, s, a);
-  return multi_column ? launch_k(k_march<T, true, false>, grid, block, 0, s, a)
-                      : launch_k(k_march<T, false, false>, grid, block, 0, s, a);
+    return multi_column ? launch_k(k_march<true, true>, grid, block, 0, s, a)
+                        : launch_k(k_march<false, true>, grid, block, 0, s, a);
+  return multi_column ? launch_k(k_march<true, false>, grid, block, 0, s, a)
+                      : launch_k(k_march<false, false>, grid, block, 0, s, a);
 }
 
 template <>
@@ -179,7 +180,6 @@ cudaError_t launch_output(const typename C2<T>::type* u, int offset, int n, doub
   template cudaError_t launch_init<T>(const double*, int, int, int, C2<T>::type*, cudaStream_t); \
   template cudaError_t launch_reduce<T>(const ReduceArgs<T>&, cudaStream_t);                    \
   template cudaError_t launch_fft<T>(const FftArgs<T>&, cudaStream_t);                          \
-  template cudaError_t launch_march<T>(const MarchArgs<T>&, bool, cudaStream_t);                \
   template cudaError_t launch_bracket<T>(const BracketArgs<T>&, cudaStream_t);                  \
   template cudaError_t launch_resum<T>(const ResumArgs<T>&, cudaStream_t);                      \
   template cudaError_t launch_output<T>(const C2<T>::type*, int, int, double*, cudaStream_t);   \

@@ -249,12 +249,16 @@ namespace {
 
 // Intervals of the FP32 medium table of one column (layout in swkb_internal.h).
 int table32_intervals(const swkb_plan* p) { return (p->mirror ? 2 : 1) * p->n_int + 1; }
-// Its columns as stored (with several, each holds the differences to the
-// next one too, so the last needs none of its own) and the values of one.
-int table32_columns(const swkb_plan* p) { return p->n_cols > 1 ? p->n_cols - 1 : 1; }
-long long table32_values(const swkb_plan* p) {
-  return (long long)table32_intervals(p) * (p->pieces > 0 ? 4 * p->pieces : 8) *
-         (p->n_cols > 1 ? 2 : 1);
+// Columns of the medium table as stored (with several, each holds the
+// differences to the next one too, so the last needs none of its own) and the
+// values of one.
+int table_columns(const swkb_plan* p) { return p->n_cols > 1 ? p->n_cols - 1 : 1; }
+long long table_values(const swkb_plan* p) {
+  const long long entries =
+      p->precision == SWKB_FP64
+          ? (long long)p->n_int * 8
+          : (long long)table32_intervals(p) * (p->pieces > 0 ? 4 * p->pieces : 8);
+  return entries * (p->n_cols > 1 ? 2 : 1);
 }
 
 // Quintic Hermite interpolant of eps - eps_ref on every profile interval, as
@@ -479,10 +483,8 @@ swkb_status build_device(swkb_plan* p, const swkb_profile* prof) {
   const int M = p->M, N = p->N;
   // medium coefficient table (eps - eps_ref), 8 slots per interval
   {
-    const std::vector<double> coef = quintic_coefficients(p, prof);
-    if (sizeof(T) == 8) {
-      TRY(upload<T>(p, &p->coef, coef));
-    } else {
+    std::vector<double> coef = quintic_coefficients(p, prof);
+    if (sizeof(T) == 4) {
       // FP32 layout: reflected intervals below z_a (grounded), the profile's
       // intervals, one continuation interval.  A reflected interval holds
       // p(1 - t) and the continuation p_last(1 + t), re-expanded in t.
@@ -517,21 +519,22 @@ swkb_status build_device(swkb_plan* p, const swkb_profile* prof) {
           for (int sp = 0; sp < S; ++sp) cubic_piece(c32.data() + k * 8, sp, S, &cub[(k * S + sp) * 4]);
         c32.swap(cub);
       }
-      if (p->n_cols > 1) {
-        // each entry of a column followed by its difference to the next one
-        const size_t w = p->pieces > 0 ? 4 : 8, per = c32.size() / p->n_cols;
-        std::vector<T> pairs((size_t)(p->n_cols - 1) * per * 2);
-        T* o = pairs.data();
-        for (size_t k = 0; k + per < c32.size(); k += w, o += 2 * w)
-          for (size_t j = 0; j < w; ++j) {
-            o[j] = (T)c32[k + j];
-            o[w + j] = (T)(c32[k + per + j] - c32[k + j]);
-          }
-        TRY(dev_alloc(p, &p->coef, pairs.size() * sizeof(T)));
-        CK(cudaMemcpy(p->coef, pairs.data(), pairs.size() * sizeof(T), cudaMemcpyHostToDevice));
-      } else {
-        TRY(upload<T>(p, &p->coef, c32));
-      }
+      coef.swap(c32);
+    }
+    if (p->n_cols > 1) {
+      // each entry of a column followed by its difference to the next one
+      const size_t w = p->pieces > 0 ? 4 : 8, per = coef.size() / p->n_cols;
+      std::vector<T> pairs((size_t)(p->n_cols - 1) * per * 2);
+      T* o = pairs.data();
+      for (size_t k = 0; k + per < coef.size(); k += w, o += 2 * w)
+        for (size_t j = 0; j < w; ++j) {
+          o[j] = (T)coef[k + j];
+          o[w + j] = (T)(coef[k + per + j] - coef[k + j]);
+        }
+      TRY(dev_alloc(p, &p->coef, pairs.size() * sizeof(T)));
+      CK(cudaMemcpy(p->coef, pairs.data(), pairs.size() * sizeof(T), cudaMemcpyHostToDevice));
+    } else {
+      TRY(upload<T>(p, &p->coef, coef));
     }
   }
   // RK4 stage columns for screens 0 .. stage_rows - 1
@@ -714,36 +717,23 @@ template <typename T>
 MarchArgs<T> march_args(const swkb_plan* p, int q) {
   MarchArgs<T> a;
   a.med.coef = (const T*)p->coef;
+  double z0 = p->z0p, hs = p->dzp;   // table origin and entry spacing
   a.med.n_int = p->n_int;
-  a.med.col_stride = (long long)p->n_int * 8;
-  a.med.z0 = (T)p->z0p;
-  a.med.inv_h = (T)(1.0 / p->dzp);
-  a.med.inv_h2 = (T)(2.0 / (p->dzp * p->dzp));
   a.med.mirrored = p->mirror != 0;
-  a.med.z_mirror = (T)p->z_a;
-  a.med.top = (T)p->n_int;
-  a.med.pieces = 0;
-  a.med.size = (long long)p->n_cols * p->n_int * 8;
-  if (sizeof(T) == 4) {
-    // reflection stored in the table; positions in table intervals
-    const double z0 = p->mirror ? p->z0p - p->n_int * p->dzp : p->z0p;
-    // with cubic pieces, positions and derivatives are in piece units
+  a.med.pieces = p->pieces;
+  if (sizeof(T) == 4) {   // the reflection stored, entries in pieces
     const int S = p->pieces > 0 ? p->pieces : 1;
-    const double hs = p->dzp / S;
-    a.med.n_int = (p->mirror ? 2 : 1) * p->n_int * S;
-    a.med.col_stride = table32_values(p);
-    a.med.z0 = (T)z0;
-    a.med.inv_h = (T)(1.0 / hs);
-    a.med.inv_h2 = (T)(2.0 / (hs * hs));
+    if (p->mirror) z0 -= p->n_int * p->dzp;
+    hs /= S;
+    a.med.n_int *= (p->mirror ? 2 : 1) * S;
     a.med.mirrored = 0;
-    a.med.pieces = p->pieces;
-    a.med.size = (long long)table32_columns(p) * a.med.col_stride;
-    a.med.top = (T)a.med.n_int;
-    a.u_lo = (T)((p->z_lo - z0) / hs);
-    a.u_dz = (T)(p->dz / hs);
-  } else {
-    a.u_lo = a.u_dz = T(0);
   }
+  a.med.col_stride = table_values(p);
+  a.med.inv_h = (T)(1.0 / hs);
+  a.med.top = (T)a.med.n_int;
+  a.med.size = (long long)table_columns(p) * a.med.col_stride;
+  a.u_lo = (T)((p->z_lo - z0) / hs);
+  a.u_dz = (T)(p->dz / hs);
   const int S = 2 * p->Nt + 1;
   const int row = std::min(std::max(q, 0), p->stage_rows - 1);
   a.st.c = p->stage_c + (size_t)row * S;
@@ -753,7 +743,7 @@ MarchArgs<T> march_args(const swkb_plan* p, int q) {
   a.pbar2 = (const T*)p->pbar2_d;
   a.Mr = p->Mr; a.mode_off = p->sym ? p->n_max : 0;
   a.NRT = p->NRT; a.G = p->G; a.R = p->R; a.Nt = p->Nt;
-  a.z_lo = (T)p->z_lo; a.dz = (T)p->dz; a.inv_dz = (T)(1.0 / p->dz);
+  a.inv_dz = (T)(1.0 / p->dz);
   a.h = (T)(p->dx / p->Nt);
   a.k_over_2pi = (T)(p->k / (2.0 * M_PI));
   a.out_d = (T*)p->rd; a.out_ph = (T*)p->rph; a.out_a = (T*)p->ra;
@@ -1696,8 +1686,7 @@ swkb_status configure(swkb_plan* p, const swkb_profile* prof, double k, const sw
 size_t device_bytes(const swkb_plan* p) {
   const size_t T = p->precision == SWKB_FP64 ? 8 : 4, V = 2 * T;
   const size_t S = 2 * (size_t)p->Nt + 1;
-  size_t b = (T == 8 ? (size_t)p->n_cols * p->n_int * 8                              // medium
-                     : (size_t)table32_columns(p) * table32_values(p)) * T;
+  size_t b = (size_t)table_columns(p) * table_values(p) * T;        // medium
   b += (size_t)p->stage_rows * S * (sizeof(int) + T);               // stage columns
   b += 3 * (size_t)p->M * T + (size_t)p->M * V;                     // mode tables
   b += (size_t)p->N * V;                                            // twiddles
@@ -1858,13 +1847,8 @@ swkb_status plan_parts(swkb_plan* p, PlanParts<T>* o) {
   o->n_cols = p->n_cols; o->pieces = p->pieces;
   o->stage_rows = p->stage_rows;
   o->stage_stride = 2 * p->Nt + 1;
-  if (sizeof(T) == 8) {
-    o->march_bx = (p->Mr + 31) / 32;
-    o->march_blocks = o->march_bx * ((p->NRT + 7) / 8);
-  } else {
-    o->march_bx = 0;
-    o->march_blocks = (int)(((long long)p->Mr * ((p->NRT + 1) / 2) + 255) / 256);
-  }
+  o->march_blocks =
+      (int)(((long long)p->Mr * (sizeof(T) == 8 ? p->NRT : (p->NRT + 1) / 2) + 255) / 256);
   o->bracket_bx = (p->Mr + 255) / 256;
   o->resum_blocks = p->n_tiles_run * p->n_groups;
   o->resum_pw = p->PW;
