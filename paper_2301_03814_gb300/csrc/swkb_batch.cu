@@ -188,10 +188,10 @@ template <typename T>
 __device__ __forceinline__ void resum_item(const ResumArgs<T>& r, int pw, int v, int tid,
                                            unsigned char* smem, int sub) {
   switch (pw) {
-    case 2: resum_body<T, 2, LD_CG, 1>(r, v, tid, smem, sub); break;
-    case 4: resum_body<T, 4, LD_CG, 1>(r, v, tid, smem, sub); break;
-    case 8: resum_body<T, 8, LD_CG, 1>(r, v, tid, smem, sub); break;
-    default: resum_body<T, 16, LD_CG, 1>(r, v, tid, smem, sub); break;
+    case 2: resum_body<2, LD_CG, 1>(r, v, tid, smem, sub); break;
+    case 4: resum_body<4, LD_CG, 1>(r, v, tid, smem, sub); break;
+    case 8: resum_body<8, LD_CG, 1>(r, v, tid, smem, sub); break;
+    default: resum_body<16, LD_CG, 1>(r, v, tid, smem, sub); break;
   }
 }
 

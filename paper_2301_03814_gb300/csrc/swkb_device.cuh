@@ -814,13 +814,284 @@ __device__ __forceinline__ void cubic_through(T f0, T f1, T f2, T f3, T r21, T r
   b3 = d0123;
 }
 
+// Fixed-order sum of a block's four warps, written as its group's partial.
+template <typename T, int PW, int BAR>
+__device__ __forceinline__ void block_sum(const ResumArgs<T>& p, const T* accr, const T* acci,
+                                          unsigned char* smem_raw, int group, int m0, int tid,
+                                          int sub, unsigned st) {
+  using V = typename C2<T>::type;
+  const int lane = tid & 31, warp = tid >> 5, TM = p.TM;
+  vb_sync<BAR>(sub);
+  // per warp TM points as 32 runs of PW, each run padded to PW + 1 entries so
+  // that the lanes' stores fall in different banks
+  V* red = reinterpret_cast<V*>(smem_raw);
+  const int TMP = 32 * (PW + 1);
+#pragma unroll
+  for (int q = 0; q < PW; ++q) {
+    V v;
+    v.x = accr[q];
+    v.y = acci[q];
+    red[warp * TMP + lane * (PW + 1) + q] = v;
+  }
+  vb_sync<BAR>(sub);
+  V* out = p.part + bchk((long long)group * p.N + m0, (long long)p.n_groups * p.N - (TM - 1), st);
+  if (st) atomicOr(p.status, st);
+  for (int x = tid; x < TM; x += RESUM_WARPS * 32) {
+    const int xs = (x / PW) * (PW + 1) + x % PW;
+    V sum = red[xs];
+#pragma unroll
+    for (int w = 1; w < RESUM_WARPS; ++w) {
+      const V v = red[w * TMP + xs];
+      sum.x += v.x; sum.y += v.y;
+    }
+    out[x] = sum;
+  }
+}
+
+// ---- FP32 ----
+// Interval row: (X_w, X_w) | (b3, a3) | (b2, a2) | (b1, a1) | (b0, a0) | X_{w+1},
+// the phase and amplitude cubics interleaved, so that three packed FMAs
+// evaluate both and three 16-byte loads fetch a row.
+struct Row32 {
+  f2 X1, c3, c2, c1, c0;
+  float X2;
+};
+__device__ __forceinline__ void load_row32(const float* p, Row32& r) {
+  const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(p);
+  const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(p + 4);
+  const float4 x = *reinterpret_cast<const float4*>(p + 8);
+  r.X1.v = u.x; r.c3.v = u.y; r.c2.v = v.x; r.c1.v = v.y;
+  r.c0 = mk2(x.x, x.y);
+  r.X2 = x.z;
+}
+
 // One resummation block: blk its index in the launch, tid its thread index
 // (0 .. 32 RESUM_WARPS - 1), smem_raw its shared memory (resum_smem_bytes),
 // sub the virtual-block slot for the barrier (BAR).
-template <typename T, int PW, int LD, int BAR>
-__device__ __forceinline__ void resum_body(const ResumArgs<T>& p, int blk, int tid,
+template <int PW, int LD, int BAR>
+__device__ __forceinline__ void resum_body(const ResumArgs<float>& p, int blk, int tid,
                                            unsigned char* smem_raw, int sub) {
-  using V = typename C2<T>::type;
+  constexpr int LDC = LD == LD_NC ? LD_PLAIN : LD;   // mode coefficients
+  constexpr unsigned ALL = 0xffffffffu;
+  const int lane = tid & 31;
+  const int warp = tid >> 5;
+  const int tt = blk % p.n_tiles_run;
+  const int group = blk / p.n_tiles_run;
+  const int half = p.n_tiles >> 1;
+  const int tile = p.sym ? (tt < half ? half + tt : 0) : tt;
+  const int wcap = p.wcap;
+  const int TM = p.TM;
+  unsigned char* wbase = smem_raw + (long long)warp * resum_warp_bytes<float>(wcap);
+  float* s_cf = reinterpret_cast<float*>(wbase);               // [wcap][RESUM_CF], 16-byte aligned
+  float2* s_pa = reinterpret_cast<float2*>(s_cf + RESUM_CF * wcap);   // phase, amplitude
+  float* s_X = reinterpret_cast<float*>(s_pa + wcap);
+  const int m0 = tile * TM;
+  const int i0 = group * p.modes_per_group;
+  const int i1 = min(p.M, i0 + p.modes_per_group);
+  const float invN = scalbn(1.f, -(__ffs(p.N) - 1));           // exact
+  const unsigned mask = (unsigned)p.N - 1u;
+  const long long nrm = (long long)p.NRT * p.Mr;
+  unsigned st = 0;
+
+  float accr[PW], acci[PW];
+#pragma unroll
+  for (int q = 0; q < PW; ++q) { accr[q] = 0.f; acci[q] = 0.f; }
+
+  // grounded: mode n < 0 is the mirror image of mode -n (column -n); its
+  // ray j' is ray NRT - j' of mode -n, landing at N - g
+  auto column = [&](int i, bool& mir) {
+    const int n = i - p.n_max;
+    mir = p.sym && n < 0;
+    return p.sym ? (n < 0 ? -n : n) : i;
+  };
+  // One ray window per mode, its first 32 rays loaded one mode ahead.  r0: ray
+  // of slot 0 (mirrored families run backwards), W: slots (0: skip the mode).
+  float rd = 0.f, rph = 0.f, ra = 0.f;
+  auto fetch = [&](int i, int r0, int w, float& d, float& ph, float& a) {
+    bool mir;
+    const int col = column(i, mir);
+    const long long o = bchk((long long)(mir ? r0 - w : r0 + w) * p.Mr + col, nrm, st);
+    d = ld<LD>(p.d + o);
+    ph = ld<LD>(p.ph + o);
+    a = ld<LD>(p.a + o);
+  };
+
+  // The warp's modes ib + RESUM_WARPS k, 32 at a time: lane k looks up the
+  // brackets and the coefficient of mode k, which the loop takes by shuffles.
+  for (int ib = i0 + warp; ib < i1; ib += 32 * RESUM_WARPS) {
+    int h_r0 = 0, h_W = 0, h_base = 0;
+    float h_mag = 0.f, h_arg = 0.f;
+    {
+      const int i = ib + RESUM_WARPS * lane;
+      if (i < i1) {
+        bool mir;
+        const int col = column(i, mir);
+        const int* jt = mir ? p.jlo_neg : p.jlo;
+        const long long nj = (long long)(p.n_tiles + 1) * p.Mr;
+        const int jl = ld<LD>(jt + bchk((long long)tile * p.Mr + col, nj, st));
+        const int jh = ld<LD>(jt + bchk((long long)(tile + 1) * p.Mr + col, nj, st));
+        // A bracket table left inconsistent by a failed screen (already flagged
+        // by k_bracket) must not send the reads out of [0, NRT); a window wider
+        // than the tile's capacity means rays compressed beyond it (flagged here).
+        if (jl >= (mir ? 2 : 1) && jh >= jl && jh <= p.NRT - 3) {
+          h_W = jh - jl + 4;
+          if (h_W > wcap) { st |= ST_CAUSTIC; h_W = 0; }
+        }
+        const int jb = jl - 1;
+        h_r0 = mir ? p.NRT - jb : jb;
+        h_base = mir ? p.N - m0 - (p.NRT - jb - p.G) * p.R : (jb - p.G) * p.R - m0;
+        // the mode coefficient in polar form (|c_n| scales the amplitudes,
+        // arg c_n / 2 pi shifts the phases, in turns), formed by the DFT, so
+        // that a term is two FMAs instead of a complex product
+        const float2 cp = ld<LDC>(p.cpol + i);
+        h_mag = cp.x;
+        h_arg = cp.y;
+      }
+    }
+    const int K = min(32, (i1 - ib + RESUM_WARPS - 1) / RESUM_WARPS);
+    int r0 = __shfl_sync(ALL, h_r0, 0), W = __shfl_sync(ALL, h_W, 0);
+    if (lane < W) fetch(ib, r0, lane, rd, rph, ra);
+    for (int k = 0; k < K; ++k) {
+      const int i = ib + RESUM_WARPS * k;
+      const int Wc = W, rc = r0;
+      const int base = __shfl_sync(ALL, h_base, k);
+      const float cmag = __shfl_sync(ALL, h_mag, k);
+      const float carg = __shfl_sync(ALL, h_arg, k);
+      const float dsign = p.sym && i < p.n_max ? -1.f : 1.f;
+      __syncwarp();
+      if (lane < Wc) {
+        s_X[lane] = fmaf(dsign, rd, (float)(base + lane * p.R));
+        s_pa[lane] = make_float2(rph + carg, ra * cmag);
+      }
+      for (int w = lane + 32; w < Wc; w += 32) {   // beyond the prefetched rays
+        float d, ph, a;
+        fetch(i, rc, w, d, ph, a);
+        s_X[w] = fmaf(dsign, d, (float)(base + w * p.R));
+        s_pa[w] = make_float2(ph + carg, a * cmag);
+      }
+      // issue the next mode's window
+      if (k + 1 < K) {
+        r0 = __shfl_sync(ALL, h_r0, k + 1);
+        W = __shfl_sync(ALL, h_W, k + 1);
+        if (lane < W) fetch(i + RESUM_WARPS, r0, lane, rd, rph, ra);
+      }
+      if (Wc == 0) continue;
+      __syncwarp();
+      // Rows of the intervals 1 .. W - 3.  The last one's end is stored as
+      // infinity: no lane steps past it.
+      bool wide = true;
+      for (int w = 1 + lane; w <= Wc - 3; w += 32) {
+        const float X0 = s_X[w - 1], X1 = s_X[w], X2 = s_X[w + 1], X3 = s_X[w + 2];
+        const float h21 = X2 - X1, h10 = X1 - X0;
+        wide = wide && h21 >= 1.f;
+        const f2 r21 = bc2(rcp_approx(h21)), r10 = bc2(rcp_approx(h10));
+        const f2 r32 = bc2(rcp_approx(X3 - X2)), r20 = bc2(rcp_approx(X2 - X0));
+        const f2 r31 = bc2(rcp_approx(X3 - X1)), r30 = bc2(rcp_approx(X3 - X0));
+        const auto val = [&](int k) {
+          f2 v;
+          v.v = *reinterpret_cast<const unsigned long long*>(s_pa + w + k);
+          return v;
+        };
+        // Newton divided differences through (X1, X2, X0, X3) of phase and
+        // amplitude together, rewritten as cubics in tau = x - X1
+        const f2 f0 = val(-1), f1 = val(0), fa = val(1), f3 = val(2);
+        const f2 d12 = mul2(sub2(fa, f1), r21), d01 = mul2(sub2(f1, f0), r10);
+        const f2 d23 = mul2(sub2(f3, fa), r32);
+        const f2 d012 = mul2(sub2(d12, d01), r20), d123 = mul2(sub2(d23, d12), r31);
+        const f2 c3 = mul2(sub2(d123, d012), r30);
+        const f2 c1 = fma2(bc2(-h21), fma2(c3, bc2(h10), d012), d12);
+        const f2 c2 = fma2(c3, bc2(h10 - h21), d012);
+        float b0, a0;
+        sp2(f1, b0, a0);
+        b0 = minus_rint(b0);                       // whole turns do not matter
+        float* row = s_cf + RESUM_CF * w;
+        *reinterpret_cast<ulonglong2*>(row) = make_ulonglong2(bc2(X1).v, c3.v);
+        *reinterpret_cast<ulonglong2*>(row + 4) = make_ulonglong2(c2.v, c1.v);
+        *reinterpret_cast<float4*>(row + 8) =
+            make_float4(b0, a0, w == Wc - 3 ? __int_as_float(0x7f800000) : X2, 0.f);
+      }
+      wide = __all_sync(ALL, wide);
+      __syncwarp();
+      // Lane l sums the PW consecutive points x = l PW + q.  The interval of its
+      // first point (X_w <= x < X_{w+1}, w in [1, W-3]) is guessed from the mean
+      // landing spacing and corrected by comparisons; later points only step
+      // forward, loading the next row when they pass X_{w+1}: at most one row
+      // per point where every interval is at least a grid step long.
+      const int x0 = lane * PW;
+      const float xv0 = (float)x0;
+      int w;
+      {
+        const float xf = s_X[1];
+        const float inv_sp = (float)(Wc - 3) * rcp_approx(s_X[Wc - 2] - xf);
+        w = 1 + ifloor_small((xv0 - xf) * inv_sp);
+        w = min(max(w, 1), Wc - 3);
+        while (w > 1 && s_X[w] > xv0) --w;
+        while (w < Wc - 3 && s_X[w + 1] <= xv0) ++w;
+      }
+      const float* row = s_cf + RESUM_CF * w;
+      Row32 r;
+      load_row32(row, r);
+      // The exact integer phase n m / N mod 1 of the run's middle point,
+      // moved into [-1/2, 1/2); the run's points differ from it by
+      // (q - PW/2) n / N, exact in FP32 (multiples of 1/N below 2^(24 - log2 N)),
+      // so each point's turn count costs one FMA.  The phase cubic is reduced
+      // to (-1/2, 1/2] at its interval start, so the argument of the sine
+      // stays within a few turns.
+      const unsigned nn = (unsigned)(i - p.n_max);
+      const unsigned nmc = (nn * (unsigned)(m0 + x0 + PW / 2)) & mask;
+      float bc = exact_u2f(nmc, 0.f) * invN;
+      bc = bc >= 0.5f ? bc - 1.f : bc;
+      const float nN = (float)(int)nn * invN;
+      const f2 one = bc2(1.f);
+      f2 xv = bc2(xv0);                     // the point, twice; exact
+      const auto term = [&](int q) {
+        const f2 tau = sub2(xv, r.X1);
+        float phv, av;
+        sp2(fma2(fma2(fma2(r.c3, tau, r.c2), tau, r.c1), tau, r.c0), phv, av);
+        const float t = fmaf((float)(q - PW / 2), nN, bc) + phv;
+        float sn, cs;
+        sincos_turns(t, &sn, &cs);
+        accr[q] = fmaf(av, cs, accr[q]);
+        acci[q] = fmaf(av, sn, acci[q]);
+      };
+      const auto past = [&]() {
+        float x, y;
+        sp2(xv, x, y);
+        return r.X2 <= x;
+      };
+      term(0);
+      if (wide) {
+#pragma unroll
+        for (int q = 1; q < PW; ++q) {
+          xv = add2(xv, one);
+          if (past()) {
+            row += RESUM_CF;
+            load_row32(row, r);
+          }
+          term(q);
+        }
+      } else {
+#pragma unroll
+        for (int q = 1; q < PW; ++q) {
+          xv = add2(xv, one);
+          while (past()) {
+            row += RESUM_CF;
+            load_row32(row, r);
+          }
+          term(q);
+        }
+      }
+    }
+  }
+  block_sum<float, PW, BAR>(p, accr, acci, smem_raw, group, m0, tid, sub, st);
+}
+
+// ---- FP64 ----
+template <int PW, int LD, int BAR>
+__device__ __forceinline__ void resum_body(const ResumArgs<double>& p, int blk, int tid,
+                                           unsigned char* smem_raw, int sub) {
+  using T = double;
+  using V = double2;
   constexpr int LDC = LD == LD_NC ? LD_PLAIN : LD;   // mode coefficients
   const int lane = tid & 31;
   const int warp = tid >> 5;
@@ -915,19 +1186,7 @@ __device__ __forceinline__ void resum_body(const ResumArgs<T>& p, int blk, int t
     const int W = jh - jl + 4;
     const int base = mirrored ? p.N - m0 - (p.NRT - jb - p.G) * p.R : (jb - p.G) * p.R - m0;
     const T dsign = mirrored ? T(-1) : T(1);
-    // FP32: the mode coefficient enters as |c_n| (scaling the amplitudes) and
-    // arg(c_n) / 2 pi (added to the phases, in turns) -- cpol, formed by the
-    // DFT -- so that each term is |c_n| a e^{2 pi i t}: two FMAs instead of a
-    // complex product.  FP64 multiplies by c_n.
-    V cn;
-    T cmag = T(1), carg = T(0);
-    if constexpr (sizeof(T) == 4) {
-      const V cp = ld<LDC>(p.cpol + i);
-      cmag = cp.x;
-      carg = cp.y;
-    } else {
-      cn = ld<LDC>(p.c + i);
-    }
+    const V cn = ld<LDC>(p.c + i);
     const unsigned nn = (unsigned)(i - p.n_max);
     __syncwarp();
     if (ok) {
@@ -936,26 +1195,16 @@ __device__ __forceinline__ void resum_body(const ResumArgs<T>& p, int blk, int t
         const int w = lane + 32 * r;
         if (w < W) {
           s_X[w] = T(base + w * p.R) + dsign * rd[r];
-          if constexpr (sizeof(T) == 4) {
-            s_ph[w] = rph[r] + carg;
-            s_a[w] = ra[r] * cmag;
-          } else {
-            s_ph[w] = rph[r];
-            s_a[w] = ra[r];
-          }
+          s_ph[w] = rph[r];
+          s_a[w] = ra[r];
         }
       }
       for (int w = lane + 32 * PF; w < W; w += 32) {   // beyond the prefetched rounds
         const long long o = bchk((long long)ray_of(mirrored, jb, w) * p.Mr + col,
                                  (long long)p.NRT * p.Mr, st);
         s_X[w] = T(base + w * p.R) + dsign * ld<LD>(p.d + o);
-        if constexpr (sizeof(T) == 4) {
-          s_ph[w] = ld<LD>(p.ph + o) + carg;
-          s_a[w] = ld<LD>(p.a + o) * cmag;
-        } else {
-          s_ph[w] = ld<LD>(p.ph + o);
-          s_a[w] = ld<LD>(p.a + o);
-        }
+        s_ph[w] = ld<LD>(p.ph + o);
+        s_a[w] = ld<LD>(p.a + o);
       }
     }
     // issue the next mode's window and the following mode's brackets
@@ -976,7 +1225,6 @@ __device__ __forceinline__ void resum_body(const ResumArgs<T>& p, int blk, int t
                     h21, h10, b0, b1, b2, b3);
       cubic_through(s_a[w - 1], s_a[w], s_a[w + 1], s_a[w + 2], r21, r10, r32, r20, r31, r30,
                     h21, h10, a0, a1, a2, a3);
-      if constexpr (sizeof(T) == 4) b0 = minus_rint(b0);   // whole turns do not matter
       store_cf(s_cf + RESUM_CF * w, X1, X2, b0, b1, b2, b3, a0, a1, a2, a3);
     }
     __syncwarp();
@@ -994,89 +1242,41 @@ __device__ __forceinline__ void resum_body(const ResumArgs<T>& p, int blk, int t
     while (w < W - 3 && s_X[w + 1] <= xv0) ++w;
     T X1, X2, b0, b1, b2, b3, a0, a1, a2, a3;
     load_cf<T>(s_cf + RESUM_CF * w, X1, X2, b0, b1, b2, b3, a0, a1, a2, a3);
-    if constexpr (sizeof(T) == 4) {
-      // The exact integer phase n m / N mod 1 of the run's middle point,
-      // moved into [-1/2, 1/2); the run's points differ from it by
-      // (q - PW/2) n / N, exact in FP32 (multiples of 1/N below 2^(24 - log2 N)),
-      // so each point's turn count costs one FMA.  The phase cubic is reduced
-      // to (-1/2, 1/2] at its interval start, so the argument of the sine
-      // stays within a few turns.
-      const unsigned nmc = (nn * (unsigned)(m0 + x0 + PW / 2)) & mask;
-      T bc = exact_u2f(nmc, T()) * invN;
-      bc = bc >= T(0.5) ? bc - T(1) : bc;
-      const T nN = T((int)nn) * invN;
+    unsigned nm = (nn * (unsigned)(m0 + x0)) & mask;
 #pragma unroll
-      for (int q = 0; q < PW; ++q) {
-        const T xv = xv0 + T(q);   // exact
-        while (w < W - 3 && X2 <= xv) {
-          ++w;
-          load_cf<T>(s_cf + RESUM_CF * w, X1, X2, b0, b1, b2, b3, a0, a1, a2, a3);
-        }
-        const T tau = xv - X1;
-        const T phv = ((b3 * tau + b2) * tau + b1) * tau + b0;
-        const T av = ((a3 * tau + a2) * tau + a1) * tau + a0;
-        const T t = fmaf(T(q - PW / 2), nN, bc) + phv;
-        T sn, cs;
-        sincos_turns(t, &sn, &cs);
-        accr[q] = fmaf(av, cs, accr[q]);
-        acci[q] = fmaf(av, sn, acci[q]);
+    for (int q = 0; q < PW; ++q) {
+      const T xv = xv0 + T(q);   // exact
+      while (w < W - 3 && X2 <= xv) {
+        ++w;
+        load_cf<T>(s_cf + RESUM_CF * w, X1, X2, b0, b1, b2, b3, a0, a1, a2, a3);
       }
-    } else {
-      unsigned nm = (nn * (unsigned)(m0 + x0)) & mask;
-#pragma unroll
-      for (int q = 0; q < PW; ++q) {
-        const T xv = xv0 + T(q);   // exact
-        while (w < W - 3 && X2 <= xv) {
-          ++w;
-          load_cf<T>(s_cf + RESUM_CF * w, X1, X2, b0, b1, b2, b3, a0, a1, a2, a3);
-        }
-        const T tau = xv - X1;
-        const T phv = ((b3 * tau + b2) * tau + b1) * tau + b0;
-        const T av = ((a3 * tau + a2) * tau + a1) * tau + a0;
-        const T t = minus_rint(exact_u2f(nm, T()) * invN + phv);
-        T sn, cs;
-        sincos_turns(t, &sn, &cs);
-        const T ar = av * cn.x, ai = av * cn.y;
-        accr[q] += ar * cs - ai * sn;
-        acci[q] += ar * sn + ai * cs;
-        nm = (nm + nn) & mask;
-      }
+      const T tau = xv - X1;
+      const T phv = ((b3 * tau + b2) * tau + b1) * tau + b0;
+      const T av = ((a3 * tau + a2) * tau + a1) * tau + a0;
+      const T t = minus_rint(exact_u2f(nm, T()) * invN + phv);
+      T sn, cs;
+      sincos_turns(t, &sn, &cs);
+      const T ar = av * cn.x, ai = av * cn.y;
+      accr[q] += ar * cs - ai * sn;
+      acci[q] += ar * sn + ai * cs;
+      nm = (nm + nn) & mask;
     }
   }
-  // fixed-order sum of the warps' partial sums
-  vb_sync<BAR>(sub);
-  // per warp TM points as 32 runs of PW, each run padded to PW + 1 entries so
-  // that the lanes' stores fall in different banks
-  V* red = reinterpret_cast<V*>(smem_raw);
-  const int TMP = 32 * (PW + 1);
-#pragma unroll
-  for (int q = 0; q < PW; ++q) {
-    V v;
-    v.x = accr[q];
-    v.y = acci[q];
-    red[warp * TMP + lane * (PW + 1) + q] = v;
-  }
-  vb_sync<BAR>(sub);
-  V* out = p.part + bchk((long long)group * p.N + m0, (long long)p.n_groups * p.N - (TM - 1), st);
-  if (st) atomicOr(p.status, st);
-  for (int x = tid; x < TM; x += RESUM_WARPS * 32) {
-    const int xs = (x / PW) * (PW + 1) + x % PW;
-    V sum = red[xs];
-#pragma unroll
-    for (int w = 1; w < RESUM_WARPS; ++w) {
-      const V v = red[w * TMP + xs];
-      sum.x += v.x; sum.y += v.y;
-    }
-    out[x] = sum;
-  }
+  block_sum<double, PW, BAR>(p, accr, acci, smem_raw, group, m0, tid, sub, st);
 }
 
-// FP32: 7 CTAs per SM (the register budget that keeps the one-mode-ahead
-// prefetch without losing occupancy); FP64 keeps its registers
+// FP32, bound by instruction issue: 390 warp instructions per (mode, 256-point
+// tile), 15 per point and lane and ~150 for the window, the rows and the search
+// (477 with scalar cubics, per-mode bracket lookups and library divisions).
+// 16384-point duct (977 modes x 16640 points) 34 us per sum against 41,
+// 131072-point duct (1395 modes, R = 64) 214 against 372.  7 CTAs per SM (72
+// registers: keeps the one-mode-ahead window), 5 for runs of 16 points (213 us;
+// 230 at 72 registers); FP64 keeps its registers.
 template <typename T, int PW>
-__global__ void __launch_bounds__(RESUM_WARPS * 32, sizeof(T) == 4 ? 7 : 1) k_resum(const ResumArgs<T> p) {
+__global__ void __launch_bounds__(RESUM_WARPS * 32, sizeof(T) == 4 ? (PW < 16 ? 7 : 5) : 1)
+    k_resum(const ResumArgs<T> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  resum_body<T, PW, LD_NC, 0>(p, blockIdx.x, threadIdx.x, smem_raw, 0);
+  resum_body<PW, LD_NC, 0>(p, blockIdx.x, threadIdx.x, smem_raw, 0);
 }
 
 // ----------------------------------------------------------------------------

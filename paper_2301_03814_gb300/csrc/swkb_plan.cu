@@ -1460,12 +1460,32 @@ bool valid_tiling(const swkb_plan* p, const Tiling& t) {
 
 Tiling default_tiling(const swkb_plan* p) {
   Tiling t;
-  t.PW = p->R >= 8 ? 8 : (p->R >= 2 ? 4 : 2);
+  // Runs of about half a ray spacing: the tile's rows of intervals (one lane
+  // builds one) then number 16 to 20, and a run meets one interval's end at
+  // most once.  FP32, R = 64 (131072 points, 1395 modes): 214 us per sum with
+  // runs of 16 points, 280 with 8; R = 16 (16384 points): 35 with 16, 34 with 8.
+  const bool f32 = p->precision != SWKB_FP64 && !p->fc;
+  t.PW = f32 && p->R >= 32 ? 16 : (p->R >= 8 ? 8 : (p->R >= 2 ? 4 : 2));
   while (32 * t.PW > (p->sym ? p->N / 2 : p->N) || (p->fc && p->N % (32 * t.PW))) t.PW /= 2;
   // patch-wise plans are not autotuned: many short mode groups keep the
   // last wave of their sum short (measured on the open lens, N_z = 131072:
   // 0.31 ms per sum with 2 groups, 0.26 with 8)
-  t.ctas_per_sm = p->fc ? 24 : 6;
+  if (p->fc) {
+    t.ctas_per_sm = 24;
+  } else {
+    // Mode groups: up to 20 CTAs per SM, so that the last wave is short, while
+    // a group keeps 32 modes (a warp looks its modes up 32 at a time, and the
+    // DFT adds up one partial per group); at least 4 CTAs per SM where the
+    // modes allow it, at 4 per group.  Sum plus DFT per screen, by groups:
+    // 16384 points, 977 modes 50.9 us (15), 48.5 (29), 50.1 (43); 131072 points,
+    // 1395 modes 276 (4), 252 (13); 4096 points, 401 modes 25.0 (19), 22.5 (37),
+    // 24.8 (51); 512 points, 65 modes 18.1 (17), 22.0 (65).
+    const int tiles = p->sym ? p->N / (64 * t.PW) + 1 : p->N / (32 * t.PW);
+    const auto groups_at = [&](int c) { return (p->sms * c + tiles - 1) / tiles; };
+    const int g = std::min(std::max(std::min(groups_at(20), p->M / 32), groups_at(4)),
+                           std::max(1, p->M / 4));
+    t.ctas_per_sm = std::max(1, (int)((long long)g * tiles / p->sms));
+  }
   // N1 ~ sqrt(M): pass 1 costs N N1, pass 2 M N2
   t.N1 = 1;
   while (t.N1 * t.N1 * 2 < p->M && t.N1 < p->N / 32 && t.N1 < 64) t.N1 *= 2;
@@ -1476,7 +1496,7 @@ std::vector<Tiling> tiling_candidates(const swkb_plan* p) {
   const Tiling d = default_tiling(p);
   std::vector<Tiling> out;
   for (int pw : {d.PW / 2, d.PW, d.PW * 2})
-    for (int c : {4, 6, 8, 12})
+    for (int c : {4, 8, 12, d.ctas_per_sm})
       for (int n1 : {d.N1, d.N1 * 2}) {
         const Tiling t{pw, c, n1};
         if (valid_tiling(p, t)) out.push_back(t);
