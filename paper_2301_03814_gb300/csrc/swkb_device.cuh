@@ -745,58 +745,11 @@ __global__ void __launch_bounds__(256) k_bracket(const BracketArgs<T> p) {
 //      phase with its integer part exact (k kappa_n (z_m - z_lo) =
 //      2 pi (n m mod N) / N), sincos, complex multiply-accumulate.
 constexpr int RESUM_WARPS = 4;
-constexpr int RESUM_CF = 12;      // X_w, 4 phase + 4 amplitude coefficients, X_{w+1}, 2 pad
+constexpr int RESUM_CF = 12;      // values per interval row (X_w, X_{w+1}, two cubics, padding)
 
 template <typename T>
 __device__ __forceinline__ int resum_warp_bytes(int wcap) {
   return ((RESUM_CF + 3) * wcap * (int)sizeof(T) + 15) & ~15;
-}
-
-// one coefficient row (X_w, phase b0..b3, amplitude a0..a3), vector stores:
-// rows are 48 B (FP32) apart, so a quarter-warp writes 32 distinct banks
-// Row of interval w: X_w, phase cubic b0..b3, amplitude cubic a0..a3, X_{w+1}.
-__device__ __forceinline__ void store_cf(float* p, float X1, float X2, float b0, float b1,
-                                         float b2, float b3, float a0, float a1, float a2,
-                                         float a3) {
-  *reinterpret_cast<float4*>(p) = make_float4(X1, b0, b1, b2);
-  *reinterpret_cast<float4*>(p + 4) = make_float4(b3, a0, a1, a2);
-  *reinterpret_cast<float4*>(p + 8) = make_float4(a3, X2, 0.f, 0.f);
-}
-__device__ __forceinline__ void store_cf(double* p, double X1, double X2, double b0, double b1,
-                                         double b2, double b3, double a0, double a1, double a2,
-                                         double a3) {
-  *reinterpret_cast<double2*>(p) = make_double2(X1, b0);
-  *reinterpret_cast<double2*>(p + 2) = make_double2(b1, b2);
-  *reinterpret_cast<double2*>(p + 4) = make_double2(b3, a0);
-  *reinterpret_cast<double2*>(p + 6) = make_double2(a1, a2);
-  *reinterpret_cast<double2*>(p + 8) = make_double2(a3, X2);
-}
-
-template <typename T>
-__device__ __forceinline__ void load_cf(const T* p, T& X1, T& X2, T& b0, T& b1, T& b2, T& b3,
-                                        T& a0, T& a1, T& a2, T& a3);
-template <>
-__device__ __forceinline__ void load_cf<float>(const float* p, float& X1, float& X2, float& b0,
-                                               float& b1, float& b2, float& b3, float& a0,
-                                               float& a1, float& a2, float& a3) {
-  const float4 u = *reinterpret_cast<const float4*>(p);
-  const float4 v = *reinterpret_cast<const float4*>(p + 4);
-  const float2 w = *reinterpret_cast<const float2*>(p + 8);
-  X1 = u.x; b0 = u.y; b1 = u.z; b2 = u.w; b3 = v.x; a0 = v.y; a1 = v.z; a2 = v.w;
-  a3 = w.x; X2 = w.y;
-}
-template <>
-__device__ __forceinline__ void load_cf<double>(const double* p, double& X1, double& X2,
-                                                double& b0, double& b1, double& b2, double& b3,
-                                                double& a0, double& a1, double& a2,
-                                                double& a3) {
-  const double2 u = *reinterpret_cast<const double2*>(p);
-  const double2 v = *reinterpret_cast<const double2*>(p + 2);
-  const double2 w = *reinterpret_cast<const double2*>(p + 4);
-  const double2 x = *reinterpret_cast<const double2*>(p + 6);
-  const double2 y = *reinterpret_cast<const double2*>(p + 8);
-  X1 = u.x; b0 = u.y; b1 = v.x; b2 = v.y; b3 = w.x; a0 = w.y; a1 = x.x; a2 = x.y;
-  a3 = y.x; X2 = y.y;
 }
 
 // Newton divided differences through (X1, X2, X0, X3), rewritten as a cubic
@@ -1087,12 +1040,41 @@ __device__ __forceinline__ void resum_body(const ResumArgs<float>& p, int blk, i
 }
 
 // ---- FP64 ----
+// sin / cos of 2 pi t: t = k / TRIG_N + r with |r| <= 1 / (2 TRIG_N); the
+// table's entry exp(2 pi i k / TRIG_N) (correctly rounded on the host) rotated by
+// the angle 2 pi r <= pi / 1024, whose sine and cosine - 1 need two and three
+// Taylor terms (the next ones are below 2e-18).  13 FP64 operations, absolute
+// error about one unit in the last place of 1; any |t| < 2^41.
+__device__ __forceinline__ void sincos_table(const double2* trig, double t, double* s, double* c) {
+  const double magic = 6755399441055744.0;   // 1.5 * 2^52: rounds to an integer
+  const double v = fma(t, (double)TRIG_N, magic);
+  const double r = fma(v - magic, -1.0 / TRIG_N, t);
+  const double2 e = __ldg(trig + (__double2loint(v) & (TRIG_N - 1)));
+  const double r2 = r * r;
+  const double sr = r * fma(r2, fma(r2, 81.60524927607503, -41.34170224039975), 6.283185307179586);
+  const double cr = r2 * fma(r2, 64.93939402266828, -19.73920880217872);   // cos - 1
+  *c = fma(e.x, cr, fma(-e.y, sr, e.x));
+  *s = fma(e.y, cr, fma(e.x, sr, e.y));
+}
+
+// Interval row: X_w, X_{w+1}, phase b0..b3, amplitude a0..a3.
+struct Row64 {
+  double X1, X2, b0, b1, b2, b3, a0, a1, a2, a3;
+};
+__device__ __forceinline__ Row64 load_row64(const double* p) {
+  const double2* q = reinterpret_cast<const double2*>(p);
+  const double2 u = q[0], v = q[1], w = q[2], x = q[3], y = q[4];
+  return Row64{u.x, u.y, v.x, v.y, w.x, w.y, x.x, x.y, y.x, y.y};
+}
+
+// As the FP32 block; bound by the FP64 pipe, so reciprocals take 3 FP64
+// operations (rcp64), a term 24, and a run's next interval is found by integer
+// comparisons.
 template <int PW, int LD, int BAR>
 __device__ __forceinline__ void resum_body(const ResumArgs<double>& p, int blk, int tid,
                                            unsigned char* smem_raw, int sub) {
-  using T = double;
-  using V = double2;
   constexpr int LDC = LD == LD_NC ? LD_PLAIN : LD;   // mode coefficients
+  constexpr unsigned ALL = 0xffffffffu;
   const int lane = tid & 31;
   const int warp = tid >> 5;
   const int tt = blk % p.n_tiles_run;
@@ -1101,165 +1083,171 @@ __device__ __forceinline__ void resum_body(const ResumArgs<double>& p, int blk, 
   const int tile = p.sym ? (tt < half ? half + tt : 0) : tt;
   const int wcap = p.wcap;
   const int TM = p.TM;
-  unsigned char* wbase = smem_raw + (long long)warp * resum_warp_bytes<T>(wcap);
-  T* s_cf = reinterpret_cast<T*>(wbase);            // [wcap][RESUM_CF], 16-byte aligned
-  T* s_X = s_cf + RESUM_CF * wcap;
-  T* s_ph = s_X + wcap;
-  T* s_a = s_ph + wcap;
+  unsigned char* wbase = smem_raw + (long long)warp * resum_warp_bytes<double>(wcap);
+  double* s_cf = reinterpret_cast<double*>(wbase);            // [wcap][RESUM_CF], 16-byte aligned
+  double2* s_pa = reinterpret_cast<double2*>(s_cf + RESUM_CF * wcap);   // phase, amplitude
+  double* s_X = reinterpret_cast<double*>(s_pa + wcap);
   const int m0 = tile * TM;
   const int i0 = group * p.modes_per_group;
   const int i1 = min(p.M, i0 + p.modes_per_group);
-  const int lgN = __ffs(p.N) - 1;
-  const T invN = scalbn(T(1), -lgN);               // exact
+  const double invN = scalbn(1.0, -(__ffs(p.N) - 1));         // exact
   const unsigned mask = (unsigned)p.N - 1u;
+  const long long nrm = (long long)p.NRT * p.Mr;
+  const int x0 = lane * PW;
+  const double xv0 = (double)x0;
   unsigned st = 0;
 
-  T accr[PW], acci[PW];
+  double accr[PW], acci[PW];
 #pragma unroll
-  for (int q = 0; q < PW; ++q) { accr[q] = T(0); acci[q] = T(0); }
+  for (int q = 0; q < PW; ++q) { accr[q] = 0.0; acci[q] = 0.0; }
 
-  // Software pipeline over this warp's modes: the bracket entries are
-  // loaded two modes ahead and the ray window (landing offset, phase,
-  // amplitude; the first 32 rays) one mode ahead into registers, so their
-  // global-memory latency overlaps the current mode's arithmetic.
-  // grounded: mode n < 0 is the mirror image of mode -n (column -n); its
-  // ray j' is ray NRT - j' of mode -n, landing at N - g
-  constexpr int PF = 1;
-  T rd[PF], rph[PF], ra[PF];
   auto column = [&](int i, bool& mir) {
     const int n = i - p.n_max;
     mir = p.sym && n < 0;
     return p.sym ? (n < 0 ? -n : n) : i;
   };
-  auto load_head = [&](int i, int& jl, int& jh) {
-    jl = -1; jh = -1;
-    if (i >= i1) return;
+  double rd = 0.0, rph = 0.0, ra = 0.0;   // the next mode's first 32 rays
+  auto fetch = [&](int i, int r0, int w, double& d, double& ph, double& a) {
     bool mir;
     const int col = column(i, mir);
-    const int* jt = mir ? p.jlo_neg : p.jlo;
-    const long long nj = (long long)(p.n_tiles + 1) * p.Mr;
-    jl = ld<LD>(jt + bchk((long long)tile * p.Mr + col, nj, st));
-    jh = ld<LD>(jt + bchk((long long)(tile + 1) * p.Mr + col, nj, st));
-  };
-  // A bracket table left inconsistent by a failed screen (already flagged by
-  // k_bracket) must not send the reads out of [0, NRT); a window wider than
-  // the tile's capacity means rays compressed beyond it (flagged here).
-  auto head_ok = [&](int i, int jl, int jh) {
-    if (i >= i1) return false;
-    bool mir;
-    column(i, mir);
-    if (jl < (mir ? 2 : 1) || jh < jl || jh > p.NRT - 3) return false;
-    if (jh - jl + 4 > wcap) { st |= ST_CAUSTIC; return false; }
-    return true;
-  };
-  // ray index of window slot w (mirrored families run backwards)
-  auto ray_of = [&](bool mir, int jb, int w) { return mir ? p.NRT - jb - w : jb + w; };
-  auto prefetch = [&](int i, int jl, int jh) {
-    bool mir;
-    const int col = column(i, mir);
-    const int jb = jl - 1, W = jh - jl + 4;
-#pragma unroll
-    for (int r = 0; r < PF; ++r) {
-      const int w = lane + 32 * r;
-      if (w < W) {
-        const long long o = bchk((long long)ray_of(mir, jb, w) * p.Mr + col,
-                                 (long long)p.NRT * p.Mr, st);
-        rd[r] = ld<LD>(p.d + o);
-        rph[r] = ld<LD>(p.ph + o);
-        ra[r] = ld<LD>(p.a + o);
-      }
-    }
+    const long long o = bchk((long long)(mir ? r0 - w : r0 + w) * p.Mr + col, nrm, st);
+    d = ld<LD>(p.d + o);
+    ph = ld<LD>(p.ph + o);
+    a = ld<LD>(p.a + o);
   };
 
-  int i = i0 + warp;
-  int jl_c, jh_c, jl_n, jh_n;
-  load_head(i, jl_c, jh_c);
-  load_head(i + RESUM_WARPS, jl_n, jh_n);
-  bool ok_c = head_ok(i, jl_c, jh_c);
-  if (ok_c) prefetch(i, jl_c, jh_c);
-  for (; i < i1; i += RESUM_WARPS) {
-    const bool ok = ok_c;
-    const int jl = jl_c, jh = jh_c;
-    bool mirrored;
-    const int col = column(i, mirrored);
-    const int jb = jl - 1;
-    const int W = jh - jl + 4;
-    const int base = mirrored ? p.N - m0 - (p.NRT - jb - p.G) * p.R : (jb - p.G) * p.R - m0;
-    const T dsign = mirrored ? T(-1) : T(1);
-    const V cn = ld<LDC>(p.c + i);
-    const unsigned nn = (unsigned)(i - p.n_max);
-    __syncwarp();
-    if (ok) {
+  for (int ib = i0 + warp; ib < i1; ib += 32 * RESUM_WARPS) {
+    // lane k: the brackets and coefficient of mode ib + RESUM_WARPS k
+    int h_r0 = 0, h_W = 0, h_base = 0;
+    double h_mag = 0.0, h_arg = 0.0;
+    {
+      const int i = ib + RESUM_WARPS * lane;
+      if (i < i1) {
+        bool mir;
+        const int col = column(i, mir);
+        const int* jt = mir ? p.jlo_neg : p.jlo;
+        const long long nj = (long long)(p.n_tiles + 1) * p.Mr;
+        const int jl = ld<LD>(jt + bchk((long long)tile * p.Mr + col, nj, st));
+        const int jh = ld<LD>(jt + bchk((long long)(tile + 1) * p.Mr + col, nj, st));
+        // (inconsistent or too wide windows: as in the FP32 block)
+        if (jl >= (mir ? 2 : 1) && jh >= jl && jh <= p.NRT - 3) {
+          h_W = jh - jl + 4;
+          if (h_W > wcap) { st |= ST_CAUSTIC; h_W = 0; }
+        }
+        const int jb = jl - 1;
+        h_r0 = mir ? p.NRT - jb : jb;
+        h_base = mir ? p.N - m0 - (p.NRT - jb - p.G) * p.R : (jb - p.G) * p.R - m0;
+        const double2 cp = ld<LDC>(p.cpol + i);
+        h_mag = cp.x;
+        h_arg = cp.y;
+      }
+    }
+    const int K = min(32, (i1 - ib + RESUM_WARPS - 1) / RESUM_WARPS);
+    int r0 = __shfl_sync(ALL, h_r0, 0), W = __shfl_sync(ALL, h_W, 0);
+    if (lane < W) fetch(ib, r0, lane, rd, rph, ra);
+    for (int k = 0; k < K; ++k) {
+      const int i = ib + RESUM_WARPS * k;
+      const int Wc = W, rc = r0;
+      const int base = __shfl_sync(ALL, h_base, k);
+      const double cmag = __shfl_sync(ALL, h_mag, k);
+      const double carg = __shfl_sync(ALL, h_arg, k);
+      const double dsign = p.sym && i < p.n_max ? -1.0 : 1.0;
+      __syncwarp();
+      if (lane < Wc) {
+        s_X[lane] = fma(dsign, rd, (double)(base + lane * p.R));
+        s_pa[lane] = make_double2(rph + carg, ra * cmag);
+      }
+      for (int w = lane + 32; w < Wc; w += 32) {   // beyond the prefetched rays
+        double d, ph, a;
+        fetch(i, rc, w, d, ph, a);
+        s_X[w] = fma(dsign, d, (double)(base + w * p.R));
+        s_pa[w] = make_double2(ph + carg, a * cmag);
+      }
+      if (k + 1 < K) {   // issue the next mode's window
+        r0 = __shfl_sync(ALL, h_r0, k + 1);
+        W = __shfl_sync(ALL, h_W, k + 1);
+        if (lane < W) fetch(i + RESUM_WARPS, r0, lane, rd, rph, ra);
+      }
+      if (Wc == 0) continue;
+      __syncwarp();
+      bool wide = true;
+      for (int w = 1 + lane; w <= Wc - 3; w += 32) {
+        const double X0 = s_X[w - 1], X1 = s_X[w], X2 = s_X[w + 1], X3 = s_X[w + 2];
+        const double2 f0 = s_pa[w - 1], f1 = s_pa[w], f2 = s_pa[w + 1], f3 = s_pa[w + 2];
+        const double h21 = X2 - X1, h10 = X1 - X0;
+        wide = wide && h21 >= 1.0;
+        const double r21 = rcp64(h21), r10 = rcp64(h10), r32 = rcp64(X3 - X2);
+        const double r20 = rcp64(X2 - X0), r31 = rcp64(X3 - X1), r30 = rcp64(X3 - X0);
+        double b0, b1, b2, b3, a0, a1, a2, a3;
+        cubic_through(f0.x, f1.x, f2.x, f3.x, r21, r10, r32, r20, r31, r30, h21, h10, b0, b1, b2,
+                      b3);
+        cubic_through(f0.y, f1.y, f2.y, f3.y, r21, r10, r32, r20, r31, r30, h21, h10, a0, a1, a2,
+                      a3);
+        double2* row = reinterpret_cast<double2*>(s_cf + RESUM_CF * w);
+        // the last row's end is stored as infinity: no lane steps past it
+        row[0] = make_double2(X1, w == Wc - 3 ? __longlong_as_double(0x7ff0000000000000ll) : X2);
+        row[1] = make_double2(b0, b1);
+        row[2] = make_double2(b2, b3);
+        row[3] = make_double2(a0, a1);
+        row[4] = make_double2(a2, a3);
+      }
+      wide = __all_sync(ALL, wide);
+      __syncwarp();
+      // interval of the lane's first point, as in the FP32 block
+      int w;
+      {
+        const float xf = (float)s_X[1];
+        const float inv_sp = (float)(Wc - 3) / ((float)s_X[Wc - 2] - xf);
+        w = 1 + ifloor_small(((float)x0 - xf) * inv_sp);
+        w = min(max(w, 1), Wc - 3);
+        while (w > 1 && s_X[w] > xv0) --w;
+        while (w < Wc - 3 && s_X[w + 1] <= xv0) ++w;
+      }
+      const double* row = s_cf + RESUM_CF * w;
+      Row64 r;
+      double t0;   // the run's first point in the row's tau
+      int q_end;   // first point of the run past the row's interval
+      const auto enter = [&]() {
+        r = load_row64(row);
+        t0 = xv0 - r.X1;
+        const double d = r.X2 - xv0;          // exact where it decides
+        q_end = d < (double)PW ? __double2int_ru(d) : PW;
+      };
+      enter();
+      // exact integer phase of the run's middle point and n / N per point from
+      // it, as in the FP32 block (exact: multiples of 1/N)
+      const unsigned nn = (unsigned)(i - p.n_max);
+      const double bc = (double)((nn * (unsigned)(m0 + x0 + PW / 2)) & mask) * invN;
+      const double nN = (double)(int)nn * invN;
+      const auto term = [&](int q) {
+        const double tau = t0 + (double)q;
+        const double phv = ((r.b3 * tau + r.b2) * tau + r.b1) * tau + r.b0;
+        const double av = ((r.a3 * tau + r.a2) * tau + r.a1) * tau + r.a0;
+        double sn, cs;
+        sincos_table(p.trig, fma((double)(q - PW / 2), nN, bc) + phv, &sn, &cs);
+        accr[q] = fma(av, cs, accr[q]);
+        acci[q] = fma(av, sn, acci[q]);
+      };
+      term(0);
+      if (wide) {
 #pragma unroll
-      for (int r = 0; r < PF; ++r) {
-        const int w = lane + 32 * r;
-        if (w < W) {
-          s_X[w] = T(base + w * p.R) + dsign * rd[r];
-          s_ph[w] = rph[r];
-          s_a[w] = ra[r];
+        for (int q = 1; q < PW; ++q) {
+          if (q >= q_end) {
+            row += RESUM_CF;
+            enter();
+          }
+          term(q);
+        }
+      } else {
+#pragma unroll
+        for (int q = 1; q < PW; ++q) {
+          while (q >= q_end) {
+            row += RESUM_CF;
+            enter();
+          }
+          term(q);
         }
       }
-      for (int w = lane + 32 * PF; w < W; w += 32) {   // beyond the prefetched rounds
-        const long long o = bchk((long long)ray_of(mirrored, jb, w) * p.Mr + col,
-                                 (long long)p.NRT * p.Mr, st);
-        s_X[w] = T(base + w * p.R) + dsign * ld<LD>(p.d + o);
-        s_ph[w] = ld<LD>(p.ph + o);
-        s_a[w] = ld<LD>(p.a + o);
-      }
-    }
-    // issue the next mode's window and the following mode's brackets
-    jl_c = jl_n;
-    jh_c = jh_n;
-    ok_c = head_ok(i + RESUM_WARPS, jl_c, jh_c);
-    if (ok_c) prefetch(i + RESUM_WARPS, jl_c, jh_c);
-    load_head(i + 2 * RESUM_WARPS, jl_n, jh_n);
-    if (!ok) continue;
-    __syncwarp();
-    for (int w = 1 + lane; w <= W - 3; w += 32) {
-      const T X0 = s_X[w - 1], X1 = s_X[w], X2 = s_X[w + 1], X3 = s_X[w + 2];
-      const T h21 = X2 - X1, h10 = X1 - X0;
-      const T r21 = T(1) / h21, r10 = T(1) / h10, r32 = T(1) / (X3 - X2);
-      const T r20 = T(1) / (X2 - X0), r31 = T(1) / (X3 - X1), r30 = T(1) / (X3 - X0);
-      T b0, b1, b2, b3, a0, a1, a2, a3;
-      cubic_through(s_ph[w - 1], s_ph[w], s_ph[w + 1], s_ph[w + 2], r21, r10, r32, r20, r31, r30,
-                    h21, h10, b0, b1, b2, b3);
-      cubic_through(s_a[w - 1], s_a[w], s_a[w + 1], s_a[w + 2], r21, r10, r32, r20, r31, r30,
-                    h21, h10, a0, a1, a2, a3);
-      store_cf(s_cf + RESUM_CF * w, X1, X2, b0, b1, b2, b3, a0, a1, a2, a3);
-    }
-    __syncwarp();
-    // Lane l sums the PW consecutive points x = l PW + q.  The interval of its
-    // first point (X_w <= x < X_{w+1}, w in [1, W-3]) is guessed from the mean
-    // landing spacing and corrected by comparisons; later points only step
-    // forward, reloading the row when they pass X_{w+1}.
-    const T xf = s_X[1];
-    const T inv_sp = T(W - 3) / (s_X[W - 2] - xf);
-    const int x0 = lane * PW;
-    const T xv0 = T(x0);
-    int w = 1 + ifloor_small(xv0 * inv_sp - xf * inv_sp);
-    w = min(max(w, 1), W - 3);
-    while (w > 1 && s_X[w] > xv0) --w;
-    while (w < W - 3 && s_X[w + 1] <= xv0) ++w;
-    T X1, X2, b0, b1, b2, b3, a0, a1, a2, a3;
-    load_cf<T>(s_cf + RESUM_CF * w, X1, X2, b0, b1, b2, b3, a0, a1, a2, a3);
-    unsigned nm = (nn * (unsigned)(m0 + x0)) & mask;
-#pragma unroll
-    for (int q = 0; q < PW; ++q) {
-      const T xv = xv0 + T(q);   // exact
-      while (w < W - 3 && X2 <= xv) {
-        ++w;
-        load_cf<T>(s_cf + RESUM_CF * w, X1, X2, b0, b1, b2, b3, a0, a1, a2, a3);
-      }
-      const T tau = xv - X1;
-      const T phv = ((b3 * tau + b2) * tau + b1) * tau + b0;
-      const T av = ((a3 * tau + a2) * tau + a1) * tau + a0;
-      const T t = minus_rint(exact_u2f(nm, T()) * invN + phv);
-      T sn, cs;
-      sincos_turns(t, &sn, &cs);
-      const T ar = av * cn.x, ai = av * cn.y;
-      accr[q] += ar * cs - ai * sn;
-      acci[q] += ar * sn + ai * cs;
-      nm = (nm + nn) & mask;
     }
   }
   block_sum<double, PW, BAR>(p, accr, acci, smem_raw, group, m0, tid, sub, st);
@@ -1271,7 +1259,9 @@ __device__ __forceinline__ void resum_body(const ResumArgs<double>& p, int blk, 
 // 16384-point duct (977 modes x 16640 points) 34 us per sum against 41,
 // 131072-point duct (1395 modes, R = 64) 214 against 372.  7 CTAs per SM (72
 // registers: keeps the one-mode-ahead window), 5 for runs of 16 points (213 us;
-// 230 at 72 registers); FP64 keeps its registers.
+// 230 at 72 registers).  FP64, bound by its pipe: 1.05 ms on the 16384-point duct
+with 29 mode groups (1.78 with sincospi, library divisions and a complex
+coefficient per term; 24 FP64 operations per term instead of ~46).
 template <typename T, int PW>
 __global__ void __launch_bounds__(RESUM_WARPS * 32, sizeof(T) == 4 ? (PW < 16 ? 7 : 5) : 1)
     k_resum(const ResumArgs<T> p) {
@@ -1400,7 +1390,8 @@ __device__ __forceinline__ typename C2<T>::type cmul(typename C2<T>::type a,
 template <typename T>
 __device__ __forceinline__ typename C2<T>::type polar_turns(typename C2<T>::type v) {
   typename C2<T>::type r;
-  r.x = sqrt(v.x * v.x + v.y * v.y);
+  if constexpr (sizeof(T) == 8) r.x = hypot(v.x, v.y);
+  else r.x = sqrt(v.x * v.x + v.y * v.y);
   r.y = atan2(v.y, v.x) * T(0.15915494309189533577);
   return r;
 }

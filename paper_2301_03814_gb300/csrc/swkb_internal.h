@@ -18,6 +18,9 @@ enum : unsigned {
   ST_BOUNDS = 16u,   // bounds-checked builds: a device index left its buffer
 };
 
+// Entries of the FP64 sums' table of exp(2 pi i k / TRIG_N) (a power of two).
+constexpr int TRIG_N = 1024;
+
 // Columns n2 of the DFT's pass 1 handled by one block.
 constexpr int FFT1_COLS = 8;
 
@@ -102,8 +105,9 @@ struct ResumArgs {
   const T* a;
   const int* jlo;
   const int* jlo_neg;
-  const typename C2<T>::type* c;   // [M] mode coefficients, range phase folded in
-  const typename C2<T>::type* cpol; // [M] FP32: (|c_n|, arg(c_n) / 2 pi), read instead of c
+  const typename C2<T>::type* cpol; // [M] mode coefficients, range phase folded in, as
+                                    // (|c_n|, arg(c_n) / 2 pi)
+  const double2* trig;              // [TRIG_N] FP64: exp(2 pi i k / TRIG_N)
   int M, Mr, NRT, G, R, N, TM, PW, n_tiles, n_groups, modes_per_group, n_max, wcap;
   int sym;          // grounded: modes n < 0 are mirror images of -n; only the
                     // tiles of the physical half and tile 0 are summed

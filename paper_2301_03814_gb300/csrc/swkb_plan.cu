@@ -112,7 +112,8 @@ struct swkb_plan {
   void* part = nullptr;
   void* Y = nullptr;
   void* c = nullptr;
-  void* cpol = nullptr;   // FP32: (|c_n|, arg(c_n) / 2 pi) of c
+  void* cpol = nullptr;   // (|c_n|, arg(c_n) / 2 pi) of c
+  void* trig = nullptr;   // FP64: exp(2 pi i k / TRIG_N)
   void* rd = nullptr;
   void* rph = nullptr;
   void* ra = nullptr;
@@ -591,6 +592,20 @@ swkb_status build_device(swkb_plan* p, const swkb_profile* prof) {
     }
     TRY(upload<T>(p, &p->tw, tw));
   }
+  if (sizeof(T) == 8) {
+    std::vector<double> e(2 * TRIG_N);
+    for (int k = 0; k < TRIG_N; ++k) {
+      // eighths of a turn by symmetry, so that the quadrants' entries are exact
+      const int o = k / (TRIG_N / 8), m = k % (TRIG_N / 4);
+      const double a = 2.0 * M_PI / TRIG_N * (m <= TRIG_N / 8 ? m : TRIG_N / 4 - m);
+      double c = cos(a), s = sin(a);
+      if (m > TRIG_N / 8) std::swap(c, s);
+      const int quad = o / 2;
+      e[2 * k] = quad == 0 ? c : (quad == 1 ? -s : (quad == 2 ? -c : s));
+      e[2 * k + 1] = quad == 0 ? s : (quad == 1 ? c : (quad == 2 ? -s : -c));
+    }
+    TRY(upload<double>(p, &p->trig, e));
+  }
   // absorber
   if (p->absorber_frac > 0) {
     std::vector<double> w(N, 1.0);
@@ -610,7 +625,7 @@ swkb_status build_device(swkb_plan* p, const swkb_profile* prof) {
   TRY(dev_alloc(p, &p->part, (size_t)p->alloc_groups * N * sizeof(V)));
   if (!p->fc) TRY(dev_alloc(p, &p->Y, (size_t)N * sizeof(V)));
   TRY(dev_alloc(p, &p->c, (size_t)M * sizeof(V)));
-  if (sizeof(T) == 4) TRY(dev_alloc(p, &p->cpol, (size_t)M * sizeof(V)));
+  TRY(dev_alloc(p, &p->cpol, (size_t)M * sizeof(V)));
   const size_t rays = (size_t)p->NRT * p->Mr;
   TRY(dev_alloc(p, &p->rd, rays * sizeof(T)));
   TRY(dev_alloc(p, &p->rph, rays * sizeof(T)));
@@ -621,7 +636,7 @@ swkb_status build_device(swkb_plan* p, const swkb_profile* prof) {
     TRY(dev_alloc(p, &p->pl_ph, pr * sizeof(T)));
     TRY(dev_alloc(p, &p->pl_a, pr * sizeof(T)));
     TRY(dev_alloc(p, &p->c_plane, (size_t)M * sizeof(V)));
-    if (sizeof(T) == 4) TRY(dev_alloc(p, &p->cpol_plane, (size_t)M * sizeof(V)));
+    TRY(dev_alloc(p, &p->cpol_plane, (size_t)M * sizeof(V)));
     TRY(dev_alloc(p, &p->ephi_pl, (size_t)(p->planes - 1) * M * sizeof(V)));
   }
   const size_t jn = (size_t)(p->alloc_tiles + 1) * p->Mr;
@@ -768,7 +783,7 @@ ResumArgs<T> resum_args(const swkb_plan* p, const T* d, const T* ph, const T* a,
   ResumArgs<T> ra;
   ra.d = d; ra.ph = ph; ra.a = a; ra.jlo = jlo ? jlo : p->jlo;
   ra.jlo_neg = jlo ? jlo_neg : p->jlo_neg;
-  ra.c = c;
+  ra.trig = (const double2*)p->trig;
   ra.cpol = (c == (const typename C2<T>::type*)p->c) ? (const V*)p->cpol : (const V*)p->cpol_plane;
   ra.M = p->M; ra.Mr = p->Mr; ra.sym = p->sym; ra.n_tiles_run = p->n_tiles_run; ra.NRT = p->NRT;
   ra.G = p->G; ra.R = p->R; ra.N = p->N; ra.TM = p->TM;
@@ -1712,11 +1727,12 @@ size_t device_bytes(const swkb_plan* p) {
   b += (size_t)p->N * V;                                            // twiddles
   if (p->absorber_frac > 0) b += (size_t)p->N * T;                  // absorber
   b += (size_t)p->N * V * (2 + (size_t)p->alloc_groups) + (size_t)p->M * V;  // u, Y, partials, c
-  if (T == 4) b += (size_t)p->M * V;                                 // polar c
+  b += (size_t)p->M * V;                                            // polar c
+  if (T == 8) b += (size_t)TRIG_N * 16;                             // trig
   b += 3 * (size_t)p->NRT * p->Mr * T * (p->overlap ? 2 : 1);     // rays (one or two sets)
   if (p->planes > 1)                                                 // inner planes
     b += (size_t)(p->planes - 1) * (3 * (size_t)p->NRT * p->Mr * T + (size_t)p->M * V) +
-         (size_t)p->M * V * (T == 4 ? 2 : 1);
+         (size_t)p->M * V * 2;
   b += (size_t)(p->alloc_tiles + 1) * p->Mr * sizeof(int) * (p->sym ? 2 : 1) *
        (p->overlap ? 2 : 1);
   b += 16 + 2 * (size_t)std::max(p->N, p->n_z) * sizeof(double);   // status, io
