@@ -1259,9 +1259,9 @@ __device__ __forceinline__ void resum_body(const ResumArgs<double>& p, int blk, 
 // 16384-point duct (977 modes x 16640 points) 34 us per sum against 41,
 // 131072-point duct (1395 modes, R = 64) 214 against 372.  7 CTAs per SM (72
 // registers: keeps the one-mode-ahead window), 5 for runs of 16 points (213 us;
-// 230 at 72 registers).  FP64, bound by its pipe: 1.05 ms on the 16384-point duct
-with 29 mode groups (1.78 with sincospi, library divisions and a complex
-coefficient per term; 24 FP64 operations per term instead of ~46).
+// 230 at 72 registers).  FP64, bound by its pipe: 1.05 ms on the 16384-point
+// duct with 29 mode groups (1.78 with sincospi, library divisions and a complex
+// coefficient per term; 24 FP64 operations per term instead of ~46).
 template <typename T, int PW>
 __global__ void __launch_bounds__(RESUM_WARPS * 32, sizeof(T) == 4 ? (PW < 16 ? 7 : 5) : 1)
     k_resum(const ResumArgs<T> p) {
