@@ -60,33 +60,26 @@ __device__ __forceinline__ void vb_sync(int sub) {
   }
 }
 
-// sin / cos of 2 pi t for |t| <= 1/2: the FP32 path uses the special-function
-// unit (absolute error ~2^-21 on [-pi, pi]); the FP64 path stays exact.
+// sin / cos of 2 pi t for |t| <= 1/2 on the special-function unit (absolute
+// error ~2^-21 on [-pi, pi]).
 __device__ __forceinline__ void sincos_turns(float t, float* s, float* c) {
   __sincosf(6.28318530717958647692f * t, s, c);
-}
-__device__ __forceinline__ void sincos_turns(double t, double* s, double* c) {
-  sincospi(2.0 * t, s, c);
 }
 
 // Exact integer/float steps of the resummation kept off the conversion units
 // in FP32: floor of |y| < 2^22 by a round-down add of 1.5 * 2^23, the float
 // of an integer k < 2^23 from its bits, and t - rint(t) for |t| < 2^22 by
-// adding and subtracting 1.5 * 2^23 (round to nearest even, as rint).  The
-// FP64 versions are the plain operations.
+// adding and subtracting 1.5 * 2^23 (round to nearest even, as rint).
 __device__ __forceinline__ int ifloor_small(float y) {
   return (int)(__float_as_uint(__fadd_rd(y, 12582912.f)) - 0x4B400000u);
 }
-__device__ __forceinline__ int ifloor_small(double y) { return (int)floor(y); }
-__device__ __forceinline__ float exact_u2f(unsigned k, float) {
+__device__ __forceinline__ float exact_u2f(unsigned k) {
   return __uint_as_float(0x4B000000u | k) - 8388608.f;
 }
-__device__ __forceinline__ double exact_u2f(unsigned k, double) { return (double)k; }
 __device__ __forceinline__ float minus_rint(float t) {
   const float r = (t + 12582912.f) - 12582912.f;
   return t - r;
 }
-__device__ __forceinline__ double minus_rint(double t) { return t - rint(t); }
 
 template <typename T>
 __device__ __forceinline__ void load6(const T* p, T& a0, T& a1, T& a2, T& a3, T& a4, T& a5);
@@ -992,7 +985,7 @@ __device__ __forceinline__ void resum_body(const ResumArgs<float>& p, int blk, i
       // stays within a few turns.
       const unsigned nn = (unsigned)(i - p.n_max);
       const unsigned nmc = (nn * (unsigned)(m0 + x0 + PW / 2)) & mask;
-      float bc = exact_u2f(nmc, 0.f) * invN;
+      float bc = exact_u2f(nmc) * invN;
       bc = bc >= 0.5f ? bc - 1.f : bc;
       const float nN = (float)(int)nn * invN;
       const f2 one = bc2(1.f);

@@ -29,11 +29,13 @@ namespace {
 constexpr int FC_MODES_THREADS = 256;
 constexpr int FC_MODES_PER_CTA = 64;   // 8 warps x 8 modes
 constexpr int FC_WARPS = 4;
-constexpr int FC_PF = 2;    // rounds of 32 rays prefetched one mode ahead
+constexpr int FC_PF = 1;    // rounds of 32 rays prefetched one mode ahead
 // Row of interval w: X_w, X_{w+1}, phase b0..b3, Re a r0..r3, Im a i0..i3.
-// 14 values accessed as 7 pairs: at a 56-byte (FP32) row stride the 16
-// lanes of a half-warp touch 32 distinct banks.
-constexpr int FC_CF = 14;
+// FP32: 20 floats (16 used) read as four 16-byte words; at an 80-byte stride
+// the 8 lanes of a load phase touch 32 distinct banks.  FP64: 14 values read as
+// 7 pairs.
+template <typename T>
+constexpr int FC_CF = sizeof(T) == 4 ? 20 : 14;
 
 // x mod Np for x < 2^32 with magic = floor(2^32 / Np): the quotient
 // estimate is floor(x / Np) or one less, so one correction finishes it.
@@ -44,7 +46,7 @@ __device__ __forceinline__ unsigned mod_np(unsigned x, unsigned Np, unsigned mag
 
 template <typename T>
 __host__ __device__ inline int fc_warp_bytes(int wcap) {
-  return ((FC_CF + 4) * wcap * (int)sizeof(T) + 15) & ~15;
+  return ((FC_CF<T> + 4) * wcap * (int)sizeof(T) + 15) & ~15;
 }
 
 // CTA (patch blockIdx.x, mode block blockIdx.y): the continuation in FP64,
@@ -130,55 +132,152 @@ __global__ void __launch_bounds__(FC_MODES_THREADS) k_fc_modes(const FcModesArgs
 }
 
 template <typename T>
-__device__ __forceinline__ void store_row(T* r, T X1, T X2, T b0, T b1, T b2, T b3, T r0, T r1,
-                                          T r2, T r3, T i0, T i1, T i2, T i3) {
-  using V = typename C2<T>::type;
-  V* q = reinterpret_cast<V*>(r);
-  q[0] = V{X1, X2};
-  q[1] = V{b0, b1};
-  q[2] = V{b2, b3};
-  q[3] = V{r0, r1};
-  q[4] = V{r2, r3};
-  q[5] = V{i0, i1};
-  q[6] = V{i2, i3};
-}
+struct FcRow;
 
-template <typename T>
-struct Row {
-  T X1, X2, b0, b1, b2, b3, r0, r1, r2, r3, i0, i1, i2, i3;
+template <>
+struct FcRow<float> {
+  f2 c3, c2, c1, c0;   // (Re, Im) of the amplitude's cubic
+  float X1, X2, b0, b1, b2, b3;
+  __device__ __forceinline__ void load(const float* p) {
+    const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(p);
+    const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(p + 4);
+    const float4 x = *reinterpret_cast<const float4*>(p + 8);
+    const float4 y = *reinterpret_cast<const float4*>(p + 12);
+    c3.v = u.x; c2.v = u.y; c1.v = v.x; c0.v = v.y;
+    X1 = x.x; X2 = x.y; b0 = x.z; b1 = x.w;
+    b2 = y.x; b3 = y.y;
+  }
 };
 
-template <typename T>
-__device__ __forceinline__ Row<T> load_row(const T* r) {
-  using V = typename C2<T>::type;
-  const V* q = reinterpret_cast<const V*>(r);
-  const V a = q[0], b = q[1], c = q[2], d = q[3], e = q[4], f = q[5], g = q[6];
-  return Row<T>{a.x, a.y, b.x, b.y, c.x, c.y, d.x, d.y, e.x, e.y, f.x, f.y, g.x, g.y};
+template <>
+struct FcRow<double> {
+  double X1, X2, b0, b1, b2, b3, r0, r1, r2, r3, i0, i1, i2, i3;
+  __device__ __forceinline__ void load(const double* p) {
+    const double2* q = reinterpret_cast<const double2*>(p);
+    const double2 a = q[0], b = q[1], c = q[2], d = q[3], e = q[4], f = q[5], g = q[6];
+    X1 = a.x; X2 = a.y; b0 = b.x; b1 = b.y; b2 = c.x; b3 = c.y; r0 = d.x; r1 = d.y;
+    r2 = e.x; r3 = e.y; i0 = f.x; i1 = f.y; i2 = g.x; i3 = g.y;
+  }
+};
+
+// Rows of the intervals 1 .. W - 3 of a window (staged landings X, phases and
+// complex amplitudes), a lane per interval; the last one's end is stored as
+// infinity, so that no lane steps past it.  Returns whether every interval the
+// lane built is at least a grid step long.
+__device__ __forceinline__ bool build_rows(float* s_cf, const float* s_X, const float* s_ph,
+                                           const float2* s_a, int W, int lane) {
+  bool wide = true;
+  for (int w = 1 + lane; w <= W - 3; w += 32) {
+    const float X0 = s_X[w - 1], X1 = s_X[w], X2 = s_X[w + 1], X3 = s_X[w + 2];
+    const float h21 = X2 - X1, h10 = X1 - X0;
+    wide = wide && h21 >= 1.f;
+    const float r21 = rcp_approx(h21), r10 = rcp_approx(h10), r32 = rcp_approx(X3 - X2);
+    const float r20 = rcp_approx(X2 - X0), r31 = rcp_approx(X3 - X1), r30 = rcp_approx(X3 - X0);
+    float b0, b1, b2, b3;
+    cubic_through(s_ph[w - 1], s_ph[w], s_ph[w + 1], s_ph[w + 2], r21, r10, r32, r20, r31, r30,
+                  h21, h10, b0, b1, b2, b3);
+    const auto val = [&](int k) {
+      f2 v;
+      v.v = *reinterpret_cast<const unsigned long long*>(s_a + w + k);
+      return v;
+    };
+    // the same Newton form for (Re, Im) together
+    const f2 f0 = val(-1), f1 = val(0), fa = val(1), f3 = val(2);
+    const f2 d12 = mul2(sub2(fa, f1), bc2(r21)), d01 = mul2(sub2(f1, f0), bc2(r10));
+    const f2 d23 = mul2(sub2(f3, fa), bc2(r32));
+    const f2 d012 = mul2(sub2(d12, d01), bc2(r20)), d123 = mul2(sub2(d23, d12), bc2(r31));
+    const f2 c3 = mul2(sub2(d123, d012), bc2(r30));
+    const f2 c1 = fma2(bc2(-h21), fma2(c3, bc2(h10), d012), d12);
+    const f2 c2 = fma2(c3, bc2(h10 - h21), d012);
+    float* row = s_cf + FC_CF<float> * w;
+    *reinterpret_cast<ulonglong2*>(row) = make_ulonglong2(c3.v, c2.v);
+    *reinterpret_cast<ulonglong2*>(row + 4) = make_ulonglong2(c1.v, f1.v);
+    *reinterpret_cast<float4*>(row + 8) =
+        make_float4(X1, w == W - 3 ? __int_as_float(0x7f800000) : X2,
+                    minus_rint(b0), b1);           // whole turns do not matter
+    *reinterpret_cast<float2*>(row + 12) = make_float2(b2, b3);
+  }
+  return wide;
+}
+__device__ __forceinline__ bool build_rows(double* s_cf, const double* s_X, const double* s_ph,
+                                           const double2* s_a, int W, int lane) {
+  bool wide = true;
+  for (int w = 1 + lane; w <= W - 3; w += 32) {
+    const double X0 = s_X[w - 1], X1 = s_X[w], X2 = s_X[w + 1], X3 = s_X[w + 2];
+    const double h21 = X2 - X1, h10 = X1 - X0;
+    wide = wide && h21 >= 1.0;
+    const double r21 = rcp64(h21), r10 = rcp64(h10), r32 = rcp64(X3 - X2);
+    const double r20 = rcp64(X2 - X0), r31 = rcp64(X3 - X1), r30 = rcp64(X3 - X0);
+    const double2 f0 = s_a[w - 1], f1 = s_a[w], f2 = s_a[w + 1], f3 = s_a[w + 2];
+    double b0, b1, b2, b3, c0, c1, c2, c3, d0, d1, d2, d3;
+    cubic_through(s_ph[w - 1], s_ph[w], s_ph[w + 1], s_ph[w + 2], r21, r10, r32, r20, r31, r30,
+                  h21, h10, b0, b1, b2, b3);
+    cubic_through(f0.x, f1.x, f2.x, f3.x, r21, r10, r32, r20, r31, r30, h21, h10, c0, c1, c2, c3);
+    cubic_through(f0.y, f1.y, f2.y, f3.y, r21, r10, r32, r20, r31, r30, h21, h10, d0, d1, d2, d3);
+    double2* row = reinterpret_cast<double2*>(s_cf + FC_CF<double> * w);
+    row[0] = make_double2(X1, w == W - 3 ? __longlong_as_double(0x7ff0000000000000ll) : X2);
+    row[1] = make_double2(b0, b1);
+    row[2] = make_double2(b2, b3);
+    row[3] = make_double2(c0, c1);
+    row[4] = make_double2(c2, c3);
+    row[5] = make_double2(d0, d1);
+    row[6] = make_double2(d2, d3);
+  }
+  return wide;
+}
+
+// The term of one point: tau from the row's X_w, t the phase in turns without
+// the row's part.
+__device__ __forceinline__ void add_term(const FcRow<float>& r, const double2*, float xv, float t,
+                                         float& sr, float& si) {
+  const float tau = xv - r.X1;
+  const f2 tau2 = bc2(tau);
+  float ar, ai, sn, cs;
+  sp2(fma2(fma2(fma2(r.c3, tau2, r.c2), tau2, r.c1), tau2, r.c0), ar, ai);
+  sincos_turns(t + (((r.b3 * tau + r.b2) * tau + r.b1) * tau + r.b0), &sn, &cs);
+  sr = fmaf(ar, cs, fmaf(-ai, sn, sr));
+  si = fmaf(ar, sn, fmaf(ai, cs, si));
+}
+__device__ __forceinline__ void add_term(const FcRow<double>& r, const double2* trig, double xv,
+                                         double t, double& sr, double& si) {
+  const double tau = xv - r.X1;
+  const double ar = ((r.r3 * tau + r.r2) * tau + r.r1) * tau + r.r0;
+  const double ai = ((r.i3 * tau + r.i2) * tau + r.i1) * tau + r.i0;
+  double sn, cs;
+  sincos_table(trig, t + (((r.b3 * tau + r.b2) * tau + r.b1) * tau + r.b0), &sn, &cs);
+  sr = fma(ar, cs, fma(-ai, sn, sr));
+  si = fma(ar, sn, fma(ai, cs, si));
 }
 
 // One CTA: tile blk % n_tiles (TM = 32 PW points), mode group blk / n_tiles;
-// its warps take the group's modes round-robin and the CTA adds the warps'
-// sums in a fixed order.
-// FP32: at most 80 registers per thread (measured faster than the
-// unbounded 93: 0.31 against 0.47 ms per sum on a 131072-point open lens)
+// its warps take the group's modes round-robin (the structure of the periodic
+// sum: brackets of 32 modes looked up at once, the next mode's first rays loaded
+// one mode ahead) and the CTA adds the warps' sums in a fixed order.
+// Bound by instruction issue and by the warps its shared memory leaves (96 bytes
+// per ray of a window): 131072-point lens, 545 modes, R = 8, 221 us per sum with
+// 128-point tiles (256-point ones 306; 261 before, with per-mode bracket
+// lookups, scalar amplitude cubics and library divisions).  FP64 8192-point lens
+// 410 us (723).  FP32 7 CTAs per SM (72 registers); 6: 223 us, 8: 289.
 template <typename T, int PW>
-__global__ void __launch_bounds__(FC_WARPS * 32, sizeof(T) == 4 ? 6 : 1)
+__global__ void __launch_bounds__(FC_WARPS * 32, sizeof(T) == 4 ? 7 : 1)
     k_fc_resum(const FcResumArgs<T> p) {
   using V = typename C2<T>::type;
+  constexpr unsigned ALL = 0xffffffffu;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int tile = blockIdx.x % p.n_tiles, group = blockIdx.x / p.n_tiles;
   const int wcap = p.wcap, TM = p.TM, m0 = tile * TM;
   T* s_cf = reinterpret_cast<T*>(smem_raw + (long long)warp * fc_warp_bytes<T>(wcap));
-  T* s_X = s_cf + FC_CF * wcap;
+  V* s_a = reinterpret_cast<V*>(s_cf + FC_CF<T> * wcap);
+  T* s_X = reinterpret_cast<T*>(s_a + wcap);
   T* s_ph = s_X + wcap;
-  T* s_ar = s_ph + wcap;
-  T* s_ai = s_ar + wcap;
   const int i0 = group * p.modes_per_group, i1 = min(p.M, i0 + p.modes_per_group);
   const unsigned Np = (unsigned)p.Np;
   const T invNp = T(1) / T(p.Np);
   const long long nrays = (long long)p.NRT * p.M;
   const long long njlo = (long long)(p.n_tiles + 1) * p.M;
+  const int x0 = lane * PW;
+  const T xv0 = T(x0);
   unsigned st = 0;
   T accr[PW], acci[PW];
 #pragma unroll
@@ -186,14 +285,16 @@ __global__ void __launch_bounds__(FC_WARPS * 32, sizeof(T) == 4 ? 6 : 1)
 
   // ray j of mode i: landing offset, phase and the complex amplitude
   // a_j (S^{p0}(z_j) cf[p0][i] + S^{p0+1}(z_j) cf[p0+1][i])
-  auto fetch = [&](int i, int j, T& d, T& ph, T& ar, T& ai) {
+  struct RayVal { T d, ph; V a; };
+  auto fetch = [&](int i, int j) {
     // NRT M < 2^32 (at most 2^20 + 2 G rays of 2047 modes)
     const unsigned o = (unsigned)bchk((long long)((unsigned)j * (unsigned)p.M + (unsigned)i),
                                       nrays, st);
-    d = ld<LD_NC>(p.d + o);
-    ph = ld<LD_NC>(p.ph + o);
+    RayVal v;
+    v.d = ld<LD_NC>(p.d + o);
+    v.ph = ld<LD_NC>(p.ph + o);
     const T a = ld<LD_NC>(p.a + o);
-    const int p0 = p.win_p[j];
+    const int p0 = __ldg(p.win_p + j);
     const V sw = p.win_s[j];
     const V c0 = p.cf[bchk((long long)p0 * p.M + i, (long long)p.P * p.M, st)];
     T cr = sw.x * c0.x, ci = sw.x * c0.y;
@@ -202,152 +303,108 @@ __global__ void __launch_bounds__(FC_WARPS * 32, sizeof(T) == 4 ? 6 : 1)
       cr += sw.y * c1.x;
       ci += sw.y * c1.y;
     }
-    ar = a * cr;
-    ai = a * ci;
+    v.a.x = a * cr;
+    v.a.y = a * ci;
+    return v;
   };
-  auto head = [&](int i, int& jl, int& jh) {
-    jl = -1;
-    jh = -1;
-    if (i >= i1) return;
-    jl = p.jlo[bchk((long long)tile * p.M + i, njlo, st)];
-    jh = p.jlo[bchk((long long)(tile + 1) * p.M + i, njlo, st)];
-  };
-  // a table left inconsistent by a failed screen (flagged by the bracket
-  // kernel) must not send the reads out of [0, NRT); a window beyond the
-  // tile's capacity means rays compressed beyond it (flagged here)
-  auto head_ok = [&](int i, int jl, int jh) {
-    if (i >= i1 || jl < 1 || jh < jl || jh > p.NRT - 3) return false;
-    if (jh - jl + 4 > wcap) {
-      st |= ST_CAUSTIC;
-      return false;
-    }
-    return true;
-  };
-  // the next mode's first FC_PF rounds of 32 rays are loaded into registers
-  // while the current mode is summed
-  T pd[FC_PF], pph[FC_PF], par[FC_PF], pai[FC_PF];
-  auto prefetch = [&](int i, int jl, int jh) {
-    const int W = jh - jl + 4;
+  RayVal pre[FC_PF];   // the next mode's first FC_PF rounds of 32 rays
+  auto prefetch = [&](int i, int jb, int W) {
 #pragma unroll
-    for (int r = 0; r < FC_PF; ++r) {
-      const int w = lane + 32 * r;
-      if (w < W) fetch(i, jl - 1 + w, pd[r], pph[r], par[r], pai[r]);
-    }
+    for (int r = 0; r < FC_PF; ++r)
+      if (lane + 32 * r < W) pre[r] = fetch(i, jb + lane + 32 * r);
   };
 
-  int i = i0 + warp;
-  int jl_c, jh_c, jl_n, jh_n;
-  head(i, jl_c, jh_c);
-  head(i + FC_WARPS, jl_n, jh_n);
-  bool ok_c = head_ok(i, jl_c, jh_c);
-  if (ok_c) prefetch(i, jl_c, jh_c);
-  for (; i < i1; i += FC_WARPS) {
-    const bool ok = ok_c;
-    const int jl = jl_c, jh = jh_c;
-    const int W = jh - jl + 4;
-    const int jb = jl - 1;
-    __syncwarp();
-    if (ok) {
-#pragma unroll
-      for (int r = 0; r < FC_PF; ++r) {
-        const int w = lane + 32 * r;
-        if (w < W) {
-          s_X[w] = T((jb + w - p.G) * p.R - m0) + pd[r];
-          s_ph[w] = pph[r];
-          s_ar[w] = par[r];
-          s_ai[w] = pai[r];
+  for (int ib = i0 + warp; ib < i1; ib += 32 * FC_WARPS) {
+    // lane k: window of mode ib + FC_WARPS k (first ray jb, W rays; 0: skip)
+    int h_jb = 0, h_W = 0;
+    {
+      const int i = ib + FC_WARPS * lane;
+      if (i < i1) {
+        const int jl = p.jlo[bchk((long long)tile * p.M + i, njlo, st)];
+        const int jh = p.jlo[bchk((long long)(tile + 1) * p.M + i, njlo, st)];
+        // a table left inconsistent by a failed screen (flagged by the bracket
+        // kernel) must not send the reads out of [0, NRT); a window beyond the
+        // tile's capacity means rays compressed beyond it (flagged here)
+        if (jl >= 1 && jh >= jl && jh <= p.NRT - 3) {
+          h_W = jh - jl + 4;
+          if (h_W > wcap) { st |= ST_CAUSTIC; h_W = 0; }
         }
-      }
-      for (int w = lane + 32 * FC_PF; w < W; w += 32) {
-        T d, ph, ar, ai;
-        fetch(i, jb + w, d, ph, ar, ai);
-        s_X[w] = T((jb + w - p.G) * p.R - m0) + d;
-        s_ph[w] = ph;
-        s_ar[w] = ar;
-        s_ai[w] = ai;
+        h_jb = jl - 1;
       }
     }
-    jl_c = jl_n;
-    jh_c = jh_n;
-    ok_c = head_ok(i + FC_WARPS, jl_c, jh_c);
-    if (ok_c) prefetch(i + FC_WARPS, jl_c, jh_c);
-    head(i + 2 * FC_WARPS, jl_n, jh_n);
-    if (!ok) continue;
-    __syncwarp();
-    for (int w = 1 + lane; w <= W - 3; w += 32) {
-      const T X0 = s_X[w - 1], X1 = s_X[w], X2 = s_X[w + 1], X3 = s_X[w + 2];
-      const T h21 = X2 - X1, h10 = X1 - X0;
-      const T r21 = T(1) / h21, r10 = T(1) / h10, r32 = T(1) / (X3 - X2);
-      const T r20 = T(1) / (X2 - X0), r31 = T(1) / (X3 - X1), r30 = T(1) / (X3 - X0);
-      T b0, b1, b2, b3, c0, c1, c2, c3, d0, d1, d2, d3;
-      cubic_through(s_ph[w - 1], s_ph[w], s_ph[w + 1], s_ph[w + 2], r21, r10, r32, r20, r31, r30,
-                    h21, h10, b0, b1, b2, b3);
-      cubic_through(s_ar[w - 1], s_ar[w], s_ar[w + 1], s_ar[w + 2], r21, r10, r32, r20, r31, r30,
-                    h21, h10, c0, c1, c2, c3);
-      cubic_through(s_ai[w - 1], s_ai[w], s_ai[w + 1], s_ai[w + 2], r21, r10, r32, r20, r31, r30,
-                    h21, h10, d0, d1, d2, d3);
-      if constexpr (sizeof(T) == 4) b0 = minus_rint(b0);   // whole turns do not matter
-      store_row(s_cf + FC_CF * w, X1, X2, b0, b1, b2, b3, c0, c1, c2, c3, d0, d1, d2, d3);
-    }
-    __syncwarp();
-    // lane l sums the PW consecutive points l PW .. l PW + PW - 1 of the tile
-    const T xf = s_X[1];
-    const T inv_sp = T(W - 3) / (s_X[W - 2] - xf);
-    const int x0 = lane * PW;
-    const T xv0 = T(x0);
-    int w = 1 + ifloor_small(xv0 * inv_sp - xf * inv_sp);
-    w = min(max(w, 1), W - 3);
-    while (w > 1 && s_X[w] > xv0) --w;
-    while (w < W - 3 && s_X[w + 1] <= xv0) ++w;
-    Row<T> r = load_row<T>(s_cf + FC_CF * w);
-    const int n = i - p.n_max;   // |n| < Np / 2
-    const unsigned nn = (unsigned)(n < 0 ? n + p.Np : n);
-    if constexpr (sizeof(T) == 4) {
+    const int K = min(32, (i1 - ib + FC_WARPS - 1) / FC_WARPS);
+    int jb = __shfl_sync(ALL, h_jb, 0), W = __shfl_sync(ALL, h_W, 0);
+    prefetch(ib, jb, W);
+    for (int k = 0; k < K; ++k) {
+      const int i = ib + FC_WARPS * k;
+      const int Wc = W, jc = jb, base = (jc - p.G) * p.R - m0;
+      const auto put = [&](int w, const RayVal& v) {
+        s_X[w] = T(base + w * p.R) + v.d;
+        s_ph[w] = v.ph;
+        s_a[w] = v.a;
+      };
+      __syncwarp();
+#pragma unroll
+      for (int r = 0; r < FC_PF; ++r)
+        if (lane + 32 * r < Wc) put(lane + 32 * r, pre[r]);
+      for (int w = lane + 32 * FC_PF; w < Wc; w += 32) put(w, fetch(i, jc + w));
+      if (k + 1 < K) {
+        jb = __shfl_sync(ALL, h_jb, k + 1);
+        W = __shfl_sync(ALL, h_W, k + 1);
+        prefetch(i + FC_WARPS, jb, W);
+      }
+      if (Wc == 0) continue;
+      __syncwarp();
+      bool wide = build_rows(s_cf, s_X, s_ph, s_a, Wc, lane);
+      wide = __all_sync(ALL, wide);
+      __syncwarp();
+      // lane l sums the PW consecutive points l PW .. l PW + PW - 1 of the tile
+      int w;
+      {
+        const float xf = (float)s_X[1];
+        const float inv_sp = (float)(Wc - 3) * rcp_approx((float)s_X[Wc - 2] - xf);
+        w = 1 + ifloor_small(((float)x0 - xf) * inv_sp);
+        w = min(max(w, 1), Wc - 3);
+        while (w > 1 && s_X[w] > xv0) --w;
+        while (w < Wc - 3 && s_X[w + 1] <= xv0) ++w;
+      }
+      const T* row = s_cf + FC_CF<T> * w;
+      FcRow<T> r;
+      r.load(row);
       // the exact integer phase n m / Np mod 1 of the run's middle point,
       // moved into [-1/2, 1/2), and n / Np (|n / Np| < 1/2) per point from it:
       // the argument of the sine stays within about two turns
-      const unsigned nmc = mod_np(nn * (unsigned)(m0 + x0 + PW / 2), Np, p.np_magic);
-      T bc = T(nmc) * invNp;
+      const int n = i - p.n_max;   // |n| < Np / 2
+      const unsigned nn = (unsigned)(n < 0 ? n + p.Np : n);
+      // nn (m0 + x0 + PW / 2) < 2^11 2^20: no overflow
+      T bc = T(mod_np(nn * (unsigned)(m0 + x0 + PW / 2), Np, p.np_magic)) * invNp;
       bc = bc >= T(0.5) ? bc - T(1) : bc;
       const T nNp = T(n) * invNp;
+      T xv = xv0;   // exact
+      if (wide) {   // at most one interval ends between two points
 #pragma unroll
-      for (int q = 0; q < PW; ++q) {
-        const T xv = xv0 + T(q);
-        while (w < W - 3 && r.X2 <= xv) {
-          ++w;
-          r = load_row<T>(s_cf + FC_CF * w);
+        for (int q = 0; q < PW; ++q) {
+          if (q > 0) {
+            xv += T(1);
+            if (r.X2 <= xv) {
+              row += FC_CF<T>;
+              r.load(row);
+            }
+          }
+          add_term(r, p.trig, xv, fma(T(q - PW / 2), nNp, bc), accr[q], acci[q]);
         }
-        const T tau = xv - r.X1;
-        const T phv = ((r.b3 * tau + r.b2) * tau + r.b1) * tau + r.b0;
-        const T ar = ((r.r3 * tau + r.r2) * tau + r.r1) * tau + r.r0;
-        const T ai = ((r.i3 * tau + r.i2) * tau + r.i1) * tau + r.i0;
-        const T t = fmaf(T(q - PW / 2), nNp, bc) + phv;
-        T sn, cs;
-        sincos_turns(t, &sn, &cs);
-        accr[q] += ar * cs - ai * sn;
-        acci[q] += ar * sn + ai * cs;
-      }
-    } else {
-      // nn (m0 + x0) < 2^11 2^20: no overflow
-      unsigned nm = mod_np(nn * (unsigned)(m0 + x0), Np, p.np_magic);
+      } else {
 #pragma unroll
-      for (int q = 0; q < PW; ++q) {
-        const T xv = xv0 + T(q);
-        while (w < W - 3 && r.X2 <= xv) {
-          ++w;
-          r = load_row<T>(s_cf + FC_CF * w);
+        for (int q = 0; q < PW; ++q) {
+          if (q > 0) {
+            xv += T(1);
+            while (r.X2 <= xv) {
+              row += FC_CF<T>;
+              r.load(row);
+            }
+          }
+          add_term(r, p.trig, xv, fma(T(q - PW / 2), nNp, bc), accr[q], acci[q]);
         }
-        const T tau = xv - r.X1;
-        const T phv = ((r.b3 * tau + r.b2) * tau + r.b1) * tau + r.b0;
-        const T ar = ((r.r3 * tau + r.r2) * tau + r.r1) * tau + r.r0;
-        const T ai = ((r.i3 * tau + r.i2) * tau + r.i1) * tau + r.i0;
-        const T t = minus_rint(T(nm) * invNp + phv);
-        T sn, cs;
-        sincos_turns(t, &sn, &cs);
-        accr[q] += ar * cs - ai * sn;
-        acci[q] += ar * sn + ai * cs;
-        nm += nn;
-        if (nm >= Np) nm -= Np;
       }
     }
   }

@@ -167,6 +167,7 @@ struct FcResumArgs {
   const typename C2<T>::type* cf;    // [P][M]
   const int* win_p;                  // [NRT] first patch with a non-zero weight at ray j
   const typename C2<T>::type* win_s; // [NRT] (S^{p0}, S^{p0+1}) at ray j
+  const double2* trig;               // [TRIG_N] FP64: exp(2 pi i k / TRIG_N)
   int M, NRT, G, R, N, TM, n_tiles, n_groups, modes_per_group, n_max, wcap, Np, P;
   unsigned np_magic;                 // floor(2^32 / Np)
   typename C2<T>::type* part;        // [n_groups][N]

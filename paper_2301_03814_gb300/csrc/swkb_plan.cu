@@ -834,6 +834,7 @@ FcResumArgs<T> fc_resum_args(const swkb_plan* p, const T* d, const T* ph, const 
   r.cf = (const V*)(cf ? cf : p->fc_cf);
   r.win_p = p->fc_win_p;
   r.win_s = (const V*)p->fc_win_s;
+  r.trig = (const double2*)p->trig;
   r.M = p->M; r.NRT = p->NRT; r.G = p->G; r.R = p->R; r.N = p->N; r.TM = p->TM;
   r.n_tiles = p->n_tiles; r.n_groups = p->n_groups; r.modes_per_group = p->modes_per_group;
   r.n_max = p->n_max; r.wcap = p->wcap; r.Np = p->fc_Np; r.P = p->fc_P;
@@ -1479,28 +1480,27 @@ Tiling default_tiling(const swkb_plan* p) {
   // builds one) then number 16 to 20, and a run meets one interval's end at
   // most once.  FP32, R = 64 (131072 points, 1395 modes): 214 us per sum with
   // runs of 16 points, 280 with 8; R = 16 (16384 points): 35 with 16, 34 with 8.
-  const bool f32 = p->precision != SWKB_FP64 && !p->fc;
-  t.PW = f32 && p->R >= 32 ? 16 : (p->R >= 8 ? 8 : (p->R >= 2 ? 4 : 2));
+  // Patch-wise windows (96 bytes of shared memory a ray) halve them: R = 8
+  // (131072 points, 545 modes) 231 us with runs of 4, 336 with 8; R = 2 (8192
+  // points) 68 with 2, 92 with 4.
+  if (p->fc) t.PW = p->R >= 8 ? 4 : 2;
+  else if (p->precision != SWKB_FP64 && p->R >= 32) t.PW = 16;
+  else t.PW = p->R >= 8 ? 8 : (p->R >= 2 ? 4 : 2);
   while (32 * t.PW > (p->sym ? p->N / 2 : p->N) || (p->fc && p->N % (32 * t.PW))) t.PW /= 2;
-  // patch-wise plans are not autotuned: many short mode groups keep the
-  // last wave of their sum short (measured on the open lens, N_z = 131072:
-  // 0.31 ms per sum with 2 groups, 0.26 with 8)
-  if (p->fc) {
-    t.ctas_per_sm = 24;
-  } else {
-    // Mode groups: up to 20 CTAs per SM, so that the last wave is short, while
-    // a group keeps 32 modes (a warp looks its modes up 32 at a time, and the
-    // DFT adds up one partial per group); at least 4 CTAs per SM where the
-    // modes allow it, at 4 per group.  Sum plus DFT per screen, by groups:
-    // 16384 points, 977 modes 50.9 us (15), 48.5 (29), 50.1 (43); 131072 points,
-    // 1395 modes 276 (4), 252 (13); 4096 points, 401 modes 25.0 (19), 22.5 (37),
-    // 24.8 (51); 512 points, 65 modes 18.1 (17), 22.0 (65).
-    const int tiles = p->sym ? p->N / (64 * t.PW) + 1 : p->N / (32 * t.PW);
-    const auto groups_at = [&](int c) { return (p->sms * c + tiles - 1) / tiles; };
-    const int g = std::min(std::max(std::min(groups_at(20), p->M / 32), groups_at(4)),
-                           std::max(1, p->M / 4));
-    t.ctas_per_sm = std::max(1, (int)((long long)g * tiles / p->sms));
-  }
+  // Mode groups: up to 20 CTAs per SM (patch-wise, where a group sums longer,
+  // 40), so that the last wave is short, while a group keeps 32 modes
+  // (patch-wise 16; a warp looks its modes up 32 at a time, and the next screen
+  // adds up one partial per group); at least 4 CTAs per SM where the modes allow it, at 4 per group.  Sum
+  // plus DFT per screen, by groups: 16384 points, 977 modes 50.9 us (15), 48.5
+  // (29), 50.1 (43); 131072 points, 1395 modes 276 (4), 252 (13); 4096 points,
+  // 401 modes 25.0 (19), 22.5 (37), 24.8 (51); 512 points, 65 modes 18.1 (17),
+  // 22.0 (65).  Patch-wise sums: 131072 points, 545 modes 261 us (2), 234 (4), 231
+  // (6); 8192 points 24.6 (10), 22.5 (29), 24.5 (54).
+  const int tiles = p->sym ? p->N / (64 * t.PW) + 1 : p->N / (32 * t.PW);
+  const auto groups_at = [&](int c) { return (p->sms * c + tiles - 1) / tiles; };
+  const int most = p->fc ? std::min(groups_at(40), p->M / 16) : std::min(groups_at(20), p->M / 32);
+  const int g = std::min(std::max(most, groups_at(4)), std::max(1, p->M / 4));
+  t.ctas_per_sm = std::max(1, (int)((long long)g * tiles / p->sms));
   // N1 ~ sqrt(M): pass 1 costs N N1, pass 2 M N2
   t.N1 = 1;
   while (t.N1 * t.N1 * 2 < p->M && t.N1 < p->N / 32 && t.N1 < 64) t.N1 *= 2;

@@ -23,6 +23,10 @@ def _lens(R):
     return w.config_gaussian_medium(a=0.02, b=0.01, ray_stride=R, n_screens=2)
 
 
+def _open(R):
+    return w.config_open_lens(n_z=8192, fc_patch=910, fc_overlap=248, n_screens=2, ray_stride=R)
+
+
 @pytest.mark.parametrize("problem,tiling", [
     (lambda: _lens(1), None),                                        # intervals below one step
     (lambda: _lens(1), (64, 1, 4)),
@@ -33,6 +37,11 @@ def _lens(R):
     (lambda: w.config_gaussian_lens_40km().with_(n_screens=2), (64, 1, 8)),    # 134 modes per group
     (lambda: w.config_gaussian_lens_40km().with_(n_screens=2), (256, 1024, 8)),  # one mode per group
     (lambda: w.config_surface_duct_small(n_screens=2).with_(theta_max=math.radians(0.02)), None),
+    # patch-wise: 36 rays per window, several hundred modes per group, R = 1
+    (lambda: _open(8), (256, 1, 32)),
+    (lambda: _open(8), (64, 1024, 32)),
+    (lambda: _open(2), (128, 1, 32)),
+    (lambda: _open(1), None),
 ])
 def test_mixed_sum_matches_fp64(problem, tiling):
     pb = problem()
