@@ -4,9 +4,8 @@
 // periodic ones: a ray depends only on its mode angle and launch point, so
 // one family per mode serves every patch.
 //
-//   k_fc_modes  one CTA per patch: the patch's samples, its FC-Gram
-//               continuation to N_p = n_pat + C points, and the kept modes of
-//               that sequence's DFT, w_n / N_p, rotated to the interval's
+//   k_fc_modes  per patch: the patch's samples, its FC-Gram continuation to
+//               N_p = n_pat + C points, and the kept modes of that sequence's DFT, w_n / N_p, rotated to the interval's
 //               origin (exp(-2 pi i n s_p / N_p)) and carried over the screen
 //               (exp(i k dx Pbar_n)): cf[p][n].  The continuation runs in
 //               FP64 in every plan (the operator's entries reach 3e3, so its
@@ -26,8 +25,11 @@ namespace swkb {
 
 namespace {
 
-constexpr int FC_MODES_THREADS = 256;
-constexpr int FC_MODES_PER_CTA = 64;   // 8 warps x 8 modes
+constexpr int FC_MODES_PARTS = 8;        // parts of the sequence in a DFT block
+constexpr int FC_MODES_BINS = 32;        // bins n >= 0 of one
+constexpr int FC_MODES_THREADS = FC_MODES_PARTS * FC_MODES_BINS;
+constexpr int FC_MODES_PATCHES = 4;      // patches sharing a block's twiddles
+constexpr int FC_CHUNK = 16;             // samples summed before they join the total
 constexpr int FC_WARPS = 4;
 constexpr int FC_PF = 1;    // rounds of 32 rays prefetched one mode ahead
 // Row of interval w: X_w, X_{w+1}, phase b0..b3, Re a r0..r3, Im a i0..i3.
@@ -49,25 +51,44 @@ __host__ __device__ inline int fc_warp_bytes(int wcap) {
   return ((FC_CF<T> + 4) * wcap * (int)sizeof(T) + 15) & ~15;
 }
 
-// CTA (patch blockIdx.x, mode block blockIdx.y): the continuation in FP64,
-// then the DFT of the FC_MODES_PER_CTA modes of the block in T (a mixed plan
-// sums in FP32: exact twiddle indices, FP32 twiddles and samples).
-template <typename T>
+// Twiddles of a DFT block, padded so that the samples behind them start on 16
+// bytes.
+__host__ __device__ inline int modes_pad(int Np) { return (Np + 1) & ~1; }
+
+// CTA (PP patches from blockIdx.x PP, mode block blockIdx.y): the continuation
+// in FP64, then the DFT in T (a mixed plan sums in FP32: exact twiddle indices,
+// FP32 twiddles and samples).  A thread forms the bins n and -n of its PP
+// patches over every eighth sample of the sequence (a warp each), from the sums of e cos and
+// e sin they share, in chunks of 16 samples; the parts are added pairwise at the end.
+// (Strided parts: neighbouring samples' terms are alike, so a part of consecutive
+// ones sums to larger values; FP32 fields were 2 to 4 % further from FP64 with.)
+//   What bounds it: per twiddle one gather from shared memory (several bank
+// conflicts: lanes are consecutive n, so its stride is the sample's index) and
+// its index, shared by PP patches and both bins.  188 patches of 945 points, 545
+// modes: 35 us, against 95 with a warp per mode and patch (a gather and a sample
+// per term); see launch_fc_modes for PP.
+template <typename T, int PP>
 __global__ void __launch_bounds__(FC_MODES_THREADS) k_fc_modes(const FcModesArgs<T> p) {
   using V = typename C2<T>::type;
+  constexpr int PARTS = FC_MODES_PARTS, BINS = FC_MODES_BINS;
+  static_assert(PARTS == 8, "the pairwise sum of the parts is written out");
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  V* e = reinterpret_cast<V*>(smem_raw);    // [N_p] the continued sequence
-  V* tw = e + p.Np;                         // [N_p] exp(-2 pi i k / N_p)
-  __shared__ double2 ends[2 * FC_D];        // the d samples at each end, FP64
-  const int pt = blockIdx.x;
-  const long long s0 = (long long)pt * p.stride;
-  for (int k = threadIdx.x; k < p.n_pat; k += blockDim.x) {
-    const V v = p.u[s0 + k];
-    e[k] = v;
-    if (k < FC_D) ends[FC_D + k] = make_double2((double)v.x, (double)v.y);
-    if (k >= p.n_pat - FC_D) ends[k - (p.n_pat - FC_D)] = make_double2((double)v.x, (double)v.y);
+  V* tw = reinterpret_cast<V*>(smem_raw);   // [N_p] exp(-2 pi i k / N_p)
+  V* e = tw + modes_pad(p.Np);              // [N_p][PP] the continued sequences
+  __shared__ double2 ends[PP][2 * FC_D];    // the d samples at each end, FP64
+  const int pt0 = blockIdx.x * PP;
+  const int np = min(PP, p.P - pt0);        // patches of this CTA
+  for (int x = threadIdx.x; x < p.n_pat * PP; x += FC_MODES_THREADS) {
+    const int k = x / PP, a = x % PP;
+    V v;
+    v.x = T(0); v.y = T(0);
+    if (a < np) v = p.u[(long long)(pt0 + a) * p.stride + k];
+    e[x] = v;
+    if (k < FC_D) ends[a][FC_D + k] = make_double2((double)v.x, (double)v.y);
+    if (k >= p.n_pat - FC_D)
+      ends[a][k - (p.n_pat - FC_D)] = make_double2((double)v.x, (double)v.y);
   }
-  for (int k = threadIdx.x; k < p.Np; k += blockDim.x) {
+  for (int k = threadIdx.x; k < p.Np; k += FC_MODES_THREADS) {
     const double2 w = p.tw[k];
     V v;
     v.x = (T)w.x;
@@ -75,59 +96,112 @@ __global__ void __launch_bounds__(FC_MODES_THREADS) k_fc_modes(const FcModesArgs
     tw[k] = v;
   }
   __syncthreads();
-  if (threadIdx.x < FC_C) {
+  for (int x = threadIdx.x; x < FC_C * PP; x += FC_MODES_THREADS) {
     // value t past the right end: the right end's d samples (ends[0 .. d-1])
     // through row t; the same value counted backwards from the left end is
     // C - t steps before sample 0: the left end read backwards (sample
     // d - 1 - i = ends[2 d - 1 - i]) through row C - 1 - t
-    const int t = threadIdx.x;
+    const int t = x / PP, a = x % PP;
     double ar = 0.0, ai = 0.0;
     for (int i = 0; i < FC_D; ++i) {
       const double cr = p.cont[t * FC_D + i];
       const double cl = p.cont[(FC_C - 1 - t) * FC_D + i];
-      const double2 fr = ends[i];
-      const double2 fl = ends[2 * FC_D - 1 - i];
+      const double2 fr = ends[a][i];
+      const double2 fl = ends[a][2 * FC_D - 1 - i];
       ar += cr * fr.x + cl * fl.x;
       ai += cr * fr.y + cl * fl.y;
     }
     V v;
     v.x = (T)ar;
     v.y = (T)ai;
-    e[p.n_pat + t] = v;
+    e[(p.n_pat + t) * PP + a] = v;
   }
   __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned Np = (unsigned)p.Np;
-  const int i_end = min(p.M, (int)(blockIdx.y + 1) * FC_MODES_PER_CTA);
-  for (int i = blockIdx.y * FC_MODES_PER_CTA + warp; i < i_end; i += FC_MODES_THREADS / 32) {
-    const int n = i - p.n_max;   // |n| < Np / 2
-    const unsigned nn = (unsigned)(n < 0 ? n + p.Np : n);
-    const unsigned step = mod_np(nn * 32u, Np, p.np_magic);
-    unsigned idx = mod_np(nn * (unsigned)lane, Np, p.np_magic);
-    T sr = T(0), si = T(0);
-    for (int k = lane; k < p.Np; k += 32) {
-      const V v = e[k], w = tw[idx];
-      sr += v.x * w.x - v.y * w.y;
-      si += v.x * w.y + v.y * w.x;
+  const int lt = threadIdx.x % BINS, part = threadIdx.x / BINS;
+  const int n = blockIdx.y * BINS + lt;      // bins n and -n, n <= n_max < Np / 2
+  const unsigned nn = (unsigned)min(n, p.n_max);
+  // sums of e cos and of e sin (the twiddle's parts) per patch
+  T cr[PP], ci[PP], sr[PP], si[PP];
+#pragma unroll
+  for (int a = 0; a < PP; ++a) cr[a] = ci[a] = sr[a] = si[a] = T(0);
+  int k = part;
+  const unsigned step = mod_np(nn * (unsigned)PARTS, Np, p.np_magic);
+  unsigned idx = mod_np(nn * (unsigned)part, Np, p.np_magic);
+  while (k < p.Np) {
+    const int stop = min(k + FC_CHUNK * PARTS, p.Np);
+    T dr[PP], di[PP], fr[PP], fi[PP];
+#pragma unroll
+    for (int a = 0; a < PP; ++a) dr[a] = di[a] = fr[a] = fi[a] = T(0);
+#pragma unroll 4
+    for (; k < stop; k += PARTS) {
+      const V w = tw[idx];
       idx += step;
-      if (idx >= Np) idx -= Np;
+      idx = min(idx, idx - Np);      // unsigned: the smaller is the one in [0, Np)
+      V ev[PP];
+      if constexpr (sizeof(T) == 4 && PP == 4) {
+        const float4 x = *reinterpret_cast<const float4*>(e + k * PP);
+        const float4 y = *reinterpret_cast<const float4*>(e + k * PP + 2);
+        ev[0] = V{x.x, x.y}; ev[1] = V{x.z, x.w}; ev[2] = V{y.x, y.y}; ev[3] = V{y.z, y.w};
+      } else {
+#pragma unroll
+        for (int a = 0; a < PP; ++a) ev[a] = e[k * PP + a];
+      }
+#pragma unroll
+      for (int a = 0; a < PP; ++a) {
+        const V v = ev[a];
+        dr[a] += v.x * w.x;
+        di[a] += v.y * w.x;
+        fr[a] += v.x * w.y;
+        fi[a] += v.y * w.y;
+      }
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      sr += __shfl_xor_sync(0xffffffffu, sr, o);
-      si += __shfl_xor_sync(0xffffffffu, si, o);
+    for (int a = 0; a < PP; ++a) { cr[a] += dr[a]; ci[a] += di[a]; sr[a] += fr[a]; si[a] += fi[a]; }
+  }
+  // the other parts' sums through shared memory (over the samples)
+  __syncthreads();
+  T* red = reinterpret_cast<T*>(e);   // [PARTS - 1][4 PP][BINS]
+  const T inv = (T)p.inv_Np;
+  if (part > 0) {
+    T* r = red + (part - 1) * 4 * PP * BINS + lt;
+#pragma unroll
+    for (int a = 0; a < PP; ++a) {
+      r[(4 * a + 0) * BINS] = cr[a];
+      r[(4 * a + 1) * BINS] = ci[a];
+      r[(4 * a + 2) * BINS] = sr[a];
+      r[(4 * a + 3) * BINS] = si[a];
     }
-    if (lane == 0) {
-      // (sr + i si) rot exp(i phi) / N_p in the plan's type; nn s0 < 2^11 2^20
-      const V rot = tw[mod_np(nn * (unsigned)s0, Np, p.np_magic)];
-      const V ep = p.ephi[i];
-      const T xr = sr * rot.x - si * rot.y, xi = sr * rot.y + si * rot.x;
-      const T inv = (T)p.inv_Np;
+  }
+  __syncthreads();
+  if (part != 0 || n > p.n_max) return;
+  const V ep = p.ephi[p.n_max + n], em = p.ephi[p.n_max - n];
+#pragma unroll
+  for (int a = 0; a < PP; ++a) {
+    if (a >= np) break;
+    const auto total = [&](T own, int v) {
+      T q[PARTS];
+      q[0] = own;
+#pragma unroll
+      for (int x = 1; x < PARTS; ++x) q[x] = red[((x - 1) * 4 * PP + 4 * a + v) * BINS + lt];
+      return ((q[0] + q[1]) + (q[2] + q[3])) + ((q[4] + q[5]) + (q[6] + q[7]));
+    };
+    const T ar = total(cr[a], 0), ai = total(ci[a], 1);
+    const T br = total(sr[a], 2), bi = total(si[a], 3);
+    // nn s0 < 2^11 2^20
+    const V rot = tw[mod_np(nn * (unsigned)((long long)(pt0 + a) * p.stride), Np, p.np_magic)];
+    // X_n = sum e w = (ar - bi) + i (ai + br), X_-n = sum e conj(w); each times
+    // the patch's rotation (conjugated for -n), exp(i phi) and 1 / N_p
+    const auto finish = [&](T xr, T xi, T ry, V ph) {
+      const T zr = xr * rot.x - xi * ry, zi = xr * ry + xi * rot.x;
       V c;
-      c.x = (xr * ep.x - xi * ep.y) * inv;
-      c.y = (xr * ep.y + xi * ep.x) * inv;
-      p.cf[(long long)pt * p.M + i] = c;
-    }
+      c.x = (zr * ph.x - zi * ph.y) * inv;
+      c.y = (zr * ph.y + zi * ph.x) * inv;
+      return c;
+    };
+    V* cf = p.cf + (long long)(pt0 + a) * p.M + p.n_max;
+    cf[n] = finish(ar - bi, ai + br, rot.y, ep);
+    if (n > 0) cf[-n] = finish(ar + bi, ai - br, -rot.y, em);
   }
 }
 
@@ -235,8 +309,8 @@ __device__ __forceinline__ void add_term(const FcRow<float>& r, const double2*, 
   float ar, ai, sn, cs;
   sp2(fma2(fma2(fma2(r.c3, tau2, r.c2), tau2, r.c1), tau2, r.c0), ar, ai);
   sincos_turns(t + (((r.b3 * tau + r.b2) * tau + r.b1) * tau + r.b0), &sn, &cs);
-  sr = fmaf(ar, cs, fmaf(-ai, sn, sr));
-  si = fmaf(ar, sn, fmaf(ai, cs, si));
+  sr += fmaf(ar, cs, -ai * sn);   // one rounding at the sum's size per term
+  si += fmaf(ar, sn, ai * cs);
 }
 __device__ __forceinline__ void add_term(const FcRow<double>& r, const double2* trig, double xv,
                                          double t, double& sr, double& si) {
@@ -245,8 +319,8 @@ __device__ __forceinline__ void add_term(const FcRow<double>& r, const double2* 
   const double ai = ((r.i3 * tau + r.i2) * tau + r.i1) * tau + r.i0;
   double sn, cs;
   sincos_table(trig, t + (((r.b3 * tau + r.b2) * tau + r.b1) * tau + r.b0), &sn, &cs);
-  sr = fma(ar, cs, fma(-ai, sn, sr));
-  si = fma(ar, sn, fma(ai, cs, si));
+  sr += fma(ar, cs, -ai * sn);
+  si += fma(ar, sn, ai * cs);
 }
 
 // One CTA: tile blk % n_tiles (TM = 32 PW points), mode group blk / n_tiles;
@@ -452,8 +526,17 @@ size_t fc_resum_smem_bytes(int wcap, int tile_points) {
 }
 
 template <typename T>
+size_t modes_smem(int Np, int patches) {
+  const size_t tw = (size_t)modes_pad(Np) * sizeof(typename C2<T>::type);
+  // the sums of the other parts overlie the samples
+  const size_t stage = (size_t)patches * Np * sizeof(typename C2<T>::type);
+  const size_t red = (size_t)(FC_MODES_PARTS - 1) * 4 * patches * FC_MODES_BINS * sizeof(T);
+  return tw + (stage > red ? stage : red);
+}
+
+template <typename T>
 size_t fc_modes_smem_bytes(int Np) {
-  return 2 * (size_t)Np * sizeof(typename C2<T>::type);
+  return modes_smem<T>(Np, FC_MODES_PATCHES);
 }
 
 template <typename T>
@@ -467,9 +550,11 @@ cudaError_t prepare_fc_kernels(int resum_smem, int modes_smem) {
   if (e == cudaSuccess)
     e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e != cudaSuccess) return e;
-  if (resum_smem > optin || modes_smem + (int)(2 * FC_D * sizeof(double2)) > optin)
+  if (resum_smem > optin ||
+      modes_smem + (int)(FC_MODES_PATCHES * 2 * FC_D * sizeof(double2)) > optin)
     return cudaErrorInvalidValue;
-  const void* fs[] = {(const void*)k_fc_modes<T>, (const void*)k_fc_resum<T, 2>,
+  const void* fs[] = {(const void*)k_fc_modes<T, 1>, (const void*)k_fc_modes<T, FC_MODES_PATCHES>,
+                      (const void*)k_fc_resum<T, 2>,
                       (const void*)k_fc_resum<T, 4>, (const void*)k_fc_resum<T, 8>};
   for (const void* f : fs) {
     // the dynamic limit plus the kernel's static shared memory must stay
@@ -507,10 +592,21 @@ cudaError_t launch_fc_cscale(const typename C2<T>::type* cf, const typename C2<T
   return cudaGetLastError();
 }
 
+// Four patches per CTA share each twiddle where that still gives 128 CTAs: 188
+// patches of 545 modes 35 us, against 49 with one patch per CTA; few patches
+// take a CTA each (12 patches of 539 modes 13.5 us; FP64 41 us, against 125 with a
+// warp per mode and patch).  Blocks of 128 bins and two parts: 32 and 22 us, and
+// longer beside the march (730 instead of 708 us per screen on the 131072-point
+// lens).
 template <typename T>
 cudaError_t launch_fc_modes(const FcModesArgs<T>& a, cudaStream_t s) {
-  const dim3 grid(a.P, (a.M + FC_MODES_PER_CTA - 1) / FC_MODES_PER_CTA);
-  k_fc_modes<T><<<grid, FC_MODES_THREADS, fc_modes_smem_bytes<T>(a.Np), s>>>(a);
+  const int bx = (a.P + FC_MODES_PATCHES - 1) / FC_MODES_PATCHES;
+  const int by = a.n_max / FC_MODES_BINS + 1;   // bins 0 .. n_max
+  if (bx * by >= 128)
+    k_fc_modes<T, FC_MODES_PATCHES><<<dim3(bx, by), FC_MODES_THREADS,
+                                      modes_smem<T>(a.Np, FC_MODES_PATCHES), s>>>(a);
+  else
+    k_fc_modes<T, 1><<<dim3(a.P, by), FC_MODES_THREADS, modes_smem<T>(a.Np, 1), s>>>(a);
   return cudaGetLastError();
 }
 
