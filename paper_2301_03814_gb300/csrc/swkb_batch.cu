@@ -64,7 +64,7 @@ constexpr int kSets = 3;          // ray-buffer sets per instance
 constexpr int kThreads = 256;
 // standalone blocks per work item (small blocks are grouped so that an item
 // is worth its claim)
-constexpr int VB_INIT = 8, VB_MARCH = 2, VB_FFT1 = 4, VB_FFT2 = 8, VB_BRACKET = 64,
+constexpr int VB_INIT = 8, VB_MARCH = 2, VB_FFT1 = 4, VB_FFT2 = 8, VB_BRACKET = 16,
               VB_REDUCE = 8, VB_OUTPUT = 8;
 // resummation blocks per item: one per 128-thread half of the CTA, or one in
 // the lower half when two blocks' shared memory does not fit (Ctl.resum_per_item)
@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 1)
         BracketArgs<T>& b = slot_bracket<T>(s_args);
         stage_args(&b, &I.bracket[set], tid);
         __syncthreads();
-        const int nb = I.bracket_bx * (b.NRT - 1);
+        const int nb = I.bracket_bx * bracket_rows(b.NRT);
         for (int v = item * VB_BRACKET; v < min(item * VB_BRACKET + VB_BRACKET, nb); ++v)
           bracket_body<T, LD_CG>(b, v % I.bracket_bx, v / I.bracket_bx, tid);
         break;
@@ -468,7 +468,7 @@ swkb_status build(swkb_batch* b, const swkb_request* reqs, const swkb_batch_opti
     it[PH_MARCH] = cdiv(pp.march_blocks, VB_MARCH);
     it[PH_FFT1] = cdiv(pp.fft1_blocks, VB_FFT1);
     it[PH_FFT2] = cdiv(pp.fft2_blocks, VB_FFT2);
-    it[PH_BRACKET] = cdiv((long long)pp.bracket_bx * (pp.NRT - 1), VB_BRACKET);
+    it[PH_BRACKET] = cdiv((long long)pp.bracket_bx * bracket_rows(pp.NRT), VB_BRACKET);
     it[PH_RESUM] = 0;   // set below, once the shared-memory budget is known
     it[PH_REDUCE] = cdiv(cdiv(pp.reduce_n, 256), VB_REDUCE);
     it[PH_OUTPUT] = cdiv(cdiv(pp.n_z, 256), VB_OUTPUT);

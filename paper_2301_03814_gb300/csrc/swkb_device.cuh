@@ -623,88 +623,80 @@ __global__ void __launch_bounds__(MARCH_THREADS, 6) k_march_x2(const MarchArgs<f
 // ----------------------------------------------------------------------------
 // Landing of ray j in grid units: g_j = (j - G) R + d_j.  Tile t starts at
 // grid point t TM; jlo[t][i] = the j with g_j <= t TM < g_{j+1}.
-// One landing pair (j, j + 1) of column i: order and coverage checks, and
-// the tile starts the pair brackets.  Returns status bits.
+
+// Coverage of the screen by the landing pair (j, j + 1).
 template <typename T>
-__device__ __forceinline__ unsigned bracket_pair(const BracketArgs<T>& p, int i, int j, T d0,
-                                                 T d1) {
-  const int b0 = (j - p.G) * p.R;   // |b0| <= N + G R < 2^31
-  const int b1 = b0 + p.R;
+__device__ __forceinline__ unsigned cover_pair(const BracketArgs<T>& p, int j, T d0, T d1) {
+  const int b0 = (j - p.G) * p.R, b1 = b0 + p.R;
   unsigned st = 0;
-  if (!(T(p.R) + d1 - d0 > T(0))) st |= ST_CAUSTIC;              // g_{j+1} > g_j
   if (j == 1 && !(d0 <= T(-b0))) st |= ST_COVER;                  // g_1 <= 0
   if (j + 1 == p.NRT - 2 && !(d1 > T(p.N - b1))) st |= ST_COVER;  // g_{NRT-2} > N
   if (p.sym) {   // the mirror family g'_{j'} = N - g_{NRT-j'} must cover too
     if (j == 2 && !(d0 < T(-b0))) st |= ST_COVER;                 // g_2 < 0
     if (j + 1 == p.NRT - 1 && !(d1 >= T(p.N - b1))) st |= ST_COVER;  // g_{NRT-1} >= N
   }
-  if (st) return st;
-  const int TM = p.TM;
-  const float inv_tm = 1.0f / (float)TM;   // exact (TM is a power of two)
-  // Both families bracket a tile start only if a multiple of TM lies in
-  // [g_j, g_{j+1}] (the mirror family's starts N - t TM are multiples of TM
-  // too).  Float estimate with a margin of TM / 1000, far above its rounding;
-  // the exact tests below decide the pairs that pass.
-  {
-    const float g0 = (float)b0 + (float)d0, g1 = (float)b1 + (float)d1;
-    if (floorf(g1 * inv_tm + 1e-3f) < ceilf(g0 * inv_tm - 1e-3f)) return 0;
-  }
-  {
-    // tile starts t TM in [g_j, g_{j+1})
-    int t0 = (int)ceilf(((float)b0 + (float)d0) * inv_tm);
-    int t1 = (int)ceilf(((float)b1 + (float)d1) * inv_tm) - 1;
-    t0 = min(max(t0, -1), p.n_tiles + 1);
-    t1 = min(max(t1, -1), p.n_tiles + 1);
-    for (int k = 0; k < 4 && d0 <= T((t0 - 1) * TM - b0); ++k) --t0;
-    for (int k = 0; k < 4 && !(d0 <= T(t0 * TM - b0)); ++k) ++t0;
-    for (int k = 0; k < 4 && !(T(t1 * TM - b1) < d1); ++k) --t1;
-    for (int k = 0; k < 4 && T((t1 + 1) * TM - b1) < d1; ++k) ++t1;
-    t0 = max(t0, 0);
-    t1 = min(t1, p.n_tiles);
-    for (int t = t0; t <= t1; ++t)
-      p.jlo[bchk((long long)t * p.Mr + i, (long long)(p.n_tiles + 1) * p.Mr, st)] = j;
-  }
-  if (p.sym) {
-    // mirror family: its bracket of tile start t TM is ray NRT - 1 - j when
-    // g_j < N - t TM <= g_{j+1}
-    int t0 = (int)ceilf(((float)p.N - (float)b1 - (float)d1) * inv_tm);
-    int t1 = (int)ceilf(((float)p.N - (float)b0 - (float)d0) * inv_tm) - 1;
-    t0 = min(max(t0, -1), p.n_tiles + 1);
-    t1 = min(max(t1, -1), p.n_tiles + 1);
-    // t0 = min t with N - t TM <= g_{j+1};  t1 = max t with g_j < N - t TM
-    for (int k = 0; k < 4 && T(p.N - (t0 - 1) * TM - b1) <= d1; ++k) --t0;
-    for (int k = 0; k < 4 && !(T(p.N - t0 * TM - b1) <= d1); ++k) ++t0;
-    for (int k = 0; k < 4 && !(d0 < T(p.N - t1 * TM - b0)); ++k) --t1;
-    for (int k = 0; k < 4 && d0 < T(p.N - (t1 + 1) * TM - b0); ++k) ++t1;
-    t0 = max(t0, 0);
-    t1 = min(t1, p.n_tiles);
-    for (int t = t0; t <= t1; ++t)
-      p.jlo_neg[bchk((long long)t * p.Mr + i, (long long)(p.n_tiles + 1) * p.Mr, st)] =
-          p.NRT - 1 - j;
-  }
   return st;
 }
 
-// One thread per landing pair (measured faster than longer per-thread runs:
-// the kernel is latency-bound and wants the parallelism).
-constexpr int BRACKET_RUN = 1;
+// A thread takes BRACKET_RUN consecutive landing pairs of one column, all its
+// loads issued first; most runs bracket no tile start and leave after one test.
+// Bound by the latency of those loads and, for large plans, by reading the
+// landings: 489 x 2086 landings 8.1 us, 545 x 16398 20 us, FP64 489 x 2086 20 us
+// (a thread per pair, each with its own estimates and loops for both families:
+// 10.2, 39 and 38; runs of 2: 8.2, 30 and 18.5).
+constexpr int BRACKET_RUN = 4;
+// blocks along the rays
+__host__ __device__ inline int bracket_rows(int NRT) {
+  return (NRT - 1 + BRACKET_RUN - 1) / BRACKET_RUN;
+}
 
 template <typename T, int LD>
 __device__ __forceinline__ void bracket_body(const BracketArgs<T>& p, int bx, int by, int tid) {
   const int i = bx * 256 + tid;
-  const int j0 = by * BRACKET_RUN;
   if (i >= p.Mr) return;
-  const int j1 = min(j0 + BRACKET_RUN, p.NRT - 1);   // pairs (j, j + 1), j < j1
+  const int j0 = by * BRACKET_RUN;
+  const int n = min(BRACKET_RUN, p.NRT - 1 - j0);   // pairs (j0 + k, j0 + k + 1), k < n
   unsigned st = 0;
-  unsigned bst = 0;
-  const long long nrm = (long long)p.NRT * p.Mr;
-  T d0 = ld<LD>(p.d + bchk((long long)j0 * p.Mr + i, nrm, bst));
-  for (int j = j0; j < j1; ++j) {
-    const T d1 = ld<LD>(p.d + bchk((long long)(j + 1) * p.Mr + i, nrm, bst));
-    st |= bracket_pair(p, i, j, d0, d1);
-    d0 = d1;
+  const long long nrm = (long long)p.NRT * p.Mr, o = (long long)j0 * p.Mr + i;
+  T d[BRACKET_RUN + 1];
+#pragma unroll
+  for (int k = 0; k <= BRACKET_RUN; ++k)
+    d[k] = ld<LD>(p.d + bchk(o + (long long)min(k, n) * p.Mr, nrm, st));
+  bool rising = true;
+#pragma unroll
+  for (int k = 0; k < BRACKET_RUN; ++k)
+    if (k < n) rising = rising && T(p.R) + d[k + 1] - d[k] > T(0);   // g_{j+1} > g_j
+  if (!rising) st |= ST_CAUSTIC;
+  if (j0 <= 2 || j0 + BRACKET_RUN >= p.NRT - 2) {
+#pragma unroll
+    for (int k = 0; k < BRACKET_RUN; ++k)
+      if (k < n) st |= cover_pair(p, j0 + k, d[k], d[k + 1]);
   }
-  st |= bst;
+  // Multiples x = t TM within the run's landings, by a float estimate with a
+  // margin of TM / 100, far above its rounding; exact tests decide.  Tile t of
+  // the family starts at x, tile n_tiles - t of its mirror image (landings
+  // N - g) at N - x.  (A run out of order, or NaN, is an error already: nothing
+  // is written, and the sums check what they take from the table.)
+  const float inv_tm = 1.0f / (float)p.TM;   // exact (TM is a power of two)
+  const int b0 = (j0 - p.G) * p.R;           // |b0| <= N + G R < 2^31
+  const float g0 = (float)b0 + (float)d[0];
+  const float g1 = (float)(b0 + n * p.R) + (float)d[BRACKET_RUN];
+  const int t0 = max((int)ceilf(g0 * inv_tm - 1e-2f), 0);
+  const int t1 = rising ? min((int)floorf(g1 * inv_tm + 1e-2f), p.n_tiles) : -1;
+  for (int t = t0; t <= t1; ++t) {
+    const int x = t * p.TM;
+    const long long nj = (long long)(p.n_tiles + 1) * p.Mr;
+#pragma unroll
+    for (int k = 0; k < BRACKET_RUN; ++k) {
+      if (k >= n) break;
+      const T lo = T(x - (b0 + k * p.R)), hi = T(x - (b0 + (k + 1) * p.R));
+      if (d[k] <= lo && hi < d[k + 1])               // g_j <= x < g_{j+1}
+        p.jlo[bchk((long long)t * p.Mr + i, nj, st)] = j0 + k;
+      // bracket of the mirror family: g_j < x <= g_{j+1}
+      if (p.sym && d[k] < lo && hi <= d[k + 1])
+        p.jlo_neg[bchk((long long)(p.n_tiles - t) * p.Mr + i, nj, st)] = p.NRT - 1 - (j0 + k);
+    }
+  }
   if (st) atomicOr(p.status, st);
 }
 
@@ -712,7 +704,7 @@ __device__ __forceinline__ void bracket_body(const BracketArgs<T>& p, int bx, in
 // strides of gridDim.y.
 template <typename T>
 __global__ void __launch_bounds__(256) k_bracket(const BracketArgs<T> p) {
-  const int rows = (p.NRT - 1 + BRACKET_RUN - 1) / BRACKET_RUN;
+  const int rows = bracket_rows(p.NRT);
   for (int by = blockIdx.y; by < rows; by += gridDim.y)
     bracket_body<T, LD_PLAIN>(p, blockIdx.x, by, threadIdx.x);
 }
