@@ -20,6 +20,10 @@
 //   4. the projections of the field on the basis (period means), the
 //      advance by exp(i alpha x) and the sum back onto the field points.
 //
+// Without eigenvalues to return, step 3 and the advance are replaced, where that
+// is shorter, by the Chebyshev expansion of exp(i sqrt(A) x) applied to the
+// projections (see chebyshev below): 641 rows at 1 and 2 km 5.3 ms instead of 60.
+//
 // FP64 throughput is the scarce resource on this GPU (two FMAs per SM and
 // clock), so the rotation tangent is found in FP32 and only c, s and the
 // updates are FP64.  A zero padding row never mixes with the others (its
@@ -135,10 +139,16 @@ __global__ void k_eps_means(const double* eps, int n_q, const double* tq, int J,
   __shared__ double sh[32];
   const int j = blockIdx.x, b = blockIdx.y;
   const double* e = eps + (size_t)b * (n_q + 1);
-  const long long two = 2LL * n_q;
+  const unsigned two = 2u * (unsigned)n_q;   // n_q <= 2^24
+  // (j i) mod 2 n_q, advanced by addition
+  const unsigned step = (unsigned)(((unsigned long long)j * blockDim.x) % two);
+  unsigned ph = (unsigned)(((unsigned long long)j * (1 + threadIdx.x)) % two);
   double acc = 0.0;
-  for (int i = 1 + threadIdx.x; i < n_q; i += blockDim.x)
-    acc += e[i] * tq[((long long)j * i) % two];
+  for (int i = 1 + threadIdx.x; i < n_q; i += blockDim.x) {
+    acc += e[i] * tq[ph];
+    ph += step;
+    ph = min(ph, ph - two);   // unsigned: the smaller is the one in [0, 2 n_q)
+  }
   acc = block_sum(acc, sh);
   if (threadIdx.x == 0)
     eh[(size_t)b * J + j] = (e[0] + 2.0 * acc + ((j & 1) ? -e[n_q] : e[n_q])) / (double)two;
@@ -517,6 +527,12 @@ __device__ inline double2 field_at(const double2* u, const FieldDims& f, int i) 
   return f.mirror > 0 ? v : make_double2(-v.x, -v.y);
 }
 
+// (n a) mod N in [0, N), n >= 0, |a| < N < 2^31
+__device__ inline unsigned phase_index(int n, int a, int N) {
+  const long long ph = ((long long)n * a) % N;
+  return (unsigned)(ph < 0 ? ph + N : ph);
+}
+
 // uh[mat][row] = w_n / N sum_i u(i) e_n(i); one CTA per (row, mat)
 __global__ void k_project(const double2* u0, FieldDims f, HillDims d, const double2* tab,
                           double2* uh) {
@@ -529,10 +545,14 @@ __global__ void k_project(const double2* u0, FieldDims f, HillDims d, const doub
   if (row < n_blk) {
     const int bn = row + odd;
     const double2* u = u0 + (size_t)b * f.n_z;
+    // (bn (i - m_c)) mod N, advanced by addition
+    const unsigned N = (unsigned)f.N;
+    const unsigned step = (unsigned)(((unsigned long long)bn * blockDim.x) % N);
+    unsigned ph = phase_index(bn, (int)threadIdx.x - f.m_c, f.N);
     for (int i = threadIdx.x; i < f.N; i += blockDim.x) {
-      long long ph = ((long long)bn * (i - f.m_c)) % f.N;
-      if (ph < 0) ph += f.N;
       const double2 cs = tab[ph];
+      ph += step;
+      ph = min(ph, ph - N);
       const double e = odd ? cs.y : cs.x;
       const double2 v = field_at(u, f, i);
       sr += v.x * e;
@@ -580,33 +600,50 @@ __global__ void k_advance_coefficients(const double* A, const double2* coef, Hil
   }
 }
 
-// u_out[b][r][m] = sum over blocks and rows of g e_n at the field point m
-__global__ void k_synthesize(const double2* g, FieldDims f, HillDims d, int batch, int n_x,
+// u_out[b][r][m] = sum over blocks and rows of g e_n at the field point m; a
+// thread takes SYN_X ranges of one point, which share the basis value.  Latency of
+// the table and the coefficients bounds it, so four rows are in flight.
+template <int SYN_X>
+__global__ void __launch_bounds__(64) k_synthesize(const double2* g, FieldDims f, HillDims d, int batch, int n_x,
                              const double2* tab, double2* out) {
-  const long long total = (long long)batch * n_x * f.n_z;
+  const int groups = (n_x + SYN_X - 1) / SYN_X;
+  const long long total = (long long)batch * groups * f.n_z;
+  const unsigned N = (unsigned)f.N;
   for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
        idx += (long long)gridDim.x * blockDim.x) {
     const int m = (int)(idx % f.n_z);
-    const long long br = idx / f.n_z;
-    const int r = (int)(br % n_x), b = (int)(br / n_x);
+    const long long bg = idx / f.n_z;
+    const int r0 = (int)(bg % groups) * SYN_X, b = (int)(bg / groups);
     const int i = f.mirror ? f.n_z + m : m;   // period point
-    double sr = 0.0, si = 0.0;
+    double sr[SYN_X], si[SYN_X];
+#pragma unroll
+    for (int x = 0; x < SYN_X; ++x) sr[x] = si[x] = 0.0;
     for (int blk = 0; blk < d.n_par; ++blk) {
       const int mat = b * d.n_par + blk;
       const int odd = parity_of(d, mat);
       const int n_blk = odd ? d.K : d.K + 1;
-      const double2* gg = g + ((size_t)mat * n_x + r) * d.P;
+      const double2* gg = g + ((size_t)mat * n_x + r0) * d.P;
+      const int nr = min(SYN_X, n_x - r0);
+      // (bn (i - m_c)) mod N, advanced by addition
+      const unsigned step = phase_index(1, i - f.m_c, f.N);
+      unsigned ph = odd ? step : 0u;
+#pragma unroll 4
       for (int row = 0; row < n_blk; ++row) {
-        const int bn = row + odd;
-        long long ph = ((long long)bn * (i - f.m_c)) % f.N;
-        if (ph < 0) ph += f.N;
         const double2 cs = tab[ph];
-        const double e = (bn == 0 ? 1.0 : M_SQRT2) * (odd ? cs.y : cs.x);
-        sr += gg[row].x * e;
-        si += gg[row].y * e;
+        ph += step;
+        ph = min(ph, ph - N);
+        const double e = (row + odd == 0 ? 1.0 : M_SQRT2) * (odd ? cs.y : cs.x);
+#pragma unroll
+        for (int x = 0; x < SYN_X; ++x) {
+          const double2 v = gg[(size_t)(x < nr ? x : 0) * d.P + row];
+          sr[x] += v.x * e;
+          si[x] += v.y * e;
+        }
       }
     }
-    out[idx] = make_double2(sr, si);
+#pragma unroll
+    for (int x = 0; x < SYN_X; ++x)
+      if (r0 + x < n_x) out[((size_t)b * n_x + r0 + x) * f.n_z + m] = make_double2(sr[x], si[x]);
   }
 }
 
@@ -638,6 +675,183 @@ __global__ void k_copy_leading(const double* A, const double* W, int n, int P, i
     const size_t src = (size_t)mat * P * P + (size_t)r * P + c;
     if (vec) vec[idx] = W[src];
     if (lam && r == c) lam[(size_t)mat * n + r] = A[src];
+  }
+}
+
+// ---------------------------------------------------------------------------
+// the field without the eigen-decomposition: Chebyshev expansion of
+// exp(i sqrt(A) x) on an interval that holds the spectrum
+// ---------------------------------------------------------------------------
+
+// range[b] = (min, max) of eps, (NaN, NaN) when an entry is not finite
+constexpr int kRangeThreads = 1024;
+
+__global__ void __launch_bounds__(kRangeThreads) k_eps_range(const double* eps, int n_q,
+                                                             double2* range) {
+  __shared__ double sh[2][32];
+  const double* e = eps + (size_t)blockIdx.x * (n_q + 1);
+  double lo = e[0], hi = e[0];
+  bool bad = false;
+#pragma unroll 8
+  for (int i = threadIdx.x; i <= n_q; i += kRangeThreads) {
+    const double v = e[i];
+    bad = bad || !isfinite(v);
+    lo = fmin(lo, v);
+    hi = fmax(hi, v);
+  }
+  bad = __syncthreads_or(bad);
+  for (int r = 0; r < 2; ++r) {   // within the warps, then over their results
+    for (int o = 16; o > 0; o >>= 1) {
+      lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+      hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    }
+    if (r == 0) {
+      if ((threadIdx.x & 31) == 0) {
+        sh[0][threadIdx.x >> 5] = lo;
+        sh[1][threadIdx.x >> 5] = hi;
+      }
+      __syncthreads();
+      lo = sh[0][threadIdx.x & 31];
+      hi = sh[1][threadIdx.x & 31];
+    }
+  }
+  if (threadIdx.x == 0) range[blockIdx.x] = bad ? make_double2(NAN, NAN) : make_double2(lo, hi);
+}
+
+// Per problem: spectrum within [mid - half, mid + half], alpha0 ~ sqrt(mid).
+struct ChebSpan {
+  double mid, half, alpha0, resid;   // resid = mid - alpha0^2
+};
+
+// f[b][r][k] = exp(i x_r (sqrt(lambda_k) - alpha0)) at the N Chebyshev nodes
+// lambda_k = mid + half cos(pi (k + 1/2) / N); the difference of the square
+// roots is formed without cancellation, so that its phase is a few hundred turns
+// at most.
+__global__ void k_cheb_nodes(const ChebSpan* span, const double* xs, int n_x, int N, int batch,
+                             double2* f) {
+  const long long total = (long long)batch * n_x * N;
+  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
+       idx += (long long)gridDim.x * blockDim.x) {
+    const int k = (int)(idx % N);
+    const long long br = idx / N;
+    const int r = (int)(br % n_x), b = (int)(br / n_x);
+    const ChebSpan s = span[b];
+    const double c = cospi((2.0 * k + 1.0) / (2.0 * N));
+    const double root = sqrt(fma(s.half, c, s.mid));
+    double sn, cs;
+    sincos(fma(s.half, c, s.resid) / (root + s.alpha0) * xs[r], &sn, &cs);
+    f[idx] = make_double2(cs, sn);
+  }
+}
+
+// coef[b][r][j] = (2 - delta_j0) / N carrier[b][r] sum_k f_k cos(pi j (2 k + 1) / (2 N)),
+// j < terms; a warp per coefficient, ct[m] = cos(pi m / (2 N)), m < 4 N (a power of two)
+__global__ void k_cheb_coef(const double2* f, const double2* carrier, const double* ct, int n_x,
+                            int N, int terms, int batch, double2* coef) {
+  const long long warp = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (warp >= (long long)batch * n_x * terms) return;
+  const int j = (int)(warp % terms);
+  const long long br = warp / terms;
+  const double2* fk = f + br * N;
+  const unsigned mask = 4u * (unsigned)N - 1u;
+  double sr = 0.0, si = 0.0;
+  for (int k = lane; k < N; k += 32) {
+    const double c = ct[((unsigned)j * (2u * (unsigned)k + 1u)) & mask];
+    const double2 v = fk[k];
+    sr += v.x * c;
+    si += v.y * c;
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    sr += __shfl_xor_sync(0xffffffffu, sr, o);
+    si += __shfl_xor_sync(0xffffffffu, si, o);
+  }
+  if (lane == 0) {
+    const double w = (j == 0 ? 1.0 : 2.0) / N;
+    const double2 c = carrier[br];
+    coef[warp] = make_double2((sr * c.x - si * c.y) * w, (sr * c.y + si * c.x) * w);
+  }
+}
+
+__global__ void k_cheb_table(double* ct, int N) {
+  for (long long m = blockIdx.x * (long long)blockDim.x + threadIdx.x; m < 4LL * N;
+       m += (long long)gridDim.x * blockDim.x)
+    ct[m] = cospi((double)m / (2.0 * N));
+}
+
+// A <- 2 (A - mid I) / half (the padding rows keep zeros off the diagonal)
+__global__ void k_cheb_scale(double* A, int P, int n_par, int n_mat, const ChebSpan* span) {
+  const long long PP = (long long)P * P, total = PP * n_mat;
+  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
+       idx += (long long)gridDim.x * blockDim.x) {
+    const int mat = (int)(idx / PP);
+    const int rem = (int)(idx - (long long)mat * PP);
+    const ChebSpan s = span[mat / n_par];
+    const int r = rem / P;
+    A[idx] = 2.0 * (A[idx] - (rem - r * P == r ? s.mid : 0.0)) / s.half;
+  }
+}
+
+// One step of the recurrence T_{j+1} = M T_j - T_{j-1} (M = 2 (A - mid) / half)
+// on a complex vector per matrix, a one-warp CTA per row (CTAs of four warps
+// spread 642 rows unevenly: 9.5 us); the new vector replaces T_{j-1} (its element
+// is read by this row only).  The ranges' sums gain coef_{j+1}
+// T_{j+1}.  FIRST: T_1 = M T_0 / 2, the sums start as coef_0 T_0 + coef_1 T_1.
+//   Bound by latency (FP64 pipe 1.4 us for 642 rows): the loads, a chain of
+// products and a shuffle tree, so what the row needs last is loaded first.  642
+// rows: 8 us per step (a row over four warps 10; programmatic dependent launches
+// with M loaded before the wait 18).
+template <bool FIRST>
+__global__ void __launch_bounds__(32) k_cheb_step(const double* __restrict__ M,
+                                                   const double2* __restrict__ cur, double2* prev,
+                                                   const double2* __restrict__ coef, int j,
+                                                   int terms, int n_par, int n_x, int P, int n_mat,
+                                                   double2* __restrict__ out) {
+  const int lane = threadIdx.x;
+  const int mat = blockIdx.x / P, row = blockIdx.x - mat * P;
+  const double2* m2 = reinterpret_cast<const double2*>(M + ((size_t)mat * P + row) * P);
+  const double2* c = cur + (size_t)mat * P;
+  const size_t at = (size_t)mat * P + row;
+  const double2 old = FIRST ? c[row] : prev[at];
+  const double2* cf = coef + (size_t)(mat / n_par) * n_x * terms;
+  double2* o = out + (size_t)mat * n_x * P + row;
+  double2 w0 = make_double2(0.0, 0.0), s0 = w0, z0 = w0;   // range `lane`
+  if (lane < n_x) {
+    w0 = cf[(size_t)lane * terms + j];
+    if (FIRST) z0 = cf[(size_t)lane * terms];
+    else s0 = o[(size_t)lane * P];
+  }
+  double sr[2] = {0.0, 0.0}, si[2] = {0.0, 0.0};
+#pragma unroll 6
+  for (int k = lane; k < P / 2; k += 32) {
+    const double2 m = __ldg(m2 + k);
+    const double2 a = c[2 * k], b = c[2 * k + 1];
+    sr[0] = fma(m.x, a.x, sr[0]);
+    si[0] = fma(m.x, a.y, si[0]);
+    sr[1] = fma(m.y, b.x, sr[1]);
+    si[1] = fma(m.y, b.y, si[1]);
+  }
+  double xr = sr[0] + sr[1], xi = si[0] + si[1];
+  for (int q = 16; q > 0; q >>= 1) {
+    xr += __shfl_xor_sync(0xffffffffu, xr, q);
+    xi += __shfl_xor_sync(0xffffffffu, xi, q);
+  }
+  const double2 t = FIRST ? make_double2(0.5 * xr, 0.5 * xi) : make_double2(xr - old.x, xi - old.y);
+  __syncwarp();
+  if (lane == 0) prev[at] = t;
+  for (int r = lane; r < n_x; r += 32) {
+    const bool pre = r < 32;
+    const double2 w = pre ? w0 : cf[(size_t)r * terms + j];
+    double2 s;
+    if (FIRST) {
+      const double2 z = pre ? z0 : cf[(size_t)r * terms];
+      s = make_double2(z.x * old.x - z.y * old.y, z.x * old.y + z.y * old.x);
+    } else {
+      s = pre ? s0 : o[(size_t)r * P];
+    }
+    s.x = fma(w.x, t.x, fma(-w.y, t.y, s.x));
+    s.y = fma(w.x, t.y, fma(w.y, t.x, s.y));
+    o[(size_t)r * P] = s;
   }
 }
 
@@ -814,6 +1028,108 @@ swkb_status replay_back(Scratch& s, const RotLog& log, int P, int n_mat, int vec
   return SWKB_OK;
 }
 
+// out[mat][r] <- exp(i sqrt(A[mat]) x_r) uh[mat] by the Chebyshev expansion, when
+// that is the shorter way (*done); else nothing has changed.  The quadrature of
+// A is exact on the basis (n_q >= 2 K), so the spectrum lies within
+// [k^2 min eps - kappa_K^2, k^2 max eps]; without evanescent modes the expansion
+// of exp(i x sqrt(lambda)) there needs about x half / (2 sqrt(lambda_min))
+// terms, each one matrix-vector product of 4 to 9 us, against the ~7 P rounds of
+// the Jacobi iteration.  Surface duct, 641 rows, 2 km: 526 terms, 59.9 -> 5.3 ms
+// for the whole call.  Both ways cost the same at 4.1 P (402 rows), 4.7 P (206), 6.1 P
+// (102) and above 7.8 P (62 and 642) terms, so 4 P is the most taken here.
+// uh and A are overwritten when done.
+swkb_status chebyshev(Scratch& s, const HillDims& d, int batch, int n_x, const double* k,
+                      const double* x, const std::vector<double2>& range, const double* xd,
+                      double* A, double2* uh, double2* out, bool* done) {
+  *done = false;
+  const int n_mat = batch * d.n_par, P = d.P;
+  double x_max = 0.0;
+  for (int r = 0; r < n_x; ++r) x_max = std::max(x_max, x[r]);
+  std::vector<ChebSpan> span(batch);
+  double terms_d = 0.0;
+  for (int b = 0; b < batch; ++b) {
+    const double kap = d.kappa1 * d.K, k2 = k[b] * k[b];
+    // (a non-finite eps gives NaN and the Jacobi path, which reports it)
+    double lo = k2 * range[b].x - kap * kap, hi = k2 * range[b].y;
+    const double pad = 1e-12 * fabs(hi) + 1e-9 * (hi - lo);   // rounding of A
+    lo -= pad;
+    hi += pad;
+    // (nor do sums of squares overflow, which it refuses)
+    if (!(lo > 0.01 * hi) || !(hi > 1e-140 && hi < 1e140)) return SWKB_OK;
+    ChebSpan& c = span[b];
+    c.mid = 0.5 * (lo + hi);
+    c.half = 0.5 * (hi - lo);
+    c.alpha0 = sqrt(c.mid);
+    c.resid = fma(-c.alpha0, c.alpha0, c.mid);
+    const double z = x_max * c.half / (2.0 * sqrt(lo));
+    const double rho = (sqrt(hi) + sqrt(lo)) / (sqrt(hi) - sqrt(lo));   // branch point at 0
+    terms_d = std::max(terms_d, z + 12.0 * cbrt(z) + 24.0 + 40.0 / log(rho));
+  }
+  if (!(terms_d <= 4.0 * P)) return SWKB_OK;
+  const int terms = std::max(4, (int)ceil(terms_d));
+  int N = 64;
+  while (N < terms + 32) N *= 2;
+  // the coefficients must cost neither more time than the products nor more
+  // memory than the Jacobi iteration's rotations (72 n_mat P^2 bytes)
+  if ((double)N * n_x * batch > 2.0 * P * P * batch + 32768.0) return SWKB_OK;
+  // carriers exp(i alpha0 x): the product exactly as hi + lo, the sine and cosine
+  // of hi reduced by the C library
+  std::vector<double2> carrier((size_t)batch * n_x);
+  for (int b = 0; b < batch; ++b)
+    for (int r = 0; r < n_x; ++r) {
+      const double hi = span[b].alpha0 * x[r], lo = fma(span[b].alpha0, x[r], -hi);
+      const double c = cos(hi), sn = sin(hi);
+      carrier[(size_t)b * n_x + r] = make_double2(c - lo * sn, sn + lo * c);
+    }
+  ChebSpan* span_d = nullptr;
+  double2 *carrier_d = nullptr, *f = nullptr, *coef = nullptr, *t1 = nullptr;
+  double* ct = nullptr;
+  const size_t n_br = (size_t)batch * n_x;
+  HTRY(s.alloc(&span_d, batch));
+  HTRY(s.alloc(&carrier_d, n_br));
+  HTRY(s.alloc(&f, n_br * N));
+  HTRY(s.alloc(&coef, n_br * terms));
+  HTRY(s.alloc(&ct, 4 * (size_t)N));
+  HTRY(s.alloc(&t1, (size_t)n_mat * P));
+  HCK(cudaMemcpyAsync(span_d, span.data(), batch * sizeof(ChebSpan), cudaMemcpyHostToDevice,
+                      s.stream));
+  HCK(cudaMemcpyAsync(carrier_d, carrier.data(), n_br * sizeof(double2), cudaMemcpyHostToDevice,
+                      s.stream));
+  k_cheb_table<<<grid_for(4LL * N), kThreads, 0, s.stream>>>(ct, N);
+  k_cheb_nodes<<<grid_for((long long)n_br * N), kThreads, 0, s.stream>>>(span_d, xd, n_x, N, batch,
+                                                                         f);
+  const long long warps = (long long)n_br * terms;
+  k_cheb_coef<<<(unsigned)((warps * 32 + kThreads - 1) / kThreads), kThreads, 0, s.stream>>>(
+      f, carrier_d, ct, n_x, N, terms, batch, coef);
+  HCK(cudaGetLastError());
+  // the last coefficients must have fallen off
+  std::vector<double2> tail(2 * n_br);
+  HCK(cudaMemcpy2DAsync(tail.data(), 2 * sizeof(double2), coef + (terms - 2),
+                        terms * sizeof(double2), 2 * sizeof(double2), n_br,
+                        cudaMemcpyDeviceToHost, s.stream));
+  HCK(cudaStreamSynchronize(s.stream));
+  for (const double2& c : tail)
+    if (!(fabs(c.x) + fabs(c.y) < 1e-14)) {
+      HTRY(s.release(f));
+      HTRY(s.release(coef));
+      return SWKB_OK;
+    }
+  k_cheb_scale<<<grid_for((long long)n_mat * P * P), kThreads, 0, s.stream>>>(A, P, d.n_par, n_mat,
+                                                                              span_d);
+  const unsigned grid = (unsigned)(n_mat * P);   // A's size bounds it
+  k_cheb_step<true><<<grid, 32, 0, s.stream>>>(A, uh, t1, coef, 1, terms, d.n_par, n_x, P, n_mat,
+                                                out);
+  double2 *cur = t1, *prev = uh;
+  for (int j = 2; j < terms; ++j) {
+    k_cheb_step<false><<<grid, 32, 0, s.stream>>>(A, cur, prev, coef, j, terms, d.n_par, n_x, P,
+                                                   n_mat, out);
+    std::swap(cur, prev);
+  }
+  HCK(cudaGetLastError());
+  *done = true;
+  return SWKB_OK;
+}
+
 swkb_status open_stream(Scratch& s, int on_device, void* user_stream) {
   // the caller's device work must be finished before the private stream reads it
   if (on_device) HCK(cudaStreamSynchronize((cudaStream_t)user_stream));
@@ -935,6 +1251,19 @@ swkb_status hill_propagate(const swkb_hill_desc* d, int batch, const double* k,
   HTRY(s.alloc(&ph, (size_t)n_mat * n_x * P));
   HCK(cudaMemcpyAsync(kd, k, batch * sizeof(double), cudaMemcpyHostToDevice, s.stream));
   HCK(cudaMemcpyAsync(xd, x, n_x * sizeof(double), cudaMemcpyHostToDevice, s.stream));
+  std::vector<double2> range;
+  if (!lam) {
+    // the eigenvalues are not asked for: chebyshev's choice, read back before
+    // the other kernels so that Jacobi's set-up still runs on the host beside them
+    double2* range_d = nullptr;
+    range.resize(batch);
+    HTRY(s.alloc(&range_d, batch));
+    k_eps_range<<<batch, kRangeThreads, 0, s.stream>>>(eps, d->n_q, range_d);
+    HCK(cudaGetLastError());
+    HCK(cudaMemcpyAsync(range.data(), range_d, batch * sizeof(double2), cudaMemcpyDeviceToHost,
+                        s.stream));
+    HCK(cudaStreamSynchronize(s.stream));
+  }
 
   k_dct_table<<<grid_for(2LL * d->n_q), kThreads, 0, s.stream>>>(tq, d->n_q);
   k_period_table<<<grid_for(f.N), kThreads, 0, s.stream>>>(tab, f.N);
@@ -946,13 +1275,19 @@ swkb_status hill_propagate(const swkb_hill_desc* d, int batch, const double* k,
   // logged rotations W = J_T^T ... J_1^T
   // the field's basis projections uh ride along the rotations: a = W uh
   k_project<<<dim3(P, n_mat), kThreads, 0, s.stream>>>(u0, f, hd, tab, uh);
-  RotLog lg;
-  HTRY(jacobi(s, A, nullptr, uh, P, n_mat, nullptr, &lg));
-  k_advance_coefficients<<<grid_for((long long)n_mat * n_x * P), kThreads, 0, s.stream>>>(
-      A, uh, hd, n_mat, xd, n_x, ph);                     // a_j exp(i alpha_j x)
-  HTRY(replay_back(s, lg, P, n_mat, n_x, ph));           // g = W^T (a exp(i alpha x))
-  k_synthesize<<<grid_for((long long)n_out), kThreads, 0, s.stream>>>(ph, f, hd, batch, n_x, tab,
-                                                                       out);
+  bool done = false;
+  if (!lam) HTRY(chebyshev(s, hd, batch, n_x, k, x, range, xd, A, uh, ph, &done));
+  if (!done) {
+    RotLog lg;
+    HTRY(jacobi(s, A, nullptr, uh, P, n_mat, nullptr, &lg));
+    k_advance_coefficients<<<grid_for((long long)n_mat * n_x * P), kThreads, 0, s.stream>>>(
+        A, uh, hd, n_mat, xd, n_x, ph);                   // a_j exp(i alpha_j x)
+    HTRY(replay_back(s, lg, P, n_mat, n_x, ph));         // g = W^T (a exp(i alpha x))
+  }
+  const auto synthesize = n_x == 1 ? k_synthesize<1> : n_x == 2 ? k_synthesize<2> : k_synthesize<4>;
+  const int per = std::min(n_x == 3 ? 4 : n_x, 4);
+  synthesize<<<grid_for((long long)batch * ((n_x + per - 1) / per) * d->n_z, 64), 64, 0, s.stream>>>(
+      ph, f, hd, batch, n_x, tab, out);
   if (lam) k_eigenvalues<<<grid_for((long long)batch * n_eig), kThreads, 0, s.stream>>>(
       A, hd, batch, lam);
   HCK(cudaGetLastError());
