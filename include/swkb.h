@@ -316,10 +316,10 @@ swkb_status swkb_plan_get_stats(const swkb_plan* plan, swkb_plan_stats* stats);
  * 65536 complex128 values) that every GPU loading this library holds until
  * the process exits.
  * The first call on a device performs a one-time set-up on that device (it
- * resolves the arrays' device addresses, initialises one of them and
+ * resolves the arrays' device addresses, initialises two of them and
  * synchronises the device); make that first call before any stream capture.
  * All calls on a device share the arrays and leave the last call's contents
- * in them (each call rewrites everything it reads, so nothing needs
+ * in them (each call rewrites what it reads besides those two, so nothing needs
  * clearing); calls that overlap on the GPU -- e.g. on two streams at once --
  * race on the arrays and must be serialised by the caller.
  */

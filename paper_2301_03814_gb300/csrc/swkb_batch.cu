@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 1)
         stage_args(&f, jb.step == 0 ? &I.fft_fresh : &I.fft_next, tid);
         __syncthreads();
         for (int v = item * VB_FFT1; v < min(item * VB_FFT1 + VB_FFT1, I.fft1_blocks); ++v) {
-          fft1_body<T, LD_CG>(f, v, tid, smem);
+          fft1_body<T, LD_CG, FFT1_COLS>(f, v, tid, smem);
           __syncthreads();   // the tile is reused by the next block
         }
         break;

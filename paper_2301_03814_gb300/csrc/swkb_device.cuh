@@ -1254,6 +1254,67 @@ __global__ void __launch_bounds__(RESUM_WARPS * 32, sizeof(T) == 4 ? (PW < 16 ? 
   resum_body<PW, LD_NC, 0>(p, blockIdx.x, threadIdx.x, smem_raw, 0);
 }
 
+// A point's partials are added in PART_SUMS interleaved sums (groups q, q +
+// PART_SUMS, ... in order), then these in order, so that in pass 1 of the DFT several
+// threads can share a point's loads.
+constexpr int PART_SUMS = 4;
+
+// interleaved sum q; loads issued 8 at a time
+template <typename V, int LD>
+__device__ __forceinline__ V parts_sum(const V* __restrict__ part, int N, int n_part, int q) {
+  V s;
+  s.x = s.y = 0;
+  int g = q;
+  for (; g + 7 * PART_SUMS < n_part; g += 8 * PART_SUMS) {
+    V v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = ld<LD>(part + (long long)(g + k * PART_SUMS) * N);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) { s.x += v[k].x; s.y += v[k].y; }
+  }
+#pragma unroll 4
+  for (; g < n_part; g += PART_SUMS) {
+    const V v = ld<LD>(part + (long long)g * N);
+    s.x += v.x; s.y += v.y;
+  }
+  return s;
+}
+
+template <typename V>
+__device__ __forceinline__ V parts_combine(V (&v)[PART_SUMS]) {
+#pragma unroll
+  for (int q = 1; q < PART_SUMS; ++q) { v[0].x += v[q].x; v[0].y += v[q].y; }
+  return v[0];
+}
+
+// the four sums of one thread side by side
+template <typename V, int LD>
+__device__ __forceinline__ V parts_total(const V* __restrict__ part, int N, int n_part) {
+  V a[PART_SUMS];
+#pragma unroll
+  for (int q = 0; q < PART_SUMS; ++q) a[q].x = a[q].y = 0;
+  int g = 0;
+  for (; g + 2 * PART_SUMS <= n_part; g += 2 * PART_SUMS) {
+    V v[2 * PART_SUMS];
+#pragma unroll
+    for (int k = 0; k < 2 * PART_SUMS; ++k) v[k] = ld<LD>(part + (long long)(g + k) * N);
+#pragma unroll
+    for (int k = 0; k < 2 * PART_SUMS; ++k) {
+      a[k % PART_SUMS].x += v[k].x;
+      a[k % PART_SUMS].y += v[k].y;
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 2 * PART_SUMS; ++k) {
+    if (g + k < n_part) {
+      const V v = ld<LD>(part + (long long)(g + k) * N);
+      a[k % PART_SUMS].x += v.x;
+      a[k % PART_SUMS].y += v.y;
+    }
+  }
+  return parts_combine(a);
+}
+
 // ----------------------------------------------------------------------------
 // field bookkeeping: partial sums, absorber, reflection, I/O
 // ----------------------------------------------------------------------------
@@ -1261,12 +1322,7 @@ template <typename T, int LD>
 __device__ __forceinline__ void reduce_body(const ReduceArgs<T>& p, int k) {
   using V = typename C2<T>::type;
   auto sum_at = [&](int mm) {
-    V s;
-    s.x = T(0); s.y = T(0);
-    for (int g = 0; g < p.n_part; ++g) {
-      const V v = ld<LD>(p.part + (long long)g * p.N + mm);
-      s.x += v.x; s.y += v.y;
-    }
+    V s = parts_total<V, LD>(p.part + mm, p.N, p.n_part);
     if (p.W) { const T w = p.W[mm]; s.x *= w; s.y *= w; }
     return s;
   };
@@ -1366,11 +1422,6 @@ __device__ __forceinline__ typename C2<T>::type cmul(typename C2<T>::type a,
   return r;
 }
 
-// pass 1: a CTA takes FFT1_COLS consecutive columns n2 (all N1 rows, one
-// tile in shared memory) and forms Y[k1][n2] = w_N^{n2 k1} sum_n1 x[n1 N2 + n2]
-// w_{N1}^{n1 k1} for all k1.  N1 <= 64.
-// FFT1_COLS (columns per pass-1 block) is in swkb_internal.h
-
 // (|v|, arg(v) / 2 pi) of a complex value, the angle in turns in [-1/2, 1/2].
 template <typename T>
 __device__ __forceinline__ typename C2<T>::type polar_turns(typename C2<T>::type v) {
@@ -1384,27 +1435,15 @@ __device__ __forceinline__ typename C2<T>::type polar_turns(typename C2<T>::type
 // Field value at grid point m formed from the resummation partials: the sum
 // over mode groups times the absorber, with the reflection of grounded plans
 // (same arithmetic as k_reduce).
-template <typename T, int LD>
-__device__ __forceinline__ typename C2<T>::type field_from_parts(const FftArgs<T>& p, int m) {
-  using V = typename C2<T>::type;
+template <typename T>
+__device__ __forceinline__ int parts_source(const FftArgs<T>& p, int m) {
+  return (p.sym && m > 0 && m < (p.N >> 1)) ? p.N - m : m;
+}
+
+template <typename T>
+__device__ __forceinline__ typename C2<T>::type parts_finish(const FftArgs<T>& p, int m, int src,
+                                                             typename C2<T>::type s) {
   const int half = p.N >> 1;
-  const int src = (p.sym && m > 0 && m < half) ? p.N - m : m;
-  V s;
-  s.x = T(0); s.y = T(0);
-  // loads issued in batches of 8, added in group order
-  const V* q = p.part + src;
-  int g = 0;
-  for (; g + 8 <= p.n_part; g += 8) {
-    V v[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) v[k] = ld<LD>(q + (long long)(g + k) * p.N);
-#pragma unroll
-    for (int k = 0; k < 8; ++k) { s.x += v[k].x; s.y += v[k].y; }
-  }
-  for (; g < p.n_part; ++g) {
-    const V v = ld<LD>(q + (long long)g * p.N);
-    s.x += v.x; s.y += v.y;
-  }
   if (p.W) { const T w = p.W[src]; s.x *= w; s.y *= w; }
   if (p.sym) {
     const T sg = T(p.mirror);
@@ -1417,38 +1456,91 @@ __device__ __forceinline__ typename C2<T>::type field_from_parts(const FftArgs<T
   return s;
 }
 
-// One pass-1 block of 256 threads (blk its index, smem_raw its shared memory).
-template <typename T, int LD>
-__device__ __forceinline__ void fft1_body(const FftArgs<T>& p, int blk, int tid,
-                                          unsigned char* smem_raw) {
-  using V = typename C2<T>::type;
-  V* tile = reinterpret_cast<V*>(smem_raw);          // [N1][FFT1_COLS]
-  V* w1 = tile + p.N1 * FFT1_COLS;                   // [N1] w_{N1}^k
-  const int c0 = blk * FFT1_COLS;
-  for (int e = tid; e < p.N1 * FFT1_COLS; e += 256) {
-    const int n1 = e / FFT1_COLS, c = e % FFT1_COLS;
-    const int m = n1 * p.N2 + c0 + c;
-    tile[e] = p.part ? field_from_parts<T, LD>(p, m) : ld<LD>(p.u + m);
-  }
-  for (int k = tid; k < p.N1; k += 256) w1[k] = p.tw[(long long)k * p.N2];
-  __syncthreads();
-  for (int e = tid; e < p.N1 * FFT1_COLS; e += 256) {
-    const int k1 = e / FFT1_COLS, c = e % FFT1_COLS;
-    V acc;
-    acc.x = T(0); acc.y = T(0);
-    for (int n1 = 0; n1 < p.N1; ++n1) {
-      const V t = cmul<T>(tile[n1 * FFT1_COLS + c], w1[(n1 * k1) & (p.N1 - 1)]);
-      acc.x += t.x; acc.y += t.y;
-    }
-    const int n2 = c0 + c;
-    p.Y[(long long)k1 * p.N2 + n2] = cmul<T>(acc, p.tw[(long long)n2 * k1]);
+// acc + a w: one rounding per product pair and sum in FP32 (as cmul and an
+// addition), four FMAs in FP64, where issue bounds the sums
+template <typename T>
+__device__ __forceinline__ void cmac(typename C2<T>::type& s, typename C2<T>::type a,
+                                     typename C2<T>::type w) {
+  if constexpr (sizeof(T) == 8) {
+    s.x = fma(a.x, w.x, fma(-a.y, w.y, s.x));
+    s.y = fma(a.x, w.y, fma(a.y, w.x, s.y));
+  } else {
+    const typename C2<T>::type t = cmul<T>(a, w);
+    s.x += t.x; s.y += t.y;
   }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(256) k_fft1(const FftArgs<T> p) {
+// pass 1: a CTA takes COLS consecutive columns n2 (all N1 rows, one tile in shared
+// memory) and forms Y[k1][n2] = w_N^{n2 k1} sum_n1 x[n1 N2 + n2] w_{N1}^{n1 k1} for
+// all k1.  Two threads form rows k1 and k1 + N1 / 2 of a column, the sum and the
+// difference of their sums over even and odd n1.  Latency bounds it on the plans'
+// chain: few columns per CTA (fft1_cols), a point's partials summed by several threads.
+// Both passes, 4096 points and 37 groups (lens): 12.1 -> 10.1 us; 8192 points (FP32
+// duct) 12.0 -> 10.0; FP64, 32768 points: 33.3 -> 27.9 (with one thread per point's
+// partials, 8 columns and every row formed alone; ~2 us are events).
+// One block of 256 threads (blk its index, smem_raw its shared memory).
+template <typename T, int LD, int COLS>
+__device__ __forceinline__ void fft1_body(const FftArgs<T>& p, int blk, int tid,
+                                          unsigned char* smem_raw) {
+  using V = typename C2<T>::type;
+  const int E = p.N1 * COLS;                         // a power of two
+  V* tile = reinterpret_cast<V*>(smem_raw);          // [N1][COLS]
+  V* w1 = tile + E;                                  // [N1] w_{N1}^k
+  const int c0 = blk * COLS;
+  for (int k = tid; k < p.N1; k += FFT1_THREADS) w1[k] = p.tw[(long long)k * p.N2 << p.tw_shift];
+  if (p.part) {
+    V* sums = w1 + p.N1;                             // [PART_SUMS][E], E < FFT1_THREADS
+    const int m0 = c0 + (tid & (COLS - 1));
+    if (E < FFT1_THREADS) {
+      for (int i = tid; i < PART_SUMS * E; i += FFT1_THREADS) {
+        const int src = parts_source(p, ((i & (E - 1)) / COLS) * p.N2 + m0);
+        sums[i] = parts_sum<V, LD>(p.part + src, p.N, p.n_part, i / E);
+      }
+      __syncthreads();
+    }
+    for (int e = tid; e < E; e += FFT1_THREADS) {
+      const int m = e / COLS * p.N2 + m0, src = parts_source(p, m);
+      V s;
+      if (E < FFT1_THREADS) {
+        V v[PART_SUMS];
+#pragma unroll
+        for (int q = 0; q < PART_SUMS; ++q) v[q] = sums[q * E + e];
+        s = parts_combine(v);
+      } else {
+        s = parts_total<V, LD>(p.part + src, p.N, p.n_part);
+      }
+      tile[e] = parts_finish(p, m, src, s);
+    }
+  } else {
+    for (int e = tid; e < E; e += FFT1_THREADS) tile[e] = ld<LD>(p.u + e / COLS * p.N2 + c0 + e % COLS);
+  }
+  __syncthreads();
+  for (int e0 = 0; e0 < E; e0 += FFT1_THREADS) {
+    const int e = e0 + tid;                          // (k1, h, c); idle threads stay for the shuffle
+    const int c = e % COLS, h = e / COLS & 1, k1 = e / (2 * COLS);
+    const int row = k1 + h * (p.N1 / 2), n2 = c0 + c;
+    V s;
+    s.x = s.y = T(0);
+    V w2 = s;
+    if (e < E) {
+      w2 = p.tw[(long long)n2 * row << p.tw_shift];
+#pragma unroll 4
+      for (int n1 = h; n1 < p.N1; n1 += 2)
+        cmac<T>(s, tile[n1 * COLS + c], w1[(n1 * k1) & (p.N1 - 1)]);
+    }
+    V o;
+    o.x = __shfl_xor_sync(0xffffffffu, s.x, COLS);
+    o.y = __shfl_xor_sync(0xffffffffu, s.y, COLS);
+    if (h) { s.x = o.x - s.x; s.y = o.y - s.y; }
+    else { s.x += o.x; s.y += o.y; }
+    if (e < E) p.Y[(long long)row * p.N2 + n2] = cmul<T>(s, w2);
+  }
+}
+
+template <typename T, int COLS>
+__global__ void __launch_bounds__(FFT1_THREADS) k_fft1(const FftArgs<T> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  fft1_body<T, LD_PLAIN>(p, blockIdx.x, threadIdx.x, smem_raw);
+  fft1_body<T, LD_PLAIN, COLS>(p, blockIdx.x, threadIdx.x, smem_raw);
 }
 
 // out_i = c_i f_i (mode coefficients of a plane between screens), and its
@@ -1467,8 +1559,8 @@ __global__ void k_cscale(const typename C2<T>::type* __restrict__ c,
 
 // w_{N2}^{idx} from the table of w_N (w_{N2} = w_N^{N1}).
 template <typename V>
-__device__ __forceinline__ V twiddle2(const V* tw, unsigned idx, int, int N1) {
-  return tw[(long long)idx * N1];
+__device__ __forceinline__ V twiddle2(const V* tw, unsigned idx, int shift, int N1) {
+  return tw[(long long)idx * N1 << shift];
 }
 
 // pass 2: one CTA (4 warps) per kept mode n:
@@ -1491,6 +1583,7 @@ __device__ __forceinline__ void fft2_body(const FftArgs<T>& p, int blk, int tid,
   const int k1 = b & (p.N1 - 1);
   const int k2 = b / p.N1;
   const V* row = (p.N1 > 1 ? p.Y : p.u) + (long long)k1 * p.N2;
+  const V ph = p.ephi[i];   // early: it is the last the chain needs
   V acc;
   acc.x = T(0); acc.y = T(0);
   // row entries and twiddles loaded 8 iterations at a time, summed in order
@@ -1503,7 +1596,7 @@ __device__ __forceinline__ void fft2_body(const FftArgs<T>& p, int blk, int tid,
       const int m = n2 + k * FFT2_THREADS;
       const unsigned e = (unsigned)(((long long)m * k2) & (p.N2 - 1));
       rv[k] = ld<LD>(row + m);
-      tv[k] = twiddle2(p.tw, e, p.log2N2, p.N1);
+      tv[k] = twiddle2(p.tw, e, p.tw_shift, p.N1);
     }
 #pragma unroll
     for (int k = 0; k < B; ++k) {
@@ -1513,7 +1606,7 @@ __device__ __forceinline__ void fft2_body(const FftArgs<T>& p, int blk, int tid,
   }
   for (; n2 < p.N2; n2 += FFT2_THREADS) {
     const unsigned e = (unsigned)(((long long)n2 * k2) & (p.N2 - 1));
-    const V t = cmul<T>(ld<LD>(row + n2), twiddle2(p.tw, e, p.log2N2, p.N1));
+    const V t = cmul<T>(ld<LD>(row + n2), twiddle2(p.tw, e, p.tw_shift, p.N1));
     acc.x += t.x; acc.y += t.y;
   }
 #pragma unroll
@@ -1528,7 +1621,7 @@ __device__ __forceinline__ void fft2_body(const FftArgs<T>& p, int blk, int tid,
 #pragma unroll
     for (int w = 1; w < FFT2_THREADS / 32; ++w) { tot.x += wsum[w].x; tot.y += wsum[w].y; }
     tot.x *= p.inv_N; tot.y *= p.inv_N;
-    const V cv = cmul<T>(tot, p.ephi[i]);
+    const V cv = cmul<T>(tot, ph);
     p.c[i] = cv;
     if (p.mirror && n > 0) {
       V cm;

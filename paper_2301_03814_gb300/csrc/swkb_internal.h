@@ -23,6 +23,11 @@ constexpr int TRIG_N = 1024;
 
 // Columns n2 of the DFT's pass 1 handled by one block.
 constexpr int FFT1_COLS = 8;
+constexpr int FFT1_THREADS = 256;
+// columns per CTA of k_fft1: 4 while 8 make fewer than two CTAs per SM
+inline int fft1_cols(int N2) { return N2 / 8 < 304 ? 4 : 8; }
+// CTAs of k_fft2_pair
+inline int fft2_pairs(int N1, int n_max) { return N1 * ((n_max + N1 - 1) / N1 + 1); }
 
 template <typename T> struct C2;
 template <> struct C2<float> { using type = float2; };
@@ -129,7 +134,8 @@ struct ReduceArgs {
 template <typename T>
 struct FftArgs {
   const typename C2<T>::type* u;     // [N]
-  const typename C2<T>::type* tw;    // [N] exp(-2 pi i k / N)
+  const typename C2<T>::type* tw;    // [N << tw_shift] exp(-2 pi i k / (N << tw_shift))
+  int tw_shift;
   typename C2<T>::type* Y;           // [N1][N2]
   int N, N1, N2, log2N2, n_max;
   int mirror;                        // 0, or +-1: the field is even / odd
@@ -193,6 +199,8 @@ template <typename T> cudaError_t launch_init(const double* u0, int n_z, int N, 
                                               typename C2<T>::type* u, cudaStream_t s);
 template <typename T> cudaError_t launch_reduce(const ReduceArgs<T>& a, cudaStream_t s);
 template <typename T> cudaError_t launch_fft(const FftArgs<T>& a, cudaStream_t s);
+// the same without a mirror, bins in pairs
+cudaError_t launch_fft_pairs(const FftArgs<double>& a, cudaStream_t s);
 template <typename T> cudaError_t launch_march(const MarchArgs<T>& a, bool multi_column,
                                                cudaStream_t s);
 template <typename T> cudaError_t launch_bracket(const BracketArgs<T>& a, cudaStream_t s);
@@ -251,7 +259,7 @@ struct PlanParts {
 // inner planes, reused rays, or a one-pass DFT (fft_n1 = 1).
 template <typename T> swkb_status plan_parts(swkb_plan* p, PlanParts<T>* out);
 // Shared-memory bytes of one pass-1 DFT block for split N1.
-template <typename T> size_t fft1_smem_bytes(int N1);
+template <typename T> size_t fft1_smem_bytes(int N1, int cols);
 
 // Plan-level hooks used by the request server (swkb_server.cu).
 cudaStream_t plan_stream(swkb_plan* p);

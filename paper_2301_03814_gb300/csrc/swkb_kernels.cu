@@ -57,19 +57,81 @@ cudaError_t launch_reduce(const ReduceArgs<T>& a, cudaStream_t s) {
 }
 
 template <typename T>
-size_t fft1_smem_bytes(int N1) {
-  return (size_t)(N1 * FFT1_COLS + N1) * sizeof(typename C2<T>::type);
+size_t fft1_smem_bytes(int N1, int cols) {
+  const int E = N1 * cols;
+  return (size_t)(E + N1 + (E < FFT1_THREADS ? PART_SUMS * E : 0)) * sizeof(typename C2<T>::type);
+}
+
+namespace {
+// Pass 2 in FP64 without a mirror: one CTA per pair of bins of a row, n = k1 + N1 k2
+// and k1 - N1 k2, which share the products of the row's entries with the cosine
+// and the sine (4 FMAs per entry for both bins; one by one 12 FP64 instructions).
+// Pairs are counted by n (fft2_pairs); where only one bin is kept the other is not
+// stored.
+// Bound by FP64 issue at large sizes, by latency at small ones.
+__global__ void __launch_bounds__(FFT2_THREADS) k_fft2_pair(const FftArgs<double> p) {
+  using V = double2;
+  __shared__ V sum[2][FFT2_THREADS / 32];
+  const int tid = threadIdx.x;
+  const int k1 = blockIdx.x & (p.N1 - 1), k2 = blockIdx.x / p.N1;
+  const V* row = (p.N1 > 1 ? p.Y : p.u) + (long long)k1 * p.N2;
+  double xc = 0.0, ys = 0.0, xs = 0.0, yc = 0.0;
+#pragma unroll 8
+  for (int n2 = tid; n2 < p.N2; n2 += FFT2_THREADS) {
+    const unsigned e = (unsigned)(((long long)n2 * k2) & (p.N2 - 1));
+    const V r = row[n2], w = twiddle2(p.tw, e, p.tw_shift, p.N1);
+    xc += r.x * w.x;
+    ys += r.y * w.y;
+    xs += r.x * w.y;
+    yc += r.y * w.x;
+  }
+  V s[2];
+  s[0].x = xc - ys; s[0].y = yc + xs;   // n = k1 + N1 k2
+  s[1].x = xc + ys; s[1].y = yc - xs;   // n = k1 - N1 k2
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      s[h].x += __shfl_xor_sync(0xffffffffu, s[h].x, o);
+      s[h].y += __shfl_xor_sync(0xffffffffu, s[h].y, o);
+    }
+    if ((tid & 31) == 0) sum[h][tid >> 5] = s[h];
+  }
+  __syncthreads();
+  if (tid > 1 || (tid == 1 && k2 == 0)) return;
+  const int n = tid == 0 ? k1 + p.N1 * k2 : k1 - p.N1 * k2;
+  if (n > p.n_max || n < -p.n_max) return;
+  V tot = sum[tid][0];
+#pragma unroll
+  for (int w = 1; w < FFT2_THREADS / 32; ++w) { tot.x += sum[tid][w].x; tot.y += sum[tid][w].y; }
+  tot.x *= p.inv_N; tot.y *= p.inv_N;
+  const int i = n + p.n_max;
+  const V cv = cmul<double>(tot, p.ephi[i]);
+  p.c[i] = cv;
+  if (p.cpol) p.cpol[i] = polar_turns<double>(cv);
 }
 
 template <typename T>
+cudaError_t launch_fft1(const FftArgs<T>& a, cudaStream_t s) {
+  if (a.N1 == 1) return cudaSuccess;
+  const int cols = fft1_cols(a.N2);
+  return launch_k(cols == 4 ? k_fft1<T, 4> : k_fft1<T, 8>, dim3(a.N2 / cols), dim3(FFT1_THREADS),
+                  fft1_smem_bytes<T>(a.N1, cols), s, a);
+}
+}  // namespace
+
+template <typename T>
 cudaError_t launch_fft(const FftArgs<T>& a, cudaStream_t s) {
-  if (a.N1 > 1) {
-    const size_t smem = fft1_smem_bytes<T>(a.N1);
-    const cudaError_t e = launch_k(k_fft1<T>, dim3(a.N2 / FFT1_COLS), dim3(256), smem, s, a);
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t e = launch_fft1<T>(a, s);
+  if (e != cudaSuccess) return e;
   const int modes = a.mirror ? a.n_max + 1 : 2 * a.n_max + 1;
   return launch_k(k_fft2<T>, dim3(modes), dim3(FFT2_THREADS), 0, s, a);
+}
+
+cudaError_t launch_fft_pairs(const FftArgs<double>& a, cudaStream_t s) {
+  const cudaError_t e = launch_fft1<double>(a, s);
+  if (e != cudaSuccess) return e;
+  return launch_k(k_fft2_pair, dim3(fft2_pairs(a.N1, a.n_max)), dim3(FFT2_THREADS), 0, s, a);
 }
 
 template <>
@@ -156,10 +218,11 @@ cudaError_t prepare_kernels(int resum_smem) {
 
 template <typename T>
 cudaError_t prepare_fft_kernels() {
-  // k_fft1's dynamic shared memory is (N1 FFT1_COLS + N1) complex values: at
-  // most 9 KB for the largest split the plans allow (N1 = 64), inside the
-  // default 48 KB limit; k_fft2 uses static shared memory only
-  static_assert((64 * FFT1_COLS + 64) * 16 <= 48 * 1024, "k_fft1 staging exceeds 48 KB");
+  // k_fft1's dynamic shared memory is at most 5 E + N1 complex values at E = 128,
+  // N1 = 32 and 9 N1 at the largest N1 = 64, inside the default 48 KB limit; k_fft2
+  // uses static shared memory only
+  static_assert((5 * 128 + 32) * 16 <= 48 * 1024 && 9 * 64 * 16 <= 48 * 1024,
+                "k_fft1 staging exceeds 48 KB");
   return cudaSuccess;
 }
 
@@ -186,7 +249,7 @@ cudaError_t launch_output(const typename C2<T>::type* u, int offset, int n, doub
   template cudaError_t launch_cscale<T>(const C2<T>::type*, const C2<T>::type*, C2<T>::type*,   \
                                         C2<T>::type*, int, cudaStream_t);                       \
   template size_t resum_smem_bytes<T>(int, int);                                                \
-  template size_t fft1_smem_bytes<T>(int);                                                      \
+  template size_t fft1_smem_bytes<T>(int, int);                                                     \
   template cudaError_t prepare_kernels<T>(int);                                                 \
   template cudaError_t prepare_fft_kernels<T>();
 

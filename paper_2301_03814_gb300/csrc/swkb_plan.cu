@@ -797,7 +797,7 @@ template <typename T>
 FftArgs<T> fft_args(const swkb_plan* p, bool fuse) {
   using V = typename C2<T>::type;
   FftArgs<T> f;
-  f.u = (const V*)p->u; f.tw = (const V*)p->tw; f.Y = (V*)p->Y;
+  f.u = (const V*)p->u; f.tw = (const V*)p->tw; f.tw_shift = 0; f.Y = (V*)p->Y;
   f.N = p->N; f.N1 = p->N1; f.N2 = p->N2; f.log2N2 = p->log2N2; f.n_max = p->n_max;
   f.mirror = p->mirror;
   f.part = fuse ? (const V*)p->part : nullptr;
@@ -884,7 +884,7 @@ swkb_status launch_screen(swkb_plan* p, int q, bool u_fresh) {
     TRY(timed(p, SWKB_KERNEL_REDUCE, 1, [&] { return launch_reduce<T>(r, s); }));
   }
   FftArgs<T> f;
-  f.u = (const V*)p->u; f.tw = (const V*)p->tw; f.Y = (V*)p->Y;
+  f.u = (const V*)p->u; f.tw = (const V*)p->tw; f.tw_shift = 0; f.Y = (V*)p->Y;
   f.N = p->N; f.N1 = p->N1; f.N2 = p->N2; f.log2N2 = p->log2N2; f.n_max = p->n_max;
   f.mirror = p->mirror;
   f.part = fuse ? (const V*)p->part : nullptr;
@@ -1019,7 +1019,7 @@ swkb_status overlapped_screen(swkb_plan* p, int q, int b, bool fresh) {
     TRY(timed(p, SWKB_KERNEL_REDUCE, 1, [&] { return launch_reduce<T>(r, s); }));
   }
   FftArgs<T> f;
-  f.u = (const V*)p->u; f.tw = (const V*)p->tw; f.Y = (V*)p->Y;
+  f.u = (const V*)p->u; f.tw = (const V*)p->tw; f.tw_shift = 0; f.Y = (V*)p->Y;
   f.N = p->N; f.N1 = p->N1; f.N2 = p->N2; f.log2N2 = p->log2N2; f.n_max = p->n_max;
   f.mirror = p->mirror;
   f.part = fuse ? (const V*)p->part : nullptr;
@@ -1193,7 +1193,7 @@ swkb_status enqueue_planes(swkb_plan* p, const double* u0, int q0, int n, int P,
   };
   for (int q = q0; q < q0 + n; ++q) {
     FftArgs<T> f;
-    f.u = (const V*)p->u; f.tw = (const V*)p->tw; f.Y = (V*)p->Y;
+    f.u = (const V*)p->u; f.tw = (const V*)p->tw; f.tw_shift = 0; f.Y = (V*)p->Y;
     f.N = p->N; f.N1 = p->N1; f.N2 = p->N2; f.log2N2 = p->log2N2; f.n_max = p->n_max;
     f.mirror = p->mirror;
     f.part = nullptr;
@@ -1899,7 +1899,7 @@ swkb_status plan_parts(swkb_plan* p, PlanParts<T>* o) {
   o->resum_smem = resum_smem_bytes<T>(p->wcap, p->TM);
   o->fft1_blocks = p->N2 / FFT1_COLS;
   o->fft2_blocks = p->mirror ? p->n_max + 1 : p->M;
-  o->fft1_smem = fft1_smem_bytes<T>(p->N1);
+  o->fft1_smem = fft1_smem_bytes<T>(p->N1, FFT1_COLS);
   o->reduce_n = (p->mirror || p->sym) ? p->N / 2 + 1 : p->N;
   o->out_off = p->mirror ? p->n_z : 0;
   o->rays = (size_t)p->NRT * p->Mr;
