@@ -1543,8 +1543,8 @@ __global__ void __launch_bounds__(FFT1_THREADS) k_fft1(const FftArgs<T> p) {
   fft1_body<T, LD_PLAIN, COLS>(p, blockIdx.x, threadIdx.x, smem_raw);
 }
 
-// out_i = c_i f_i (mode coefficients of a plane between screens), and its
-// polar form when pol is given.
+// out_i = c_i f_i (mode coefficients of the planes between screens, one per
+// blockIdx.y), and its polar form when pol is given.
 template <typename T>
 __global__ void k_cscale(const typename C2<T>::type* __restrict__ c,
                          const typename C2<T>::type* __restrict__ f,
@@ -1552,9 +1552,10 @@ __global__ void k_cscale(const typename C2<T>::type* __restrict__ c,
                          typename C2<T>::type* __restrict__ pol, int M) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= M) return;
-  const typename C2<T>::type v = cmul<T>(c[i], f[i]);
-  out[i] = v;
-  if (pol) pol[i] = polar_turns<T>(v);
+  const long long o = (long long)blockIdx.y * M + i;
+  const typename C2<T>::type v = cmul<T>(c[i], f[o]);
+  if (out) out[o] = v;
+  if (pol) pol[o] = polar_turns<T>(v);
 }
 
 // w_{N2}^{idx} from the table of w_N (w_{N2} = w_N^{N1}).

@@ -121,6 +121,11 @@ struct ResumArgs {
   unsigned* status;
 };
 
+// Elements from one inner plane's arrays to the next one's.
+struct PlaneStrides {
+  long long rays, jlo, modes, part;
+};
+
 template <typename T>
 struct ReduceArgs {
   const typename C2<T>::type* part;  // [n_part][N]
@@ -207,11 +212,23 @@ template <typename T> cudaError_t launch_bracket(const BracketArgs<T>& a, cudaSt
 template <typename T> cudaError_t launch_resum(const ResumArgs<T>& a, cudaStream_t s);
 template <typename T> cudaError_t launch_output(const typename C2<T>::type* u, int offset, int n,
                                                 double* out, cudaStream_t s);
+// n planes: f, out and pol hold M values per plane; out may be NULL
 template <typename T> cudaError_t launch_cscale(const typename C2<T>::type* c,
                                                 const typename C2<T>::type* f,
                                                 typename C2<T>::type* out,
-                                                typename C2<T>::type* pol, int M,
+                                                typename C2<T>::type* pol, int M, int n,
                                                 cudaStream_t s);
+// k_bracket, k_resum, and k_reduce with k_output (no absorber; u is not written) of
+// n inner planes in one launch each; a holds the first plane's arrays
+template <typename T> cudaError_t launch_bracket_planes(const BracketArgs<T>& a,
+                                                        const PlaneStrides& ps, int n,
+                                                        cudaStream_t s);
+template <typename T> cudaError_t launch_resum_planes(const ResumArgs<T>& a,
+                                                      const PlaneStrides& ps, int n,
+                                                      cudaStream_t s);
+template <typename T> cudaError_t launch_output_planes(const ReduceArgs<T>& a,
+                                                       const PlaneStrides& ps, int offset, int n_z,
+                                                       int n, double* out, cudaStream_t s);
 template <typename T> size_t resum_smem_bytes(int wcap, int tile_points);
 // Raise the dynamic shared-memory limit of the resummation kernels
 // on the current device (call once per device before launching).

@@ -117,9 +117,14 @@ struct swkb_plan {
   void* rd = nullptr;
   void* rph = nullptr;
   void* ra = nullptr;
-  // fields between screens: ray data of planes - 1 inner planes, the mode
-  // coefficients of one plane, its range-phase factors
+  // fields between screens: ray data of planes - 1 inner planes, their range-phase
+  // factors; mode coefficients, brackets and partials of pl_batch planes at a time
+  // (with one plane at a time the screen's brackets and partials serve)
   int planes = 0;
+  int pl_batch = 1;
+  int* pl_jlo = nullptr;
+  int* pl_jneg = nullptr;
+  void* pl_part = nullptr;
   void* pl_d = nullptr;
   void* pl_ph = nullptr;
   void* pl_a = nullptr;
@@ -636,7 +641,7 @@ swkb_status build_device(swkb_plan* p, const swkb_profile* prof) {
     TRY(dev_alloc(p, &p->pl_ph, pr * sizeof(T)));
     TRY(dev_alloc(p, &p->pl_a, pr * sizeof(T)));
     TRY(dev_alloc(p, &p->c_plane, (size_t)M * sizeof(V)));
-    TRY(dev_alloc(p, &p->cpol_plane, (size_t)M * sizeof(V)));
+    TRY(dev_alloc(p, &p->cpol_plane, (size_t)p->pl_batch * M * sizeof(V)));
     TRY(dev_alloc(p, &p->ephi_pl, (size_t)(p->planes - 1) * M * sizeof(V)));
   }
   const size_t jn = (size_t)(p->alloc_tiles + 1) * p->Mr;
@@ -645,6 +650,16 @@ swkb_status build_device(swkb_plan* p, const swkb_profile* prof) {
   if (p->sym) {
     TRY(dev_alloc(p, (void**)&p->jlo_neg, jn * sizeof(int)));
     CK(cudaMemsetAsync(p->jlo_neg, 0, jn * sizeof(int), p->stream));
+  }
+  if (p->pl_batch > 1) {
+    const size_t n = (size_t)p->pl_batch;
+    TRY(dev_alloc(p, &p->pl_part, n * p->alloc_groups * N * sizeof(V)));
+    TRY(dev_alloc(p, (void**)&p->pl_jlo, n * jn * sizeof(int)));
+    CK(cudaMemsetAsync(p->pl_jlo, 0, n * jn * sizeof(int), p->stream));
+    if (p->sym) {
+      TRY(dev_alloc(p, (void**)&p->pl_jneg, n * jn * sizeof(int)));
+      CK(cudaMemsetAsync(p->pl_jneg, 0, n * jn * sizeof(int), p->stream));
+    }
   }
   if (p->overlap) {
     TRY(dev_alloc(p, &p->rd1, rays * sizeof(T)));
@@ -1210,20 +1225,41 @@ swkb_status enqueue_planes(swkb_plan* p, const double* u0, int q0, int n, int P,
     }
     const bool multi = p->n_cols > 1;
     TRY(timed(p, SWKB_KERNEL_MARCH, 1, [&] { return launch_march<T>(ma, multi, s); }));
-    for (int j = 1; j < P; ++j) {
+    for (int j = 1; j < P; j += p->pl_batch) {   // pl_batch inner planes at once
+      const int n_pl = std::min(p->pl_batch, P - j);
       const size_t o = (size_t)(j - 1) * rays;
-      const BracketArgs<T> b = bracket_args<T>(p, (const T*)p->pl_d + o);
-      TRY(timed(p, SWKB_KERNEL_BRACKET, 1, [&] { return launch_bracket<T>(b, s); }));
+      const bool own = p->pl_batch > 1;
+      const PlaneStrides ps{(long long)rays, (long long)(p->alloc_tiles + 1) * p->Mr,
+                            (long long)p->M, (long long)p->alloc_groups * p->N};
+      const BracketArgs<T> b = own ? bracket_args<T>(p, (const T*)p->pl_d + o, p->pl_jlo, p->pl_jneg)
+                                   : bracket_args<T>(p, (const T*)p->pl_d + o);
+      TRY(timed(p, SWKB_KERNEL_BRACKET, 1,
+                [&] { return launch_bracket_planes<T>(b, ps, n_pl, s); }));
       // c_n of plane j: the screen's c_n (carried over dx) times exp(i k (j/P - 1) dx P_bar_n)
       const V* fj = (const V*)p->ephi_pl + (size_t)(j - 1) * p->M;
       TRY(timed(p, SWKB_KERNEL_REDUCE, 1, [&] {
-        return launch_cscale<T>((const V*)p->c, fj, (V*)p->c_plane, (V*)p->cpol_plane, p->M, s);
+        return launch_cscale<T>((const V*)p->c, fj, (V*)nullptr, (V*)p->cpol_plane, p->M, n_pl, s);
       }));
-      const ResumArgs<T> ra = resum_args<T>(p, (const T*)p->pl_d + o, (const T*)p->pl_ph + o,
-                                            (const T*)p->pl_a + o, (const V*)p->c_plane);
-      TRY(timed(p, SWKB_KERNEL_RESUM, 1, [&] { return launch_resum<T>(ra, s); }));
-      TRY(reduce(nullptr));
-      TRY(emit());
+      ResumArgs<T> ra = resum_args<T>(p, (const T*)p->pl_d + o, (const T*)p->pl_ph + o,
+                                      (const T*)p->pl_a + o, (const V*)p->c_plane, b.jlo,
+                                      b.jlo_neg);
+      if (own) ra.part = (V*)p->pl_part;
+      TRY(timed(p, SWKB_KERNEL_RESUM, 1,
+                [&] { return launch_resum_planes<T>(ra, ps, n_pl, s); }));
+      // staged rows go to the host one by one
+      const int at_once = out_dev ? n_pl : 1;
+      for (int l = 0; l < n_pl; l += at_once) {
+        const ReduceArgs<T> r{ra.part + l * ps.part, p->n_groups, p->N, nullptr, p->mirror, p->sym,
+                              nullptr};
+        double* dst = out_dev ? out_dev + 2 * (size_t)row * p->n_z : p->io;
+        TRY(timed(p, SWKB_KERNEL_OUTPUT, 1, [&] {
+          return launch_output_planes<T>(r, ps, off, p->n_z, at_once, dst, s);
+        }));
+        if (!out_dev)
+          CK(cudaMemcpyAsync(out_host + 2 * (size_t)row * p->n_z, p->io, nb,
+                             cudaMemcpyDeviceToHost, s));
+        row += at_once;
+      }
     }
     const BracketArgs<T> b = bracket_args<T>(p, (const T*)p->rd);
     TRY(timed(p, SWKB_KERNEL_BRACKET, 1, [&] { return launch_bracket<T>(b, s); }));
@@ -1537,6 +1573,13 @@ void apply_tiling(swkb_plan* p, const Tiling& t) {
   p->log2N2 = ilog2(p->N2);
 }
 
+// Brackets and partials of one inner plane taken together with others.
+size_t plane_bytes(const swkb_plan* p) {
+  const size_t V = p->precision == SWKB_FP64 ? 16 : 8;
+  return (size_t)p->alloc_groups * p->N * V +
+         (size_t)(p->alloc_tiles + 1) * p->Mr * sizeof(int) * (p->sym ? 2 : 1);
+}
+
 // Validate the arguments and derive every size of the plan (host only).
 swkb_status configure(swkb_plan* p, const swkb_profile* prof, double k, const swkb_domain* dom,
                       int32_t n_z, double screen_dx, const swkb_options& opt) {
@@ -1722,6 +1765,11 @@ swkb_status configure(swkb_plan* p, const swkb_profile* prof, double k, const sw
     }
     apply_tiling(p, def);
   }
+  if (p->planes > 1 && !p->fc) {
+    // inner planes at once: their extra arrays stay within 256 MB
+    const size_t one = plane_bytes(p);
+    p->pl_batch = (int)std::max<size_t>(1, std::min<size_t>(p->planes - 1, (256u << 20) / one));
+  }
   return SWKB_OK;
 }
 
@@ -1740,7 +1788,8 @@ size_t device_bytes(const swkb_plan* p) {
   b += 3 * (size_t)p->NRT * p->Mr * T * (p->overlap ? 2 : 1);     // rays (one or two sets)
   if (p->planes > 1)                                                 // inner planes
     b += (size_t)(p->planes - 1) * (3 * (size_t)p->NRT * p->Mr * T + (size_t)p->M * V) +
-         (size_t)p->M * V * 2;
+         (size_t)p->M * V * (1 + (size_t)p->pl_batch) +
+         (p->pl_batch > 1 ? p->pl_batch * plane_bytes(p) : 0);
   b += (size_t)(p->alloc_tiles + 1) * p->Mr * sizeof(int) * (p->sym ? 2 : 1) *
        (p->overlap ? 2 : 1);
   b += 16 + 2 * (size_t)std::max(p->N, p->n_z) * sizeof(double);   // status, io
