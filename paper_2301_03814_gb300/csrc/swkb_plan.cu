@@ -165,7 +165,9 @@ struct swkb_plan {
   // stream, and per set an event "rays ready" and "set free again"
   bool overlap = false;
   cudaStream_t ray_stream = nullptr;
+  cudaStream_t bracket_stream = nullptr;
   cudaEvent_t ev_rays[2] = {nullptr, nullptr};
+  cudaEvent_t ev_brackets[2] = {nullptr, nullptr};
   cudaEvent_t ev_free[2] = {nullptr, nullptr};
   void* rd1 = nullptr;
   void* rph1 = nullptr;
@@ -991,13 +993,13 @@ swkb_status enqueue(swkb_plan* p, const double* u0, int q0, int n, double* out_d
 }
 
 // One screen of the overlapped sequence: rays of screen q into ray-buffer set
-// b on ray_stream, modes of the field on the plan stream, then brackets and
-// sum once the rays are there.  ev_free[b] must have been recorded (set free).
+// b on ray_stream, their brackets on bracket_stream, modes of the field on the plan
+// stream, then the sum once the brackets are there.  ev_free[b] must have been recorded (set free).
 template <typename T>
 swkb_status overlapped_screen(swkb_plan* p, int q, int b, bool fresh) {
   Range range("swkb_screen");
   using V = typename C2<T>::type;
-  cudaStream_t s = p->stream, sr = p->ray_stream;
+  cudaStream_t s = p->stream, sr = p->ray_stream, sb = p->bracket_stream;
   T* rd[2] = {(T*)p->rd, (T*)p->rd1};
   T* rph[2] = {(T*)p->rph, (T*)p->rph1};
   T* ra[2] = {(T*)p->ra, (T*)p->ra1};
@@ -1010,6 +1012,11 @@ swkb_status overlapped_screen(swkb_plan* p, int q, int b, bool fresh) {
   ma.out_d = rd[b]; ma.out_ph = rph[b]; ma.out_a = ra[b];
   TRY(timed_on(p, sr, SWKB_KERNEL_MARCH, 1, [&] { return launch_march<T>(ma, multi, sr); }));
   CK(cudaEventRecord(p->ev_rays[b], sr));
+  // their brackets, which do not wait for the field either
+  CK(cudaStreamWaitEvent(sb, p->ev_rays[b], 0));
+  const BracketArgs<T> br = bracket_args<T>(p, rd[b], jlo[b], jneg[b]);
+  TRY(timed_on(p, sb, SWKB_KERNEL_BRACKET, 1, [&] { return launch_bracket<T>(br, sb); }));
+  CK(cudaEventRecord(p->ev_brackets[b], sb));
   if (p->fc) {
     if (!fresh) {
       ReduceArgs<T> r{(const V*)p->part, p->n_groups, p->N, nullptr, 0, 0, (V*)p->u};
@@ -1017,9 +1024,7 @@ swkb_status overlapped_screen(swkb_plan* p, int q, int b, bool fresh) {
     }
     const FcModesArgs<T> fm = fc_modes_args<T>(p);
     TRY(timed(p, SWKB_KERNEL_FFT, 1, [&] { return launch_fc_modes<T>(fm, s); }));
-    CK(cudaStreamWaitEvent(s, p->ev_rays[b], 0));
-    const BracketArgs<T> br = bracket_args<T>(p, rd[b], jlo[b], jneg[b]);
-    TRY(timed(p, SWKB_KERNEL_BRACKET, 1, [&] { return launch_bracket<T>(br, s); }));
+    CK(cudaStreamWaitEvent(s, p->ev_brackets[b], 0));
     const FcResumArgs<T> rs = fc_resum_args<T>(p, rd[b], rph[b], ra[b], jlo[b]);
     TRY(timed(p, SWKB_KERNEL_RESUM, 1, [&] { return launch_fc_resum<T>(rs, s); }));
     CK(cudaEventRecord(p->ev_free[b], s));
@@ -1044,11 +1049,9 @@ swkb_status overlapped_screen(swkb_plan* p, int q, int b, bool fresh) {
   f.inv_N = (T)(1.0 / p->N);
   f.ephi = (const V*)p->ephi_d; f.c = (V*)p->c; f.cpol = (V*)p->cpol;
   TRY(timed(p, SWKB_KERNEL_FFT, p->N1 > 1 ? 2 : 1, [&] { return launch_fft<T>(f, s); }));
-  // brackets and sum of screen q, once its rays are there (the ray stream
-  // goes on with the next march)
-  CK(cudaStreamWaitEvent(s, p->ev_rays[b], 0));
-  const BracketArgs<T> br = bracket_args<T>(p, rd[b], jlo[b], jneg[b]);
-  TRY(timed(p, SWKB_KERNEL_BRACKET, 1, [&] { return launch_bracket<T>(br, s); }));
+  // sum of screen q, once its rays and brackets are there (the ray stream goes
+  // on with the next march)
+  CK(cudaStreamWaitEvent(s, p->ev_brackets[b], 0));
   const ResumArgs<T> rs = resum_args<T>(p, rd[b], rph[b], ra[b], (const V*)p->c, jlo[b],
                                         jneg[b]);
   TRY(timed(p, SWKB_KERNEL_RESUM, 1, [&] { return launch_resum<T>(rs, s); }));
@@ -1057,13 +1060,15 @@ swkb_status overlapped_screen(swkb_plan* p, int q, int b, bool fresh) {
   return SWKB_OK;
 }
 
-// enqueue() with the rays on a second stream.  A screen's rays depend only on
-// the medium and the mode angles, never on the field, so the march of screen
-// q (into ray-buffer set (q - q0) % 2, on ray_stream) runs beside the DFT of
-// screen q and the bracket and resummation of screen q - 1 on the plan stream.
-// The bracket of screen q waits for its set's "rays" event; the march of
-// screen q + 2 waits for the "free" event recorded after the resummation of
-// screen q, the last reader of that set.  Same kernels and
+// enqueue() with the rays on a second stream and their brackets on a third.  A
+// screen's rays depend only on the medium and the mode angles, never on the field,
+// so the march of screen q (into ray-buffer set (q - q0) % 2, on ray_stream) and its
+// brackets run beside the DFT of screen q and the resummation of screen q - 1 on the
+// plan stream.  The bracket of screen q waits for its set's "rays" event, the
+// resummation for its "brackets"; the march of screen q + 2 waits for the "free"
+// event recorded after the resummation of screen q, the last reader of that set.
+// (Brackets on the plan stream: open lens of 131072 points 2860 us for 4 screens, now
+// 2748; 131072-point duct 3520 / 3474 for 6; 4096 points 274 / 267 for 12.)  Same kernels and
 // arguments as enqueue(): the fields are bit-identical.
 template <typename T>
 swkb_status enqueue_overlapped(swkb_plan* p, const double* u0, int q0, int n, double* out_dev,
@@ -1436,14 +1441,17 @@ void release(swkb_plan* p) {
   // a sequence that failed between a march and the wait that joins it may
   // leave work on the ray stream: finish it before its buffers go
   if (p->ray_stream) cudaStreamSynchronize(p->ray_stream);
+  if (p->bracket_stream) cudaStreamSynchronize(p->bracket_stream);
   drop_graphs(p);
   for (void* ptr : p->allocs) cudaFree(ptr);
   for (cudaEvent_t e : p->events) cudaEventDestroy(e);
   for (int b = 0; b < 2; ++b) {
     if (p->ev_rays[b]) cudaEventDestroy(p->ev_rays[b]);
+    if (p->ev_brackets[b]) cudaEventDestroy(p->ev_brackets[b]);
     if (p->ev_free[b]) cudaEventDestroy(p->ev_free[b]);
   }
   if (p->ray_stream) cudaStreamDestroy(p->ray_stream);
+  if (p->bracket_stream) cudaStreamDestroy(p->bracket_stream);
   if (p->own_stream && p->stream) cudaStreamDestroy(p->stream);
   cudaSetDevice(cur);
   delete p;
@@ -2056,8 +2064,10 @@ swkb_status swkb_plan_create(const swkb_profile* prof, double k, const swkb_doma
     }
     if (p->overlap) {
       CK(cudaStreamCreateWithFlags(&p->ray_stream, cudaStreamNonBlocking));
+      CK(cudaStreamCreateWithFlags(&p->bracket_stream, cudaStreamNonBlocking));
       for (int b = 0; b < 2; ++b) {
         CK(cudaEventCreateWithFlags(&p->ev_rays[b], cudaEventDisableTiming));
+        CK(cudaEventCreateWithFlags(&p->ev_brackets[b], cudaEventDisableTiming));
         CK(cudaEventCreateWithFlags(&p->ev_free[b], cudaEventDisableTiming));
       }
     }
