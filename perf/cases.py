@@ -365,7 +365,7 @@ class _Table:
             sign = torch.where(z < self.ground, -1.0, 1.0)
             z = self.ground + (z - self.ground).abs()
         u = (z - self.z0) / self.h
-        i = u.floor().nan_to_num(0.0).clamp(0, self.c.shape[1] - 1)      # a ray gone NaN reads in bounds
+        i = u.floor().clamp(0, self.c.shape[1] - 1)
         t = u - i
         i = i.long()
         e = ez = ezz = 0.0
@@ -430,7 +430,6 @@ def _mode_sum(n, amp, shift, excess, a, k, dz, G, R, period, points, chunk=24):
         land = launch + shift[i:i + chunk] / dz
         rows = land.shape[0]
         j = torch.searchsorted(land, x.expand(rows, -1).contiguous(), right=True) - 1
-        j = j.clamp(1, land.shape[1] - 3)        # a screen its rays do not cover (an error of run) reads in bounds
         X = [land.gather(1, j + o) for o in (-1, 0, 1, 2)]
         wgt = []
         for p in range(4):
