@@ -239,9 +239,9 @@ __device__ __forceinline__ void march64_body(const MarchArgs<double>& p, int blk
   if (!(P0sq > 0.0)) { st |= ST_TURNING; P0sq = pb2; }
   const double P0 = sqrt(P0sq);
   Ray y{0.0, 0.0, 0.0, -1.0, 0.0};
-  const double H = 0.5 * p.med.inv_h * p.h;
-  const double H2 = 0.5 * H, H6 = H / 6.0, H3 = H / 3.0, W1 = 2.0 * H, W3 = 2.0 * H3;
-  const double h6 = p.h / 6.0, h3 = p.h / 3.0;
+  const double H2 = p.s2, H = 2.0 * H2, W1 = 2.0 * H;
+  const double H6 = p.s6, H3 = 2.0 * H6, W3 = 2.0 * H3;
+  const double h6 = p.h6, h3 = 2.0 * h6;
   int P2_lo = 0x7fefffff, N_hi = (int)0x80000000;
   // landing quantities at RK4 stage l (the screen's end, or a plane inside it)
   auto land = [&](int l, double* od, double* oph, double* oa) {
@@ -252,8 +252,8 @@ __device__ __forceinline__ void march64_body(const MarchArgs<double>& p, int blk
     double P1sq = pb2 + e1 - y.dQ * (2.0 * kap + y.dQ);
     if (!(P1sq > 0.0)) { st |= ST_TURNING; P1sq = pb2; }
     const double Zs = y.N < 0.0 ? -y.N : 1.0;
-    od[o] = y.w * (p.inv_dz / p.med.inv_h);
-    oph[o] = y.rh * p.k_over_2pi;
+    od[o] = y.w * p.w_out;
+    oph[o] = y.rh * p.ph_out;
     oa[o] = sqrt(P0 * rsqrt(P1sq) / Zs);
   };
   // RK4 accumulated as the stages complete; a stage state needs no rh, and its
@@ -527,13 +527,13 @@ __device__ __forceinline__ void march_x2_body(const MarchArgs<float>& p, int blk
   P0a = sqrtf(P0a);
   P0b = sqrtf(P0b);
   Ray2 y{zero, zero, zero, bc2(-1.f), zero};
-  const float c = 0.5f * p.med.inv_h, H = c * p.h;
   // RK4 weights 1/2, 1, 1/6, 1/3 times the factors of the scaled system
-  const f2 H2 = bc2(0.5f * H), H1 = bc2(H), H6 = bc2(H / 6.f), H3 = bc2(H / 3.f);
-  const f2 W1 = bc2(2.f * H), W3 = bc2(2.f * H / 3.f);          // w: H1, W1, H3, W3
-  const f2 n2 = bc2(-0.5f * H), n1 = bc2(-H), n6 = bc2(-H / 6.f), n3 = bc2(-H / 3.f);
-  const f2 h6 = bc2(p.h / 6.f), h3 = bc2(p.h / 3.f);
-  const float w_out = p.inv_dz / p.med.inv_h;
+  const float s2 = p.s2, s6 = p.s6;
+  const f2 H2 = bc2(s2), H1 = bc2(2.f * s2), H6 = bc2(s6), H3 = bc2(2.f * s6);
+  const f2 W1 = bc2(4.f * s2), W3 = bc2(4.f * s6);              // w: H1, W1, H3, W3
+  const f2 n2 = bc2(-s2), n1 = bc2(-2.f * s2), n6 = bc2(-s6), n3 = bc2(-2.f * s6);
+  const f2 h6 = bc2(p.h6), h3 = bc2(2.f * p.h6);
+  const float w_out = p.w_out;
   // landing quantities at RK4 stage l (the screen's end, or a plane inside it)
   const auto land = [&](int l, float* od, float* oph, float* oam) {
     const long long nrm = (long long)p.NRT * p.Mr;
@@ -558,11 +558,11 @@ __device__ __forceinline__ void march_x2_body(const MarchArgs<float>& p, int blk
     if (!(P1b > 0.f)) { st |= ST_TURNING; P1b = pb2; }
     const float Za = Na < 0.f ? -Na : 1.f, Zb = Nb < 0.f ? -Nb : 1.f;
     od[oa] = wa * w_out;
-    oph[oa] = rha * p.k_over_2pi;
+    oph[oa] = rha * p.ph_out;
     oam[oa] = sqrtf(P0a * rsqrtf(P1a) / Za);
     if (has_b) {
       od[ob] = wb * w_out;
-      oph[ob] = rhb * p.k_over_2pi;
+      oph[ob] = rhb * p.ph_out;
       oam[ob] = sqrtf(P0b * rsqrtf(P1b) / Zb);
     }
   };

@@ -45,7 +45,7 @@ template <> struct C2<double> { using type = double2; };
 //   before that pad and top = n_int as a float.  When pieces = S > 0 every
 //   interval is stored as S cubic Hermite pieces of its quintic (value and
 //   slope matched at the piece ends; 4 slots b0..b3 in the piece's own
-//   tau in [0, 1]) and n_int, top, inv_h count pieces.
+//   tau in [0, 1]) and n_int, top count pieces.
 // With several columns every entry is followed by its difference to the next
 // column's entry (twice the slots), and the last column has no rows of its own.
 template <typename T>
@@ -53,7 +53,6 @@ struct Medium {
   const T* coef;
   int n_int;
   long long col_stride;
-  T inv_h;
   int mirrored;
   T top;
   int pieces;   // FP32: > 0 when each entry is a cubic piece (4 slots), in piece units
@@ -78,7 +77,11 @@ struct MarchArgs {
   int Mr;           // marched modes (row length of the outputs)
   int mode_off;     // marched mode r is mode index r + mode_off (n = r + mode_off - n_max)
   int NRT, G, R, Nt;
-  T inv_dz, h, k_over_2pi;
+  // RK4 constants, formed on the host so that each is rounded once (H = h / (2 h_table),
+  // h the step): stage weight H / 2, sum weights H / 6 and h / 6 (the kernels use
+  // these times 2 and 4, exact); w_out and ph_out carry the displacement to grid units
+  // and the phase to turns, for the weights as rounded
+  T s2, s6, h6, w_out, ph_out;
   T u_lo, u_dz;     // table position of grid point 0 and per grid point
   T* out_d;         // [NRT][Mr] landing offset from the launch grid point, grid units
   T* out_ph;        // [NRT][Mr] residual phase k (r - x P_bar) / (2 pi), turns

@@ -761,7 +761,6 @@ MarchArgs<T> march_args(const swkb_plan* p, int q) {
     a.med.mirrored = 0;
   }
   a.med.col_stride = table_values(p);
-  a.med.inv_h = (T)(1.0 / hs);
   a.med.top = (T)a.med.n_int;
   a.med.size = (long long)table_columns(p) * a.med.col_stride;
   a.u_lo = (T)((p->z_lo - z0) / hs);
@@ -775,9 +774,13 @@ MarchArgs<T> march_args(const swkb_plan* p, int q) {
   a.pbar2 = (const T*)p->pbar2_d;
   a.Mr = p->Mr; a.mode_off = p->sym ? p->n_max : 0;
   a.NRT = p->NRT; a.G = p->G; a.R = p->R; a.Nt = p->Nt;
-  a.inv_dz = (T)(1.0 / p->dz);
-  a.h = (T)(p->dx / p->Nt);
-  a.k_over_2pi = (T)(p->k / (2.0 * M_PI));
+  // in long double: an FP64 plan's constants are rounded once too
+  const long double h = (long double)p->dx / p->Nt, H = h / (2.0L * hs);
+  a.s2 = (T)(H / 2.0L);
+  a.s6 = (T)(H / 6.0L);
+  a.h6 = (T)(h / 6.0L);
+  a.w_out = (T)(h / ((long double)p->dz * 12.0L * a.s6));   // a step's weights of w: 12 s6
+  a.ph_out = (T)((long double)p->k * h / (2.0L * acosl(-1.0L) * 6.0L * a.h6));   // of rh: 6 h6
   a.out_d = (T*)p->rd; a.out_ph = (T*)p->rph; a.out_a = (T*)p->ra;
   a.plane_steps = 0;
   a.pl_d = a.pl_ph = a.pl_a = nullptr;
