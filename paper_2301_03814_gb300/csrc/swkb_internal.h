@@ -79,7 +79,7 @@ struct MarchArgs {
   int NRT, G, R, Nt;
   // RK4 constants, formed on the host so that each is rounded once (H = h / (2 h_table),
   // h the step): stage weight H / 2, sum weights H / 6 and h / 6 (the kernels use
-  // these times 2 and 4, exact); w_out and ph_out carry the displacement to grid units
+  // these times 2 or 4, exact); w_out and ph_out carry the displacement to grid units
   // and the phase to turns, for the weights as rounded
   T s2, s6, h6, w_out, ph_out;
   T u_lo, u_dz;     // table position of grid point 0 and per grid point
