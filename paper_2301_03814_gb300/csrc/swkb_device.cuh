@@ -1027,15 +1027,18 @@ __device__ __forceinline__ void resum_body(const ResumArgs<float>& p, int blk, i
 }
 
 // ---- FP64 ----
-// sin / cos of 2 pi t: t = k / TRIG_N + r with |r| <= 1 / (2 TRIG_N); the
-// table's entry exp(2 pi i k / TRIG_N) (correctly rounded on the host) rotated by
-// the angle 2 pi r <= pi / 1024, whose sine and cosine - 1 need two and three
-// Taylor terms (the next ones are below 2e-18).  13 FP64 operations, absolute
-// error about one unit in the last place of 1; any |t| < 2^41.
-__device__ __forceinline__ void sincos_table(const double2* trig, double t, double* s, double* c) {
+// sin / cos of 2 pi (a + b), a + b = k / TRIG_N + r with |r| <= 1 / (2 TRIG_N):
+// the table's entry exp(2 pi i k / TRIG_N) rotated by the angle 2 pi r <= pi / 1024,
+// whose sine and cosine - 1 need two and three Taylor terms (the next ones are
+// below 2e-18).  a is a multiple of a small fraction of a turn (n m / N), so a - k /
+// TRIG_N is exact and r takes no rounding of the size of a + b, only b's own.  14 FP64
+// operations, absolute error about one unit in the last place of 1, small sines to
+// a few units of their own; any |a + b| < 2^41.
+__device__ __forceinline__ void sincos_table(const double2* trig, double a, double b, double* s,
+                                             double* c) {
   const double magic = 6755399441055744.0;   // 1.5 * 2^52: rounds to an integer
-  const double v = fma(t, (double)TRIG_N, magic);
-  const double r = fma(v - magic, -1.0 / TRIG_N, t);
+  const double v = fma(a + b, (double)TRIG_N, magic);
+  const double r = fma(v - magic, -1.0 / TRIG_N, a) + b;
   const double2 e = __ldg(trig + (__double2loint(v) & (TRIG_N - 1)));
   const double r2 = r * r;
   const double sr = r * fma(r2, fma(r2, 81.60524927607503, -41.34170224039975), 6.283185307179586);
@@ -1055,7 +1058,7 @@ __device__ __forceinline__ Row64 load_row64(const double* p) {
 }
 
 // As the FP32 block; bound by the FP64 pipe, so reciprocals take 3 FP64
-// operations (rcp64), a term 24, and a run's next interval is found by integer
+// operations (rcp64), a term 25, and a run's next interval is found by integer
 // comparisons.
 template <int PW, int LD, int BAR>
 __device__ __forceinline__ void resum_body(const ResumArgs<double>& p, int blk, int tid,
@@ -1211,7 +1214,7 @@ __device__ __forceinline__ void resum_body(const ResumArgs<double>& p, int blk, 
         const double phv = ((r.b3 * tau + r.b2) * tau + r.b1) * tau + r.b0;
         const double av = ((r.a3 * tau + r.a2) * tau + r.a1) * tau + r.a0;
         double sn, cs;
-        sincos_table(p.trig, fma((double)(q - PW / 2), nN, bc) + phv, &sn, &cs);
+        sincos_table(p.trig, fma((double)(q - PW / 2), nN, bc), phv, &sn, &cs);
         accr[q] = fma(av, cs, accr[q]);
         acci[q] = fma(av, sn, acci[q]);
       };
@@ -1248,7 +1251,7 @@ __device__ __forceinline__ void resum_body(const ResumArgs<double>& p, int blk, 
 // registers: keeps the one-mode-ahead window), 5 for runs of 16 points (213 us;
 // 230 at 72 registers).  FP64, bound by its pipe: 1.05 ms on the 16384-point
 // duct with 29 mode groups (1.78 with sincospi, library divisions and a complex
-// coefficient per term; 24 FP64 operations per term instead of ~46).
+// coefficient per term; 25 FP64 operations per term instead of ~46).
 template <typename T, int PW>
 __global__ void __launch_bounds__(RESUM_WARPS * 32, sizeof(T) == 4 ? (PW < 16 ? 7 : 5) : 1)
     k_resum(const ResumArgs<T> p) {

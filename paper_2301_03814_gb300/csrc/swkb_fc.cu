@@ -318,7 +318,7 @@ __device__ __forceinline__ void add_term(const FcRow<double>& r, const double2* 
   const double ar = ((r.r3 * tau + r.r2) * tau + r.r1) * tau + r.r0;
   const double ai = ((r.i3 * tau + r.i2) * tau + r.i1) * tau + r.i0;
   double sn, cs;
-  sincos_table(trig, t + (((r.b3 * tau + r.b2) * tau + r.b1) * tau + r.b0), &sn, &cs);
+  sincos_table(trig, t, ((r.b3 * tau + r.b2) * tau + r.b1) * tau + r.b0, &sn, &cs);
   sr += fma(ar, cs, -ai * sn);
   si += fma(ar, sn, ai * cs);
 }

@@ -3,7 +3,11 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
+
+#include <utility>
+#include <vector>
 
 #include "swkb.h"
 
@@ -20,6 +24,22 @@ enum : unsigned {
 
 // Entries of the FP64 sums' table of exp(2 pi i k / TRIG_N) (a power of two).
 constexpr int TRIG_N = 1024;
+
+// That table as (cos, sin) pairs, from long double; the quadrants' entries are exact.
+inline std::vector<double> trig_table() {
+  std::vector<double> e(2 * TRIG_N);
+  const long double turn = 2.0L * acosl(-1.0L);
+  for (int k = 0; k < TRIG_N; ++k) {
+    const int o = k / (TRIG_N / 8), m = k % (TRIG_N / 4);   // eighths of a turn by symmetry
+    const long double a = turn * (m <= TRIG_N / 8 ? m : TRIG_N / 4 - m) / TRIG_N;
+    double c = (double)cosl(a), s = (double)sinl(a);
+    if (m > TRIG_N / 8) std::swap(c, s);
+    const int quad = o / 2;
+    e[2 * k] = quad == 0 ? c : (quad == 1 ? -s : (quad == 2 ? -c : s));
+    e[2 * k + 1] = quad == 0 ? s : (quad == 1 ? c : (quad == 2 ? -s : -c));
+  }
+  return e;
+}
 
 // Columns n2 of the DFT's pass 1 handled by one block.
 constexpr int FFT1_COLS = 8;

@@ -599,20 +599,7 @@ swkb_status build_device(swkb_plan* p, const swkb_profile* prof) {
     }
     TRY(upload<T>(p, &p->tw, tw));
   }
-  if (sizeof(T) == 8) {
-    std::vector<double> e(2 * TRIG_N);
-    for (int k = 0; k < TRIG_N; ++k) {
-      // eighths of a turn by symmetry, so that the quadrants' entries are exact
-      const int o = k / (TRIG_N / 8), m = k % (TRIG_N / 4);
-      const double a = 2.0 * M_PI / TRIG_N * (m <= TRIG_N / 8 ? m : TRIG_N / 4 - m);
-      double c = cos(a), s = sin(a);
-      if (m > TRIG_N / 8) std::swap(c, s);
-      const int quad = o / 2;
-      e[2 * k] = quad == 0 ? c : (quad == 1 ? -s : (quad == 2 ? -c : s));
-      e[2 * k + 1] = quad == 0 ? s : (quad == 1 ? c : (quad == 2 ? -s : -c));
-    }
-    TRY(upload<double>(p, &p->trig, e));
-  }
+  if (sizeof(T) == 8) TRY(upload<double>(p, &p->trig, trig_table()));
   // absorber
   if (p->absorber_frac > 0) {
     std::vector<double> w(N, 1.0);
