@@ -314,28 +314,25 @@ void cubic_piece(const double* a, int s, int S, double* b) {
   b[3] = 2.0 * (f0 - f1) + d0 + d1;
 }
 
-// The smallest curvature deviation an FP32 march can tell: over one screen a
-// deviation d of eps_zz moves Z_s by at most d dx^2 / (4 P^2), P^2 >= eps_ref -
-// kappa_max^2; at 2^-26 P^2 / dx^2 that is an eighth of the rounding of Z_s.
-double curvature_floor(const swkb_plan* p) {
-  const double kmax = 2.0 * M_PI * p->n_max / (p->k * p->L);
-  return ldexp(std::max(p->eps_ref - kmax * kmax, 0.0), -26) / (p->dx * p->dx);
-}
-
 // FP32 plans evaluate each interval's quintic through S cubic Hermite pieces
 // (6 FMAs per lookup instead of 12).  S is the smallest of 1, 2, 4, 8, 16 for
 // which, at the quarter points of every piece, value, slope and curvature of
 // the pieces stay within 1e-7, 1e-6 and 1e-4 of the table's largest |e|, |e_z|
 // and |e_zz| (e = eps - eps_ref): far below what the FP32 march resolves.  The
-// curvature's bound is not taken below curvature_floor: media broad against
-// the table spacing (or linear) have an e_zz of the order of the table's own
-// rounding, which no number of pieces reproduces (open lens of 131072 points,
-// spacing 1/16, width 7282: one piece instead of the quintic, 425 against 495
-// us per march).  0 when none does (the quintic itself is evaluated).
-int choose_pieces(const swkb_plan* p, const std::vector<double>& coef) {
+// curvature's bound is not taken below what the rounding of the table's eps does
+// to it: an error d in the difference of two nodes puts up to 5.6 d / h^2 into the
+// quintic's curvature at the quarter points and 3 d / h^2 into one cubic's, so with
+// d <= 2 x 2^-53 max |eps| they differ by up to 6 x 2^-53 max |eps| / h^2.  Media broad
+// against the table spacing (or linear) have an e_zz below that, and no number of
+// pieces reproduces the noise (open lens of 131072 points, spacing 1/16, width 7282:
+// one piece, at 0.87 of that bound, instead of the quintic, 425 against 495 us per
+// march).  0 when none does (the quintic itself is evaluated).
+int choose_pieces(const swkb_plan* p, const swkb_profile* prof, const std::vector<double>& coef) {
   const double h = p->dzp;
   const size_t n = (size_t)p->n_cols * p->n_int;
-  double E0 = 0, E1 = 0, E2 = 0;
+  double E0 = 0, E1 = 0, E2 = 0, eps_max = 0;
+  for (size_t i = 0; i < (size_t)p->n_cols * p->n_p; ++i)
+    eps_max = std::max(eps_max, fabs(prof->eps[i]));
   for (size_t i = 0; i < n; ++i) {
     const double* a = coef.data() + i * 8;
     for (double t : {0.0, 1.0}) {
@@ -346,7 +343,7 @@ int choose_pieces(const swkb_plan* p, const std::vector<double>& coef) {
       E2 = std::max(E2, fabs(d2) / (h * h));
     }
   }
-  const double tol[3] = {1e-7 * E0, 1e-6 * E1, std::max(1e-4 * E2, curvature_floor(p))};
+  const double tol[3] = {1e-7 * E0, 1e-6 * E1, std::max(1e-4 * E2, 6.0 * ldexp(eps_max, -53) / (h * h))};
   // largest deviations of S pieces from the quintic (value, slope, curvature);
   // with stop set, returns as soon as one exceeds its bound
   auto worst = [&](int S, double dev[3], bool stop) {
@@ -389,7 +386,7 @@ int choose_pieces(const swkb_plan* p, const std::vector<double>& coef) {
 }
 
 // choose_pieces depends only on the table (and eps_ref, the ground
-// reflection, the curvature floor): remembered by a 64-bit FNV-1a hash of those, so that the
+// reflection): remembered by a 64-bit FNV-1a hash of those, so that the
 // budget estimate and the creation of the same request's plan scan it once.
 uint64_t table_hash(const swkb_plan* p, const swkb_profile* prof) {
   uint64_t h = 1469598103934665603ull;
@@ -401,7 +398,7 @@ uint64_t table_hash(const swkb_plan* p, const swkb_profile* prof) {
   mix(prof->eps, nt * sizeof(double));
   mix(prof->eps_z, nt * sizeof(double));
   mix(prof->eps_zz, nt * sizeof(double));
-  const double sc[3] = {p->eps_ref, p->dzp, curvature_floor(p)};
+  const double sc[2] = {p->eps_ref, p->dzp};
   const int ic[3] = {p->n_cols, p->n_p, p->mirror};
   mix(sc, sizeof(sc));
   mix(ic, sizeof(ic));
@@ -418,7 +415,7 @@ int pieces_for(const swkb_plan* p, const swkb_profile* prof) {
     auto it = g_pieces_cache.find(key);
     if (it != g_pieces_cache.end()) return it->second;
   }
-  const int S = choose_pieces(p, quintic_coefficients(p, prof));
+  const int S = choose_pieces(p, prof, quintic_coefficients(p, prof));
   std::lock_guard<std::mutex> lk(g_pieces_mutex);
   if (g_pieces_cache.size() >= 256) g_pieces_cache.clear();
   g_pieces_cache[key] = S;

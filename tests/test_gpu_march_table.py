@@ -67,3 +67,12 @@ def test_pieces_and_mixed_parity(problem, pieces):
     assert plan.info.medium_pieces in pieces
     # the mixed path's bar against the FP64 path
     assert rel_l2(plan.propagate(), swkb.Plan(pb, swkb.SWKB_FP64).propagate()) < 1e-4
+
+
+@pytest.mark.parametrize("dx", [50.0, 5.0, 1.0])
+def test_pieces_follow_the_table_alone(dx):
+    # the duct's 1 m blends ask for 16 pieces however short the screens are; a linear medium's curvature
+    # is the table's rounding, for which one piece does
+    duct = w.config_surface_duct_small().with_(dx=dx)
+    assert swkb.Plan(duct, swkb.SWKB_MIXED).info.medium_pieces == 16
+    assert swkb.Plan(w.config_unit_periodic().with_(dx=20.0 * dx / 50.0), swkb.SWKB_MIXED).info.medium_pieces == 1
