@@ -323,6 +323,144 @@ __device__ __forceinline__ void add_term(const FcRow<double>& r, const double2* 
   si += fma(ar, sn, ai * cs);
 }
 
+template <typename T>
+struct FcRay {
+  T d, ph;
+  typename C2<T>::type a;
+};
+
+// ray j of mode i: landing offset, phase and the complex amplitude
+// a_j (S^{p0}(z_j) cf[p0][i] + S^{p0+1}(z_j) cf[p0+1][i])
+template <typename T>
+__device__ __forceinline__ FcRay<T> fc_ray(const FcResumArgs<T>& p, int i, int j, unsigned& st) {
+  using V = typename C2<T>::type;
+  // NRT M < 2^32 (at most 2^20 + 2 G rays of 2047 modes)
+  const unsigned o = (unsigned)bchk((long long)((unsigned)j * (unsigned)p.M + (unsigned)i),
+                                    (long long)p.NRT * p.M, st);
+  FcRay<T> v;
+  v.d = ld<LD_NC>(p.d + o);
+  v.ph = ld<LD_NC>(p.ph + o);
+  const T a = ld<LD_NC>(p.a + o);
+  const int p0 = __ldg(p.win_p + j);
+  const V sw = p.win_s[j];
+  const V c0 = p.cf[bchk((long long)p0 * p.M + i, (long long)p.P * p.M, st)];
+  T cr = sw.x * c0.x, ci = sw.x * c0.y;
+  if (p0 + 1 < p.P) {
+    const V c1 = p.cf[(long long)(p0 + 1) * p.M + i];
+    cr += sw.y * c1.x;
+    ci += sw.y * c1.y;
+  }
+  v.a.x = a * cr;
+  v.a.y = a * ci;
+  return v;
+}
+
+// Rays of the window between two brackets (0: skip).  A table left inconsistent by a
+// failed screen (flagged by the bracket kernel) must not send the reads out of
+// [0, NRT).
+template <typename T>
+__device__ __forceinline__ int fc_window(const FcResumArgs<T>& p, int jl, int jh) {
+  return jl >= 1 && jh >= jl && jh <= p.NRT - 3 ? jh - jl + 4 : 0;
+}
+
+// The warps' sums in a fixed order, written as (ADD: added to) the group's partial.
+template <typename T, int PW, bool ADD>
+__device__ __forceinline__ void fc_block_sum(const FcResumArgs<T>& p, unsigned char* smem_raw,
+                                             const T* accr, const T* acci, int tile, int group,
+                                             unsigned st) {
+  using V = typename C2<T>::type;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, TM = p.TM, m0 = tile * TM;
+  V* red = reinterpret_cast<V*>(smem_raw);
+  const int TMP = 32 * (PW + 1);
+#pragma unroll
+  for (int q = 0; q < PW; ++q) {
+    V v;
+    v.x = accr[q];
+    v.y = acci[q];
+    red[warp * TMP + lane * (PW + 1) + q] = v;
+  }
+  __syncthreads();
+  V* out = p.part + bchk((long long)group * p.N + m0, (long long)p.n_groups * p.N - (TM - 1), st);
+  if (st) atomicOr(p.status, st);
+  for (int x = threadIdx.x; x < TM; x += FC_WARPS * 32) {
+    const int xs = (x / PW) * (PW + 1) + x % PW;
+    V sum = red[xs];
+#pragma unroll
+    for (int k = 1; k < FC_WARPS; ++k) {
+      const V v = red[k * TMP + xs];
+      sum.x += v.x;
+      sum.y += v.y;
+    }
+    if (ADD) { sum.x += out[x].x; sum.y += out[x].y; }
+    out[x] = sum;
+  }
+}
+
+// The modes of a tile whose rays are compressed beyond a window (wcap rays), up to wlim
+// on the tile or its pair of tiles (lim_pair): wcap rays at a time.  A function of its
+// own: within the main loop it takes that loop's registers (235 instead of 224 us on
+// the 131072-point lens).
+template <typename T, int PW>
+__device__ __noinline__ void fc_resum_split(const FcResumArgs<T>& p, unsigned char* smem_raw,
+                                            int tile, int group) {
+  using V = typename C2<T>::type;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int wcap = p.wcap, m0 = tile * p.TM, x0 = lane * PW;
+  T* s_cf = reinterpret_cast<T*>(smem_raw + (long long)warp * fc_warp_bytes<T>(wcap));
+  V* s_a = reinterpret_cast<V*>(s_cf + FC_CF<T> * wcap);
+  T* s_X = reinterpret_cast<T*>(s_a + wcap);
+  T* s_ph = s_X + wcap;
+  const int i1 = min(p.M, (group + 1) * p.modes_per_group);
+  const unsigned Np = (unsigned)p.Np;
+  const T invNp = T(1) / T(p.Np);
+  unsigned st = 0;
+  T accr[PW], acci[PW];
+#pragma unroll
+  for (int q = 0; q < PW; ++q) { accr[q] = T(0); acci[q] = T(0); }
+  __syncthreads();   // the block's first sums are read
+  for (int i = group * p.modes_per_group + warp; i < i1; i += FC_WARPS) {
+    const auto bracket = [&](int t) {
+      return p.jlo[bchk((long long)t * p.M + i, (long long)(p.n_tiles + 1) * p.M, st)];
+    };
+    const int jb = bracket(tile) - 1, W = fc_window(p, jb + 1, bracket(tile + 1));
+    if (W <= wcap) continue;
+    if ((p.lim_pair ? fc_window(p, bracket(tile & ~1), bracket((tile | 1) + 1)) : W) > p.wlim) {
+      st |= ST_CAUSTIC;
+      continue;
+    }
+    const int base = (jb - p.G) * p.R - m0, n = i - p.n_max;
+    const unsigned nn = (unsigned)(n < 0 ? n + p.Np : n);   // phases as in k_fc_resum
+    T bc = T(mod_np(nn * (unsigned)(m0 + x0 + PW / 2), Np, p.np_magic)) * invNp;
+    bc = bc >= T(0.5) ? bc - T(1) : bc;
+    for (int w0 = 0; w0 < W - 3; w0 += wcap - 3) {
+      const int Wp = min(wcap, W - w0);
+      __syncwarp();
+      for (int s = lane; s < Wp; s += 32) {
+        const FcRay<T> v = fc_ray(p, i, jb + w0 + s, st);
+        s_X[s] = T(base + (w0 + s) * p.R) + v.d;
+        s_ph[s] = v.ph;
+        s_a[s] = v.a;
+      }
+      __syncwarp();
+      build_rows(s_cf, s_X, s_ph, s_a, Wp, lane);
+      __syncwarp();
+      int w = 1;
+#pragma unroll
+      for (int q = 0; q < PW; ++q) {   // the points of these rays' intervals
+        const T xv = T(x0 + q);
+        if ((w0 == 0 || s_X[1] <= xv) && (w0 + Wp == W || xv < s_X[Wp - 2])) {
+          while (w < Wp - 3 && s_X[w + 1] <= xv) ++w;
+          FcRow<T> r;
+          r.load(s_cf + FC_CF<T> * w);
+          add_term(r, p.trig, xv, fma(T(q - PW / 2), T(n) * invNp, bc), accr[q], acci[q]);
+        }
+      }
+    }
+  }
+  __syncthreads();
+  fc_block_sum<T, PW, true>(p, smem_raw, accr, acci, tile, group, st);
+}
+
 // One CTA: tile blk % n_tiles (TM = 32 PW points), mode group blk / n_tiles;
 // its warps take the group's modes round-robin (the structure of the periodic
 // sum: brackets of 32 modes looked up at once, the next mode's first rays loaded
@@ -357,30 +495,10 @@ __global__ void __launch_bounds__(FC_WARPS * 32, sizeof(T) == 4 ? 7 : 1)
 #pragma unroll
   for (int q = 0; q < PW; ++q) { accr[q] = T(0); acci[q] = T(0); }
 
-  // ray j of mode i: landing offset, phase and the complex amplitude
-  // a_j (S^{p0}(z_j) cf[p0][i] + S^{p0+1}(z_j) cf[p0+1][i])
-  struct RayVal { T d, ph; V a; };
-  auto fetch = [&](int i, int j) {
-    // NRT M < 2^32 (at most 2^20 + 2 G rays of 2047 modes)
-    const unsigned o = (unsigned)bchk((long long)((unsigned)j * (unsigned)p.M + (unsigned)i),
-                                      nrays, st);
-    RayVal v;
-    v.d = ld<LD_NC>(p.d + o);
-    v.ph = ld<LD_NC>(p.ph + o);
-    const T a = ld<LD_NC>(p.a + o);
-    const int p0 = __ldg(p.win_p + j);
-    const V sw = p.win_s[j];
-    const V c0 = p.cf[bchk((long long)p0 * p.M + i, (long long)p.P * p.M, st)];
-    T cr = sw.x * c0.x, ci = sw.x * c0.y;
-    if (p0 + 1 < p.P) {
-      const V c1 = p.cf[(long long)(p0 + 1) * p.M + i];
-      cr += sw.y * c1.x;
-      ci += sw.y * c1.y;
-    }
-    v.a.x = a * cr;
-    v.a.y = a * ci;
-    return v;
-  };
+  using RayVal = FcRay<T>;
+  auto fetch = [&](int i, int j) { return fc_ray(p, i, j, st); };
+  auto window = [&](int jl, int jh) { return fc_window(p, jl, jh); };
+  constexpr unsigned OVER = 1u << 31;   // (in st) windows left to fc_resum_split
   RayVal pre[FC_PF];   // the next mode's first FC_PF rounds of 32 rays
   auto prefetch = [&](int i, int jb, int W) {
 #pragma unroll
@@ -396,13 +514,8 @@ __global__ void __launch_bounds__(FC_WARPS * 32, sizeof(T) == 4 ? 7 : 1)
       if (i < i1) {
         const int jl = p.jlo[bchk((long long)tile * p.M + i, njlo, st)];
         const int jh = p.jlo[bchk((long long)(tile + 1) * p.M + i, njlo, st)];
-        // a table left inconsistent by a failed screen (flagged by the bracket
-        // kernel) must not send the reads out of [0, NRT); a window beyond the
-        // tile's capacity means rays compressed beyond it (flagged here)
-        if (jl >= 1 && jh >= jl && jh <= p.NRT - 3) {
-          h_W = jh - jl + 4;
-          if (h_W > wcap) { st |= ST_CAUSTIC; h_W = 0; }
-        }
+        h_W = window(jl, jh);
+        if (h_W > wcap) { st |= OVER; h_W = 0; }
         h_jb = jl - 1;
       }
     }
@@ -482,30 +595,9 @@ __global__ void __launch_bounds__(FC_WARPS * 32, sizeof(T) == 4 ? 7 : 1)
       }
     }
   }
-  __syncthreads();
-  V* red = reinterpret_cast<V*>(smem_raw);
-  const int TMP = 32 * (PW + 1);
-#pragma unroll
-  for (int q = 0; q < PW; ++q) {
-    V v;
-    v.x = accr[q];
-    v.y = acci[q];
-    red[warp * TMP + lane * (PW + 1) + q] = v;
-  }
-  __syncthreads();
-  V* out = p.part + bchk((long long)group * p.N + m0, (long long)p.n_groups * p.N - (TM - 1), st);
-  if (st) atomicOr(p.status, st);
-  for (int x = threadIdx.x; x < TM; x += FC_WARPS * 32) {
-    const int xs = (x / PW) * (PW + 1) + x % PW;
-    V sum = red[xs];
-#pragma unroll
-    for (int k = 1; k < FC_WARPS; ++k) {
-      const V v = red[k * TMP + xs];
-      sum.x += v.x;
-      sum.y += v.y;
-    }
-    out[x] = sum;
-  }
+  const bool over = __syncthreads_or(st & OVER);
+  fc_block_sum<T, PW, false>(p, smem_raw, accr, acci, tile, group, st & ~OVER);
+  if (over) fc_resum_split<T, PW>(p, smem_raw, tile, group);
 }
 
 template <typename T, int PW>

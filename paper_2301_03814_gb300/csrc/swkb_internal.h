@@ -204,6 +204,7 @@ struct FcResumArgs {
   const double2* trig;               // [TRIG_N] FP64: exp(2 pi i k / TRIG_N)
   int M, NRT, G, R, N, TM, n_tiles, n_groups, modes_per_group, n_max, wcap, Np, P;
   unsigned np_magic;                 // floor(2^32 / Np)
+  int wlim, lim_pair;                // most rays on a tile (on a pair of tiles)
   typename C2<T>::type* part;        // [n_groups][N]
   unsigned* status;
 };

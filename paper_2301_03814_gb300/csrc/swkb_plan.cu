@@ -84,6 +84,7 @@ struct swkb_plan {
   double eps_ref = 0, absorber_frac = 0;
   // resummation tiling
   int PW = 8, TM = 256, n_tiles = 0, n_groups = 1, modes_per_group = 1, wcap = 0;
+  int fc_wlim = 0, fc_lim_pair = 0;   // most rays on a tile (on a pair of tiles)
   int ctas_per_sm = 6, sms = 1;
   int alloc_groups = 0, alloc_tiles = 0;   // buffer sizes: max over tuning candidates
   // medium
@@ -842,6 +843,7 @@ FcResumArgs<T> fc_resum_args(const swkb_plan* p, const T* d, const T* ph, const 
   r.M = p->M; r.NRT = p->NRT; r.G = p->G; r.R = p->R; r.N = p->N; r.TM = p->TM;
   r.n_tiles = p->n_tiles; r.n_groups = p->n_groups; r.modes_per_group = p->modes_per_group;
   r.n_max = p->n_max; r.wcap = p->wcap; r.Np = p->fc_Np; r.P = p->fc_P;
+  r.wlim = p->fc_wlim; r.lim_pair = p->fc_lim_pair;
   r.np_magic = (unsigned)((1ULL << 32) / (unsigned long long)p->fc_Np);
   r.part = (V*)p->part; r.status = p->status;
   return r;
@@ -1555,9 +1557,14 @@ void apply_tiling(swkb_plan* p, const Tiling& t) {
   p->TM = 32 * t.PW;
   p->n_tiles = p->N / p->TM;
   p->n_tiles_run = p->sym ? p->n_tiles / 2 + 1 : p->n_tiles;
-  // rays per tile window: up to 4x compression (patch-wise plans: exactly,
-  // which keeps six FP32 sums of 4 warps within an SM's shared memory)
-  p->wcap = 4 * p->TM / p->R + (p->fc ? 4 : 8);
+  // rays per tile window: up to 4x compression.  Periodic tiles of 512 points take 4
+  // rays more, so that they hold what two tiles of 256 points would.  Patch-wise plans
+  // have no slack, which keeps six FP32 sums of 4 warps within an SM's shared memory
+  // (but at least one interval between two landings): a window may hold more rays, up
+  // to 4x on the tile or its pair of tiles, and is then summed in parts.
+  const auto fc_window = [&](int points) { return std::max(4 * points / p->R, 2) + 4; };
+  p->wcap = p->fc ? fc_window(p->TM) : 4 * p->TM / p->R + (p->TM > 256 ? 12 : 8);
+  p->fc_wlim = fc_window(p->fc_lim_pair ? 2 * p->TM : p->TM);
   p->ctas_per_sm = t.ctas_per_sm;
   const int target_ctas = p->sms * t.ctas_per_sm;
   p->n_groups = std::max(1, std::min(p->M, (target_ctas + p->n_tiles_run - 1) / p->n_tiles_run));
@@ -1727,6 +1734,13 @@ swkb_status configure(swkb_plan* p, const swkb_profile* prof, double k, const sw
   if (p->planes && (p->planes > p->Nt || p->Nt % p->planes))
     return fail(SWKB_ERR_INVALID_ARG, "planes (%d) must divide rk4_steps (%d)", p->planes, p->Nt);
   Tiling def = default_tiling(p);
+  if (p->fc) {
+    // the compression limit holds on tiles of 256 points (64 to 128 at R < 8), twice the
+    // default ones where such tiles divide N; on the tile itself if its size is asked for
+    int lim = p->R >= 8 ? 8 : (p->R >= 2 ? 4 : 2);
+    while (32 * lim > p->N || p->N % (32 * lim)) lim /= 2;
+    p->fc_lim_pair = lim > def.PW && opt.tile_points == 0;
+  }
   if (opt.tile_points != 0 || opt.ctas_per_sm != 0 || opt.fft_n1 != 0) {
     const Tiling t{opt.tile_points / 32, opt.ctas_per_sm, opt.fft_n1};
     if (opt.tile_points % 32 || opt.ctas_per_sm > 1024 || !valid_tiling(p, t))
