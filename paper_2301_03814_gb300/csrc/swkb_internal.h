@@ -313,7 +313,11 @@ swkb_status plan_advance(swkb_plan* p, int q, int n, bool first);
 swkb_status plan_finish(swkb_plan* p, bool fresh);
 // Wait for the plan's stream, map its status, copy the result to the host.
 swkb_status plan_collect(swkb_plan* p, double* out_host);
-// Device bytes a plan with these arguments would hold (no allocation).
+// swkb_plan_create.  served: the plan of a served request, which calls for no inner
+// planes (no memory is taken to sum several at once).
+swkb_status create_plan(const swkb_profile* prof, double k, const swkb_domain* dom, int32_t n_z,
+                        double screen_dx, const swkb_options* opt, bool served, swkb_plan** out);
+// Device bytes such a plan with these arguments would hold (no allocation).
 swkb_status estimate_plan_bytes(const swkb_profile* prof, double k, const swkb_domain* dom,
                                 int32_t n_z, double screen_dx, const swkb_options* opt,
                                 size_t* bytes);

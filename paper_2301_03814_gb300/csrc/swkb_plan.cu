@@ -123,6 +123,7 @@ struct swkb_plan {
   // (with one plane at a time the screen's brackets and partials serve)
   int planes = 0;
   int pl_batch = 1;
+  bool pl_single = false;   // one inner plane at a time (served requests call for none)
   int* pl_jlo = nullptr;
   int* pl_jneg = nullptr;
   void* pl_part = nullptr;
@@ -483,6 +484,45 @@ swkb_status build_fc(swkb_plan* p) {
   return SWKB_OK;
 }
 
+// Brackets, coefficients and partials of one inner plane taken together with others.
+size_t plane_bytes(const swkb_plan* p) {
+  const size_t V = p->precision == SWKB_FP64 ? 16 : 8;
+  return (size_t)p->alloc_groups * p->N * V + (size_t)p->M * V +
+         (size_t)(p->alloc_tiles + 1) * p->Mr * sizeof(int) * (p->sym ? 2 : 1);
+}
+
+// Arrays for pl_batch inner planes at once: taken last, and only from memory to spare
+// (an eighth of what is free); without them the planes go one at a time.
+template <typename T>
+swkb_status alloc_plane_batch(swkb_plan* p) {
+  using V = typename C2<T>::type;
+  if (p->pl_batch <= 1) return SWKB_OK;
+  size_t free_b = 0, total_b = 0;
+  CK(cudaMemGetInfo(&free_b, &total_b));
+  const size_t one = plane_bytes(p), jn = (size_t)(p->alloc_tiles + 1) * p->Mr * sizeof(int);
+  p->pl_batch = (int)std::min<size_t>(p->pl_batch, free_b / 8 / one);
+  const size_t held = p->allocs.size(), bytes = p->bytes, n = (size_t)std::max(p->pl_batch, 0);
+  void* cpol = nullptr;
+  const bool ok =
+      n > 1 && dev_alloc(p, &cpol, n * p->M * sizeof(V)) == SWKB_OK &&
+      dev_alloc(p, &p->pl_part, n * p->alloc_groups * p->N * sizeof(V)) == SWKB_OK &&
+      dev_alloc(p, (void**)&p->pl_jlo, n * jn) == SWKB_OK &&
+      (!p->sym || dev_alloc(p, (void**)&p->pl_jneg, n * jn) == SWKB_OK);
+  if (!ok) {
+    for (size_t i = held; i < p->allocs.size(); ++i) cudaFree(p->allocs[i]);
+    p->allocs.resize(held);
+    p->bytes = bytes;
+    p->pl_part = nullptr;
+    p->pl_jlo = p->pl_jneg = nullptr;
+    p->pl_batch = 1;
+    return SWKB_OK;
+  }
+  p->cpol_plane = cpol;
+  CK(cudaMemsetAsync(p->pl_jlo, 0, n * jn, p->stream));
+  if (p->sym) CK(cudaMemsetAsync(p->pl_jneg, 0, n * jn, p->stream));
+  return SWKB_OK;
+}
+
 template <typename T>
 swkb_status build_device(swkb_plan* p, const swkb_profile* prof) {
   using V = typename C2<T>::type;
@@ -628,7 +668,7 @@ swkb_status build_device(swkb_plan* p, const swkb_profile* prof) {
     TRY(dev_alloc(p, &p->pl_ph, pr * sizeof(T)));
     TRY(dev_alloc(p, &p->pl_a, pr * sizeof(T)));
     TRY(dev_alloc(p, &p->c_plane, (size_t)M * sizeof(V)));
-    TRY(dev_alloc(p, &p->cpol_plane, (size_t)p->pl_batch * M * sizeof(V)));
+    TRY(dev_alloc(p, &p->cpol_plane, (size_t)M * sizeof(V)));
     TRY(dev_alloc(p, &p->ephi_pl, (size_t)(p->planes - 1) * M * sizeof(V)));
   }
   const size_t jn = (size_t)(p->alloc_tiles + 1) * p->Mr;
@@ -637,16 +677,6 @@ swkb_status build_device(swkb_plan* p, const swkb_profile* prof) {
   if (p->sym) {
     TRY(dev_alloc(p, (void**)&p->jlo_neg, jn * sizeof(int)));
     CK(cudaMemsetAsync(p->jlo_neg, 0, jn * sizeof(int), p->stream));
-  }
-  if (p->pl_batch > 1) {
-    const size_t n = (size_t)p->pl_batch;
-    TRY(dev_alloc(p, &p->pl_part, n * p->alloc_groups * N * sizeof(V)));
-    TRY(dev_alloc(p, (void**)&p->pl_jlo, n * jn * sizeof(int)));
-    CK(cudaMemsetAsync(p->pl_jlo, 0, n * jn * sizeof(int), p->stream));
-    if (p->sym) {
-      TRY(dev_alloc(p, (void**)&p->pl_jneg, n * jn * sizeof(int)));
-      CK(cudaMemsetAsync(p->pl_jneg, 0, n * jn * sizeof(int), p->stream));
-    }
   }
   if (p->overlap) {
     TRY(dev_alloc(p, &p->rd1, rays * sizeof(T)));
@@ -662,6 +692,7 @@ swkb_status build_device(swkb_plan* p, const swkb_profile* prof) {
   TRY(dev_alloc(p, (void**)&p->status, sizeof(unsigned)));
   CK(cudaMemsetAsync(p->status, 0, sizeof(unsigned), p->stream));
   TRY(dev_alloc(p, (void**)&p->io, 2 * (size_t)std::max(N, p->n_z) * sizeof(double)));
+  TRY(alloc_plane_batch<T>(p));
   if (p->fc)
     CK(prepare_fc_kernels<T>((int)fc_resum_smem_bytes<T>(p->wcap, p->TM),
                              (int)fc_modes_smem_bytes<T>(p->fc_Np)));
@@ -1575,13 +1606,6 @@ void apply_tiling(swkb_plan* p, const Tiling& t) {
   p->log2N2 = ilog2(p->N2);
 }
 
-// Brackets and partials of one inner plane taken together with others.
-size_t plane_bytes(const swkb_plan* p) {
-  const size_t V = p->precision == SWKB_FP64 ? 16 : 8;
-  return (size_t)p->alloc_groups * p->N * V +
-         (size_t)(p->alloc_tiles + 1) * p->Mr * sizeof(int) * (p->sym ? 2 : 1);
-}
-
 // Validate the arguments and derive every size of the plan (host only).
 swkb_status configure(swkb_plan* p, const swkb_profile* prof, double k, const swkb_domain* dom,
                       int32_t n_z, double screen_dx, const swkb_options& opt) {
@@ -1774,7 +1798,7 @@ swkb_status configure(swkb_plan* p, const swkb_profile* prof, double k, const sw
     }
     apply_tiling(p, def);
   }
-  if (p->planes > 1 && !p->fc) {
+  if (p->planes > 1 && !p->fc && !p->pl_single) {
     // inner planes at once: their extra arrays stay within 256 MB
     const size_t one = plane_bytes(p);
     p->pl_batch = (int)std::max<size_t>(1, std::min<size_t>(p->planes - 1, (256u << 20) / one));
@@ -1797,7 +1821,7 @@ size_t device_bytes(const swkb_plan* p) {
   b += 3 * (size_t)p->NRT * p->Mr * T * (p->overlap ? 2 : 1);     // rays (one or two sets)
   if (p->planes > 1)                                                 // inner planes
     b += (size_t)(p->planes - 1) * (3 * (size_t)p->NRT * p->Mr * T + (size_t)p->M * V) +
-         (size_t)p->M * V * (1 + (size_t)p->pl_batch) +
+         2 * (size_t)p->M * V +
          (p->pl_batch > 1 ? p->pl_batch * plane_bytes(p) : 0);
   b += (size_t)(p->alloc_tiles + 1) * p->Mr * sizeof(int) * (p->sym ? 2 : 1) *
        (p->overlap ? 2 : 1);
@@ -2029,6 +2053,7 @@ swkb_status estimate_plan_bytes(const swkb_profile* prof, double k, const swkb_d
     swkb_options opt;
     if (opt_in) opt = *opt_in; else swkb_options_default(&opt);
     swkb_plan tmp;
+    tmp.pl_single = true;
     TRY(configure(&tmp, prof, k, dom, n_z, screen_dx, opt));
     *bytes = device_bytes(&tmp);
     return SWKB_OK;
@@ -2044,6 +2069,14 @@ extern "C" {
 swkb_status swkb_plan_create(const swkb_profile* prof, double k, const swkb_domain* dom,
                              int32_t n_z, double screen_dx, const swkb_options* opt_in,
                              swkb_plan** out) {
+  return swkb::create_plan(prof, k, dom, n_z, screen_dx, opt_in, false, out);
+}
+
+}  // extern "C"
+
+swkb_status swkb::create_plan(const swkb_profile* prof, double k, const swkb_domain* dom,
+                              int32_t n_z, double screen_dx, const swkb_options* opt_in,
+                              bool served, swkb_plan** out) {
   Range range("swkb_plan_create");
   try {
     if (!out) return fail(SWKB_ERR_INVALID_ARG, "out is NULL");
@@ -2052,6 +2085,7 @@ swkb_status swkb_plan_create(const swkb_profile* prof, double k, const swkb_doma
     if (opt_in) opt = *opt_in; else swkb_options_default(&opt);
     swkb_plan* p = new swkb_plan();
     struct Guard { swkb_plan*& p; ~Guard() { if (p) release(p); } } guard{p};
+    p->pl_single = served;
     TRY(configure(p, prof, k, dom, n_z, screen_dx, opt));
     const char* ge = getenv("SWKB_GRAPHS");
     p->use_graphs = !(ge && ge[0] == '0');
@@ -2089,6 +2123,8 @@ swkb_status swkb_plan_create(const swkb_profile* prof, double k, const swkb_doma
     return fail(SWKB_ERR_INVALID_ARG, "unexpected exception");
   }
 }
+
+extern "C" {
 
 swkb_status swkb_plan_get_info(const swkb_plan* p, swkb_plan_info* info) {
   if (!p || !info) return fail(SWKB_ERR_INVALID_ARG, "NULL argument");

@@ -146,7 +146,7 @@ void worker_main(swkb_server* s) {
         std::this_thread::sleep_for(std::chrono::milliseconds(atoi(d)));
     for (Request* r : admit) {
       swkb_plan* plan = nullptr;
-      swkb_status st = swkb_plan_create(&r->prof, r->k, &r->dom, r->n_z, r->dx, &r->opt, &plan);
+      swkb_status st = swkb::create_plan(&r->prof, r->k, &r->dom, r->n_z, r->dx, &r->opt, true, &plan);
       std::string err = st == SWKB_OK ? "" : swkb_last_error();
       if (st == SWKB_OK) {
         r->plan = plan;
