@@ -25,7 +25,8 @@ enum : unsigned {
 // Entries of the FP64 sums' table of exp(2 pi i k / TRIG_N) (a power of two).
 constexpr int TRIG_N = 1024;
 
-// That table as (cos, sin) pairs, from long double; the quadrants' entries are exact.
+// That table as (cos, sin) pairs, from long double (0.5 ms where that is software); the
+// quadrants' entries are exact.
 inline std::vector<double> trig_table() {
   std::vector<double> e(2 * TRIG_N);
   const long double turn = 2.0L * acosl(-1.0L);

@@ -637,7 +637,10 @@ swkb_status build_device(swkb_plan* p, const swkb_profile* prof) {
     }
     TRY(upload<T>(p, &p->tw, tw));
   }
-  if (sizeof(T) == 8) TRY(upload<double>(p, &p->trig, trig_table()));
+  if (sizeof(T) == 8) {
+    static const std::vector<double> trig = trig_table();
+    TRY(upload<double>(p, &p->trig, trig));
+  }
   // absorber
   if (p->absorber_frac > 0) {
     std::vector<double> w(N, 1.0);
