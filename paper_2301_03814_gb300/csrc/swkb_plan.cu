@@ -324,11 +324,12 @@ void cubic_piece(const double* a, int s, int S, double* b) {
 // curvature's bound is not taken below what the rounding of the table's eps does
 // to it: an error d in the difference of two nodes puts up to 5.6 d / h^2 into the
 // quintic's curvature at the quarter points and 3 d / h^2 into one cubic's, so with
-// d <= 2 x 2^-53 max |eps| they differ by up to 6 x 2^-53 max |eps| / h^2.  Media broad
-// against the table spacing (or linear) have an e_zz below that, and no number of
-// pieces reproduces the noise (open lens of 131072 points, spacing 1/16, width 7282:
-// one piece, at 0.87 of that bound, instead of the quintic, 425 against 495 us per
-// march).  0 when none does (the quintic itself is evaluated).
+// nodes good to two units in the last place (d <= 8 x 2^-53 max |eps|) they differ by
+// up to 24 x 2^-53 max |eps| / h^2.  Media broad against the table spacing (or linear)
+// have an e_zz below that, and no number of pieces reproduces the noise (open lens of
+// 131072 points, spacing 1/16, width 7282: one piece, at 0.22 of that bound, instead of
+// the quintic, 425 against 495 us per march).  0 when none does (the quintic itself is
+// evaluated).
 int choose_pieces(const swkb_plan* p, const swkb_profile* prof, const std::vector<double>& coef) {
   const double h = p->dzp;
   const size_t n = (size_t)p->n_cols * p->n_int;
@@ -345,7 +346,7 @@ int choose_pieces(const swkb_plan* p, const swkb_profile* prof, const std::vecto
       E2 = std::max(E2, fabs(d2) / (h * h));
     }
   }
-  const double tol[3] = {1e-7 * E0, 1e-6 * E1, std::max(1e-4 * E2, 6.0 * ldexp(eps_max, -53) / (h * h))};
+  const double tol[3] = {1e-7 * E0, 1e-6 * E1, std::max(1e-4 * E2, 24.0 * ldexp(eps_max, -53) / (h * h))};
   // largest deviations of S pieces from the quintic (value, slope, curvature);
   // with stop set, returns as soon as one exceeds its bound
   auto worst = [&](int S, double dev[3], bool stop) {

@@ -76,3 +76,11 @@ def test_pieces_follow_the_table_alone(dx):
     duct = w.config_surface_duct_small().with_(dx=dx)
     assert swkb.Plan(duct, swkb.SWKB_MIXED).info.medium_pieces == 16
     assert swkb.Plan(w.config_unit_periodic().with_(dx=20.0 * dx / 50.0), swkb.SWKB_MIXED).info.medium_pieces == 1
+
+
+def test_tables_with_ordinary_rounding_take_one_piece():
+    # a broad lens given by its refractive index: eps = n^2 is rounded once more
+    pb = w.config_gaussian_medium(a=2e-4, b=1e-6)
+    pr = pb.profile
+    pb = pb.with_(profile=w.Profile(pr.x_cols, pr.z0, pr.dz, np.sqrt(pr.eps) ** 2, pr.eps_z, pr.eps_zz))
+    assert swkb.Plan(pb, swkb.SWKB_MIXED).info.medium_pieces == 1
