@@ -179,8 +179,9 @@ __device__ __forceinline__ void march_item(const Inst<T>& I, int set, int step, 
       else march_x2_body<false, false, false, kThreads>(a, item, tid);
     }
   } else {
-    if (I.multi) march64_body<true, false, kThreads>(a, item, tid);
-    else march64_body<false, false, kThreads>(a, item, tid);
+    if (!I.multi) march64_body<ONE_COLUMN, false, kThreads>(a, item, tid);
+    else if (a.med.pairs) march64_body<PAIRS, false, kThreads>(a, item, tid);
+    else march64_body<COLUMNS, false, kThreads>(a, item, tid);
   }
 }
 

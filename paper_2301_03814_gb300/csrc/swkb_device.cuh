@@ -142,13 +142,13 @@ __device__ __forceinline__ double rcp64(double x) {
 // p''(t)/2 of the interval's quintic.  The interval comes from the low bits of
 // a round-down add of 1.5 * 2^52, so that only three additions of the lookup
 // are FP64 work; positions outside the table (or its very top) take the slow
-// branch.  MULTI: the entry holds a column's coefficients and their
-// differences to the next column, blended with weight th (6 FMAs; a second
-// polynomial and its blend would take 18).
-template <bool MULTI>
+// branch.  The coefficients of two columns are blended with weight th: 12 FMAs, 6 where
+// the table holds differences (PAIRS); a second polynomial and its blend would take 18.
+enum { ONE_COLUMN = 0, COLUMNS = 1, PAIRS = 2 };
+template <int MULTI>
 __device__ __forceinline__ void med64(const MarchArgs<double>& p, int l, double u, double& e,
                                       double& d1, double& d2, unsigned& st) {
-  constexpr int W = MULTI ? 16 : 8;
+  constexpr int W = MULTI == PAIRS ? 16 : 8;
   const double magic = 6755399441055744.0;
   const double z = p.med.mirrored ? fabs(u) : u;
   const double v = __dadd_rd(z, magic);
@@ -162,18 +162,20 @@ __device__ __forceinline__ void med64(const MarchArgs<double>& p, int l, double 
   const double* q = p.med.coef;
   long long o = (long long)i * W;
   double th = 0.0;
-  if constexpr (MULTI) {
+  if constexpr (MULTI != ONE_COLUMN) {
     o += (long long)__ldg(p.st.c + l) * p.med.col_stride;
     th = __ldg(p.st.th + l);
   }
-  q += bchk(o, p.med.size - (W - 1), st);
+  const long long next = MULTI == COLUMNS ? p.med.col_stride : MULTI == PAIRS ? 8 : 0;
+  q += bchk(o, p.med.size - next - 7, st);
   double a[6];
   load6<double>(q, a[0], a[1], a[2], a[3], a[4], a[5]);
-  if constexpr (MULTI) {
+  if constexpr (MULTI != ONE_COLUMN) {
     double d[6];
-    load6<double>(q + 8, d[0], d[1], d[2], d[3], d[4], d[5]);
+    load6<double>(q + next, d[0], d[1], d[2], d[3], d[4], d[5]);
 #pragma unroll
-    for (int k = 0; k < 6; ++k) a[k] = fma(th, d[k], a[k]);
+    for (int k = 0; k < 6; ++k)
+      a[k] = fma(th, d[k], MULTI == PAIRS ? a[k] : fma(-th, a[k], a[k]));
   }
   // Horner with derivatives (synthetic division)
   double b = a[5] * t + a[4];                             // coefficient 4
@@ -197,7 +199,7 @@ struct Ray {
 // Right-hand side without the factors 2c, c, 1, -c, c.  Turning points (P^2 <=
 // 0) and caustics (N >= 0) are running extremes of the high words (as integers,
 // off the FP64 pipe), tested once per ray.
-template <bool MULTI>
+template <int MULTI>
 __device__ __forceinline__ Ray rhs64(const MarchArgs<double>& p, int l, double u, double kap,
                                      double pb, double pb2, const Ray& y, int& P2_lo, int& N_hi,
                                      unsigned& st) {
@@ -223,7 +225,7 @@ __device__ __forceinline__ Ray rhs64(const MarchArgs<double>& p, int l, double u
 // Thread t marches ray j of mode r, t = j Mr + r: a warp's lanes are
 // consecutive modes at one launch height, so their table reads stay within a
 // few intervals.  THREADS threads per block.
-template <bool MULTI, bool PLANES, int THREADS>
+template <int MULTI, bool PLANES, int THREADS>
 __device__ __forceinline__ void march64_body(const MarchArgs<double>& p, int blk, int tid) {
   const long long t = (long long)blk * THREADS + tid;
   if (t >= (long long)p.Mr * p.NRT) return;
@@ -302,7 +304,7 @@ __device__ __forceinline__ void march64_body(const MarchArgs<double>& p, int blk
 // evaluated both columns of a lookup.
 constexpr int MARCH64_THREADS = 64;
 
-template <bool MULTI, bool PLANES>
+template <int MULTI, bool PLANES>
 __global__ void __launch_bounds__(MARCH64_THREADS) k_march(const MarchArgs<double> p) {
   march64_body<MULTI, PLANES, MARCH64_THREADS>(p, blockIdx.x, threadIdx.x);
 }
@@ -389,22 +391,25 @@ __device__ __forceinline__ void horner3(const float4 v, float t, float& e, float
   e = b; d1 = c1; d2 = c2;
 }
 
+// Two coefficients of two columns blended with weight th (m = -th), exact at both ends.
+__device__ __forceinline__ f2 blend2(f2 th, f2 m, f2 a, f2 b) {
+  return fma2(th, b, fma2(m, a, a));
+}
+
 // One entry of the FP32 medium table at its local coordinate t: p(t), p'(t)
-// and p''(t)/2.  MULTI: the entry holds a column's coefficients and their
-// differences to the next column, blended with weight th before the
-// polynomial is evaluated (4 + 6 FMAs for a cubic piece; evaluating both
-// columns and blending the results takes 18).
+// and p''(t)/2.  MULTI: blended with the next column's entry (next values on)
+// before the polynomial is evaluated (4 packed and 6 FMAs for a cubic piece;
+// evaluating both columns and blending the results takes 18).
 template <bool MULTI, bool CUBIC>
-__device__ __forceinline__ void table_eval(const float* q, float t, float th, float& e, float& d1,
-                                           float& d2) {
+__device__ __forceinline__ void table_eval(const float* q, long long next, float t, float th,
+                                           float& e, float& d1, float& d2) {
+  const f2 th2 = bc2(th), m2 = bc2(-th);
   if constexpr (CUBIC) {
     float4 v = __ldg(reinterpret_cast<const float4*>(q));
     if constexpr (MULTI) {
-      const float4 d = __ldg(reinterpret_cast<const float4*>(q + 4));
-      v.x = fmaf(th, d.x, v.x);
-      v.y = fmaf(th, d.y, v.y);
-      v.z = fmaf(th, d.z, v.z);
-      v.w = fmaf(th, d.w, v.w);
+      const float4 d = __ldg(reinterpret_cast<const float4*>(q + next));
+      sp2(blend2(th2, m2, mk2(v.x, v.y), mk2(d.x, d.y)), v.x, v.y);
+      sp2(blend2(th2, m2, mk2(v.z, v.w), mk2(d.z, d.w)), v.z, v.w);
     }
     horner3(v, t, e, d1, d2);
   } else {
@@ -412,9 +417,10 @@ __device__ __forceinline__ void table_eval(const float* q, float t, float th, fl
     load6<float>(q, a[0], a[1], a[2], a[3], a[4], a[5]);
     if constexpr (MULTI) {
       float d[6];
-      load6<float>(q + 8, d[0], d[1], d[2], d[3], d[4], d[5]);
+      load6<float>(q + next, d[0], d[1], d[2], d[3], d[4], d[5]);
 #pragma unroll
-      for (int k = 0; k < 6; ++k) a[k] = fmaf(th, d[k], a[k]);
+      for (int k = 0; k < 6; k += 2)
+        sp2(blend2(th2, m2, mk2(a[k], a[k + 1]), mk2(d[k], d[k + 1])), a[k], a[k + 1]);
     }
     horner5(a, t, e, d1, d2);
   }
@@ -435,7 +441,7 @@ struct Extremes {
 template <bool MULTI, bool CUBIC>
 __device__ __forceinline__ void med32x2(const MarchArgs<float>& p, int l, f2 u2, f2& e, f2& d1,
                                         float& d2a, float& d2b, Extremes& x, unsigned& st) {
-  constexpr int W = (CUBIC ? 4 : 8) * (MULTI ? 2 : 1);
+  constexpr int W = CUBIC ? 4 : 8;
   const f2 magic = bc2(12582912.f);
   const f2 v = add2_rd(u2, magic);
   const f2 t = sub2(u2, sub2(v, magic));
@@ -455,12 +461,13 @@ __device__ __forceinline__ void med32x2(const MarchArgs<float>& p, int l, f2 u2,
     base += (long long)__ldg(p.st.c + l) * p.med.col_stride;
     th = __ldg(p.st.th + l);
   }
-  const long long off = base - p.med.coef;
+  const long long off = base - p.med.coef, next = MULTI ? p.med.col_stride : 0;
+  const long long end = p.med.size - next - (W - 1);
   float ea, eb, d1a, d1b;
-  table_eval<MULTI, CUBIC>(base + (bchk(off + (long long)ia * W, p.med.size - (W - 1), st) - off),
-                           ta, th, ea, d1a, d2a);
-  table_eval<MULTI, CUBIC>(base + (bchk(off + (long long)ib * W, p.med.size - (W - 1), st) - off),
-                           tb, th, eb, d1b, d2b);
+  table_eval<MULTI, CUBIC>(base + (bchk(off + (long long)ia * W, end, st) - off), next, ta, th,
+                           ea, d1a, d2a);
+  table_eval<MULTI, CUBIC>(base + (bchk(off + (long long)ib * W, end, st) - off), next, tb, th,
+                           eb, d1b, d2b);
   e = mk2(ea, eb);
   d1 = mk2(d1a, d1b);
 }

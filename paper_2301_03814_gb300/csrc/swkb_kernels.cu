@@ -28,6 +28,8 @@
 
 #include <utility>
 
+#include <type_traits>
+
 #include "swkb_device.cuh"
 
 namespace swkb {
@@ -223,11 +225,13 @@ cudaError_t launch_march<double>(const MarchArgs<double>& a, bool multi_column, 
   const long long threads = (long long)a.Mr * a.NRT;
   const dim3 block(MARCH64_THREADS),
       grid((unsigned)((threads + MARCH64_THREADS - 1) / MARCH64_THREADS));
-  if (a.plane_steps > 0)
-    return multi_column ? launch_k(k_march<true, true>, grid, block, 0, s, a)
-                        : launch_k(k_march<false, true>, grid, block, 0, s, a);
-  return multi_column ? launch_k(k_march<true, false>, grid, block, 0, s, a)
-                      : launch_k(k_march<false, false>, grid, block, 0, s, a);
+  const auto launch = [&](auto planes) {
+    constexpr bool P = decltype(planes)::value;
+    return !multi_column ? launch_k(k_march<ONE_COLUMN, P>, grid, block, 0, s, a)
+           : a.med.pairs ? launch_k(k_march<PAIRS, P>, grid, block, 0, s, a)
+                         : launch_k(k_march<COLUMNS, P>, grid, block, 0, s, a);
+  };
+  return a.plane_steps > 0 ? launch(std::true_type{}) : launch(std::false_type{});
 }
 
 template <>

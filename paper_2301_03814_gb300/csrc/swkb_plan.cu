@@ -259,16 +259,17 @@ namespace {
 
 // Intervals of the FP32 medium table of one column (layout in swkb_internal.h).
 int table32_intervals(const swkb_plan* p) { return (p->mirror ? 2 : 1) * p->n_int + 1; }
-// Columns of the medium table as stored (with several, each holds the
-// differences to the next one too, so the last needs none of its own) and the
-// values of one.
-int table_columns(const swkb_plan* p) { return p->n_cols > 1 ? p->n_cols - 1 : 1; }
+// Whether the medium table's entries are followed by their differences, its columns as
+// stored, and the values of one.
+bool table_pairs(const swkb_plan* p) {
+  return p->precision == SWKB_FP64 && p->n_cols > 1 &&
+         (p->n_cols - 1) * (long long)p->n_int * 16 * (long long)sizeof(double) <= PAIRS_MAX;
+}
+int table_columns(const swkb_plan* p) { return table_pairs(p) ? p->n_cols - 1 : p->n_cols; }
 long long table_values(const swkb_plan* p) {
-  const long long entries =
-      p->precision == SWKB_FP64
-          ? (long long)p->n_int * 8
-          : (long long)table32_intervals(p) * (p->pieces > 0 ? 4 * p->pieces : 8);
-  return entries * (p->n_cols > 1 ? 2 : 1);
+  return p->precision == SWKB_FP64
+             ? (long long)p->n_int * (table_pairs(p) ? 16 : 8)
+             : (long long)table32_intervals(p) * (p->pieces > 0 ? 4 * p->pieces : 8);
 }
 
 // Quintic Hermite interpolant of eps - eps_ref on every profile interval, as
@@ -568,21 +569,19 @@ swkb_status build_device(swkb_plan* p, const swkb_profile* prof) {
       }
       coef.swap(c32);
     }
-    if (p->n_cols > 1) {
+    if (table_pairs(p)) {
       // each entry of a column followed by its difference to the next one
-      const size_t w = p->pieces > 0 ? 4 : 8, per = coef.size() / p->n_cols;
-      std::vector<T> pairs((size_t)(p->n_cols - 1) * per * 2);
-      T* o = pairs.data();
-      for (size_t k = 0; k + per < coef.size(); k += w, o += 2 * w)
-        for (size_t j = 0; j < w; ++j) {
-          o[j] = (T)coef[k + j];
-          o[w + j] = (T)(coef[k + per + j] - coef[k + j]);
+      const size_t per = coef.size() / p->n_cols;
+      std::vector<double> pairs(2 * (coef.size() - per));
+      double* o = pairs.data();
+      for (size_t k = 0; k + per < coef.size(); k += 8, o += 16)
+        for (size_t j = 0; j < 8; ++j) {
+          o[j] = coef[k + j];
+          o[8 + j] = coef[k + per + j] - coef[k + j];
         }
-      TRY(dev_alloc(p, &p->coef, pairs.size() * sizeof(T)));
-      CK(cudaMemcpy(p->coef, pairs.data(), pairs.size() * sizeof(T), cudaMemcpyHostToDevice));
-    } else {
-      TRY(upload<T>(p, &p->coef, coef));
+      coef.swap(pairs);
     }
+    TRY(upload<T>(p, &p->coef, coef));
   }
   // RK4 stage columns for screens 0 .. stage_rows - 1
   {
@@ -772,6 +771,7 @@ MarchArgs<T> march_args(const swkb_plan* p, int q) {
   double z0 = p->z0p, hs = p->dzp;   // table origin and entry spacing
   a.med.n_int = p->n_int;
   a.med.mirrored = p->mirror != 0;
+  a.med.pairs = table_pairs(p);
   a.med.pieces = p->pieces;
   if (sizeof(T) == 4) {   // the reflection stored, entries in pieces
     const int S = p->pieces > 0 ? p->pieces : 1;

@@ -84,3 +84,56 @@ def test_tables_with_ordinary_rounding_take_one_piece():
     pr = pb.profile
     pb = pb.with_(profile=w.Profile(pr.x_cols, pr.z0, pr.dz, np.sqrt(pr.eps) ** 2, pr.eps_z, pr.eps_zz))
     assert swkb.Plan(pb, swkb.SWKB_MIXED).info.medium_pieces == 1
+
+
+def _columns(pb, x_cols):
+    """The problem with the medium of its first two columns on other range columns."""
+    pr = pb.profile
+    i = np.arange(len(x_cols)) % 2
+    return pb.with_(profile=w.Profile(np.asarray(x_cols, float), pr.z0, pr.dz, pr.eps[i], pr.eps_z[i], pr.eps_zz[i]))
+
+
+def _ducts():
+    pb = w.config_surface_duct_small(n_screens=2)
+    pr = pb.profile
+    return pb.with_(profile=w._table([0.0, 50.0], pr.z0, pr.dz, pr.n_p,
+                                     [w.f_trilinear_duct(12.0, -0.1), w.f_trilinear_duct(15.0, -0.1)]))
+
+
+def test_mixed_tables_hold_each_column_once():
+    pb = _ducts()
+    infos = {n: swkb.Plan(_columns(pb, np.linspace(0.0, 200.0, n)), swkb.SWKB_MIXED).info for n in (3, 5, 9)}
+    bytes_of = {n: i.device_bytes for n, i in infos.items()}
+    column = (2 * (pb.profile.n_p - 1) + 1) * 16 * infos[3].medium_pieces   # mirrored and one more, 4 floats a piece
+    assert bytes_of[5] - bytes_of[3] == 2 * column and bytes_of[9] - bytes_of[5] == 4 * column
+
+
+@pytest.mark.parametrize("make", [_ducts, w.config_unit_periodic], ids=["grounded", "periodic"])
+def test_small_and_large_tables_blend_alike(make):
+    # FP64: small tables hold differences, larger ones (here by columns beyond the screens) do not; the blended
+    # coefficients differ by a unit in the last place of e = eps - eps_ref, which is below 0.1 here: 2e-17 of k x / 2
+    pb = make().with_(n_screens=2)
+    xs = [0.0, 0.7 * pb.dx, 2.5 * pb.dx]
+    small = swkb.Plan(_columns(pb, xs), swkb.SWKB_FP64)
+    per = (pb.profile.n_p - 1) * 128
+    far = 2.5 * pb.dx + np.arange(1, (8 << 20) // per + 3)
+    large = swkb.Plan(_columns(pb, np.concatenate([xs, far])), swkb.SWKB_FP64)
+    assert large.info.device_bytes - small.info.device_bytes < 0.6 * per * len(far) + (1 << 20)
+    a, b = small.propagate(), large.propagate()
+    assert rel_l2(a, b) < 1e-12
+
+
+@pytest.mark.parametrize("precision", [swkb.SWKB_FP64, swkb.SWKB_MIXED])
+def test_a_column_met_exactly_is_taken_exactly(precision):
+    # screens between equal columns: whatever the blend's weight, the field of the column alone.  FP64 small tables
+    # add zero differences, FP32 blends th c + (c - th c), a rounding per coefficient at most
+    pb = _ducts()
+    pr = pb.profile
+    same = pb.with_(profile=w.Profile(np.array([0.0, 30.0, 110.0]), pr.z0, pr.dz, pr.eps[[0, 0, 0]], pr.eps_z[[0, 0, 0]],
+                                      pr.eps_zz[[0, 0, 0]]))
+    one = pb.with_(profile=w.Profile(np.array([0.0]), pr.z0, pr.dz, pr.eps[:1], pr.eps_z[:1], pr.eps_zz[:1]))
+    a, b = (swkb.Plan(p, precision).propagate() for p in (same, one))
+    if precision == swkb.SWKB_FP64:
+        assert np.array_equal(a, b)
+    else:
+        assert rel_l2(a, b) < 1e-6
