@@ -619,11 +619,14 @@ __device__ __forceinline__ void march_x2_body(const MarchArgs<float>& p, int blk
 // with the unscaled system (35 packed operations, 80 instructions); 326
 // against 485 us on a range-dependent table (698 modes x 4118 rays).
 // 6 CTAs of 128 threads per SM (80 registers): 102 us; 3 of 256: 104; 4 of
-// 256 (64 registers, spills): 112; 2 of 256: 107; all-scalar arithmetic: 110.
+// 256 (64 registers, spills): 112; 2 of 256: 107; all-scalar arithmetic: 110.  With
+// inner planes 5 per SM (96 registers; 80 spill): 8192 points, 3 screens of 4 planes 447
+// against 458 us per call.
 constexpr int MARCH_THREADS = 128;
 
 template <bool MULTI, bool PLANES, bool CUBIC>
-__global__ void __launch_bounds__(MARCH_THREADS, 6) k_march_x2(const MarchArgs<float> p) {
+__global__ void __launch_bounds__(MARCH_THREADS, PLANES ? 5 : 6)
+    k_march_x2(const MarchArgs<float> p) {
   march_x2_body<MULTI, PLANES, CUBIC, MARCH_THREADS>(p, blockIdx.x, threadIdx.x);
 }
 
