@@ -115,10 +115,14 @@ typedef struct {
                              fastest; cached per shape for the process       */
   void* cuda_stream;      /* cudaStream_t to run on; NULL = a library stream.
                              The plan also owns a second stream for the ray
-                             march (unless SWKB_OVERLAP=0 or reuse_rays):
-                             within every call it forks from this stream and
-                             joins back into it, so results are ordered on
-                             this stream as if one stream ran everything     */
+                             march and a third for the landing brackets
+                             (unless reuse_rays, or the environment has
+                             SWKB_OVERLAP=0; FP64 plans of fewer than 400000
+                             rays and FP64 patch-wise plans only where it has
+                             SWKB_OVERLAP=1): within every call they fork from
+                             this stream and join back into it, so results
+                             are ordered on this stream as if one stream ran
+                             everything                                      */
   int32_t device;         /* CUDA device ordinal                              */
   int32_t reuse_rays;     /* 1: for a range-independent medium (one table
                              column) march the rays once per propagate call

@@ -1744,19 +1744,19 @@ swkb_status configure(swkb_plan* p, const swkb_profile* prof, double k, const sw
   CK(cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, p->device));
   p->autotune = opt.autotune != 0 && !p->fc;
   p->reuse_rays = opt.reuse_rays != 0 && p->n_cols == 1;
-  // rays on a second stream unless they are reused (SWKB_OVERLAP=0: one
-  // stream, one ray-buffer set)
+  // rays and their brackets on streams of their own unless they are reused.
+  // SWKB_OVERLAP=0: one stream, one ray-buffer set; any other value: streams of their
+  // own; unset: FP64 plans only if the march is long.  FP64 kernels all wait for the
+  // same pipe, so beside the march the rest of a screen only takes its share of it, and
+  // march blocks that start among the others' spread unevenly over the SMs (per screen,
+  // own stream against one: 46 K rays 290 / 206 us, 68 K 706 / 535, 260 K 2078 / 2068,
+  // 518 K 3622 / 3714, 1.02 M 7478 / 7533; patch-wise 559 K 2926 / 2689).
   {
     const char* oe = getenv("SWKB_OVERLAP");
-    p->overlap = !(oe && oe[0] == '0') && !p->reuse_rays;
-    // FP64 kernels all wait for the same pipe, so beside the march the rest of
-    // a screen only takes its share of it, and march blocks that start among the
-    // others' spread unevenly over the SMs: one stream, unless the march is long
-    // (per screen, own stream against one: 46 K rays 290 / 206 us, 68 K 706 /
-    // 535, 260 K 2078 / 2068, 518 K 3622 / 3714, 1.02 M 7478 / 7533;
-    // patch-wise 559 K 2926 / 2689).
-    if (p->precision == SWKB_FP64 && (p->fc || (long long)p->Mr * p->NRT < 400000))
-      p->overlap = false;
+    p->overlap = !p->reuse_rays &&
+                 (oe ? oe[0] != '0'
+                     : p->precision != SWKB_FP64 ||
+                           (!p->fc && (long long)p->Mr * p->NRT >= 400000));
   }
   p->planes = opt.planes > 1 ? opt.planes : 0;
   if (p->planes && (p->planes > p->Nt || p->Nt % p->planes))
