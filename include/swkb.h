@@ -520,6 +520,14 @@ swkb_status swkb_hill_propagate(const swkb_hill_desc* desc, int32_t batch, const
                                 const double* x, double* u_out, double* lambda_out,
                                 int32_t on_device, void* cuda_stream);
 
+/*
+ * How the calling thread's last swkb_hill_propagate formed its fields: the
+ * matrix-vector products of the Chebyshev expansion of exp(i sqrt(A) x)
+ * (taken when no eigenvalues are asked for and it is the shorter way), or 0
+ * when it went through the eigen-decomposition.
+ */
+int32_t swkb_hill_last_products(void);
+
 const char* swkb_last_error(void);
 const char* swkb_status_string(swkb_status s);
 

@@ -1028,6 +1028,9 @@ swkb_status replay_back(Scratch& s, const RotLog& log, int P, int n_mat, int vec
   return SWKB_OK;
 }
 
+// matrix products of this thread's last swkb_hill_propagate (0: eigenvectors)
+thread_local int g_products = 0;
+
 // out[mat][r] <- exp(i sqrt(A[mat]) x_r) uh[mat] by the Chebyshev expansion, when
 // that is the shorter way (*done); else nothing has changed.  The quadrature of
 // A is exact on the basis (n_q >= 2 K), so the spectrum lies within
@@ -1126,6 +1129,7 @@ swkb_status chebyshev(Scratch& s, const HillDims& d, int batch, int n_x, const d
     std::swap(cur, prev);
   }
   HCK(cudaGetLastError());
+  g_products = terms - 1;
   *done = true;
   return SWKB_OK;
 }
@@ -1178,6 +1182,7 @@ swkb_status sym_eig(int batch, int n, const double* A_in, double* lam_out, doubl
 swkb_status hill_propagate(const swkb_hill_desc* d, int batch, const double* k,
                            const double* eps_in, const double* u0_in, int n_x, const double* x,
                            double* u_out, double* lam_out, int on_device, void* user_stream) {
+  g_products = 0;
   if (!d || !k || !eps_in || !u0_in || !x || !u_out)
     return hfail(SWKB_ERR_INVALID_ARG, "NULL argument");
   if (d->bc < SWKB_BC_PERIODIC || d->bc > SWKB_BC_DIRICHLET)
@@ -1330,5 +1335,7 @@ swkb_status swkb_hill_propagate(const swkb_hill_desc* desc, int32_t batch, const
     return hfail(SWKB_ERR_OOM, "host allocation failed");
   }
 }
+
+int32_t swkb_hill_last_products(void) { return g_products; }
 
 }  // extern "C"

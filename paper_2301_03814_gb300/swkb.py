@@ -39,8 +39,8 @@ EXPORTED = ("swkb_options_default", "swkb_plan_create", "swkb_plan_get_info", "s
             "swkb_plan_get_stats", "swkb_server_create", "swkb_submit",
             "swkb_poll", "swkb_cancel", "swkb_server_get_stats", "swkb_server_destroy",
             "swkb_last_error", "swkb_status_string", "swkb_modes_noalloc", "swkb_sym_eig",
-            "swkb_hill_propagate", "swkb_batch_options_default", "swkb_batch_create",
-            "swkb_batch_run", "swkb_batch_get_info", "swkb_batch_destroy")
+            "swkb_hill_propagate", "swkb_hill_last_products", "swkb_batch_options_default",
+            "swkb_batch_create", "swkb_batch_run", "swkb_batch_get_info", "swkb_batch_destroy")
 
 
 class SwkbError(RuntimeError):
@@ -159,6 +159,8 @@ def lib():
                                           c_void_p, c_int32, c_void_p, c_void_p, c_void_p,
                                           c_int32, c_void_p]
         L.swkb_hill_propagate.restype = c_int32
+        L.swkb_hill_last_products.argtypes = []
+        L.swkb_hill_last_products.restype = c_int32
         L.swkb_batch_options_default.argtypes = [POINTER(swkb_batch_options)]
         L.swkb_batch_options_default.restype = None
         L.swkb_batch_create.argtypes = [c_int32, POINTER(swkb_request), POINTER(swkb_batch_options),
@@ -386,6 +388,11 @@ def swkb_hill_propagate(desc: swkb_hill_desc, k, eps, u0, xs, eigenvalues=False)
                                     lam.ctypes.data_as(c_void_p) if eigenvalues else None, 0,
                                     None))
     return (out, lam) if eigenvalues else out
+
+
+def swkb_hill_last_products() -> int:
+    """Matrix products of this thread's last call (0: it went through the eigen-decomposition)."""
+    return int(lib().swkb_hill_last_products())
 
 
 def swkb_hill_propagate_device(desc: swkb_hill_desc, k, eps_ptr, u0_ptr, xs, out_ptr,
