@@ -62,3 +62,11 @@ def test_expansion_is_taken_and_agrees(bc, K, n_z, n_q, batch, xs):
 ])
 def test_eigenvectors_are_taken(bc, K, n_z, n_q, height, xs):
     assert _both(_inputs(bc, K, n_z, n_q, 1, height), xs) == 0
+
+
+@pytest.mark.parametrize("K,n_z,height,xs", [
+    (1501, 2048, 50.0, [185.0, 190.0, 195.0, 200.0, 204.0, 205.0]),      # 5750 terms: near 4 P
+    (3001, 4096, 100.0, [195.0, 200.0, 205.0, 210.0]),                   # about 2 P
+])
+def test_large_expansions_are_not_given_up_for_rounding(K, n_z, height, xs):
+    assert _both(_inputs(swkb.SWKB_BC_NEUMANN, K, n_z, 2 * K + 100, 1, height), xs) > 5000
