@@ -1558,19 +1558,16 @@ __global__ void __launch_bounds__(FFT1_THREADS) k_fft1(const FftArgs<T> p) {
   fft1_body<T, LD_PLAIN, COLS>(p, blockIdx.x, threadIdx.x, smem_raw);
 }
 
-// out_i = c_i f_i (mode coefficients of the planes between screens, one per
-// blockIdx.y), and its polar form when pol is given.
+// Polar form of c_i f_i (mode coefficients of the planes between screens, one per
+// blockIdx.y).
 template <typename T>
 __global__ void k_cscale(const typename C2<T>::type* __restrict__ c,
                          const typename C2<T>::type* __restrict__ f,
-                         typename C2<T>::type* __restrict__ out,
                          typename C2<T>::type* __restrict__ pol, int M) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= M) return;
   const long long o = (long long)blockIdx.y * M + i;
-  const typename C2<T>::type v = cmul<T>(c[i], f[o]);
-  if (out) out[o] = v;
-  if (pol) pol[o] = polar_turns<T>(v);
+  pol[o] = polar_turns<T>(cmul<T>(c[i], f[o]));
 }
 
 // w_{N2}^{idx} from the table of w_N (w_{N2} = w_N^{N1}).

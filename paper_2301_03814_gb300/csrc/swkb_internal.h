@@ -244,10 +244,9 @@ template <typename T> cudaError_t launch_bracket(const BracketArgs<T>& a, cudaSt
 template <typename T> cudaError_t launch_resum(const ResumArgs<T>& a, cudaStream_t s);
 template <typename T> cudaError_t launch_output(const typename C2<T>::type* u, int offset, int n,
                                                 double* out, cudaStream_t s);
-// n planes: f, out and pol hold M values per plane; out may be NULL
+// n planes: f and pol hold M values per plane
 template <typename T> cudaError_t launch_cscale(const typename C2<T>::type* c,
                                                 const typename C2<T>::type* f,
-                                                typename C2<T>::type* out,
                                                 typename C2<T>::type* pol, int M, int n,
                                                 cudaStream_t s);
 // k_bracket, k_resum, and k_reduce with k_output (no absorber; u is not written) of

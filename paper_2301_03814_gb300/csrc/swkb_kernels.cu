@@ -363,18 +363,17 @@ cudaError_t prepare_kernels(int resum_smem) {
 template <typename T>
 cudaError_t prepare_fft_kernels() {
   // k_fft1's dynamic shared memory is at most 5 E + N1 complex values at E = 128,
-  // N1 = 32 and 9 N1 at the largest N1 = 64, inside the default 48 KB limit; k_fft2
+  // N1 = 32 and 9 N1 (k_fft1_pairs: 10 N1) at the largest N1 = 64, inside 48 KB; k_fft2
   // uses static shared memory only
-  static_assert((5 * 128 + 32) * 16 <= 48 * 1024 && 9 * 64 * 16 <= 48 * 1024,
+  static_assert((5 * 128 + 32) * 16 <= 48 * 1024 && 10 * 64 * 16 <= 48 * 1024,
                 "k_fft1 staging exceeds 48 KB");
   return cudaSuccess;
 }
 
 template <typename T>
 cudaError_t launch_cscale(const typename C2<T>::type* c, const typename C2<T>::type* f,
-                          typename C2<T>::type* out, typename C2<T>::type* pol, int M, int n,
-                          cudaStream_t s) {
-  return launch_k(k_cscale<T>, dim3((M + 255) / 256, n), dim3(256), 0, s, c, f, out, pol, M);
+                          typename C2<T>::type* pol, int M, int n, cudaStream_t s) {
+  return launch_k(k_cscale<T>, dim3((M + 255) / 256, n), dim3(256), 0, s, c, f, pol, M);
 }
 
 template <typename T>
@@ -420,7 +419,7 @@ cudaError_t launch_output(const typename C2<T>::type* u, int offset, int n, doub
   template cudaError_t launch_resum<T>(const ResumArgs<T>&, cudaStream_t);                      \
   template cudaError_t launch_output<T>(const C2<T>::type*, int, int, double*, cudaStream_t);   \
   template cudaError_t launch_cscale<T>(const C2<T>::type*, const C2<T>::type*, C2<T>::type*,   \
-                                        C2<T>::type*, int, int, cudaStream_t);                  \
+                                        int, int, cudaStream_t);                                \
   template cudaError_t launch_bracket_planes<T>(const BracketArgs<T>&, const PlaneStrides&, int, \
                                                 cudaStream_t);                                  \
   template cudaError_t launch_resum_planes<T>(const ResumArgs<T>&, const PlaneStrides&, int,    \

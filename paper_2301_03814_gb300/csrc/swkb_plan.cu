@@ -130,7 +130,6 @@ struct swkb_plan {
   void* pl_d = nullptr;
   void* pl_ph = nullptr;
   void* pl_a = nullptr;
-  void* c_plane = nullptr;
   void* cpol_plane = nullptr;
   void* ephi_pl = nullptr;
   int* jlo = nullptr;
@@ -660,7 +659,7 @@ swkb_status build_device(swkb_plan* p, const swkb_profile* prof) {
   TRY(dev_alloc(p, &p->part, (size_t)p->alloc_groups * N * sizeof(V)));
   if (!p->fc) TRY(dev_alloc(p, &p->Y, (size_t)N * sizeof(V)));
   TRY(dev_alloc(p, &p->c, (size_t)M * sizeof(V)));
-  TRY(dev_alloc(p, &p->cpol, (size_t)M * sizeof(V)));
+  if (!p->fc) TRY(dev_alloc(p, &p->cpol, (size_t)M * sizeof(V)));
   const size_t rays = (size_t)p->NRT * p->Mr;
   TRY(dev_alloc(p, &p->rd, rays * sizeof(T)));
   TRY(dev_alloc(p, &p->rph, rays * sizeof(T)));
@@ -670,8 +669,7 @@ swkb_status build_device(swkb_plan* p, const swkb_profile* prof) {
     TRY(dev_alloc(p, &p->pl_d, pr * sizeof(T)));
     TRY(dev_alloc(p, &p->pl_ph, pr * sizeof(T)));
     TRY(dev_alloc(p, &p->pl_a, pr * sizeof(T)));
-    TRY(dev_alloc(p, &p->c_plane, (size_t)M * sizeof(V)));
-    TRY(dev_alloc(p, &p->cpol_plane, (size_t)M * sizeof(V)));
+    if (!p->fc) TRY(dev_alloc(p, &p->cpol_plane, (size_t)M * sizeof(V)));
     TRY(dev_alloc(p, &p->ephi_pl, (size_t)(p->planes - 1) * M * sizeof(V)));
   }
   const size_t jn = (size_t)(p->alloc_tiles + 1) * p->Mr;
@@ -817,14 +815,14 @@ BracketArgs<T> bracket_args(const swkb_plan* p, const T* d, int* jlo = nullptr,
 
 template <typename T>
 ResumArgs<T> resum_args(const swkb_plan* p, const T* d, const T* ph, const T* a,
-                        const typename C2<T>::type* c, const int* jlo = nullptr,
+                        const typename C2<T>::type* cpol, const int* jlo = nullptr,
                         const int* jlo_neg = nullptr) {
   using V = typename C2<T>::type;
   ResumArgs<T> ra;
   ra.d = d; ra.ph = ph; ra.a = a; ra.jlo = jlo ? jlo : p->jlo;
   ra.jlo_neg = jlo ? jlo_neg : p->jlo_neg;
   ra.trig = (const double2*)p->trig;
-  ra.cpol = (c == (const typename C2<T>::type*)p->c) ? (const V*)p->cpol : (const V*)p->cpol_plane;
+  ra.cpol = cpol;
   ra.M = p->M; ra.Mr = p->Mr; ra.sym = p->sym; ra.n_tiles_run = p->n_tiles_run; ra.NRT = p->NRT;
   ra.G = p->G; ra.R = p->R; ra.N = p->N; ra.TM = p->TM;
   ra.PW = p->PW; ra.n_tiles = p->n_tiles; ra.n_groups = p->n_groups;
@@ -946,7 +944,7 @@ swkb_status launch_screen(swkb_plan* p, int q, bool u_fresh) {
   if (march) TRY(timed(p, SWKB_KERNEL_BRACKET, 1, [&] { return launch_bracket<T>(b, s); }));
   p->rays_ready = true;
   const ResumArgs<T> ra = resum_args<T>(p, (const T*)p->rd, (const T*)p->rph, (const T*)p->ra,
-                                        (const V*)p->c);
+                                        (const V*)p->cpol);
   TRY(timed(p, SWKB_KERNEL_RESUM, 1, [&] { return launch_resum<T>(ra, s); }));
   p->stats.screens += 1;
   return SWKB_OK;
@@ -1076,7 +1074,7 @@ swkb_status overlapped_screen(swkb_plan* p, int q, int b, bool fresh) {
   // sum of screen q, once its rays and brackets are there (the ray stream goes
   // on with the next march)
   CK(cudaStreamWaitEvent(s, p->ev_brackets[b], 0));
-  const ResumArgs<T> rs = resum_args<T>(p, rd[b], rph[b], ra[b], (const V*)p->c, jlo[b],
+  const ResumArgs<T> rs = resum_args<T>(p, rd[b], rph[b], ra[b], (const V*)p->cpol, jlo[b],
                                         jneg[b]);
   TRY(timed(p, SWKB_KERNEL_RESUM, 1, [&] { return launch_resum<T>(rs, s); }));
   CK(cudaEventRecord(p->ev_free[b], s));
@@ -1267,10 +1265,10 @@ swkb_status enqueue_planes(swkb_plan* p, const double* u0, int q0, int n, int P,
       // c_n of plane j: the screen's c_n (carried over dx) times exp(i k (j/P - 1) dx P_bar_n)
       const V* fj = (const V*)p->ephi_pl + (size_t)(j - 1) * p->M;
       TRY(timed(p, SWKB_KERNEL_REDUCE, 1, [&] {
-        return launch_cscale<T>((const V*)p->c, fj, (V*)nullptr, (V*)p->cpol_plane, p->M, n_pl, s);
+        return launch_cscale<T>((const V*)p->c, fj, (V*)p->cpol_plane, p->M, n_pl, s);
       }));
       ResumArgs<T> ra = resum_args<T>(p, (const T*)p->pl_d + o, (const T*)p->pl_ph + o,
-                                      (const T*)p->pl_a + o, (const V*)p->c_plane, b.jlo,
+                                      (const T*)p->pl_a + o, (const V*)p->cpol_plane, b.jlo,
                                       b.jlo_neg);
       if (own) ra.part = (V*)p->pl_part;
       TRY(timed(p, SWKB_KERNEL_RESUM, 1,
@@ -1293,7 +1291,7 @@ swkb_status enqueue_planes(swkb_plan* p, const double* u0, int q0, int n, int P,
     const BracketArgs<T> b = bracket_args<T>(p, (const T*)p->rd);
     TRY(timed(p, SWKB_KERNEL_BRACKET, 1, [&] { return launch_bracket<T>(b, s); }));
     const ResumArgs<T> ra = resum_args<T>(p, (const T*)p->rd, (const T*)p->rph, (const T*)p->ra,
-                                          (const V*)p->c);
+                                          (const V*)p->cpol);
     TRY(timed(p, SWKB_KERNEL_RESUM, 1, [&] { return launch_resum<T>(ra, s); }));
     TRY(reduce((const T*)p->W));
     TRY(emit());
@@ -1820,12 +1818,12 @@ size_t device_bytes(const swkb_plan* p) {
   b += (size_t)p->N * V;                                            // twiddles
   if (p->absorber_frac > 0) b += (size_t)p->N * T;                  // absorber
   b += (size_t)p->N * V * (2 + (size_t)p->alloc_groups) + (size_t)p->M * V;  // u, Y, partials, c
-  b += (size_t)p->M * V;                                            // polar c
+  if (!p->fc) b += (size_t)p->M * V;                                // polar c
   if (T == 8) b += (size_t)TRIG_N * 16;                             // trig
   b += 3 * (size_t)p->NRT * p->Mr * T * (p->overlap ? 2 : 1);     // rays (one or two sets)
   if (p->planes > 1)                                                 // inner planes
     b += (size_t)(p->planes - 1) * (3 * (size_t)p->NRT * p->Mr * T + (size_t)p->M * V) +
-         2 * (size_t)p->M * V +
+         (p->fc ? 0 : (size_t)p->M * V) +
          (p->pl_batch > 1 ? p->pl_batch * plane_bytes(p) : 0);
   b += (size_t)(p->alloc_tiles + 1) * p->Mr * sizeof(int) * (p->sym ? 2 : 1) *
        (p->overlap ? 2 : 1);
@@ -2004,7 +2002,7 @@ swkb_status plan_parts(swkb_plan* p, PlanParts<T>* o) {
   o->march = march_args<T>(p, 0);
   o->bracket = bracket_args<T>(p, (const T*)p->rd);
   o->resum = resum_args<T>(p, (const T*)p->rd, (const T*)p->rph, (const T*)p->ra,
-                           (const V*)p->c);
+                           (const V*)p->cpol);
   return SWKB_OK;
 }
 template swkb_status plan_parts<float>(swkb_plan*, PlanParts<float>*);

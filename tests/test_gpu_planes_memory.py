@@ -64,3 +64,12 @@ def test_served_requests_take_no_plane_arrays():
         assert np.array_equal(out, swkb.Plan(pb, swkb.SWKB_MIXED).propagate())
     finally:
         srv.close()
+
+
+@pytest.mark.parametrize("precision", [swkb.SWKB_FP64, swkb.SWKB_MIXED])
+def test_an_inner_plane_holds_its_rays_and_coefficients(precision):
+    # three arrays of rays, the range-phase factors and the coefficients in polar form; nothing else
+    pb = _duct()
+    i, j = (swkb.Plan(pb, precision, planes=n).info for n in (0, 2))
+    size = 8 if precision == swkb.SWKB_FP64 else 4
+    assert j.device_bytes - i.device_bytes == (3 * i.march_modes * i.n_rays_total + 4 * i.n_modes) * size
