@@ -66,7 +66,7 @@ size_t fft1_smem_bytes(int N1, int cols) {
 
 namespace {
 // cos(2 pi k / 64) as the nearest double and what is missing from it
-__device__ const double kRoot64[17][2] = {
+__constant__ double kRoot64[17][2] = {
     {1.0, 0.0}, {0.9951847266721969, -4.248691367830441e-17},
     {0.9807852804032304, 1.8546939997825006e-17}, {0.9569403357322088, 4.05538698618757e-17},
     {0.9238795325112867, 1.7645047084336677e-17}, {0.881921264348355, -1.9843248405890562e-17},
@@ -82,17 +82,19 @@ __device__ __forceinline__ void root64(int k, double2& w, double2& lo) {
   const int q = k >> 4 & 3, m = k & 15;
   const double* c = kRoot64[q & 1 ? 16 - m : m];   // |cos|, |sin| of the angle
   const double* s = kRoot64[q & 1 ? m : 16 - m];
-  const double sc = q == 1 || q == 2 ? -1.0 : 1.0, ss = q < 2 ? -1.0 : 1.0;
-  w = make_double2(sc * c[0], ss * s[0]);
-  lo = make_double2(sc * c[1], ss * s[1]);
+  const bool nc = q == 1 || q == 2, ns = q < 2;
+  w = make_double2(nc ? -c[0] : c[0], ns ? -s[0] : s[0]);
+  lo = make_double2(nc ? -c[1] : c[1], ns ? -s[1] : s[1]);
 }
 
 // Pass 1 in FP64 on a field read directly, rounding no more than rows of 2048 points
-// summed directly would: the first radix-4 step of the columns (exact factors) in
-// shared memory, then sums of N1 / 4 terms in two chains, with what the roots of unity
+// summed directly would: the first radix-4 step of the columns (exact factors) as
+// they are loaded, then sums of N1 / 4 terms in two chains, with what the roots of unity
 // lack added back.  4096 to 65536 points, error 0.89 to 0.99 of the direct sums', against
-// 1.05 to 1.09 with sums of N1 / 2 terms and rounded roots (k_fft1).  COLS columns per
-// CTA, N1 >= 2.
+// 1.05 to 1.09 with sums of N1 / 2 terms and rounded roots (k_fft1).  Latency bounds it,
+// so every load is issued before the first wait and the roots come from constant memory
+// (both passes back to back, 2048 points 12.4 -> 11.4 us, 4096 points, 201 modes 12.4 ->
+// 11.4; k_fft1 10.4; 65536 points 80.0 either way).  COLS columns per CTA, N1 >= 2.
 template <int COLS>
 __global__ void __launch_bounds__(FFT1_THREADS) k_fft1_pairs(const FftArgs<double> p) {
   using V = double2;
@@ -100,22 +102,30 @@ __global__ void __launch_bounds__(FFT1_THREADS) k_fft1_pairs(const FftArgs<doubl
   const int N1 = p.N1, E = N1 * COLS, tid = threadIdx.x, c0 = blockIdx.x * COLS;
   V* tile = reinterpret_cast<V*>(smem_raw);          // [N1][COLS]
   V* w1 = tile + E;                                  // [N1] roots, then what they lack
-  for (int k = tid; k < N1; k += FFT1_THREADS) root64(k * (64 / N1), w1[k], w1[N1 + k]);
-  for (int e = tid; e < E; e += FFT1_THREADS) tile[e] = p.u[(long long)(e / COLS) * p.N2 + c0 + e % COLS];
-  __syncthreads();
+  const auto twiddle = [&](int e) {
+    return p.tw[(long long)(c0 + e % COLS) * (e / COLS) << p.tw_shift];
+  };
   // residue q of k1 modulo radix: tile rows q L .. q L + L - 1 hold its inputs n1 = 0 .. L - 1
-  const int radix = N1 < 4 ? 2 : 4, L = N1 / radix;
-  if (tid < L * COLS) {   // at most 16 x 8
+  const int radix = N1 < 4 ? 2 : 4, L = N1 / radix, o = L * COLS;   // o <= 16 x 8
+  V x[4], w2;   // every load before the first wait
+  if (tid < o) {
+    const V* u = p.u + (long long)(tid / COLS) * p.N2 + c0 + tid % COLS;
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (j < radix) x[j] = u[(long long)j * L * p.N2];
+  }
+  if (tid < E) w2 = twiddle(tid);
+  for (int k = tid; k < N1; k += FFT1_THREADS) root64(k * (64 / N1), w1[k], w1[N1 + k]);
+  if (tid < o) {
     V* t = tile + tid;
-    const int o = L * COLS;
-    const V a = t[0], b = t[o];
     if (radix == 2) {
-      t[0] = make_double2(a.x + b.x, a.y + b.y);
-      t[o] = make_double2(a.x - b.x, a.y - b.y);
+      t[0] = make_double2(x[0].x + x[1].x, x[0].y + x[1].y);
+      t[o] = make_double2(x[0].x - x[1].x, x[0].y - x[1].y);
     } else {
-      const V c = t[2 * o], d = t[3 * o];
-      const V s0 = make_double2(a.x + c.x, a.y + c.y), s1 = make_double2(b.x + d.x, b.y + d.y);
-      const V d0 = make_double2(a.x - c.x, a.y - c.y), d1 = make_double2(b.x - d.x, b.y - d.y);
+      const V s0 = make_double2(x[0].x + x[2].x, x[0].y + x[2].y);
+      const V s1 = make_double2(x[1].x + x[3].x, x[1].y + x[3].y);
+      const V d0 = make_double2(x[0].x - x[2].x, x[0].y - x[2].y);
+      const V d1 = make_double2(x[1].x - x[3].x, x[1].y - x[3].y);
       t[0] = make_double2(s0.x + s1.x, s0.y + s1.y);
       t[o] = make_double2(d0.x + d1.y, d0.y - d1.x);       // d0 - i d1
       t[2 * o] = make_double2(s0.x - s1.x, s0.y - s1.y);
@@ -125,7 +135,7 @@ __global__ void __launch_bounds__(FFT1_THREADS) k_fft1_pairs(const FftArgs<doubl
   __syncthreads();
   for (int e = tid; e < E; e += FFT1_THREADS) {
     const int c = e % COLS, k1 = e / COLS, n2 = c0 + c;
-    const V w2 = p.tw[(long long)n2 * k1 << p.tw_shift];
+    if (e != tid) w2 = twiddle(e);
     const V* t = tile + (k1 & (radix - 1)) * L * COLS + c;
     const auto mac = [&](V& sum, int n1) {
       const int i = (n1 * k1) & (N1 - 1);
