@@ -1554,17 +1554,18 @@ Tiling default_tiling(const swkb_plan* p) {
   else t.PW = p->R >= 8 ? 8 : (p->R >= 2 ? 4 : 2);
   while (32 * t.PW > (p->sym ? p->N / 2 : p->N) || (p->fc && p->N % (32 * t.PW))) t.PW /= 2;
   // Mode groups: up to 20 CTAs per SM (patch-wise, where a group sums longer,
-  // 40), so that the last wave is short, while a group keeps 32 modes
+  // 60), so that the last wave is short, while a group keeps 32 modes
   // (patch-wise 16; a warp looks its modes up 32 at a time, and the next screen
-  // adds up one partial per group); at least 4 CTAs per SM where the modes allow it, at 4 per group.  Sum
-  // plus DFT per screen, by groups: 16384 points, 977 modes 50.9 us (15), 48.5
-  // (29), 50.1 (43); 131072 points, 1395 modes 276 (4), 252 (13); 4096 points,
-  // 401 modes 25.0 (19), 22.5 (37), 24.8 (51); 512 points, 65 modes 18.1 (17),
-  // 22.0 (65).  Patch-wise sums: 131072 points, 545 modes 261 us (2), 234 (4), 231
-  // (6); 8192 points 24.6 (10), 22.5 (29), 24.5 (54).
+  // adds up one partial per group); at least 4 CTAs per SM where the modes allow
+  // it, at 4 per group.  Sum plus DFT per screen, by groups: 16384 points, 977 modes
+  // 50.9 us (15), 48.5 (29), 50.1 (43); 131072 points, 1395 modes 276 (4), 252 (13);
+  // 4096 points, 401 modes 25.0 (19), 22.5 (37), 24.8 (51); 512 points, 65 modes 18.1
+  // (17), 22.0 (65).  Patch-wise sums: 131072 points, 545 modes 225 us (6), 226 (9), 230
+  // (15), and with 6 groups, 23 modes per warp, FP32 fields are 2 to 4 % further from
+  // FP64 ones after a screen than with 9; 8192 points 24.6 (10), 22.5 (29), 24.5 (54).
   const int tiles = p->sym ? p->N / (64 * t.PW) + 1 : p->N / (32 * t.PW);
   const auto groups_at = [&](int c) { return (p->sms * c + tiles - 1) / tiles; };
-  const int most = p->fc ? std::min(groups_at(40), p->M / 16) : std::min(groups_at(20), p->M / 32);
+  const int most = p->fc ? std::min(groups_at(60), p->M / 16) : std::min(groups_at(20), p->M / 32);
   const int g = std::min(std::max(most, groups_at(4)), std::max(1, p->M / 4));
   t.ctas_per_sm = std::max(1, (int)((long long)g * tiles / p->sms));
   // N1 ~ sqrt(M): pass 1 costs N N1, pass 2 M N2
