@@ -1592,12 +1592,14 @@ void apply_tiling(swkb_plan* p, const Tiling& t) {
   p->n_tiles = p->N / p->TM;
   p->n_tiles_run = p->sym ? p->n_tiles / 2 + 1 : p->n_tiles;
   // rays per tile window: up to 4x compression.  Periodic tiles of 512 points take 4
-  // rays more, so that they hold what two tiles of 256 points would.  Patch-wise plans
+  // rays more where they are the default (R >= 32), so that they hold what two tiles of
+  // 256 points would; at R = 16 the 1 KB more would take the batch kernel's three CTAs
+  // per SM past 196 KB of shared memory and halve its L1.  Patch-wise plans
   // have no slack, which keeps six FP32 sums of 4 warps within an SM's shared memory
   // (but at least one interval between two landings): a window may hold more rays, up
   // to 4x on the tile or its pair of tiles, and is then summed in parts.
   const auto fc_window = [&](int points) { return std::max(4 * points / p->R, 2) + 4; };
-  p->wcap = p->fc ? fc_window(p->TM) : 4 * p->TM / p->R + (p->TM > 256 ? 12 : 8);
+  p->wcap = p->fc ? fc_window(p->TM) : 4 * p->TM / p->R + (p->TM > 256 && p->R >= 32 ? 12 : 8);
   p->fc_wlim = fc_window(p->fc_lim_pair ? 2 * p->TM : p->TM);
   p->ctas_per_sm = t.ctas_per_sm;
   const int target_ctas = p->sms * t.ctas_per_sm;
