@@ -60,8 +60,10 @@ __device__ __forceinline__ void vb_sync(int sub) {
   }
 }
 
-// sin / cos of 2 pi t for |t| <= 1/2 on the special-function unit (absolute
-// error ~2^-21 on [-pi, pi]).
+// sin / cos of 2 pi t on the special-function unit: absolute error ~2^-21 for
+// |t| <= 1/2.  The sums pass t within a turn and a half plus (q - PW / 2) n / N, so up to
+// four turns more for the steepest modes of 16-point runs, whose argument's rounding (up to
+// 1e-6) adds to it.
 __device__ __forceinline__ void sincos_turns(float t, float* s, float* c) {
   __sincosf(6.28318530717958647692f * t, s, c);
 }
@@ -296,7 +298,7 @@ __device__ __forceinline__ void march64_body(const MarchArgs<double>& p, int blk
 
 // Bound by the FP64 pipe (2 operations per SM and clock, ~87 % busy): ~49 FP64
 // operations per stage (12 of them the quintic, 8 the two special functions).
-// On the 16384-point duct (489 modes x 2086 rays, 16 RK4 steps) 6.4 ms, against
+// On the 16384-point duct (489 modes x 2086 rays, 16 RK4 steps) 6.3 ms, against
 // 9.1 ms with the unscaled system, library rsqrt and division, and FP64
 // comparisons and conversions in the lookup (~66).  CTAs of 64 threads spread
 // small plans evenly: 65 modes x 704 rays on 152 SMs take 0.18 ms, against
@@ -612,12 +614,13 @@ __device__ __forceinline__ void march_x2_body(const MarchArgs<float>& p, int blk
   if (st) atomicOr(p.status, st);
 }
 
-// Bound by the FMA pipe: ~72 of its cycles per ray-pair stage (14 FFMA2, 8
-// FMUL2, 6 FADD2 at two cycles each, 12 FFMA of the medium, 2 IMAD), busy 64 %
-// of the time that CTAs are resident; 61 instructions in all.  On the
-// 16384-point duct (489 modes x 2086 rays, 16 RK4 steps) 102 us, against 121
-// with the unscaled system (35 packed operations, 80 instructions); 326
-// against 485 us on a range-dependent table (698 modes x 4118 rays).
+// Bound by the FMA pipe: ~71 of its cycles per ray-pair stage (13 FFMA2, 8
+// FMUL2, 7 FADD2 at two cycles each, 12 FFMA of the medium, 2 IMAD), busy 64 %
+// of the time that CTAs are resident; 58 instructions in all.  On the
+// 16384-point duct (489 modes x 2086 rays, 16 RK4 steps) 103 us, against 121
+// with the unscaled system (35 packed operations, 80 instructions); 347
+// against 485 us on a range-dependent table (698 modes x 4118 rays; 331 with the
+// columns' differences stored, which doubles the table).
 // 6 CTAs of 128 threads per SM (80 registers): 102 us; 3 of 256: 104; 4 of
 // 256 (64 registers, spills): 112; 2 of 256: 107; all-scalar arithmetic: 110.  With
 // inner planes 5 per SM (96 registers; 80 spill): 8192 points, 3 screens of 4 planes 447
@@ -1257,9 +1260,9 @@ __device__ __forceinline__ void resum_body(const ResumArgs<double>& p, int blk, 
 // tile), 15 per point and lane and ~150 for the window, the rows and the search
 // (477 with scalar cubics, per-mode bracket lookups and library divisions).
 // 16384-point duct (977 modes x 16640 points) 34 us per sum against 41,
-// 131072-point duct (1395 modes, R = 64) 214 against 372.  7 CTAs per SM (72
-// registers: keeps the one-mode-ahead window), 5 for runs of 16 points (213 us;
-// 230 at 72 registers).  FP64, bound by its pipe: 1.05 ms on the 16384-point
+// 131072-point duct (1395 modes, R = 64) 221 against 372.  7 CTAs per SM (72
+// registers: keeps the one-mode-ahead window), 5 for runs of 16 points (213 us,
+// 230 at 72 registers, in an earlier build).  FP64, bound by its pipe: 1.04 ms on the 16384-point
 // duct with 29 mode groups (1.78 with sincospi, library divisions and a complex
 // coefficient per term; 25 FP64 operations per term instead of ~46).
 template <typename T, int PW>

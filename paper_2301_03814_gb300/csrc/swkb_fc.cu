@@ -466,10 +466,10 @@ __device__ __noinline__ void fc_resum_split(const FcResumArgs<T>& p, unsigned ch
 // sum: brackets of 32 modes looked up at once, the next mode's first rays loaded
 // one mode ahead) and the CTA adds the warps' sums in a fixed order.
 // Bound by instruction issue and by the warps its shared memory leaves (96 bytes
-// per ray of a window): 131072-point lens, 545 modes, R = 8, 221 us per sum with
+// per ray of a window): 131072-point lens, 545 modes, R = 8, 225 us per sum with
 // 128-point tiles (256-point ones 306; 261 before, with per-mode bracket
 // lookups, scalar amplitude cubics and library divisions).  FP64 8192-point lens
-// 410 us (723).  FP32 7 CTAs per SM (72 registers); 6: 223 us, 8: 289.
+// 415 us (723).  FP32 7 CTAs per SM (72 registers); 6: 223 us, 8: 289.
 template <typename T, int PW>
 __global__ void __launch_bounds__(FC_WARPS * 32, sizeof(T) == 4 ? 7 : 1)
     k_fc_resum(const FcResumArgs<T> p) {

@@ -22,7 +22,7 @@
 //
 // Without eigenvalues to return, step 3 and the advance are replaced, where that
 // is shorter, by the Chebyshev expansion of exp(i sqrt(A) x) applied to the
-// projections (see chebyshev below): 641 rows at 1 and 2 km 5.3 ms instead of 60.
+// projections (see chebyshev below): 641 rows at 1 and 2 km 5.3 ms instead of 58.
 //
 // FP64 throughput is the scarce resource on this GPU (two FMAs per SM and
 // clock), so the rotation tangent is found in FP32 and only c, s and the
@@ -1037,7 +1037,7 @@ thread_local int g_products = 0;
 // [k^2 min eps - kappa_K^2, k^2 max eps]; without evanescent modes the expansion
 // of exp(i x sqrt(lambda)) there needs about x half / (2 sqrt(lambda_min))
 // terms, each one matrix-vector product of 4 to 9 us, against the ~7 P rounds of
-// the Jacobi iteration.  Surface duct, 641 rows, 2 km: 526 terms, 59.9 -> 5.3 ms
+// the Jacobi iteration.  Surface duct, 641 rows, 2 km: 526 terms, 58 -> 5.3 ms
 // for the whole call.  Both ways cost the same at 4.1 P (402 rows), 4.7 P (206), 6.1 P
 // (102) and above 7.8 P (62 and 642) terms, so 4 P is the most taken here.
 // uh and A are overwritten when done.

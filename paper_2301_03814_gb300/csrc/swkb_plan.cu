@@ -1544,7 +1544,7 @@ Tiling default_tiling(const swkb_plan* p) {
   Tiling t;
   // Runs of about half a ray spacing: the tile's rows of intervals (one lane
   // builds one) then number 16 to 20, and a run meets one interval's end at
-  // most once.  FP32, R = 64 (131072 points, 1395 modes): 214 us per sum with
+  // most once.  FP32, R = 64 (131072 points, 1395 modes): 221 us per sum with
   // runs of 16 points, 280 with 8; R = 16 (16384 points): 35 with 16, 34 with 8.
   // Patch-wise windows (96 bytes of shared memory a ray) halve them: R = 8
   // (131072 points, 545 modes) 231 us with runs of 4, 336 with 8; R = 2 (8192
