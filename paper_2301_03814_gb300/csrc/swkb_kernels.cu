@@ -65,8 +65,13 @@ size_t fft1_smem_bytes(int N1, int cols) {
 }
 
 namespace {
-// cos(2 pi k / 64) as the nearest double and what is missing from it
-__constant__ double kRoot64[17][2] = {
+// cos(2 pi k / 64) as the nearest double and what is missing from it.  A kernel argument:
+// in constant memory it would be a bank more for every kernel of the library (0.3 us a
+// launch: 40 screens on reused rays 488 -> 503 us).
+struct Roots64 {
+  double c[17][2];
+};
+constexpr Roots64 kRoots64 = {{
     {1.0, 0.0}, {0.9951847266721969, -4.248691367830441e-17},
     {0.9807852804032304, 1.8546939997825006e-17}, {0.9569403357322088, 4.05538698618757e-17},
     {0.9238795325112867, 1.7645047084336677e-17}, {0.881921264348355, -1.9843248405890562e-17},
@@ -75,13 +80,13 @@ __constant__ double kRoot64[17][2] = {
     {0.5555702330196022, 4.709410940561677e-17}, {0.47139673682599764, 6.516678136069013e-18},
     {0.3826834323650898, -1.0050772696461588e-17}, {0.2902846772544624, -1.892797870777425e-17},
     {0.19509032201612828, -7.991079068461731e-18}, {0.0980171403295606, -1.634582362244256e-18},
-    {0.0, 0.0}};
+    {0.0, 0.0}}};
 
 // exp(-2 pi i k / 64) and what is missing from it
-__device__ __forceinline__ void root64(int k, double2& w, double2& lo) {
+__device__ __forceinline__ void root64(const Roots64& r, int k, double2& w, double2& lo) {
   const int q = k >> 4 & 3, m = k & 15;
-  const double* c = kRoot64[q & 1 ? 16 - m : m];   // |cos|, |sin| of the angle
-  const double* s = kRoot64[q & 1 ? m : 16 - m];
+  const double* c = r.c[q & 1 ? 16 - m : m];   // |cos|, |sin| of the angle
+  const double* s = r.c[q & 1 ? m : 16 - m];
   const bool nc = q == 1 || q == 2, ns = q < 2;
   w = make_double2(nc ? -c[0] : c[0], ns ? -s[0] : s[0]);
   lo = make_double2(nc ? -c[1] : c[1], ns ? -s[1] : s[1]);
@@ -92,11 +97,12 @@ __device__ __forceinline__ void root64(int k, double2& w, double2& lo) {
 // they are loaded, then sums of N1 / 4 terms in two chains, with what the roots of unity
 // lack added back.  4096 to 65536 points, error 0.89 to 0.99 of the direct sums', against
 // 1.05 to 1.09 with sums of N1 / 2 terms and rounded roots (k_fft1).  Latency bounds it,
-// so every load is issued before the first wait and the roots come from constant memory
-// (both passes back to back, 2048 points 12.4 -> 11.4 us, 4096 points, 201 modes 12.4 ->
-// 11.4; k_fft1 10.4; 65536 points 80.0 either way).  COLS columns per CTA, N1 >= 2.
+// so every load is issued before the first wait and the roots are an argument (both
+// passes back to back, 4096 points, 201 modes 12.4 -> 10.4 us, 489 modes 12.4; k_fft1 10.4
+// and 11.4; 65536 points, 8001 modes 80.0 either way).  COLS columns per CTA, N1 >= 2.
 template <int COLS>
-__global__ void __launch_bounds__(FFT1_THREADS) k_fft1_pairs(const FftArgs<double> p) {
+__global__ void __launch_bounds__(FFT1_THREADS)
+    k_fft1_pairs(const FftArgs<double> p, const __grid_constant__ Roots64 roots) {
   using V = double2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int N1 = p.N1, E = N1 * COLS, tid = threadIdx.x, c0 = blockIdx.x * COLS;
@@ -115,7 +121,7 @@ __global__ void __launch_bounds__(FFT1_THREADS) k_fft1_pairs(const FftArgs<doubl
       if (j < radix) x[j] = u[(long long)j * L * p.N2];
   }
   if (tid < E) w2 = twiddle(tid);
-  for (int k = tid; k < N1; k += FFT1_THREADS) root64(k * (64 / N1), w1[k], w1[N1 + k]);
+  for (int k = tid; k < N1; k += FFT1_THREADS) root64(roots, k * (64 / N1), w1[k], w1[N1 + k]);
   if (tid < o) {
     V* t = tile + tid;
     if (radix == 2) {
@@ -224,7 +230,7 @@ cudaError_t launch_fft_pairs(const FftArgs<double>& a, cudaStream_t s) {
     const int cols = fft1_cols(a.N2);
     const cudaError_t e =
         launch_k(cols == 4 ? k_fft1_pairs<4> : k_fft1_pairs<8>, dim3(a.N2 / cols),
-                 dim3(FFT1_THREADS), (size_t)(cols + 2) * a.N1 * sizeof(double2), s, a);
+                 dim3(FFT1_THREADS), (size_t)(cols + 2) * a.N1 * sizeof(double2), s, a, kRoots64);
     if (e != cudaSuccess) return e;
   }
   return launch_k(k_fft2_pair, dim3(fft2_pairs(a.N1, a.n_max)), dim3(FFT2_THREADS), 0, s, a);
