@@ -133,7 +133,9 @@ typedef struct {
   int32_t planes;         /* P > 1 (dividing rk4_steps): allocate ray buffers
                              for P - 1 planes inside each screen, enabling
                              swkb_propagate_planes with up to P planes per
-                             screen (0 or 1 = none)                           */
+                             screen (0 or 1 = none).  Where device memory is
+                             to spare, up to 256 MB more let several planes
+                             be summed at once                                */
   /* Fixed launch shapes, e.g. those an autotuned plan reported in
      swkb_plan_info.  All three > 0 replaces the default and the autotuned
      shapes (autotune is then skipped): tile_points in {64, 128, 256, 512}

@@ -424,7 +424,9 @@ __device__ __noinline__ void fc_resum_split(const FcResumArgs<T>& p, unsigned ch
     };
     const int jb = bracket(tile) - 1, W = fc_window(p, jb + 1, bracket(tile + 1));
     if (W <= wcap) continue;
-    if ((p.lim_pair ? fc_window(p, bracket(tile & ~1), bracket((tile | 1) + 1)) : W) > p.wlim) {
+    // (its own window too: beside an inconsistent bracket the pair's may be empty)
+    if (W > p.wlim ||
+        (p.lim_pair && fc_window(p, bracket(tile & ~1), bracket((tile | 1) + 1)) > p.wlim)) {
       st |= ST_CAUSTIC;
       continue;
     }
