@@ -10,9 +10,9 @@
 // file-scope device arrays of a fixed size that every GPU loading this library
 // holds until the process exits (3 MB per device).
 //
-// The arithmetic is the library's FP64 pruned two-pass DFT (k_fft1, then bins in
-// pairs, k_fft2_pair).  The twiddles are those of the largest length, filled once:
-// shorter ones are strided in it.  4096 points, 489 modes: 30.7 -> 11.3 us per call
+// The arithmetic is an FP64 pruned two-pass DFT (k_fft1_pairs, then bins in pairs,
+// k_fft2_pair).  The twiddles are those of the largest length, filled once:
+// shorter ones are strided in it.  4096 points, 489 modes: 30.7 -> 12.3 us per call
 // (before, each call filled a table and split the points into two rows only).
 
 #include <mutex>
@@ -86,10 +86,11 @@ swkb_status setup(int dev, DeviceScratch** out) {
 }
 
 // N1 of n_fft = N1 N2: the smallest estimate of the FP64 instructions of the
-// busiest of 152 SMs.  A pass-1 CTA of c columns forms c N1 sums of N1 / 2 terms,
-// a pass-2 CTA a pair of sums of N2 terms, 4 instructions per term; the second
+// busiest of 152 SMs.  A pass-1 CTA of c columns forms c N1 sums of N1 / 4 terms of 8
+// instructions, a pass-2 CTA a pair of sums of N2 terms of 4; the second
 // kernel costs what an SM issues in 3 us.  Measured with about 11 us of launch and
-// event overhead, one kernel / the best split / this rule:
+// event overhead (pass 1 as N1 / 2 terms of 4 then, up to 1 us less), one kernel / the
+// best split / this rule:
 //   1024 points,   101 modes    14.8 / 14.8 / 14.9 us
 //   4096 points,   489 modes    23.6 / 18.5 / 18.0
 //   16384 points, 8001 modes     475 / 57.9 / 57.7
