@@ -504,6 +504,19 @@ __device__ __forceinline__ Ray2 rhs2(const MarchArgs<float>& p, int l, f2 u2, f2
   return d;
 }
 
+// Amplitude factor sqrt(P0 / (P1 Z)) of P0^2, P1^2 and Z, rounded once: the approximate
+// roots and the quotient lose 5e-8 on average where all three are near 1, the same
+// way for every ray, and the field that much of its length at each screen.  One
+// Newton step on a^4 P1^2 Z^2 = P0^2, whose left side is formed in two parts.
+__device__ __forceinline__ float amplitude(float P0sq, float P1sq, float Z) {
+  const float a = sqrtf(sqrtf(P0sq) * rsqrtf(P1sq) / Z);
+  const float h = a * a, hl = fmaf(a, a, -h);
+  const float u = h * Z, ul = fmaf(hl, Z, fmaf(h, Z, -u));
+  const float w = u * u, wl = fmaf(2.f * u, ul, fmaf(u, u, -w));
+  const float q = w * P1sq, ql = fmaf(wl, P1sq, fmaf(w, P1sq, -q));
+  return fmaf(0.25f * a * rcp_approx(P0sq), (P0sq - q) - ql, a);
+}
+
 // Thread t marches rays q and q + NH of mode r, t = q Mr + r (NH = ceil(NRT / 2)):
 // a warp's lanes are consecutive modes at one launch height (their table
 // reads stay within a few intervals) and no lane idles at the end of a row.
@@ -534,8 +547,6 @@ __device__ __forceinline__ void march_x2_body(const MarchArgs<float>& p, int blk
   sp2(add2(pb2v, e0), P0a, P0b);
   if (!(P0a > 0.f)) { st |= ST_TURNING; P0a = pb2; }
   if (!(P0b > 0.f)) { st |= ST_TURNING; P0b = pb2; }
-  P0a = sqrtf(P0a);
-  P0b = sqrtf(P0b);
   Ray2 y{zero, zero, zero, bc2(-1.f), zero};
   // RK4 weights 1/2, 1, 1/6 times the factors of the scaled system
   const float s2 = p.s2, s6 = p.s6;
@@ -568,11 +579,11 @@ __device__ __forceinline__ void march_x2_body(const MarchArgs<float>& p, int blk
     const float Za = Na < 0.f ? -Na : 1.f, Zb = Nb < 0.f ? -Nb : 1.f;
     od[oa] = wa * w_out;
     oph[oa] = rha * p.ph_out;
-    oam[oa] = sqrtf(P0a * rsqrtf(P1a) / Za);
+    oam[oa] = amplitude(P0a, P1a, Za);
     if (has_b) {
       od[ob] = wb * w_out;
       oph[ob] = rhb * p.ph_out;
-      oam[ob] = sqrtf(P0b * rsqrtf(P1b) / Zb);
+      oam[ob] = amplitude(P0b, P1b, Zb);
     }
   };
   // A step's slopes are summed (k1 + 2 k2 + 2 k3 + k4) before they join the state, so
@@ -1441,11 +1452,17 @@ __device__ __forceinline__ typename C2<T>::type cmul(typename C2<T>::type a,
 }
 
 // (|v|, arg(v) / 2 pi) of a complex value, the angle in turns in [-1/2, 1/2].
+// FP32: |v| makes up for what sincos_turns falls short of (its square by 1.47e-7),
+// which a field would lose at each screen whatever its shape; the root is the rounded
+// one, since the approximate one loses 1.5e-8 more.
 template <typename T>
 __device__ __forceinline__ typename C2<T>::type polar_turns(typename C2<T>::type v) {
   typename C2<T>::type r;
   if constexpr (sizeof(T) == 8) r.x = hypot(v.x, v.y);
-  else r.x = sqrt(v.x * v.x + v.y * v.y);
+  else {
+    const float q = fmaf(v.x, v.x, v.y * v.y);
+    r.x = __fsqrt_rn(fmaf(q, 1.47e-7f, q));
+  }
   r.y = atan2(v.y, v.x) * T(0.15915494309189533577);
   return r;
 }
